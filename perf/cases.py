@@ -285,3 +285,71 @@ def tolerance(case):
     # A block's activations pass through four projections and its gradients through four more, each rounded to bf16 (seen:
     # 5.4e-3 and 2.9e-2).
     return {"rel": 2e-2, "max": 1e-1}
+
+
+# The same results in 64 bits, by plain torch.  Only the inputs come from prepare().
+
+def _weight(p):
+    """W [N, K] = scale * (q - zero): 32 consecutive codes of a column are a little-endian bit stream in `bits` words."""
+    b, K, N = p.desc.bits, p.K, p.N
+    words = (p.Q.long() & 0xFFFFFFFF).reshape(K // 32, b, N)
+    codes = torch.empty((K // 32, 32, N), dtype=torch.int64, device=words.device)
+    for i in range(32):
+        w, off = divmod(i * b, 32)
+        q = words[:, w] >> off
+        if off + b > 32:
+            q = q | (words[:, w + 1] << (32 - off))
+        codes[:, i] = q & ((1 << b) - 1)
+    groups = p.scales.shape[0]
+    W = p.scales.double()[:, None] * (codes.reshape(groups, K // groups, N).double() - p.zeros.double()[:, None])
+    return W.reshape(K, N).t()
+
+
+def _exact_forward(p, X):
+    W, s, A, B = _weight(p), p.desc.alpha / p.desc.r if p.desc.r else 0.0, p.A_user if hasattr(p, "A_user") else p.A, p.B
+    A, B = A.double(), B.double()
+    if hasattr(p, "inverse"):
+        W = W[:, p.inverse.long()]
+    XD = X * p.mask.double() * p.keep_scale if hasattr(p, "mask") else X
+    H = XD @ A.t()
+    return X @ W.t() + s * (H @ B.t()), (W, s, A, B, XD, H)
+
+
+def _exact_backward(p, dY, kept):
+    W, s, A, B, XD, H = kept
+    G = dY @ B
+    low = s * (G @ A)
+    if hasattr(p, "mask"):
+        low = low * p.mask.double() * p.keep_scale
+    return dY @ W + low, s * (G.t() @ XD), s * (dY.t() @ H)
+
+
+def exact(case, seed):
+    kind = case["kind"]
+    state = prepare(case, seed)
+    if kind == "quantize":
+        return None                       # whole numbers and bytes: compared bit by bit
+    if kind == "loss":
+        logp, logq = (torch.log_softmax(state[k].double(), dim=1) for k in ("student", "teacher"))
+        p, labels = logp.exp(), state["labels"].long()[:, None]
+        kl = (p * (logp - logq)).sum(dim=1)
+        grad = p * (logp - logq - kl[:, None]) + 0.5 * p
+        grad.scatter_add_(1, labels, torch.full_like(labels, -0.5, dtype=torch.float64))
+        return kl - 0.5 * logp.gather(1, labels)[:, 0], grad * state["grad_scale"]
+    if kind == "step":
+        out = []
+        for i, p in enumerate(state["projections"]):
+            Y, kept = _exact_forward(p, state["X"][i].double())
+            out.append((Y, *_exact_backward(p, state["dY"][i].double(), kept)) if case["backward"] else (Y,))
+        return [torch.stack(parts) for parts in zip(*out)]
+    source = {"o": "q", "gate": "o", "up": "o", "down": "gate"}
+    below = {"gate": "down", "o": "gate", "q": "o"}
+    Y, kept, back = {}, {}, {}
+    for name, p in state["P"].items():
+        Y[name], kept[name] = _exact_forward(p, Y[source[name]] if name in source else state["x"].double())
+    if not case["backward"]:
+        return {name: (y,) for name, y in Y.items()}
+    for name in reversed(state["P"]):
+        dY = back[below[name]][0] if name in below else state["dY"][name].double()
+        back[name] = _exact_backward(state["P"][name], dY, kept[name])
+    return {name: (Y[name], *back[name]) for name in Y}
