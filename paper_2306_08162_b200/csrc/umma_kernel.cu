@@ -52,6 +52,10 @@ constexpr int kWaitLimitUs = 250000;   // default limit of a wait, a launch para
 
 struct Params {
     int M, N, K, bits, g, r, r_pad;
+    // r_pad: columns of the LoRA operands, a multiple of 16.  lora_lo: ranks [r, 2r) hold, beside the same adapter rows again,
+    // what the rounding of s * P to bf16 left over, so the update keeps P's fp32 bits: where the second r columns cost nothing
+    // (r == 8, half an MMA's contraction is padding) and for groups of 32 (whose products the CUDA-core kernel gave in fp32).
+    int lora_lo;
     int C;               // output columns (N forward, K backward)
     int BT;              // token rows per tile (MMA N): 32, 64, 128 or 256
     int n_tok_tiles, n_tiles, steps;
@@ -200,6 +204,22 @@ __device__ __forceinline__ bool wait_counter(const unsigned* ctr, unsigned targe
 }
 
 #include "lora_down_stream.cuh"
+
+// Eight of s * P as bf16 (the LoRA operand), or -- low != 0 -- what that rounding left over, again as bf16.
+__device__ __forceinline__ uint4 lora_p_chunk(const float4& a, const float4& b, float s, bool low) {
+    const float f[8] = {s * a.x, s * a.y, s * a.z, s * a.w, s * b.x, s * b.y, s * b.z, s * b.w};
+    uint32_t o[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        __nv_bfloat162 h = __floats2bfloat162_rn(f[2 * i], f[2 * i + 1]);
+        if (low) {                       // (nothing is left of a value that became infinite or was no number)
+            const float l0 = f[2 * i] - __low2float(h), l1 = f[2 * i + 1] - __high2float(h);
+            h = __floats2bfloat162_rn(fabsf(l0) < INFINITY ? l0 : 0.f, fabsf(l1) < INFINITY ? l1 : 0.f);
+        }
+        o[i] = *reinterpret_cast<const uint32_t*>(&h);
+    }
+    return make_uint4(o[0], o[1], o[2], o[3]);
+}
 
 // Shared-memory matrix descriptor (version 1).  Offsets in bytes; layout 0 = no swizzle, 2 = 128-byte swizzle.
 __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint32_t sbo, uint32_t layout) {
@@ -412,14 +432,15 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
                 const int row = et, wrow = w0 + row;
                 for (int jc = 0; jc < p.r_pad / 8; ++jc) {
                     uint4 v = make_uint4(0, 0, 0, 0);
-                    if (jc * 8 < p.r && wrow < p.C) {
+                    const int js = p.lora_lo && jc * 8 >= p.r ? jc * 8 - p.r : jc * 8;   // first rank of the chunk
+                    if (js < p.r && wrow < p.C) {
                         if (!TRANSPOSED) {
-                            v = __ldg(reinterpret_cast<const uint4*>(p.L + (size_t)wrow * p.r + jc * 8));      // B[n, j..j+7]
+                            v = __ldg(reinterpret_cast<const uint4*>(p.L + (size_t)wrow * p.r + js));      // B[n, j..j+7]
                         } else {
                             uint32_t e[8];
 #pragma unroll
                             for (int j = 0; j < 8; ++j)
-                                e[j] = __bfloat16_as_ushort(__ldg(p.L + (size_t)(jc * 8 + j) * p.K + wrow));     // A[j, k]
+                                e[j] = __bfloat16_as_ushort(__ldg(p.L + (size_t)(js + j) * p.K + wrow));     // A[j, k]
                             v = make_uint4(e[0] | (e[1] << 16), e[2] | (e[3] << 16), e[4] | (e[5] << 16), e[6] | (e[7] << 16));
                         }
                     }
@@ -429,14 +450,12 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
                     const int m = m0 + row_t;
                     for (int jc = 0; jc < p.r_pad / 8; ++jc) {
                         uint4 v = make_uint4(0, 0, 0, 0);
-                        if (jc * 8 < p.r && m < p.M) {
+                        const bool low = p.lora_lo && jc * 8 >= p.r;
+                        const int js = low ? jc * 8 - p.r : jc * 8;
+                        if (js < p.r && m < p.M) {
                             // (not the read-only path: P may have been written by this launch's producer clusters)
-                            const float4 a = __ldcg(reinterpret_cast<const float4*>(p.Pmat + (size_t)m * p.r + jc * 8));
-                            const float4 b = __ldcg(reinterpret_cast<const float4*>(p.Pmat + (size_t)m * p.r + jc * 8 + 4));
-                            __nv_bfloat162 h0 = __floats2bfloat162_rn(p.s * a.x, p.s * a.y), h1 = __floats2bfloat162_rn(p.s * a.z, p.s * a.w);
-                            __nv_bfloat162 h2 = __floats2bfloat162_rn(p.s * b.x, p.s * b.y), h3 = __floats2bfloat162_rn(p.s * b.z, p.s * b.w);
-                            v = make_uint4(*reinterpret_cast<uint32_t*>(&h0), *reinterpret_cast<uint32_t*>(&h1),
-                                           *reinterpret_cast<uint32_t*>(&h2), *reinterpret_cast<uint32_t*>(&h3));
+                            const float4* src = reinterpret_cast<const float4*>(p.Pmat + (size_t)m * p.r + js);
+                            v = lora_p_chunk(__ldcg(src), __ldcg(src + 1), p.s, low);
                         }
                         *reinterpret_cast<uint4*>(lp + jc * (p.BT * 16) + (row_t >> 3) * 128 + (row_t & 7) * 16) = v;
                     }
@@ -500,7 +519,7 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
             const int kb = kb0 + b * kb_stride;                   // 32-code block along k: 0..1 forward, 0..3 backward
             w_off[b] = row_base + (TRANSPOSED ? (uint32_t)(kb >> 1) * 8192u : 0u);
             chunk0[b] = (uint32_t)((TRANSPOSED ? (kb & 1) : kb) * 4);
-            srow[b] = TRANSPOSED ? (uint32_t)(((kb * 32) / p.g) % p.scale_rows) : 0u;
+            srow[b] = (uint32_t)(((kb * 32) / p.g) % p.scale_rows);   // (a stage holds several group rows when groups are short)
         }
         const uint32_t pcols = (uint32_t)p.packed_cols;
         const int my_tiles = first_tile < p.n_tiles ? (p.n_tiles - first_tile + tile_stride - 1) / tile_stride : 0;
@@ -692,10 +711,21 @@ int launch_lora_down_stream(int M, int T, int r, bool l_is_A, const void* In, co
     return launch_lora_down_stream_impl(M, T, r, l_is_A, In, L, P, st);
 }
 
+static int keep_lora_low(const qlora_desc& d) { return d.r == 8 || d.group_size == 32 ? 1 : 0; }
+
+// Rows of scales / zeros that go with the k range of one pipeline stage (64 rows of W forward, 128 backward).
+static int scale_rows_per_stage(const qlora_desc& d, bool transposed) {
+    const int k_rows = transposed ? kWRows : kStepC;
+    return d.group_size >= k_rows ? 1 : k_rows / d.group_size;
+}
+
 bool umma_supported(const qlora_desc& d, int M) {
     if (M < 1) return false;
     if (d.K % 64 != 0 || d.N % 64 != 0) return false;              // contraction steps of 64 in both directions
-    if (!(d.group_size == 64 || d.group_size % 128 == 0)) return false;
+    // a stage's 64 (forward) or 128 (backward) rows along k hold whole groups, or lie inside one: every 32-code block then has
+    // its scale row at the same place in every stage.  (Groups of 32 on the CUDA cores instead: 4130 us for a step of 333 tokens
+    // on 11008 -> 4096, against 153 here.)
+    if (!(d.group_size == 32 || d.group_size == 64 || d.group_size % 128 == 0)) return false;
     if (d.r > 64) return false;
     return true;
 }
@@ -733,7 +763,7 @@ static int launch_umma_pair(const qlora_desc& d, int M, bool transposed, const v
     // plan_only: nothing is launched and no pointer is looked at; the return value is the number of producer pairs when a
     // backward call with every optional workspace area would form dB on them, else 0
     PairParams p{};
-    p.M = M; p.N = d.N; p.K = d.K; p.bits = d.bits; p.g = d.group_size; p.r = d.r; p.r_pad = (d.r + 15) / 16 * 16;
+    p.M = M; p.N = d.N; p.K = d.K; p.bits = d.bits; p.g = d.group_size; p.r = d.r; p.lora_lo = keep_lora_low(d); p.r_pad = ((p.lora_lo ? 2 : 1) * d.r + 15) / 16 * 16;
     p.C = transposed ? d.K : d.N;
     const int T = transposed ? d.N : d.K;
     p.n_tok_tiles = (M + 4 * kPairTok - 1) / (4 * kPairTok);
@@ -742,7 +772,7 @@ static int launch_umma_pair(const qlora_desc& d, int M, bool transposed, const v
     p.steps = T / kStepC;
     p.packed_cols = transposed ? 64 : 128;
     p.packed_rows = (transposed ? 128 : 64) * d.bits / 32;
-    p.scale_rows = transposed ? (d.group_size >= 128 ? 1 : 128 / d.group_size) : 1;
+    p.scale_rows = scale_rows_per_stage(d, transposed);
     p.words_bytes = (uint32_t)(p.packed_rows * p.packed_cols * 4);
     p.scale_bytes = (uint32_t)(p.scale_rows * p.packed_cols * 2);
     p.packed_slot_bytes = (p.words_bytes + 2 * p.scale_bytes + 127u) / 128u * 128u;
@@ -752,10 +782,11 @@ static int launch_umma_pair(const qlora_desc& d, int M, bool transposed, const v
     uint32_t lora_l = (uint32_t)(kPairW * p.r_pad * 2), lora_p = (uint32_t)(2 * kPairTok * p.r_pad * 2);
     if (lora_l + lora_p < 8192) lora_p = 8192 - lora_l;   // the area doubles as the epilogue's staging slices (4 warps x 2 KiB)
     const uint32_t budget = 232448 - 1024 /*alignment slack*/ - 2048 /*static, barriers, padding*/;
-    p.P = 4;
-    const uint32_t fixed = lora_l + lora_p + p.P * p.packed_slot_bytes + 512;
     const uint32_t per_stage = kPairXStage + kWStageBytes;
-    int S = (int)((budget - fixed) / per_stage);
+    int S = 0;
+    for (p.P = 4; p.P >= 2 && S < 2; --p.P)                 // (the packed ring gives way where the LoRA operands are at their largest)
+        S = (int)((budget - (lora_l + lora_p + p.P * p.packed_slot_bytes + 512)) / per_stage);
+    ++p.P;
     if (S > 8) S = 8;
     if (S < 2) return QLORA_ERR_UNSUPPORTED;
     p.S = S;
@@ -876,7 +907,7 @@ int launch_umma_gemm(const qlora_desc& d, int M, bool transposed, const void* In
     if (prefer_pair_kernel(d, M, transposed))
         return launch_umma_pair(d, M, transposed, In, Q, scales, zeros, L, Pmat, Out, st, Ldown, sync, split_buf, split_bytes, db);
     Params p{};
-    p.M = M; p.N = d.N; p.K = d.K; p.bits = d.bits; p.g = d.group_size; p.r = d.r; p.r_pad = (d.r + 15) / 16 * 16;
+    p.M = M; p.N = d.N; p.K = d.K; p.bits = d.bits; p.g = d.group_size; p.r = d.r; p.lora_lo = keep_lora_low(d); p.r_pad = ((p.lora_lo ? 2 : 1) * d.r + 15) / 16 * 16;
     p.C = transposed ? d.K : d.N;
     const int T = transposed ? d.N : d.K;
     p.BT = M > 128 ? 256 : (M > 64 ? 128 : (M > 32 ? 64 : 32));
@@ -886,7 +917,7 @@ int launch_umma_gemm(const qlora_desc& d, int M, bool transposed, const void* In
     p.steps = T / kStepC;
     p.packed_cols = transposed ? 64 : 128;
     p.packed_rows = (transposed ? 128 : 64) * d.bits / 32;
-    p.scale_rows = transposed ? (d.group_size >= 128 ? 1 : 128 / d.group_size) : 1;
+    p.scale_rows = scale_rows_per_stage(d, transposed);
     p.words_bytes = (uint32_t)(p.packed_rows * p.packed_cols * 4);
     p.scale_bytes = (uint32_t)(p.scale_rows * p.packed_cols * 2);
     p.packed_slot_bytes = (p.words_bytes + 2 * p.scale_bytes + 127u) / 128u * 128u;
@@ -902,10 +933,10 @@ int launch_umma_gemm(const qlora_desc& d, int M, bool transposed, const void* In
     const uint32_t per_stage = p.x_stage_bytes + kWStageBytes;
     int S = 0;
     uint32_t fixed = 0;
-    for (p.P = p.BT <= 128 ? 16 : 8; p.P >= 4; p.P -= 4) {   // the packed ring gives way until three operand stages fit
+    for (p.P = p.BT <= 128 ? 16 : 8;; p.P -= p.P > 4 ? 4 : 1) {   // the packed ring gives way until three operand stages fit (two, below four slots)
         fixed = lora_a + lora_p + p.P * p.packed_slot_bytes + 512;
         S = budget > fixed ? (int)((budget - fixed) / per_stage) : 0;
-        if (S >= 3 || p.P == 4) break;
+        if (S >= (p.P > 4 ? 3 : 2) || p.P == 2) break;
     }
     if (S > 8) S = 8;
     if (S < 2) return QLORA_ERR_UNSUPPORTED;

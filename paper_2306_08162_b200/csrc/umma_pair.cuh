@@ -39,6 +39,7 @@ constexpr int kPairXStage = 2 * kPairXSub;             // two accumulators' sub-
 
 struct PairParams {
     int M, N, K, bits, g, r, r_pad;
+    int lora_lo;                 // as in Params
     int C;                       // output columns (N forward, K backward)
     int n_tok_tiles, n_tiles, steps;
     // Last wave split along the contraction: tiles [n_full, n_tiles) are each worked on by two SM pairs (nsplit == 2), one
@@ -406,14 +407,15 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
                     const int row = et, wrow = w0 + (int)cta * kPairW + row;
                     for (int jc = 0; jc < p.r_pad / 8; ++jc) {
                         uint4 v = make_uint4(0, 0, 0, 0);
-                        if (jc * 8 < p.r && wrow < p.C) {
+                        const int js = p.lora_lo && jc * 8 >= p.r ? jc * 8 - p.r : jc * 8;   // first rank of the chunk
+                        if (js < p.r && wrow < p.C) {
                             if (!TRANSPOSED) {
-                                v = __ldg(reinterpret_cast<const uint4*>(p.L + (size_t)wrow * p.r + jc * 8));      // B[n, j..j+7]
+                                v = __ldg(reinterpret_cast<const uint4*>(p.L + (size_t)wrow * p.r + js));      // B[n, j..j+7]
                             } else {
                                 uint32_t e[8];
 #pragma unroll
                                 for (int j = 0; j < 8; ++j)
-                                    e[j] = __bfloat16_as_ushort(__ldg(p.L + (size_t)(jc * 8 + j) * p.K + wrow));     // A[j, k]
+                                    e[j] = __bfloat16_as_ushort(__ldg(p.L + (size_t)(js + j) * p.K + wrow));     // A[j, k]
                                 v = make_uint4(e[0] | (e[1] << 16), e[2] | (e[3] << 16), e[4] | (e[5] << 16), e[6] | (e[7] << 16));
                             }
                         }
@@ -425,14 +427,12 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
                     const int m = m0 + a * (2 * kPairTok) + et;
                     for (int jc = 0; jc < p.r_pad / 8; ++jc) {
                         uint4 v = make_uint4(0, 0, 0, 0);
-                        if (jc * 8 < p.r && m < p.M) {
+                        const bool low = p.lora_lo && jc * 8 >= p.r;
+                        const int js = low ? jc * 8 - p.r : jc * 8;
+                        if (js < p.r && m < p.M) {
                             // (not the read-only path: P may have been written by this launch's producer clusters)
-                            const float4 x = __ldcg(reinterpret_cast<const float4*>(p.Pmat + (size_t)m * p.r + jc * 8));
-                            const float4 y = __ldcg(reinterpret_cast<const float4*>(p.Pmat + (size_t)m * p.r + jc * 8 + 4));
-                            __nv_bfloat162 h0 = __floats2bfloat162_rn(p.s * x.x, p.s * x.y), h1 = __floats2bfloat162_rn(p.s * x.z, p.s * x.w);
-                            __nv_bfloat162 h2 = __floats2bfloat162_rn(p.s * y.x, p.s * y.y), h3 = __floats2bfloat162_rn(p.s * y.z, p.s * y.w);
-                            v = make_uint4(*reinterpret_cast<uint32_t*>(&h0), *reinterpret_cast<uint32_t*>(&h1),
-                                           *reinterpret_cast<uint32_t*>(&h2), *reinterpret_cast<uint32_t*>(&h3));
+                            const float4* src = reinterpret_cast<const float4*>(p.Pmat + (size_t)m * p.r + js);
+                            v = lora_p_chunk(__ldcg(src), __ldcg(src + 1), p.s, low);
                         }
                         *reinterpret_cast<uint4*>(lp + a * (kPairTok * p.r_pad * 2) + jc * (kPairTok * 16) + (et >> 3) * 128 + (et & 7) * 16) = v;
                     }
@@ -573,7 +573,7 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
             const int kb = kb0 + b * kb_stride;                   // 32-code block along k: 0..1 forward, 0..3 backward
             w_off[b] = row_base + (TRANSPOSED ? (uint32_t)(kb >> 1) * 8192u : 0u);
             chunk0[b] = (uint32_t)((TRANSPOSED ? (kb & 1) : kb) * 4);
-            srow[b] = TRANSPOSED ? (uint32_t)(((kb * 32) / p.g) % p.scale_rows) : 0u;
+            srow[b] = (uint32_t)(((kb * 32) / p.g) % p.scale_rows);   // (a stage holds several group rows when groups are short)
         }
         const uint32_t pcols = (uint32_t)p.packed_cols;
         const uint32_t leader_full_w = map_to_cta(bar_full_w, 0);
