@@ -59,6 +59,30 @@ def test_ragged_shapes_and_special_rows(N, K, g, bits):
     check(W, bits, g)
 
 
+@pytest.mark.parametrize("N,K", [(8, 128), (33 * 8, 640), (64, 224), (40, 64)])
+@pytest.mark.parametrize("g", [32, 64, 128])
+@pytest.mark.parametrize("bits", [2, 3, 4, 8])
+def test_one_pass_groups_ties_and_extreme_scales(N, K, g, bits):
+    """Groups of 32, 64 and 128 (one pass, codes from the product with the reciprocal except near ties): strips and row blocks that are
+    not full, weights on and next to every tie, scales that are subnormal, replaced by 1 or infinite."""
+    if K % g:
+        pytest.skip("the group divides K")
+    qmax = 2 ** bits - 1
+    rng = np.random.default_rng(N + K + g + bits)
+    W = qi.gaussian_weight(N + K + bits + g, N, K, 0.05, outlier_frac=0.01)
+    half = rng.integers(-2 * qmax, 2 * qmax + 1, size=(4, K)).astype(np.float32) * np.float32(0.5)      # halves of a unit step: every second one a tie
+    half[:, ::g] = 0.0; half[:, 1::g] = np.float32(qmax)                                                  # (range 0 .. qmax where the rest stays inside)
+    W[0] = np.clip(half[0], 0, qmax)
+    W[1] = np.nextafter(np.clip(half[1], 0, qmax), np.float32(0))
+    W[2] = np.nextafter(np.clip(half[2], 0, qmax), np.float32(np.inf)).clip(max=qmax)
+    W[3] = np.clip(half[3], 0, qmax) * np.float32(1.5e-7)          # scale subnormal in fp16
+    W[4] = np.clip(half[0], 0, qmax) * np.float32(1e-12)           # scale rounds to zero, replaced by 1
+    W[5] = np.clip(half[1], -qmax, qmax) * np.float32(1e6)         # scale infinite in fp16
+    W[6, ::7] *= np.float32(-3.0)
+    with np.errstate(all="ignore"):
+        check(W, bits, g)
+
+
 def test_quantized_layer_runs_through_the_library():
     """Quantize on the device, then run the layer on the result: the same Y as with the oracle-quantized layer."""
     layer = qi.make_layer(K=512, N=512, bits=4, group_size=128, r=8, alpha=16.0, M=64, seed=0)
