@@ -35,6 +35,27 @@ def test_loss_and_gradient_match_the_oracle(T, V):
     run_case(T, V, 0.8, 1.2, seed=T + V, scale=1.0 / T)
 
 
+@pytest.mark.parametrize("V", [8, 256, 264, 2056, 8192, 8200, 20000, 24584, 32760])
+@pytest.mark.parametrize("T", [1, 700])
+def test_row_lengths_at_the_edges_of_the_block_plan(T, V):
+    """One chunk, a full warp of chunks and one more, several short rows per SM, rows that need a third and fourth chunk per
+    thread; more rows than resident blocks (700 x short rows) and a single one."""
+    if T * V > 6_000_000:
+        T = 160                                             # still more rows than SMs
+    run_case(T, V, 0.7, 0.9, seed=T + V, scale=0.5)
+
+
+def test_rows_with_infinitely_unlikely_teacher_tokens():
+    """A stretch of -inf teacher logits (whole warps of them) where the student has mass: KL is infinite, not NaN; the other
+    rows of the launch are untouched."""
+    z = torch.randn((3, 32000), device="cuda").bfloat16()
+    t = z.clone()
+    t[1, :24000] = float("-inf")
+    loss = torch.empty(3, dtype=torch.float32, device="cuda")
+    ql.qlora_lrec_loss(z, t, None, 1.0, 0.0, 1.0, loss, None)
+    assert torch.isinf(loss[1]) and loss[1] > 0 and loss[0].abs() < 1e-5 and loss[2].abs() < 1e-5
+
+
 def test_loss_only_and_pure_terms_and_determinism():
     a = run_case(16, 32000, 1.0, 0.0, seed=1, with_grad=False)
     run_case(16, 32000, 0.0, 1.0, seed=2)
