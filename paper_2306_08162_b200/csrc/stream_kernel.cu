@@ -1,35 +1,36 @@
 // Few-token kernels (M <= 16) of the quantized-linear + LoRA layer, both directions.
 //
-// With a handful of tokens the layer is bound by reading the packed weights once, so these kernels are built around
-// bytes in flight and around what a thread has to issue per weight:
-//   - every warp streams its own slice of the packed matrix with 16-byte cp.async copies from all lanes into a private
-//     shared-memory ring (no barrier between warps in the main loop); the copies of the first ring-full are issued before
-//     the kernel waits for its predecessor in the stream (griddepcontrol.wait), so the frozen weights of a call are in
-//     flight while the preceding call is still computing.  Only Q, scales and zeros are touched before that wait: the
-//     activations, the adapters (which an optimizer rewrites every step), H / G and the outputs come after it;
+// With a handful of tokens the layer is bound by reading the packed weights once -- in bytes; in time, by the chain of dependent
+// steps of a call (activations arrive, products, exchange of partial sums, store) and by what a thread issues per weight.  So:
+//   - a warp loads its packed words straight into registers, 16 bytes per lane, several hundred contraction elements ahead and
+//     before the kernel waits for its predecessor in the stream (griddepcontrol.wait); scales and zeros go to shared memory at the
+//     same time.  A CTA is 256 threads x 128 registers with at most half an SM's shared memory where the shape allows it, so the
+//     CTAs of the NEXT call move in beside those of the current one and have their weights under way when it ends.  Only Q, scales
+//     and zeros are touched before the wait: the activations, the adapters (which an optimizer rewrites every step), H / G and the
+//     outputs come after it;
 //   - the codes go to the warp-level tensor-core instruction (mma.sync m16n8k16, weights as the 16-row operand, tokens as
 //     the 8 columns) as RAW integers: a code is ORed into the mantissa of the bf16 constant 128 (one shift + one logic
 //     operation per pair of codes), so the operand is 128 + q.  The group scale and the zero-point are applied outside the
 //     per-weight path:
 //       forward   Y[m,n] = sum_groups s[G,n] * ( sum_{k in G} X[m,k] (128 + q[k,n])  -  (128 + z[G,n]) * sum_{k in G} X[m,k] )
-//                 (one accumulator per group; the scaling is a few FMAs per group, the activation sums are made once
-//                 per CTA when the activation slice is staged);
+//                 (one accumulator per group segment; the sums of the activations come from the staging pass);
 //       backward  dX[m,k] = sum_n dYs[m,n] (128 + q[k,n])  -  sum_n dYs[m,n] (128 + z[G(k),n]),   dYs = bf16(dY[m,n] * s[G(k),n])
 //                 (the scale varies along the contraction, so it is folded into a per-group copy of the activation slice,
-//                 rounded once to bf16 -- the same relative rounding the dequantised weight would get; the second sum is
-//                 one extra MMA row per 16 columns).
+//                 rounded once to bf16 -- the same relative rounding the dequantised weight would get; the second sum comes from
+//                 the staging pass, in fp32).
 //     8-bit codes take an fp32 detour (byte -> 2^23 + q -> q -> bf16, exact), offset 0 instead of 128;
-//   - backward: the contraction runs across packed columns, so a fragment register needs two columns for one feature.
-//     Each lane builds pairs of features of its own column and the 8 x 8 tile is transposed across the warp with
-//     movmatrix: the register form of the transposition of the packed matrix (Section 3.1, "Implementation Details");
-//   - the contraction is split over a cluster of up to 8 CTAs, and inside a CTA over up to four sets of warps (sixteen
-//     warps per SM keep the schedulers busy).  CTA i of a cluster finishes a slice of the columns: every CTA stores its
-//     partial sums for that slice straight into i's shared memory (distributed shared memory; nothing waits on a remote
-//     store), one cluster barrier later i adds them in a fixed order.  No workspace, no counters, and the result is the
-//     same on every run;
-//   - the LoRA down-projection (H = X A^T, G = dY B) over the CTA's part of the contraction comes from a few MMAs fed
-//     straight from global memory (ranks up to 16), reduced with the partial tiles; the update s P L is added in the
-//     epilogue in fp32 before the one rounding to bf16.
+//   - backward: the contraction runs across packed columns, so an operand register needs one feature's codes of two columns.  A lane
+//     holds the words of the same features for neighbouring columns and merges their halves (one byte permute per eight codes):
+//     the register form of the transposition of the packed matrix (Section 3.1, "Implementation Details");
+//   - one staging pass after the wait: warps take 32-wide slices of the activations, keep them in the order the products ask for,
+//     and feed the LoRA down-projection (H = X A^T, G = dY B, ranks up to 16) from the same registers;
+//   - the contraction is split over a cluster of up to 8 CTAs, and inside a CTA over its warps.  A CTA adds its warps' partial sums
+//     in order; CTA i of a cluster finishes a slice of the columns: every CTA stores its sums for that slice straight into i's
+//     shared memory (distributed shared memory; nothing waits on a remote store), one cluster barrier later i adds them in a fixed
+//     order, adds s P L in fp32 and rounds once to bf16.  No workspace, no counters, and the result is the same on every run;
+//   - at these sizes a warp has little main loop (two chunks of 128 x 32 weights at 4096 x 4096), so what it issues before and after
+//     counts as much: no divisions (the host passes reciprocals and logarithms), loads without per-lane predicates where a whole
+//     warp is inside, and only the tokens and ranks that exist are exchanged.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -43,41 +44,35 @@
 namespace qlora {
 namespace {
 
-constexpr int ST_MAX_DEVICES = kMaxDevices;
+constexpr int ST_WARPS = 8, ST_THREADS = 32 * ST_WARPS;
+constexpr int ST_CHUNK = 128;                                // forward: contraction elements per step of a warp
 
 template <int BITS>
 struct Fmt {
     static constexpr float OFF = BITS == 8 ? 0.f : 128.f;   // what the integer operand carries on top of the code
-    // forward: a ring stage = KB contraction elements x 32 columns of one warp (+ the scale / zero chunk of its group)
+    // forward: a block = KB contraction elements x 32 columns of one warp; lane (g, q) has columns 4g .. 4g+3 of packed row q
     static constexpr int KB = BITS == 2 ? 64 : 32;
-    static constexpr int ROWS = KB * BITS / 32;              // packed rows per stage: 4, 3, 4, 8
-    static constexpr int SLOT = ROWS * 128 + 128;
-    static constexpr int NS = BITS == 8 ? 5 : 8;            // ring stages per warp: 4 - 5.6 KB in flight per warp
-    static constexpr int STEPS = KB / 16;                    // k16 MMA steps per stage
+    static constexpr int BPC = ST_CHUNK / KB;                // blocks per chunk
+    static constexpr int STEPS = KB / 16;                    // k16 MMA steps per block
     static constexpr int NPAIR = 2 * STEPS;                  // bf16 pairs per column and lane
-    static constexpr int NLD = (BITS == 3 || BITS == 8) ? 2 : 1;
-    static constexpr int XPAD = BITS == 2 ? 16 : (BITS == 8 ? 32 : 64);   // pitch of an activation row = 2 xc + XPAD bytes
-    // backward: a warp owns FW output features (BROWS packed rows); a ring stage = SU units of 32 columns
-    static constexpr int FW = BITS == 2 ? 16 : 32;
-    static constexpr int BROWS = FW * BITS / 32;             // 1, 3, 4, 8
-    static constexpr int SU = BITS == 2 ? 4 : 1;
-    static constexpr int BSLOT = BROWS * 128 * SU;
-    static constexpr int BNS = BITS == 8 ? 4 : 8;
-    static constexpr int BPAIR = BITS == 2 ? 2 : 4;          // pairs per column and lane
+    static constexpr int NLD = (BITS == 3 || BITS == 8) ? 2 : 1;   // 16-byte loads per lane and block
+    static constexpr int LPC = BPC * NLD;
+    static constexpr int DEPTH = BITS == 2 ? 4 : 2;          // chunks in flight per warp: 32 registers (64 for 3 and 8 bits), 4 KB
 };
 
 struct StreamParams {
     int M, K, N, g, r;
     int C;                       // output columns (N forward, K backward)
-    int ks;                      // CTAs per cluster = ways the contraction is split
-    int wc;                      // warps side by side in a CTA (32 columns forward, FW features backward each)
-    int khs;                     // log2 of the parts the warps of a CTA split each staged slice of the contraction into
-    int sls;                     // log2 of the columns a CTA of the cluster finishes (32 wc / ks or FW wc / ks)
-    int lwc, lks;                // log2 of wc and of ks
-    int xc;                      // contraction elements of the activations staged per pass (a power of two, all parts together)
-    int copies;                  // backward: groups a CTA's features span (1 or 2)
+    int ks, lks;                 // CTAs per cluster = ways the contraction is split, and its log2
+    int wc, lwc;                 // warps side by side in a CTA (32 columns forward, 8 FL features backward each), and its log2
+    int lwp;                     // log2 of the parts the warps of a CTA split its range of the contraction into (wc << lwp == ST_WARPS)
+    int lsl;                     // log2 of the columns a CTA of the cluster finishes
+    int pitch;                   // bytes of a staged activation row
+    int range;                   // contraction elements a CTA stages at most
+    int ngl;                     // forward: group rows of a CTA's range at most; backward: groups its features span (1 or 2)
+    int gd;                      // g / 32, and ceil(2^32 / gd): a group index is a multiplication
+    uint32_t gm;
     int fused;                   // H / G is computed here (ranks up to 16) and written to P; else P is an input
-    int lup_staged;              // the epilogue's slice of the second adapter fits its shared-memory area
     float s;
     const __nv_bfloat16* In;
     const uint32_t* Q;
@@ -89,15 +84,32 @@ struct StreamParams {
     __nv_bfloat16* Out;
 };
 
-constexpr int ST_LUP_BYTES = 4096;
-
 __device__ __forceinline__ uint32_t s_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void cp16(uint32_t dst, const void* src, int bytes) {   // bytes = 16, or 0 to zero-fill
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
 }
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+__device__ __forceinline__ void cp_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// 16 bytes of packed words, kept in program order with griddepcontrol.wait.
+__device__ __forceinline__ void ldg_words(uint4& v, const uint32_t* src) {
+    asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(src));
+}
+// Shared memory, where `ok`; otherwise the registers keep what they hold.
+__device__ __forceinline__ void lds16(uint32_t& a, uint32_t& b, uint32_t& c, uint32_t& d, uint32_t addr, bool ok) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %5, 0;\n\t@p ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];\n\t}"
+                 : "+r"(a), "+r"(b), "+r"(c), "+r"(d) : "r"(addr), "r"((uint32_t)ok) : "memory");
+}
+__device__ __forceinline__ void lds8(uint32_t& a, uint32_t& b, uint32_t addr, bool ok) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %3, 0;\n\t@p ld.shared.v2.u32 {%0, %1}, [%2];\n\t}"
+                 : "+r"(a), "+r"(b) : "r"(addr), "r"((uint32_t)ok) : "memory");
+}
+// Group of the u-th 32 rows along k (u < 2^16, gd < 2^16: exact).
+__device__ __forceinline__ int st_group(const StreamParams& p, int u) { return p.gd == 1 ? u : (int)__umulhi((uint32_t)u, p.gm); }
+__device__ __forceinline__ uint4 ldg16(const void* src, bool ok) {      // plain global load, zero without `ok`
+    return ok ? *reinterpret_cast<const uint4*>(src) : make_uint4(0, 0, 0, 0);
+}
+__device__ __forceinline__ uint32_t ldg32(const void* p) { return *reinterpret_cast<const uint32_t*>(p); }
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
 __device__ __forceinline__ uint32_t st_cluster_rank() {
     uint32_t r;
@@ -109,13 +121,15 @@ __device__ __forceinline__ uint32_t st_map(uint32_t addr, uint32_t rank) {
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
     return r;
 }
+__device__ __forceinline__ void st_cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+__device__ __forceinline__ void st_cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void st_cluster_sync() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void st_mma(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-                 : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 __device__ __forceinline__ uint32_t st_movm(uint32_t a) {
     uint32_t d;
@@ -123,38 +137,18 @@ __device__ __forceinline__ uint32_t st_movm(uint32_t a) {
     return d;
 }
 __device__ __forceinline__ uint32_t st_comp(const uint4& v, int i) { return i == 0 ? v.x : (i == 1 ? v.y : (i == 2 ? v.z : v.w)); }
-__device__ __forceinline__ uint32_t ldg32(const void* p) { return *reinterpret_cast<const uint32_t*>(p); }
-
-// A ring stage holds packed rows of 32 columns (128 bytes); row `row`, 16-byte chunk `ch` sits at a swizzled place so that
-// the lanes (g, q) of a quarter-warp, which read chunk g of four different rows, hit different banks.
-__device__ __forceinline__ int st_swz(int row, int ch) { return row * 128 + (((ch ^ (2 * row)) & 7) << 4); }
-
-// The packed words a lane needs for its four columns 4g .. 4g+3: lane q takes the q-th quarter of the stage's contraction
-// range (row q; 3-bit: the 24 stream bits [24 q, 24 q + 24) of the 96-bit block, which may lie in two rows; 8-bit: rows
-// q and q + 4).
-template <int BITS>
-__device__ __forceinline__ void st_load_words(const uint8_t* slot, int g, int q, uint4 (&w)[Fmt<BITS>::NLD]) {
-    if constexpr (BITS == 3) {
-        w[0] = *reinterpret_cast<const uint4*>(slot + st_swz((24 * q) >> 5, g));
-        w[1] = *reinterpret_cast<const uint4*>(slot + st_swz((24 * q + 23) >> 5, g));
-    } else if constexpr (BITS == 8) {
-        w[0] = *reinterpret_cast<const uint4*>(slot + st_swz(q, g));
-        w[1] = *reinterpret_cast<const uint4*>(slot + st_swz(q + 4, g));
-    } else {
-        w[0] = *reinterpret_cast<const uint4*>(slot + st_swz(q, g));
-    }
-}
-
-__device__ __forceinline__ uint32_t st_u8_pair(uint32_t w, int j) {   // bytes 2j, 2j+1 -> (bf16, bf16), exact
-    const float f0 = __uint_as_float(__byte_perm(w, 0x4B000000u, 0x7540 + 2 * j)) - 8388608.f;
-    const float f1 = __uint_as_float(__byte_perm(w, 0x4B000000u, 0x7541 + 2 * j)) - 8388608.f;
-    const __nv_bfloat162 pr = __floats2bfloat162_rn(f0, f1);
+__device__ __forceinline__ uint32_t st_pack(float a, float b) {
+    const __nv_bfloat162 pr = __floats2bfloat162_rn(a, b);
     return *reinterpret_cast<const uint32_t*>(&pr);
+}
+__device__ __forceinline__ float st_byte(uint32_t w, int j) {            // byte j as fp32, exact
+    return __uint_as_float(__byte_perm(w, 0x4B000000u, 0x7540 + j)) - 8388608.f;
 }
 
 // One column's codes of this lane -> bf16 pairs holding OFF + q.  With c_0 .. c_{n-1} the lane's codes in contraction order:
 //   2-bit (16 codes): p[t] = (c_t, c_{t+8}), t < 8        3- and 4-bit (8 codes): p[t] = (c_t, c_{t+4}), t < 4
 //   8-bit (row q: c_0..3, row q + 4: c_4..7): p = (c_0,c_1), (c_2,c_3), (c_4,c_5), (c_6,c_7)
+// (3-bit: w0, w1 are the rows of stream bits 24 q and 24 q + 23 of the block.)
 template <int BITS>
 __device__ __forceinline__ void st_unpack(uint32_t w0, uint32_t w1, int q, uint32_t (&p)[Fmt<BITS>::NPAIR]) {
     if constexpr (BITS == 4) {
@@ -169,830 +163,759 @@ __device__ __forceinline__ void st_unpack(uint32_t w0, uint32_t w1, int q, uint3
 #pragma unroll
         for (int t = 0; t < 4; ++t) p[t] = ((m >> (3 * t)) & 0x00070007u) | 0x43004300u;
     } else {
-        p[0] = st_u8_pair(w0, 0); p[1] = st_u8_pair(w0, 1);
-        p[2] = st_u8_pair(w1, 0); p[3] = st_u8_pair(w1, 1);
+        p[0] = st_pack(st_byte(w0, 0), st_byte(w0, 1)); p[1] = st_pack(st_byte(w0, 2), st_byte(w0, 3));
+        p[2] = st_pack(st_byte(w1, 0), st_byte(w1, 1)); p[3] = st_pack(st_byte(w1, 2), st_byte(w1, 3));
     }
 }
 
-// 16 bytes of activations (8 consecutive contraction elements) -> the order the lanes' pairs ask for: (x0,x4) (x1,x5)
-// (x2,x6) (x3,x7); the 8-bit forward path pairs neighbours and keeps the natural order.
-__device__ __forceinline__ uint4 st_permute8(const uint4& v) {
-    return make_uint4(__byte_perm(v.x, v.z, 0x5410), __byte_perm(v.x, v.z, 0x7632), __byte_perm(v.y, v.w, 0x5410), __byte_perm(v.y, v.w, 0x7632));
-}
 __device__ __forceinline__ float st_sum8(const uint4& v) {
     return ((bf16_lo(v.x) + bf16_hi(v.x)) + (bf16_lo(v.y) + bf16_hi(v.y))) + ((bf16_lo(v.z) + bf16_hi(v.z)) + (bf16_lo(v.w) + bf16_hi(v.w)));
 }
-
-// ---- reduction across the cluster: push, barrier, add locally -------------------------------------------------------
-// The CTAs of a cluster hold partial tiles of the same output columns.  CTA `o` finishes the slice of tile_c / ks columns
-// [o sl, o sl + sl): every CTA stores its partial sums for those columns straight into o's shared memory (remote stores,
-// nothing waits on them), one cluster barrier later o adds what it received in a fixed order.  recv layout in the owner:
-//   recv_part [ks][KH][sl][16 tokens] fp32      recv_h [ks][16 ranks][16 tokens] fp32
-// Nobody reads a peer's shared memory, so a CTA may leave as soon as it has stored its own outputs.
-struct RecvLayout {
-    uint32_t part_addr, h_addr;   // shared-space addresses (the same in every CTA of the cluster)
-    int sls, khs;                 // log2 of the slice width and of the parts per CTA
-};
-
-__device__ __forceinline__ void st_push2(const RecvLayout& rl, int src_rank, int kh, int cl, int tok, float v0, float v1) {
-    const int owner = cl >> rl.sls, c = cl & ((1 << rl.sls) - 1);
-    const uint32_t off = (uint32_t)(((((src_rank << rl.khs) + kh) << rl.sls) + c) * 16 + tok) * 4u;
-    asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(st_map(rl.part_addr + off, (uint32_t)owner)), "f"(v0), "f"(v1) : "memory");
+__device__ __forceinline__ float st_quad_sum(float v) {
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    return v + __shfl_xor_sync(0xffffffffu, v, 2);
 }
 
-// This CTA's part of H / G (hs [16][16]) goes to every CTA of the cluster.
-__device__ __forceinline__ void st_push_h(const RecvLayout& rl, const float* hs, int src_rank, int ks) {
-    for (int e = threadIdx.x; e < 256 * ks; e += blockDim.x) {
-        const int peer = e >> 8, i = e & 255;
-        asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(st_map(rl.h_addr + (uint32_t)(src_rank * 256 + i) * 4u, (uint32_t)peer)), "f"(hs[i]) : "memory");
+// ---- shared memory ------------------------------------------------------------------------------------------------------
+// Everything but the staged activations (which come first) and the staged group parameters (second):
+//   sums   forward: [range / 32][TOKS] sums of 32 activations;  backward: [ST_WARPS][2][16] zero-point sums
+//   hp     [ST_WARPS][M][16] the warps' parts of H / G (16 ranks)   hfull  [M][16 or r] the whole of it
+//   lup    this CTA's slice of the second adapter
+//   part   [parts][M][tile_c] the warps' partial sums
+//   recv_h [ks][M][16], recv [ks][M][sl]: what the CTAs of the cluster send this one
+struct SmemPlan { uint32_t sz, sums, hp, hfull, lup, recv_h, part, recv, total; };
+__host__ __device__ inline SmemPlan st_plan(const StreamParams& p, bool transposed, int toks, int tile_c) {
+    SmemPlan s;
+    const uint32_t rows = (uint32_t)p.M * (transposed ? (uint32_t)p.ngl : 1u);
+    s.sz = (rows * (uint32_t)p.pitch + 127u) / 128u * 128u;
+    s.sums = s.sz + (transposed ? 4u * (uint32_t)p.ngl * (uint32_t)p.range : 4u * (uint32_t)p.ngl * (uint32_t)tile_c);
+    s.hp = s.sums + (transposed ? ST_WARPS * 128u : (uint32_t)(p.range / 32 * toks) * 4u);
+    s.hfull = s.hp + (p.fused ? ST_WARPS * 64u * (uint32_t)p.M : 0u);
+    s.lup = s.hfull + (p.r > 0 ? (uint32_t)(p.r < 16 ? 16 : p.r) * 4u * (uint32_t)p.M : 0u);
+    s.recv_h = s.lup + (((uint32_t)(p.r * 2) << p.lsl) + 15u) / 16u * 16u;
+    s.part = s.recv_h + (p.fused ? (uint32_t)p.ks * 64u * (uint32_t)p.M : 0u);
+    s.recv = s.part + ((uint32_t)(p.M * tile_c * 4) << p.lwp);
+    s.total = s.recv + (p.ks > 1 ? (uint32_t)(p.M * tile_c * 4) : 0u);
+    return s;
+}
+
+// A warp's partial H / G tile (MMA accumulator layout: rows = ranks, columns = tokens) -> its slot of hp.
+template <int NT>
+__device__ __forceinline__ void st_store_hp(const StreamParams& p, const float (&ah)[NT][4], float* hp, int warp, int g, int q) {
+    float* mine = hp + warp * 16 * p.M + g;
+#pragma unroll
+    for (int tt = 0; tt < NT; ++tt)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const int tok = 8 * tt + 2 * q + e;
+            if (tok < p.M) { mine[tok * 16] = ah[tt][e]; mine[tok * 16 + 8] = ah[tt][2 + e]; }
+        }
+}
+
+// The CTA's part of H / G: the warps' parts added in order, sent to every CTA of the cluster.
+__device__ __forceinline__ void st_share_h(const StreamParams& p, const float* hp, uint32_t recv_h_addr, int rank) {
+    const int n = 16 * p.M;
+    if ((int)threadIdx.x < n) {
+        float h = 0.f;
+#pragma unroll
+        for (int w = 0; w < ST_WARPS; ++w) h += hp[w * n + threadIdx.x];
+#pragma unroll 1
+        for (int peer = 0; peer < p.ks; ++peer)
+            asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(st_map(recv_h_addr + (uint32_t)(rank * n + (int)threadIdx.x) * 4u, (uint32_t)peer)), "f"(h) : "memory");
     }
 }
 
-__device__ __forceinline__ void st_cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
-__device__ __forceinline__ void st_cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// This CTA's slice of the second adapter, and H / G where it is an input.  After griddepcontrol.wait.
+template <bool TRANSPOSED>
+__device__ __forceinline__ void st_stage_lup(const StreamParams& p, uint8_t* lup, float* hfull, int c_lo) {
+    if (p.r == 0) return;
+    const int tid = threadIdx.x;
+    if (TRANSPOSED) {                                     // A [r, K]: [r][sl]
+        const int lc8 = p.lsl - 3;                        // log2 of the 16-byte pieces per rank
+        for (int e = tid; e < p.r << lc8; e += ST_THREADS) {
+            const int j = e >> lc8, col = c_lo + 8 * (e & ((1 << lc8) - 1));
+            cp16(s_u32(lup) + e * 16, col < p.K ? p.Lup + (size_t)j * p.K + col : p.Lup, col < p.K ? 16 : 0);
+        }
+    } else {                                              // B [N, r]: [sl][r], contiguous
+        const int pieces = ((1 << p.lsl) * p.r) >> 3, valid = max(0, p.N - c_lo) * p.r >> 3;
+        for (int e = tid; e < pieces; e += ST_THREADS)
+            cp16(s_u32(lup) + e * 16, e < valid ? p.Lup + (size_t)c_lo * p.r + 8 * e : p.Lup, e < valid ? 16 : 0);
+    }
+    if (!p.fused)
+        for (int e = tid; e < p.M * p.r; e += ST_THREADS) hfull[e] = p.P[e];
+}
 
-// After the pushes: one cluster barrier, then the owner adds (source rank, part) in order, adds s P L, stores bf16.
-template <bool TRANSPOSED, int TOKS>
-__device__ __forceinline__ void st_finish(const StreamParams& p, const float* recv_part, const float* recv_h, float* hfull,
-                                          const __nv_bfloat16* lup, int tile_c, int rank) {
-    const int tid = threadIdx.x, nthr = blockDim.x;
-    const int sl = tile_c / p.ks, KH = 1 << p.khs;
-    st_cluster_sync();                                    // every CTA's stores into this CTA's shared memory are visible
-    if (p.r > 0 && p.fused) {
-        for (int e = tid; e < 256; e += nthr) {
+// The end of a call, once the warps' partial sums are in `part`: the CTA's sums go to the owners of their columns, one cluster
+// barrier later the owner adds them (CTA by CTA, in order), adds s P L, stores bf16.  A CTA alone adds its warps' parts directly.
+template <bool TRANSPOSED>
+__device__ __forceinline__ void st_finish(const StreamParams& p, uint8_t* smem, const SmemPlan& sp, int c_lo, int rank, bool writes_p) {
+    const int tid = threadIdx.x, sl = 1 << p.lsl;
+    const float* src = reinterpret_cast<const float*>(smem + sp.part);
+    const float* recv_h = reinterpret_cast<const float*>(smem + sp.recv_h);
+    float* hfull = reinterpret_cast<float*>(smem + sp.hfull);
+    const __nv_bfloat16* lup = reinterpret_cast<const __nv_bfloat16*>(smem + sp.lup);
+    int nsrc = 1 << p.lwp;
+    __syncthreads();
+    if (p.ks > 1) {
+        const int ltc = p.lsl + p.lks;                    // log2 of the tile's columns
+        const uint32_t recv_addr = s_u32(smem + sp.recv);
+#pragma unroll 1
+        for (int e = tid; e < p.M << (ltc - 2); e += ST_THREADS) {
+            const int c = 4 * (e & ((1 << (ltc - 2)) - 1)), tok = e >> (ltc - 2);
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 2
+            for (int i = 0; i < nsrc; ++i) {
+                const float4 x = *reinterpret_cast<const float4*>(src + (((i * p.M + tok) << ltc) + c));
+                v.x += x.x; v.y += x.y; v.z += x.z; v.w += x.w;
+            }
+            const uint32_t off = (uint32_t)(((rank * p.M + tok) << p.lsl) + (c & (sl - 1))) * 4u;
+            asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(st_map(recv_addr + off, (uint32_t)(c >> p.lsl))), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+        }
+        src = reinterpret_cast<const float*>(smem + sp.recv);
+        nsrc = p.ks;
+        st_cluster_sync();                                // every CTA's stores into this CTA's shared memory are visible
+    }
+    const int hs = p.fused ? 16 : p.r;                    // ranks per row of hfull
+    if (p.fused) {
+        const int n = 16 * p.M;
+        if (tid < n) {
             float h = 0.f;
-            for (int rk = 0; rk < p.ks; ++rk) h += recv_h[rk * 256 + e];
-            hfull[e] = h;
-            const int j = e >> 4, tok = e & 15;
-            if (blockIdx.y == 0 && rank == 0 && tok < p.M && j < p.r) p.P[(size_t)tok * p.r + j] = h;
+#pragma unroll 4
+            for (int rk = 0; rk < p.ks; ++rk) h += recv_h[rk * n + tid];
+            hfull[tid] = h;
+            const int tok = tid >> 4, j = tid & 15;
+            if (writes_p && j < p.r) p.P[(size_t)tok * p.r + j] = h;
         }
         __syncthreads();
     }
-    for (int e = tid; e < sl * TOKS; e += nthr) {
-        const int tok = e % TOKS, c = e / TOKS;           // TOKS is a power of two
-        const int col = blockIdx.y * tile_c + rank * sl + c;
-        float v = 0.f;
-        for (int i = 0; i < p.ks * KH; ++i) v += recv_part[(i * sl + c) * 16 + tok];
-        if (tok >= p.M || col >= p.C) continue;
-        if (p.r > 0) {
-            float lo = 0.f;
-            for (int j = 0; j < p.r; ++j) {
-                float l;
-                if (p.lup_staged) l = __bfloat162float(TRANSPOSED ? lup[j * sl + c] : lup[c * p.r + j]);
-                else l = __bfloat162float(TRANSPOSED ? p.Lup[(size_t)j * p.K + col] : p.Lup[(size_t)col * p.r + j]);
-                lo = fmaf(hfull[j * 16 + tok], l, lo);
-            }
-            v += p.s * lo;
-        }
-        p.Out[(size_t)tok * p.C + col] = __float2bfloat16_rn(v);
-    }
-}
-
-// After griddepcontrol.wait: this CTA's slice of the second adapter (the columns it will finish) and, when H / G is an
-// input, the whole of it.
-template <bool TRANSPOSED>
-__device__ __forceinline__ void st_stage_lup(const StreamParams& p, __nv_bfloat16* lup, float* hfull, int tile_c, int rank) {
-    const int tid = threadIdx.x, nthr = blockDim.x;
-    if (p.r == 0) return;
-    const int sl = tile_c / p.ks;
-    if (p.lup_staged) {
-        for (int e = tid; e < sl * p.r; e += nthr) {
-            int c, j;
-            if (TRANSPOSED) { j = e / sl; c = e % sl; } else { c = e / p.r; j = e % p.r; }
-            const int col = blockIdx.y * tile_c + rank * sl + c;
-            __nv_bfloat16 v = __float2bfloat16_rn(0.f);
-            if (col < p.C) v = TRANSPOSED ? p.Lup[(size_t)j * p.K + col] : p.Lup[(size_t)col * p.r + j];
-            lup[e] = v;
-        }
-    }
-    if (!p.fused) {
-        for (int e = tid; e < 16 * p.r; e += nthr) {      // hfull[j][tok]; rows beyond M are zero
-            const int j = e >> 4, tok = e & 15;
-            hfull[e] = tok < p.M ? p.P[(size_t)tok * p.r + j] : 0.f;
-        }
-    }
-}
-
-// Before griddepcontrol.wait nothing but the frozen weights may be READ, but lines can be asked into L2 (the point of
-// coherence: a line the predecessor rewrites afterwards is simply updated there); the kernels do that for the slices of
-// the activations and adapters they load right after the wait.
-
-// A warp's partial H / G tile ([16 ranks][16 tokens], MMA accumulator layout) -> its slot of hp.
-template <int NT>
-__device__ __forceinline__ void st_store_hp(float (&ah)[NT][4], float* hp, int warp, int g, int q) {
-    float* mine = hp + warp * 256;
-#pragma unroll
-    for (int tt = 0; tt < 2; ++tt)
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-            mine[(g + ((e & 2) ? 8 : 0)) * 16 + 8 * tt + 2 * q + (e & 1)] = tt < NT ? ah[tt < NT ? tt : 0][e] : 0.f;
-}
-
-// ------------------------------------------------------------------------------------------------------------
-// Forward: Y = X W^T + s H B^T.  CTA (rank, tile): columns [32 wc tile, + 32 wc), contraction blocks [kb0, kb1) of KB
-// elements.  Warp (cg, kh): 32 columns and the kh-th of KH consecutive parts of [kb0, kb1).  The activations of the
-// parts are staged side by side, xpb blocks of every part per pass (one pass when the CTA's range fits the buffer).
-// ------------------------------------------------------------------------------------------------------------
-constexpr int ST_HSTEPS = 4;   // k16 steps of the fused down-projection whose operands a warp loads in one go
-
-struct PartInfo { int k0, k1, gf, nseg; };   // a part's share of the current pass: contraction range, first group, segments
-
-template <int BITS, int NT>
-__global__ void __launch_bounds__(512, 1) stream_fwd_kernel(const StreamParams p) {
-    using F = Fmt<BITS>;
-    constexpr int TOKS = 8 * NT, LTOKS = NT == 1 ? 3 : 4;
-    constexpr int KP = BITS == 2 ? 16 : 8;                 // contraction elements per staged item
-    constexpr int LKB = BITS == 2 ? 6 : 5;
-    pdl_launch_dependents();
-    st_cluster_arrive_relaxed();                           // waited for before the first store into a peer's shared memory
-    extern __shared__ __align__(128) uint8_t smem[];
-    __shared__ PartInfo tab[4];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, q = lane & 3;
-    const int nthr = blockDim.x, nw = nthr >> 5, tile_c = 32 * p.wc, KH = 1 << p.khs;
-    const int cg = warp & (p.wc - 1), kh = warp >> p.lwc;
-    const int rank = (int)st_cluster_rank();
-    const int col0 = blockIdx.y * tile_c + 32 * cg;
-    const int nblk = (p.K + F::KB - 1) >> LKB;
-    const int kb0 = (nblk * rank) >> p.lks, kb1 = (nblk * (rank + 1)) >> p.lks, nb = kb1 - kb0;
-    const int wb0 = kb0 + ((nb * kh) >> p.khs), wb1 = kb0 + ((nb * (kh + 1)) >> p.khs);
-    const int xp = p.xc * 2 + F::XPAD;
-    const int xpb = (p.xc >> LKB) >> p.khs;                // blocks of a part staged per pass
-    const int bpg = p.g >> LKB;                            // blocks per group
-    const int sl = tile_c >> p.lks;
-    uint8_t* ring = smem + warp * (F::NS * F::SLOT);
-    uint8_t* xs = smem + nw * (F::NS * F::SLOT);           // [TOKS][xp] permuted activations: KH parts side by side
-    float* sxc = reinterpret_cast<float*>(xs + TOKS * xp); // [TOKS][xc / 8] sums of 8 activations
-    float* sxs = sxc + TOKS * (p.xc >> 3);                 // [KH][xpb + 1][TOKS] sums per (part, group) segment of the pass
-    float* hs = sxs + KH * (xpb + 1) * TOKS;               // [16][16] this CTA's part of H
-    float* hfull = hs + 256;                               // [r <= 64][16] the whole of H
-    __nv_bfloat16* lup = reinterpret_cast<__nv_bfloat16*>(hfull + 1024);
-    float* hp = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(lup) + ST_LUP_BYTES);   // [nw][16][16]
-    float* recv_h = hp + nw * 256;                         // [ks][16][16]
-    float* recv_part = recv_h + p.ks * 256;                // [ks][KH][sl][16]
-    RecvLayout rl;
-    rl.part_addr = s_u32(recv_part); rl.h_addr = s_u32(recv_h); rl.sls = p.sls; rl.khs = p.khs;
-
-    // ---- the copy side of this warp: blocks wb0 .. wb1 - 1 in order, NS ahead of the arithmetic ----
-    const int i_row = lane >> 3, i_ch = lane & 7;
-    const bool i_col_ok = col0 + 4 * i_ch < p.N;
-    const uint32_t* i_src = p.Q + (size_t)(wb0 * F::ROWS + i_row) * p.N + col0 + 4 * i_ch;   // row i_row of block wb0
-    const size_t i_stride = (size_t)F::ROWS * p.N;
-    const uint32_t i_dst = s_u32(ring) + st_swz(i_row, i_ch);
-    const bool i_sz_lane = lane < 8 && col0 + 8 * (lane & 3) < p.N;
-    const __half* i_sz = (lane < 4 ? p.scales : p.zeros) + col0 + 8 * (lane & 3);
-    int i_blk = wb0, i_gpos = wb0 % bpg, i_slot = 0;
-    bool i_first = true;
-    auto issue = [&]() {
-        if (i_blk < wb1) {
-            const uint32_t dst = i_dst + i_slot * F::SLOT;
-            if (BITS != 3 || i_row < 3) {
-                const bool ok = i_col_ok && (BITS != 2 || i_blk * F::ROWS + i_row < (p.K >> 4));
-                cp16(dst, ok ? i_src : p.Q, ok ? 16 : 0);
-                if (BITS == 8) cp16(dst + 512, i_col_ok ? i_src + 4 * (size_t)p.N : p.Q, i_col_ok ? 16 : 0);
-            }
-            if ((i_gpos == 0 || i_first) && lane < 8)      // first block of a group in this part: its scales and zeros
-                cp16(s_u32(ring) + i_slot * F::SLOT + F::ROWS * 128 + lane * 16, i_sz_lane ? i_sz + (size_t)(i_blk / bpg) * p.N : p.scales,
-                     i_sz_lane ? 16 : 0);
-            i_first = false;
-            i_src += i_stride;
-            ++i_blk;
-            if (++i_gpos == bpg) i_gpos = 0;
-        }
-        if (++i_slot == F::NS) i_slot = 0;
-        cp_commit();
-    };
 #pragma unroll 1
-    for (int it = 0; it < F::NS; ++it) issue();            // frozen weights only: in flight while the predecessor finishes
-    {   // ask the lines this CTA will read right after the wait into L2: its slices of X, A and B
-        const int k_lo = kb0 << LKB, kbytes = (min(kb1 << LKB, p.K) - k_lo) * 2;
-        const int lines = (kbytes + 127) >> 7, rows = p.M + ((p.r > 0 && p.fused) ? p.r : 0);
-        for (int e = tid; e < rows * lines; e += nthr) {
-            const int rr = e / lines, i = e - rr * lines;
-            const __nv_bfloat16* base = rr < p.M ? p.In + (size_t)rr * p.K : p.Ldown + (size_t)(rr - p.M) * p.K;
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(base + k_lo) + (size_t)i * 128));
+    for (int e = tid; e < p.M << (p.lsl - 1); e += ST_THREADS) {          // two columns per thread
+        const int c = 2 * (e & ((sl >> 1) - 1)), tok = e >> (p.lsl - 1), col = c_lo + c;
+        float v0 = 0.f, v1 = 0.f, l0 = 0.f, l1 = 0.f;
+#pragma unroll 4
+        for (int i = 0; i < nsrc; ++i) {
+            const float2 x = *reinterpret_cast<const float2*>(src + (((i * p.M + tok) << p.lsl) + c));
+            v0 += x.x; v1 += x.y;
         }
-        const int c_lo = blockIdx.y * tile_c + rank * sl;
-        if (p.r > 0 && c_lo < p.N && tid * 64 < min(sl, p.N - c_lo) * p.r)
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(p.Lup + (size_t)c_lo * p.r + tid * 64));
+#pragma unroll 4
+        for (int j = 0; j < p.r; ++j) {
+            const float h = hfull[tok * hs + j];
+            l0 = fmaf(h, __bfloat162float(TRANSPOSED ? lup[j * sl + c] : lup[c * p.r + j]), l0);
+            l1 = fmaf(h, __bfloat162float(TRANSPOSED ? lup[j * sl + c + 1] : lup[(c + 1) * p.r + j]), l1);
+        }
+        if (p.r > 0) { v0 += p.s * l0; v1 += p.s * l1; }
+        if (col < p.C) *reinterpret_cast<uint32_t*>(p.Out + (size_t)tok * p.C + col) = st_pack(v0, v1);   // (C is a multiple of 8)
+    }
+}
+
+// ------------------------------------------------------------------------------------------------------------
+// Forward: Y = X W^T + s H B^T.  CTA (rank, tile): columns [32 wc tile, + 32 wc), contraction chunks [c0, c1) of 128 elements.
+// Warp (cg, part): 32 columns and its share of the chunks.  GPC: scale segments per chunk -- 1 for groups that are multiples of
+// 128, 2 for multiples of 64, 4 for multiples of 32 (the segment, not the group, is what one accumulator spans).
+// ------------------------------------------------------------------------------------------------------------
+template <int BITS, int NT, int GPC>
+__global__ void __launch_bounds__(ST_THREADS, 2) stream_fwd_kernel(const StreamParams p) {
+    using F = Fmt<BITS>;
+    constexpr int TOKS = 8 * NT, SB = 2;                   // SB: slices of the staging pass whose loads a warp has in flight
+    pdl_launch_dependents();
+    if (p.ks > 1) st_cluster_arrive_relaxed();             // waited for before the first store into a peer's shared memory
+    extern __shared__ __align__(128) uint8_t smem[];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, q = lane & 3;
+    const int tile_c = 32 * p.wc, cg = warp & (p.wc - 1), part = warp >> p.lwc;
+    const int rank = p.ks > 1 ? (int)st_cluster_rank() : 0;
+    const int tile_c0 = (int)blockIdx.y * tile_c, c_lo = tile_c0 + (rank << p.lsl);
+    const int nch = (p.K + ST_CHUNK - 1) / ST_CHUNK;
+    const int c0 = (nch * rank) >> p.lks, c1 = (nch * (rank + 1)) >> p.lks;
+    const int w0 = c0 + (((c1 - c0) * part) >> p.lwp), w1 = c0 + (((c1 - c0) * (part + 1)) >> p.lwp);
+    const SmemPlan sp = st_plan(p, false, TOKS, tile_c);
+    uint8_t* xs = smem;                                    // [M][pitch] activations in fragment order
+    const __half* sz = reinterpret_cast<const __half*>(smem + sp.sz);       // [group][scales, zeros][tile_c]
+    float* xsum = reinterpret_cast<float*>(smem + sp.sums);                 // [slice of 32][TOKS]
+    float* hp = reinterpret_cast<float*>(smem + sp.hp);
+    float* hfull = reinterpret_cast<float*>(smem + sp.hfull);
+
+    // ---- frozen weights only: in flight while the predecessor finishes ----
+    const int rows_total = p.K * BITS / 32;
+    const int row_a = BITS == 3 ? (24 * q) >> 5 : q, row_b = BITS == 3 ? (24 * q + 23) >> 5 : q + 4;   // of a block
+    const int col = tile_c0 + 32 * cg + 4 * g;
+    const uint32_t* qcol = p.Q + (col < p.N ? col : 0);    // (a column beyond the last loads another one's words and is dropped)
+    auto load_chunk = [&](uint4 (&w)[F::LPC], int ch) {
+        if (ch >= w1) return;
+        const int r0 = ch * (4 * BITS), last = rows_total - 1;
+        const bool full = (ch + 1) * ST_CHUNK <= p.K;       // (rows beyond the last: any words will do, their activations are zero)
+#pragma unroll
+        for (int b = 0; b < F::BPC; ++b) {
+            int ra = r0 + b * (F::KB * BITS / 32) + row_a;
+            if (!full) ra = min(ra, last);
+            ldg_words(w[b * F::NLD], qcol + (size_t)ra * p.N);
+            if constexpr (F::NLD == 2) {
+                int rb = r0 + b * (F::KB * BITS / 32) + row_b;
+                if (!full) rb = min(rb, last);
+                ldg_words(w[b * F::NLD + 1], qcol + (size_t)rb * p.N);
+            }
+        }
+    };
+    uint4 w[F::DEPTH][F::LPC];
+#pragma unroll
+    for (int d = 0; d < F::DEPTH; ++d) load_chunk(w[d], w0 + d);
+    const int g_first = st_group(p, c0 * (ST_CHUNK / 32));
+    {
+        const int g_last = c1 > c0 ? st_group(p, min(c1 * (ST_CHUNK / 32), p.K >> 5) - 1) : g_first - 1;
+        const int lper = p.lwc + 2, n = (g_last - g_first + 1) << (lper + 1);             // 16-byte pieces
+        for (int e = tid; e < n; e += ST_THREADS) {
+            const int row = e >> lper, c = tile_c0 + 8 * (e & ((1 << lper) - 1));
+            const __half* src = ((row & 1) ? p.zeros : p.scales) + (size_t)(g_first + (row >> 1)) * p.N + c;
+            cp16(s_u32(sz) + e * 16, c < p.N ? src : p.scales, c < p.N ? 16 : 0);
+        }
+    }
+    constexpr int SEG_K = ST_CHUNK / GPC, SEG_B = F::BPC / GPC;             // contraction elements and blocks of a segment
+    const int spg = p.gd / (SEG_K / 32);                                    // segments per group
+    const int g_w0 = st_group(p, w0 * (ST_CHUNK / 32));
+    int gpos = w0 * GPC - g_w0 * spg;
+    const __half* sz_lane = sz + (g_w0 - g_first) * 2 * tile_c + 32 * cg + 4 * g;
+    const int k_lo = c0 * ST_CHUNK, n_slices = (c1 - c0) * (ST_CHUNK / 32), n_valid = min(n_slices, (p.K - k_lo) >> 5);
+    {   // ask the lines this CTA will read right after the wait into L2 (nothing is read into the SM): its slices of X, A and B
+        const int rows = p.M + (p.fused ? p.r : 0);
+        for (int j = warp; j < rows; j += ST_WARPS) {
+            const __nv_bfloat16* base = (j < p.M ? p.In + (size_t)j * p.K : p.Ldown + (size_t)(j - p.M) * p.K) + k_lo;
+            for (int l = lane; 2 * l < n_valid; l += 32) prefetch_l2(base + 64 * l);
+        }
+        if (tid * 64 < min(1 << p.lsl, p.N - c_lo) * p.r) prefetch_l2(p.Lup + (size_t)c_lo * p.r + tid * 64);
     }
 
     pdl_wait();
 
-    // ---- LoRA: this CTA's part of H = X A^T (k16 steps dealt to the warps, operands straight from global memory); the
-    // loads of the first ST_HSTEPS steps are issued here and used once the activation slice is on its way too ----
-    const bool fused = p.r > 0 && p.fused;
-    const int h_k0 = (kb0 << LKB) + 16 * warp, h_ke = min(kb1 << LKB, p.K);
-    uint32_t ha[ST_HSTEPS][4], hb[ST_HSTEPS][NT][2];
-    auto h_load = [&](int kk) {
-        const __nv_bfloat16* a_lo = p.Ldown + (size_t)g * p.K + 2 * q;
-        const __nv_bfloat16* a_hi = a_lo + 8 * (size_t)p.K;
-        const __nv_bfloat16* x_lo = p.In + (size_t)g * p.K + 2 * q;
+    // ---- staging: activations into fragment order, their sums, and this CTA's part of H = X A^T ----
+    const bool tok_ok[2] = {g < p.M, g + 8 < p.M};
+    {
+        bool first = true;                                 // (every warp stages its share of the second adapter once)
+        float hacc[NT][4];
 #pragma unroll
-        for (int h = 0; h < ST_HSTEPS; ++h) {
-            const int k0 = kk + 16 * nw * h;
-            const bool in = k0 < h_ke;
-            ha[h][0] = (in && g < p.r) ? ldg32(a_lo + k0) : 0u; ha[h][2] = (in && g < p.r) ? ldg32(a_lo + k0 + 8) : 0u;
-            ha[h][1] = (in && g + 8 < p.r) ? ldg32(a_hi + k0) : 0u; ha[h][3] = (in && g + 8 < p.r) ? ldg32(a_hi + k0 + 8) : 0u;
+        for (int tt = 0; tt < NT; ++tt) hacc[tt][0] = hacc[tt][1] = hacc[tt][2] = hacc[tt][3] = 0.f;
+        const __nv_bfloat16* xr = p.In + (size_t)g * p.K + k_lo + 8 * q;
+        const __nv_bfloat16* ar = p.Ldown + (size_t)g * p.K + k_lo + 8 * q;
+        const bool a_lo = p.fused && g < p.r, a_hi = p.fused && g + 8 < p.r;
+#pragma unroll 1
+        for (int s0 = warp; s0 < n_slices || first; s0 += SB * ST_WARPS) {
+            uint4 xv[SB][NT], al[SB], ah[SB];
 #pragma unroll
-            for (int tt = 0; tt < NT; ++tt) {
-                const bool tin = in && g + 8 * tt < p.M;
-                hb[h][tt][0] = tin ? ldg32(x_lo + 8 * tt * (size_t)p.K + k0) : 0u;
-                hb[h][tt][1] = tin ? ldg32(x_lo + 8 * tt * (size_t)p.K + k0 + 8) : 0u;
+            for (int s = 0; s < SB; ++s) {
+                const int sl = s0 + s * ST_WARPS;
+                const bool in = sl < n_valid;              // (slices of a last chunk that is not full are zero)
+#pragma unroll
+                for (int tt = 0; tt < NT; ++tt) xv[s][tt] = ldg16(xr + 8 * tt * (size_t)p.K + 32 * sl, in && tok_ok[tt]);
+                al[s] = ldg16(ar + 32 * sl, in && a_lo);
+                ah[s] = ldg16(ar + 8 * (size_t)p.K + 32 * sl, in && a_hi);
+            }
+            if (first) st_stage_lup<false>(p, smem + sp.lup, hfull, c_lo);   // (with the first loads on their way)
+            first = false;
+#pragma unroll
+            for (int s = 0; s < SB; ++s) {
+                const int sl = s0 + s * ST_WARPS;
+                if (sl >= n_slices) break;
+#pragma unroll
+                for (int tt = 0; tt < NT; ++tt) {
+                    const uint4 v = xv[s][tt];
+                    st_mma(hacc[tt], al[s].x, ah[s].x, al[s].y, ah[s].y, v.x, v.y);
+                    st_mma(hacc[tt], al[s].z, ah[s].z, al[s].w, ah[s].w, v.z, v.w);
+                    const float sum = st_quad_sum(st_sum8(v));
+                    if (q == 0) xsum[sl * TOKS + 8 * tt + g] = sum;
+                    uint4 o;
+                    if constexpr (BITS == 2) {             // (x0,x8) (x1,x9) ... (x7,x15) of 16 elements = two lanes
+                        const uint32_t s0v = (q & 1) ? v.x : v.z, s1v = (q & 1) ? v.y : v.w;
+                        const uint32_t r0v = __shfl_xor_sync(0xffffffffu, s0v, 1), r1v = __shfl_xor_sync(0xffffffffu, s1v, 1);
+                        const uint32_t a0 = (q & 1) ? r0v : v.x, a1 = (q & 1) ? r1v : v.y, b0 = (q & 1) ? v.z : r0v, b1 = (q & 1) ? v.w : r1v;
+                        o = make_uint4(__byte_perm(a0, b0, 0x5410), __byte_perm(a0, b0, 0x7632), __byte_perm(a1, b1, 0x5410), __byte_perm(a1, b1, 0x7632));
+                    } else if constexpr (BITS == 8) {
+                        o = v;
+                    } else {                               // (x0,x4) (x1,x5) (x2,x6) (x3,x7)
+                        o = make_uint4(__byte_perm(v.x, v.z, 0x5410), __byte_perm(v.x, v.z, 0x7632), __byte_perm(v.y, v.w, 0x5410), __byte_perm(v.y, v.w, 0x7632));
+                    }
+                    if (tok_ok[tt]) *reinterpret_cast<uint4*>(xs + (g + 8 * tt) * p.pitch + sl * 64 + q * 16) = o;
+                }
             }
         }
-    };
-    if (fused) h_load(h_k0);
-    st_stage_lup<false>(p, lup, hfull, tile_c, rank);
+        if (p.fused) st_store_hp<NT>(p, hacc, hp, warp, g, q);
+    }
+    cp_wait_all();
+    __syncthreads();
+    const uint32_t recv_h_addr = s_u32(smem + sp.recv_h);
+    if (p.ks > 1) st_cluster_wait();                       // every CTA of the cluster is running: its shared memory may be written
+    if (p.fused) st_share_h(p, hp, recv_h_addr, rank);
 
     // ---- main loop ----
-    float acc[2][NT][4], grp[2][NT][4];
+    float acc[2][NT][4];
 #pragma unroll
     for (int u = 0; u < 2; ++u)
 #pragma unroll
-        for (int tt = 0; tt < NT; ++tt)
+        for (int tt = 0; tt < NT; ++tt) acc[u][tt][0] = acc[u][tt][1] = acc[u][tt][2] = acc[u][tt][3] = 0.f;
+    const uint32_t xl = s_u32(xs) + (uint32_t)(g * p.pitch + q * (BITS == 2 ? 32 : (BITS == 8 ? 8 : 16)));
+    uint32_t xf[NT][F::NPAIR];                             // activation fragments: token g (+ 8), this lane's quarter of a block
 #pragma unroll
-            for (int e = 0; e < 4; ++e) acc[u][tt][e] = grp[u][tt][e] = 0.f;
-    float sc[4] = {0.f, 0.f, 0.f, 0.f}, cz[4] = {0.f, 0.f, 0.f, 0.f};   // this lane's four columns: scale, -scale (OFF + zero)
-    int c_slot = 0;
-    const int lcpt = 31 - __clz(p.xc / KP), lcpp = lcpt - p.khs;          // log2: items per token row, per part of it
-    const int npass = (((nb + KH - 1) >> p.khs) + xpb - 1) / xpb;
-    if (npass == 0) st_cluster_wait();                     // (an empty range: the wait below is never reached)
-    for (int ps = 0; ps < npass; ++ps) {
-        // this warp's blocks of the pass, and what the staging needs to know about every part
-        const int pb0 = min(wb0 + ps * xpb, wb1), pb1 = min(wb1, pb0 + xpb);
-        const int wk0 = pb0 << LKB, wk1 = min(pb1 << LKB, p.K);
-        const int gf = wk0 / p.g;
-        if (cg == 0 && lane == 0) { tab[kh].k0 = wk0; tab[kh].k1 = wk1; tab[kh].gf = gf; tab[kh].nseg = wk1 > wk0 ? (wk1 - 1) / p.g - gf + 1 : 0; }
-        // stage the activations: permuted for the fragment loads, plus the sums the zero-points need
-        {
-            constexpr int NB = BITS == 2 ? 2 : 4;          // items per round, their loads issued together
-            const int n_items = TOKS << lcpt;
-            for (int e0 = tid; e0 < n_items; e0 += NB * nthr) {
-                uint4 v0[NB], v1[NB];
-                int tk[NB], ci[NB];
+    for (int tt = 0; tt < NT; ++tt)
 #pragma unroll
-                for (int j = 0; j < NB; ++j) {
-                    const int e = e0 + j * nthr;
-                    tk[j] = e >> lcpt; ci[j] = e & ((1 << lcpt) - 1);
-                    const int h = ci[j] >> lcpp, cl = ci[j] & ((1 << lcpp) - 1);
-                    const int hb0 = kb0 + ((nb * h) >> p.khs), hb1 = kb0 + ((nb * (h + 1)) >> p.khs);
-                    const int k = (min(hb0 + ps * xpb, hb1) << LKB) + cl * KP, kend = min(min(hb1, hb0 + (ps + 1) * xpb) << LKB, p.K);
-                    v0[j] = make_uint4(0, 0, 0, 0); v1[j] = make_uint4(0, 0, 0, 0);
-                    if (e < n_items && tk[j] < p.M && k < kend) {
-                        v0[j] = *reinterpret_cast<const uint4*>(p.In + (size_t)tk[j] * p.K + k);
-                        if (KP == 16 && k + 8 < kend) v1[j] = *reinterpret_cast<const uint4*>(p.In + (size_t)tk[j] * p.K + k + 8);
-                    }
-                }
+        for (int i = 0; i < F::NPAIR; ++i) xf[tt][i] = 0u; // (stays zero for tokens that do not exist)
+    auto compute = [&](const uint4 (&wd)[F::LPC], int ch) {
+        const uint32_t xc = xl + (uint32_t)(ch - c0) * (ST_CHUNK * 2);
+        const float* sumc = xsum + (ch - c0) * (ST_CHUNK / 32) * TOKS + 2 * q;
 #pragma unroll
-                for (int j = 0; j < NB; ++j) {
-                    if (e0 + j * nthr >= n_items) break;
-                    uint8_t* dst = xs + tk[j] * xp + ci[j] * (2 * KP);
-                    if constexpr (BITS == 2) {             // (x0,x8) (x1,x9) ... (x7,x15)
-                        *reinterpret_cast<uint4*>(dst) = make_uint4(__byte_perm(v0[j].x, v1[j].x, 0x5410), __byte_perm(v0[j].x, v1[j].x, 0x7632),
-                                                                    __byte_perm(v0[j].y, v1[j].y, 0x5410), __byte_perm(v0[j].y, v1[j].y, 0x7632));
-                        *reinterpret_cast<uint4*>(dst + 16) = make_uint4(__byte_perm(v0[j].z, v1[j].z, 0x5410), __byte_perm(v0[j].z, v1[j].z, 0x7632),
-                                                                         __byte_perm(v0[j].w, v1[j].w, 0x5410), __byte_perm(v0[j].w, v1[j].w, 0x7632));
-                        sxc[tk[j] * (p.xc >> 3) + 2 * ci[j]] = st_sum8(v0[j]);
-                        sxc[tk[j] * (p.xc >> 3) + 2 * ci[j] + 1] = st_sum8(v1[j]);
+        for (int sg = 0; sg < GPC; ++sg) {
+            if (GPC > 1 && ch * ST_CHUNK + sg * SEG_K >= p.K) break;        // (a last chunk that is not full: no such group)
+            float grp[2][NT][4];
+#pragma unroll
+            for (int u = 0; u < 2; ++u)
+#pragma unroll
+                for (int tt = 0; tt < NT; ++tt) grp[u][tt][0] = grp[u][tt][1] = grp[u][tt][2] = grp[u][tt][3] = 0.f;
+#pragma unroll
+            for (int bs = 0; bs < SEG_B; ++bs) {
+                const int b = sg * SEG_B + bs;
+#pragma unroll
+                for (int tt = 0; tt < NT; ++tt) {
+                    const uint32_t x = xc + (uint32_t)(8 * tt * p.pitch + b * (F::KB * 2));
+                    if constexpr (BITS == 8) {
+                        lds8(xf[tt][0], xf[tt][1], x, tok_ok[tt]);
+                        lds8(xf[tt][2], xf[tt][3], x + 32, tok_ok[tt]);
                     } else {
-                        *reinterpret_cast<uint4*>(dst) = BITS == 8 ? v0[j] : st_permute8(v0[j]);
-                        sxc[tk[j] * (p.xc >> 3) + ci[j]] = st_sum8(v0[j]);
+#pragma unroll
+                        for (int h = 0; h < F::NPAIR / 4; ++h) lds16(xf[tt][4 * h], xf[tt][4 * h + 1], xf[tt][4 * h + 2], xf[tt][4 * h + 3], x + 16 * h, tok_ok[tt]);
                     }
                 }
-            }
-            if (ps == 0 && fused) {                        // the down-projection's MMAs, with the activations' loads behind them
-                float ah[NT][4];
+                uint32_t pc[4][F::NPAIR];                  // [column i of the lane's four][pair]
 #pragma unroll
-                for (int tt = 0; tt < NT; ++tt) ah[tt][0] = ah[tt][1] = ah[tt][2] = ah[tt][3] = 0.f;
-                for (int kk = h_k0;;) {
+                for (int i = 0; i < 4; ++i) st_unpack<BITS>(st_comp(wd[b * F::NLD], i), F::NLD > 1 ? st_comp(wd[b * F::NLD + F::NLD - 1], i) : 0u, q, pc[i]);
+                // two tiles of 16 columns: rows g / g + 8 of tile u are columns 4g + 2u / 4g + 2u + 1
 #pragma unroll
-                    for (int h = 0; h < ST_HSTEPS; ++h)
+                for (int s = 0; s < F::STEPS; ++s)
 #pragma unroll
-                        for (int tt = 0; tt < NT; ++tt) st_mma(ah[tt], ha[h][0], ha[h][1], ha[h][2], ha[h][3], hb[h][tt][0], hb[h][tt][1]);
-                    kk += 16 * nw * ST_HSTEPS;
-                    if (kk >= h_ke) break;
-                    h_load(kk);
-                }
-                st_store_hp<NT>(ah, hp, warp, g, q);
+                    for (int u = 0; u < 2; ++u)
+#pragma unroll
+                        for (int tt = 0; tt < NT; ++tt)
+                            st_mma(grp[u][tt], pc[2 * u][2 * s], pc[2 * u + 1][2 * s], pc[2 * u][2 * s + 1], pc[2 * u + 1][2 * s + 1], xf[tt][2 * s], xf[tt][2 * s + 1]);
             }
-            __syncthreads();
-            {   // sums per (part, group segment): four lanes per (token, segment), segments numbered through the parts
-                int n_all = 0;
-                for (int h = 0; h < KH; ++h) n_all += tab[h].nseg;
-                const int total = n_all << LTOKS;
-                for (int base = 0; base < total; base += nthr >> 2) {      // the same trip count for every thread
-                    const int task = base + (tid >> 2), sub = tid & 3;
-                    const bool on = task < total;
-                    const int tok = task & (TOKS - 1);
-                    int h = 0, sg = on ? task >> LTOKS : 0;
-                    while (on && sg >= tab[h].nseg) { sg -= tab[h].nseg; ++h; }
-                    const PartInfo pi = tab[h];
-                    const int a = max(pi.k0, (pi.gf + sg) * p.g), b = min(pi.k1, (pi.gf + sg + 1) * p.g);
-                    const float* src = sxc + tok * (p.xc >> 3) + ((h << lcpp) * KP + (a - pi.k0)) / 8;
-                    float sum = 0.f;
-                    if (on)
-                        for (int c8 = sub; c8 < (b - a) >> 3; c8 += 4) sum += src[c8];
-                    sum += __shfl_xor_sync(0xffffffffu, sum, 1);
-                    sum += __shfl_xor_sync(0xffffffffu, sum, 2);
-                    if (on && sub == 0) sxs[(h * (xpb + 1) + sg) * TOKS + tok] = sum;
-                }
-            }
-            if (ps == 0 && fused) {
-                for (int e = tid; e < 256; e += nthr) {
-                    float h = 0.f;
-                    for (int w = 0; w < nw; ++w) h += hp[w * 256 + e];
-                    hs[e] = h;
-                }
-            }
-            __syncthreads();
-            if (ps == 0) {
-                st_cluster_wait();                         // every CTA of the cluster is running: its shared memory may be written
-                if (fused) st_push_h(rl, hs, rank, p.ks);
-            }
-        }
-        int gpos = pb0 - gf * bpg, grpi = gf;
-        const uint8_t* xw = xs + (kh * xpb << (LKB + 1)) + (BITS == 2 ? 32 * q : (BITS == 8 ? 8 * q : 16 * q)) + g * xp;
-#pragma unroll 2
-        for (int blk = pb0; blk < pb1; ++blk) {
-            cp_wait<F::NS - 1>();
-            __syncwarp();
-            const uint8_t* slot = ring + c_slot * F::SLOT;
-            if (gpos == 0 || blk == wb0) {                 // a new group: this lane's scales and zero-points
-                const uint2 s2 = *reinterpret_cast<const uint2*>(slot + F::ROWS * 128 + 8 * g);
-                const uint2 z2 = *reinterpret_cast<const uint2*>(slot + F::ROWS * 128 + 64 + 8 * g);
-                const float2 sa = __half22float2(*reinterpret_cast<const __half2*>(&s2.x)), sb = __half22float2(*reinterpret_cast<const __half2*>(&s2.y));
-                const float2 za = __half22float2(*reinterpret_cast<const __half2*>(&z2.x)), zb = __half22float2(*reinterpret_cast<const __half2*>(&z2.y));
-                sc[0] = sa.x; sc[1] = sa.y; sc[2] = sb.x; sc[3] = sb.y;
-                cz[0] = -sa.x * (F::OFF + za.x); cz[1] = -sa.y * (F::OFF + za.y); cz[2] = -sb.x * (F::OFF + zb.x); cz[3] = -sb.y * (F::OFF + zb.y);
-            }
-            uint4 w[F::NLD];
-            st_load_words<BITS>(slot, g, q, w);
-            // activation fragments: token g (+ 8), this lane's quarter of the block
-            uint32_t xf[NT][F::NPAIR];
-            const uint8_t* xb = xw + ((blk - pb0) << (LKB + 1));
+            // end of a segment: scale, correct for offset and zero-point
+            const uint2 s2 = *reinterpret_cast<const uint2*>(sz_lane), z2 = *reinterpret_cast<const uint2*>(sz_lane + tile_c);
+            const float2 sa = __half22float2(*reinterpret_cast<const __half2*>(&s2.x)), sb = __half22float2(*reinterpret_cast<const __half2*>(&s2.y));
+            const float2 za = __half22float2(*reinterpret_cast<const __half2*>(&z2.x)), zb = __half22float2(*reinterpret_cast<const __half2*>(&z2.y));
+            const float sc[4] = {sa.x, sa.y, sb.x, sb.y};
+            const float oz[4] = {F::OFF + za.x, F::OFF + za.y, F::OFF + zb.x, F::OFF + zb.y};
 #pragma unroll
             for (int tt = 0; tt < NT; ++tt) {
-                const uint8_t* xr = xb + 8 * tt * xp;
-                if constexpr (BITS == 2) {
-                    const uint4 v0 = *reinterpret_cast<const uint4*>(xr);
-                    const uint4 v1 = *reinterpret_cast<const uint4*>(xr + 16);
-                    xf[tt][0] = v0.x; xf[tt][1] = v0.y; xf[tt][2] = v0.z; xf[tt][3] = v0.w;
-                    xf[tt][4] = v1.x; xf[tt][5] = v1.y; xf[tt][6] = v1.z; xf[tt][7] = v1.w;
-                } else if constexpr (BITS == 8) {
-                    const uint2 v0 = *reinterpret_cast<const uint2*>(xr);
-                    const uint2 v1 = *reinterpret_cast<const uint2*>(xr + 32);
-                    xf[tt][0] = v0.x; xf[tt][1] = v0.y; xf[tt][2] = v1.x; xf[tt][3] = v1.y;
-                } else {
-                    const uint4 v0 = *reinterpret_cast<const uint4*>(xr);
-                    xf[tt][0] = v0.x; xf[tt][1] = v0.y; xf[tt][2] = v0.z; xf[tt][3] = v0.w;
+                float sx0 = 0.f, sx1 = 0.f;
+#pragma unroll
+                for (int i = 0; i < SEG_K / 32; ++i) {
+                    const float2 v = *reinterpret_cast<const float2*>(sumc + (sg * (SEG_K / 32) + i) * TOKS + 8 * tt);
+                    sx0 += v.x; sx1 += v.y;
                 }
-            }
-            // two tiles of 16 columns: rows g / g + 8 of tile u are columns 4g + 2u / 4g + 2u + 1
-            uint32_t pc[4][F::NPAIR];                      // [column i of the lane's four][pair]
-#pragma unroll
-            for (int i = 0; i < 4; ++i) st_unpack<BITS>(st_comp(w[0], i), F::NLD > 1 ? st_comp(w[F::NLD - 1], i) : 0u, q, pc[i]);
-#pragma unroll
-            for (int s = 0; s < F::STEPS; ++s)             // MMAs into the same accumulator are 2 NT instructions apart
 #pragma unroll
                 for (int u = 0; u < 2; ++u)
 #pragma unroll
-                    for (int tt = 0; tt < NT; ++tt)
-                        st_mma(grp[u][tt], pc[2 * u][2 * s], pc[2 * u + 1][2 * s], pc[2 * u][2 * s + 1], pc[2 * u + 1][2 * s + 1], xf[tt][2 * s], xf[tt][2 * s + 1]);
-            if (gpos == bpg - 1 || blk + 1 == pb1) {       // end of a group segment: scale, correct, start afresh
-                const float* sxr = sxs + (kh * (xpb + 1) + grpi - gf) * TOKS + 2 * q;
-#pragma unroll
-                for (int tt = 0; tt < NT; ++tt) {
-                    const float2 sx = *reinterpret_cast<const float2*>(sxr + 8 * tt);
-#pragma unroll
-                    for (int u = 0; u < 2; ++u) {
-                        acc[u][tt][0] += sc[2 * u] * grp[u][tt][0] + cz[2 * u] * sx.x;
-                        acc[u][tt][1] += sc[2 * u] * grp[u][tt][1] + cz[2 * u] * sx.y;
-                        acc[u][tt][2] += sc[2 * u + 1] * grp[u][tt][2] + cz[2 * u + 1] * sx.x;
-                        acc[u][tt][3] += sc[2 * u + 1] * grp[u][tt][3] + cz[2 * u + 1] * sx.y;
-                        grp[u][tt][0] = grp[u][tt][1] = grp[u][tt][2] = grp[u][tt][3] = 0.f;
+                    for (int h = 0; h < 2; ++h) {
+                        acc[u][tt][2 * h] = fmaf(sc[2 * u + h], fmaf(-oz[2 * u + h], sx0, grp[u][tt][2 * h]), acc[u][tt][2 * h]);
+                        acc[u][tt][2 * h + 1] = fmaf(sc[2 * u + h], fmaf(-oz[2 * u + h], sx1, grp[u][tt][2 * h + 1]), acc[u][tt][2 * h + 1]);
                     }
-                }
             }
-            if (++gpos == bpg) { gpos = 0; ++grpi; }
-            if (++c_slot == F::NS) c_slot = 0;
-            __syncwarp();
-            issue();
+            if (++gpos == spg) { gpos = 0; sz_lane += 2 * tile_c; }
         }
-        if (ps + 1 < npass) __syncthreads();               // the staged activations may be overwritten
+    };
+#pragma unroll 1
+    for (int ch = w0; ch < w1; ch += F::DEPTH) {
+#pragma unroll
+        for (int d = 0; d < F::DEPTH; ++d) {
+            if (ch + d < w1) {
+                compute(w[d], ch + d);
+                load_chunk(w[d], ch + d + F::DEPTH);
+            }
+        }
     }
-    // accumulator element (u, tt, e): column 4g + 2u + (e >> 1) of this warp's 32, token 2q + (e & 1) + 8 tt; sent to the
-    // CTA that finishes that column
+    // accumulator element (u, tt, e): column 4g + 2u + (e >> 1) of this warp's 32, token 2q + (e & 1) + 8 tt
+    float* mine = reinterpret_cast<float*>(smem + sp.part) + part * p.M * tile_c + 32 * cg + 4 * g;
 #pragma unroll
-    for (int u = 0; u < 2; ++u)
+    for (int tt = 0; tt < NT; ++tt)
 #pragma unroll
-        for (int tt = 0; tt < NT; ++tt) {
-            st_push2(rl, rank, kh, 32 * cg + 4 * g + 2 * u, 2 * q + 8 * tt, acc[u][tt][0], acc[u][tt][1]);
-            st_push2(rl, rank, kh, 32 * cg + 4 * g + 2 * u + 1, 2 * q + 8 * tt, acc[u][tt][2], acc[u][tt][3]);
+        for (int e = 0; e < 2; ++e) {
+            const int tok = 8 * tt + 2 * q + e;
+            if (tok < p.M) *reinterpret_cast<float4*>(mine + tok * tile_c) = make_float4(acc[0][tt][e], acc[0][tt][2 + e], acc[1][tt][e], acc[1][tt][2 + e]);
         }
-    st_finish<false, TOKS>(p, recv_part, recv_h, hfull, lup, tile_c, rank);
+    st_finish<false>(p, smem, sp, c_lo, rank, blockIdx.y == 0 && rank == 0);
 }
 
 // ------------------------------------------------------------------------------------------------------------
-// Backward: dX = dY W + s G A.  CTA (rank, tile): output features [FW wc tile, + FW wc), contraction stages [st0, st1)
-// of 32 SU packed columns.  Warp (fw, kh): FW features (all inside one group) and the kh-th of KH consecutive parts of
-// [st0, st1).  The slices of dY of the parts are staged side by side, xps stages of every part per pass.
+// Backward: dX = dY W + s G A.  CTA (rank, tile): output features [8 FL wc tile, + 8 FL wc), contraction units [u0, u1) of 32
+// packed columns.  Warp (fw, part): 8 FL features (all inside one group) and its share of the units.  Lane (g, q) has features
+// FL g .. FL g + FL - 1 of the warp's, columns 4q .. 4q+3 (+ 16) of a unit.  FL = 8, or 4 where groups are not multiples of 64.
 // ------------------------------------------------------------------------------------------------------------
-template <int BITS, int NT>
-__global__ void __launch_bounds__(512, 1) stream_bwd_kernel(const StreamParams p) {
+template <int BITS, int FL>
+struct BFmt {
+    static constexpr int NLD = (BITS == 3 || (BITS == 8 && FL == 8)) ? 2 : 1;   // packed rows a lane reads per column
+    static constexpr int DEPTH = 4;                                             // units in flight per warp: 32 or 64 registers, 4 KB
+};
+
+// FL features of two neighbouring columns (words a0 / a1 and b0 / b1) -> pairs (column a, column b) of OFF + q per feature.
+template <int BITS, int FL>
+__device__ __forceinline__ void st_bwd_pairs(uint32_t a0, uint32_t a1, uint32_t b0, uint32_t b1, uint32_t sh, uint32_t sel, uint32_t (&p)[FL]) {
+    if constexpr (BITS == 8) {
+#pragma unroll
+        for (int t = 0; t < FL; ++t) p[t] = st_pack(st_byte(t < 4 ? a0 : a1, t & 3), st_byte(t < 4 ? b0 : b1, t & 3));
+    } else {
+        constexpr uint32_t M2 = BITS == 2 ? 0x00030003u : (BITS == 3 ? 0x00070007u : 0x000F000Fu);
+        uint32_t x, y = 0u;
+        if constexpr (BITS == 3) {
+            const uint32_t va = __funnelshift_r(a0, a1, sh), vb = __funnelshift_r(b0, b1, sh);
+            x = __byte_perm(va, vb, 0x5410);
+            if constexpr (FL == 8) y = __byte_perm(va >> 12, vb >> 12, 0x5410);
+        } else {
+            x = __byte_perm(a0, b0, sel);
+            if constexpr (BITS == 4 && FL == 8) y = __byte_perm(a0, b0, 0x7632);
+        }
+        constexpr int IN_X = BITS == 2 ? 8 : 4;
+#pragma unroll
+        for (int t = 0; t < FL; ++t) p[t] = (((t < IN_X ? x : y) >> (BITS * (t % IN_X))) & M2) | 0x43004300u;
+    }
+}
+
+template <int BITS, int NT, int FL>
+__global__ void __launch_bounds__(ST_THREADS, 2) stream_bwd_kernel(const StreamParams p) {
     using F = Fmt<BITS>;
-    constexpr int TOKS = 8 * NT;
-    constexpr int NTILE = F::BPAIR / 2;                    // 16-feature MMA tiles per warp
-    constexpr int LSW = BITS == 2 ? 7 : 5;                 // log2 of the packed columns per stage
+    using BF = BFmt<BITS, FL>;
+    constexpr int TOKS = 8 * NT, SB = 2;
     pdl_launch_dependents();
-    st_cluster_arrive_relaxed();                           // waited for before the first store into a peer's shared memory
+    if (p.ks > 1) st_cluster_arrive_relaxed();             // waited for before the first store into a peer's shared memory
     extern __shared__ __align__(128) uint8_t smem[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, q = lane & 3;
-    const int nthr = blockDim.x, nw = nthr >> 5, tile_c = F::FW * p.wc, sl = tile_c >> p.lks, KH = 1 << p.khs;
-    const int fw = warp & (p.wc - 1), kh = warp >> p.lwc;
-    const int rank = (int)st_cluster_rank();
-    const int tile_f0 = blockIdx.y * tile_c, f0 = tile_f0 + F::FW * fw;
-    const bool live = f0 < p.K;                            // a warp beyond the last feature only keeps the barriers company
-    const int row0 = f0 * BITS / 32;
-    const int nst = (p.N + (1 << LSW) - 1) >> LSW;
-    const int st0 = (nst * rank) >> p.lks, st1 = (nst * (rank + 1)) >> p.lks, ns = st1 - st0;
-    const int ws0 = st0 + ((ns * kh) >> p.khs), ws1 = st0 + ((ns * (kh + 1)) >> p.khs);
-    const int xp = p.xc * 2 + 64;
-    const int xps = (p.xc >> LSW) >> p.khs;                // stages of a part staged per pass
-    const int gk0 = tile_f0 / p.g;                         // group of the CTA's first feature
-    const int ngroups = p.K / p.g;
-    const int copy = p.copies > 1 ? (f0 - tile_f0) / p.g : 0;
-    uint8_t* ring = smem + warp * (F::BNS * F::BSLOT);
-    uint8_t* ys = smem + nw * (F::BNS * F::BSLOT);         // [copies][TOKS][xp] scaled, permuted slices of dY
-    float* zp = reinterpret_cast<float*>(ys + p.copies * TOKS * xp);   // [nw][2][16] zero-point sums, per warp
-    float* zc = zp + nw * 32;                              // [2][16] their total
-    float* hs = zc + 32;
-    float* hfull = hs + 256;
-    __nv_bfloat16* lup = reinterpret_cast<__nv_bfloat16*>(hfull + 1024);
-    float* hp = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(lup) + ST_LUP_BYTES);   // [nw][16][16]
-    float* recv_h = hp + nw * 256;                         // [ks][16][16]
-    float* recv_part = recv_h + p.ks * 256;                // [ks][KH][sl][16]
-    RecvLayout rl;
-    rl.part_addr = s_u32(recv_part); rl.h_addr = s_u32(recv_h); rl.sls = p.sls; rl.khs = p.khs;
+    const int tile_c = 8 * FL * p.wc, fw = warp & (p.wc - 1), part = warp >> p.lwc;
+    const int rank = p.ks > 1 ? (int)st_cluster_rank() : 0;
+    const int tile_f0 = (int)blockIdx.y * tile_c, c_lo = tile_f0 + (rank << p.lsl), f0 = tile_f0 + 8 * FL * fw;
+    const int nun = (p.N + 31) >> 5;
+    const int u0 = (nun * rank) >> p.lks, u1 = (nun * (rank + 1)) >> p.lks;
+    const int w0 = u0 + (((u1 - u0) * part) >> p.lwp), w1 = u0 + (((u1 - u0) * (part + 1)) >> p.lwp);
+    const int gk0 = st_group(p, tile_f0 >> 5), ngroups = st_group(p, p.K >> 5);    // group of the CTA's first feature
+    const int copy = min(st_group(p, f0 >> 5) - gk0, p.ngl - 1);
+    const SmemPlan sp = st_plan(p, true, TOKS, tile_c);
+    uint8_t* ys = smem;                                    // [groups][M][pitch] scaled slices of dY
+    const __half* sz = reinterpret_cast<const __half*>(smem + sp.sz);       // [group][scales, zeros][range]
+    float* zp = reinterpret_cast<float*>(smem + sp.sums);                   // [ST_WARPS][2][16] zero-point sums, per warp
+    float* hp = reinterpret_cast<float*>(smem + sp.hp);
+    float* hfull = reinterpret_cast<float*>(smem + sp.hfull);
 
-    // ---- the copy side of this warp: stages ws0 .. ws1 - 1 in order, BNS ahead of the arithmetic ----
-    const int i_row = BITS == 2 ? 0 : lane >> 3;
-    const int i_coff = BITS == 2 ? 32 * (lane >> 3) + 4 * (lane & 7) : 4 * (lane & 7);   // column inside the stage
-    const uint32_t* i_src = p.Q + (size_t)(row0 + i_row) * p.N;
-    const uint32_t i_dst = s_u32(ring) + (BITS == 2 ? lane * 16 : st_swz(i_row, lane & 7));
-    int i_stg = ws0, i_slot = 0;
-    auto issue = [&]() {
-        if (i_stg < ws1 && live) {
-            const uint32_t dst = i_dst + i_slot * F::BSLOT;
-            const int col = (i_stg << LSW) + i_coff;
-            const bool ok = col < p.N;
-            if (BITS != 3 || i_row < 3) {
-                cp16(dst, ok ? i_src + col : p.Q, ok ? 16 : 0);
-                if (BITS == 8) cp16(dst + 512, ok ? i_src + 4 * (size_t)p.N + col : p.Q, ok ? 16 : 0);
-            }
-            ++i_stg;
+    // ---- frozen weights only: in flight while the predecessor finishes ----
+    const int bitpos = FL * BITS * g, row = f0 * BITS / 32 + (bitpos >> 5);
+    const uint32_t sh = (uint32_t)bitpos & 31u;
+    const uint32_t byte = sh >> 3;
+    const uint32_t sel = BITS == 2 && FL == 4 ? byte * 0x0011u + (byte + 4u) * 0x1100u : (sh ? 0x7632u : 0x5410u);
+    const int rows_total = p.K * BITS / 32;
+    // (rows and columns beyond the last load other words: their results are dropped, their activations are zero)
+    const int row2 = BITS == 8 || (int)sh + FL * BITS > 32 ? row + 1 : row;
+    const uint32_t* qrow = p.Q + (size_t)min(row, rows_total - 1) * p.N;
+    const uint32_t* qrow2 = p.Q + (size_t)min(row2, rows_total - 1) * p.N;
+    auto load_unit = [&](uint4 (&w)[2 * BF::NLD], int un) {
+        if (un >= w1) return;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int n = min(32 * un + 16 * h + 4 * q, p.N - 4);
+            ldg_words(w[h * BF::NLD], qrow + n);
+            if constexpr (BF::NLD == 2) ldg_words(w[h * BF::NLD + 1], qrow2 + n);
         }
-        if (++i_slot == F::BNS) i_slot = 0;
-        cp_commit();
     };
-#pragma unroll 1
-    for (int it = 0; it < F::BNS; ++it) issue();
-
-    const int n_lo_cta = st0 << LSW, n_hi_cta = min(st1 << LSW, p.N);
-    {   // ask the lines this CTA will read right after the wait into L2: its slices of dY, B, A and of the group parameters
-        const int nbytes = (n_hi_cta - n_lo_cta) * 2, lines = (nbytes + 127) >> 7;
-        const int rows = p.M + 2 * p.copies;
-        for (int e = tid; e < rows * lines; e += nthr) {
-            const int rr = e / lines, i = e - rr * lines;
-            const char* base;
-            if (rr < p.M) base = reinterpret_cast<const char*>(p.In + (size_t)rr * p.N + n_lo_cta);
-            else {
-                const int c = (rr - p.M) >> 1, gk = min(gk0 + c, ngroups - 1);
-                base = reinterpret_cast<const char*>(((rr - p.M) & 1 ? p.zeros : p.scales) + (size_t)gk * p.N + n_lo_cta);
+    uint4 w[BF::DEPTH][2 * BF::NLD];
+#pragma unroll
+    for (int d = 0; d < BF::DEPTH; ++d) load_unit(w[d], w0 + d);
+    const int n_lo = u0 << 5, nu = u1 - u0;
+    {
+        const int per = nu * 4;                            // 16-byte pieces of a row
+        for (int rr = 0; rr < 2 * p.ngl; ++rr) {
+            const int gk = gk0 + (rr >> 1);
+            const __half* src = ((rr & 1) ? p.zeros : p.scales) + (size_t)min(gk, ngroups - 1) * p.N;
+            for (int i = tid; i < per; i += ST_THREADS) {
+                const int c = n_lo + 8 * i;
+                cp16(s_u32(sz) + (uint32_t)(rr * p.range + 8 * i) * 2u, src + min(c, p.N - 8), c < p.N ? 16 : 0);
             }
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(base + (size_t)i * 128));
         }
-        if (p.r > 0 && p.fused)
-            for (int e = tid; e * 64 < (n_hi_cta - n_lo_cta) * p.r; e += nthr)
-                asm volatile("prefetch.global.L2 [%0];" ::"l"(p.Ldown + (size_t)n_lo_cta * p.r + (size_t)e * 64));
-        const int c_lo = tile_f0 + rank * sl;
-        if (p.r > 0 && c_lo < p.K && tid < p.r) asm volatile("prefetch.global.L2 [%0];" ::"l"(p.Lup + (size_t)tid * p.K + c_lo));
+    }
+    {   // ask the lines this CTA will read right after the wait into L2 (nothing is read into the SM): its slices of dY, B and A
+        const int n = min(32 * nu, p.N - n_lo);
+        for (int j = warp; j < p.M; j += ST_WARPS)
+            for (int l = lane; 64 * l < n; l += 32) prefetch_l2(p.In + (size_t)j * p.N + n_lo + 64 * l);
+        if (p.fused)
+            for (int e = tid * 64; e < n * p.r; e += ST_THREADS * 64) prefetch_l2(p.Ldown + (size_t)n_lo * p.r + e);
+        if (tid < p.r && c_lo < p.K) prefetch_l2(p.Lup + (size_t)tid * p.K + c_lo);
     }
 
     pdl_wait();
 
-    // ---- LoRA: this CTA's part of G = dY B.  B [N, r] has the ranks contiguous, so a lane loads two ranks of its own
-    // contraction column and movmatrix turns them into two columns of one rank.  The loads of the first ST_HSTEPS steps are
-    // issued here and used once the slice of dY is on its way too ----
-    const bool fused = p.r > 0 && p.fused;
-    const int h_n0 = n_lo_cta + 16 * warp;
-    uint32_t ha[ST_HSTEPS][4], hb[ST_HSTEPS][NT][2];
-    auto h_load = [&](int nn) {
+    const bool tok_ok[2] = {g < p.M, g + 8 < p.M};
+    // ---- staging: slices of dY, scaled by each group's scales (one rounding); the zero-point sums; this CTA's part of G = dY B ----
+    {
+        float hacc[NT][4], zacc[2][NT];
 #pragma unroll
-        for (int h = 0; h < ST_HSTEPS; ++h) {
-            const int nb = nn + 16 * nw * h;
-            const bool in = nb < n_hi_cta;
-            const bool v0 = in && nb + g < p.N, v1 = in && nb + 8 + g < p.N;
-            const __nv_bfloat16* b_lo = p.Ldown + (size_t)(nb + g) * p.r + 2 * q;
-            const __nv_bfloat16* b_hi = b_lo + 8 * p.r;
-            ha[h][0] = v0 ? ldg32(b_lo) : 0u; ha[h][2] = v1 ? ldg32(b_hi) : 0u;
-            ha[h][1] = (v0 && p.r > 8) ? ldg32(b_lo + 8) : 0u; ha[h][3] = (v1 && p.r > 8) ? ldg32(b_hi + 8) : 0u;
-#pragma unroll
-            for (int tt = 0; tt < NT; ++tt) {
-                const int tok = g + 8 * tt;
-                const __nv_bfloat16* y = p.In + (size_t)tok * p.N + nb + 2 * q;
-                hb[h][tt][0] = (in && tok < p.M && nb + 2 * q < p.N) ? ldg32(y) : 0u;
-                hb[h][tt][1] = (in && tok < p.M && nb + 8 + 2 * q < p.N) ? ldg32(y + 8) : 0u;
-            }
+        for (int tt = 0; tt < NT; ++tt) {
+            hacc[tt][0] = hacc[tt][1] = hacc[tt][2] = hacc[tt][3] = 0.f;
+            zacc[0][tt] = zacc[1][tt] = 0.f;
         }
-    };
-    if (fused) h_load(h_n0);
-    st_stage_lup<true>(p, lup, hfull, tile_c, rank);
-    for (int e = tid; e < nw * 32; e += nthr) zp[e] = 0.f;
-
-    float acc[NTILE][NT][4];
+        const __nv_bfloat16* yr = p.In + (size_t)g * p.N + n_lo + 8 * q;
+        const int n_left = p.N - n_lo - 8 * q;             // columns from this lane's first on
+        bool staged = false;
+#pragma unroll 1
+        for (int s0 = warp; s0 < nu || !staged; s0 += SB * ST_WARPS) {
+            uint4 yv[SB][NT];
+            uint32_t bl[SB][4], bh[SB][4];
 #pragma unroll
-    for (int t = 0; t < NTILE; ++t)
+            for (int s = 0; s < SB; ++s) {
+                const int sl = s0 + s * ST_WARPS;
+                const bool in = sl < nu && 32 * sl < n_left;               // (N is a multiple of 8)
 #pragma unroll
-        for (int tt = 0; tt < NT; ++tt) acc[t][tt][0] = acc[t][tt][1] = acc[t][tt][2] = acc[t][tt][3] = 0.f;
-    int c_slot = 0;
-    const int lcpt = 31 - __clz(p.xc >> 3), lcpp = lcpt - p.khs;          // log2: 8-column items per token row, per part of it
-    const int npass = (((ns + KH - 1) >> p.khs) + xps - 1) / xps;
-    if (npass == 0) st_cluster_wait();                     // (an empty range: the wait below is never reached)
-    for (int ps = 0; ps < npass; ++ps) {
-        const int pb0 = min(ws0 + ps * xps, ws1), pb1 = min(ws1, pb0 + xps);     // this warp's stages of the pass
-        // stage the slices of dY, once per group the CTA's features span, scaled by that group's scales (one rounding)
-        {
-            const int n_items = TOKS << lcpt;
-            for (int e0 = tid; e0 < n_items; e0 += 2 * nthr) {                   // two items per round, loads first
-                uint4 v[2], s8[2][2];
-                int tk[2], ci[2];
+                for (int tt = 0; tt < NT; ++tt) yv[s][tt] = ldg16(yr + 8 * tt * (size_t)p.N + 32 * sl, in && tok_ok[tt]);
+                // row rho of 8 x 8 tile t <-> column 8 (rho / 2) + rho % 2 + 2 t
+                const int n8 = n_lo + 32 * sl + 8 * (g >> 1);
+                const bool on = p.fused && sl < nu && n8 < p.N;
+                const __nv_bfloat16* src = p.Ldown + (size_t)(n8 + (g & 1)) * p.r + 2 * q;
 #pragma unroll
-                for (int j = 0; j < 2; ++j) {
-                    const int e = e0 + j * nthr;
-                    tk[j] = e >> lcpt; ci[j] = e & ((1 << lcpt) - 1);
-                    const int h = ci[j] >> lcpp, cl = ci[j] & ((1 << lcpp) - 1);
-                    const int hs0 = st0 + ((ns * h) >> p.khs), hs1 = st0 + ((ns * (h + 1)) >> p.khs);
-                    const int n = (min(hs0 + ps * xps, hs1) << LSW) + cl * 8, nend = min(min(hs1, hs0 + (ps + 1) * xps) << LSW, p.N);
-                    v[j] = s8[j][0] = s8[j][1] = make_uint4(0, 0, 0, 0);
-                    if (e < n_items && tk[j] < p.M && n < nend) {
-                        v[j] = *reinterpret_cast<const uint4*>(p.In + (size_t)tk[j] * p.N + n);
-#pragma unroll
-                        for (int c = 0; c < 2; ++c)
-                            if (c < p.copies && gk0 + c < ngroups) s8[j][c] = *reinterpret_cast<const uint4*>(p.scales + (size_t)(gk0 + c) * p.N + n);
-                    }
-                }
-#pragma unroll
-                for (int j = 0; j < 2; ++j) {
-                    if (e0 + j * nthr >= n_items) break;
-#pragma unroll
-                    for (int c = 0; c < 2; ++c) {
-                        if (c >= p.copies) break;
-                        const float2 s0 = __half22float2(*reinterpret_cast<const __half2*>(&s8[j][c].x)), s1 = __half22float2(*reinterpret_cast<const __half2*>(&s8[j][c].y));
-                        const float2 s2 = __half22float2(*reinterpret_cast<const __half2*>(&s8[j][c].z)), s3 = __half22float2(*reinterpret_cast<const __half2*>(&s8[j][c].w));
-                        const __nv_bfloat162 o0 = __floats2bfloat162_rn(bf16_lo(v[j].x) * s0.x, bf16_hi(v[j].x) * s0.y);
-                        const __nv_bfloat162 o1 = __floats2bfloat162_rn(bf16_lo(v[j].y) * s1.x, bf16_hi(v[j].y) * s1.y);
-                        const __nv_bfloat162 o2 = __floats2bfloat162_rn(bf16_lo(v[j].z) * s2.x, bf16_hi(v[j].z) * s2.y);
-                        const __nv_bfloat162 o3 = __floats2bfloat162_rn(bf16_lo(v[j].w) * s3.x, bf16_hi(v[j].w) * s3.y);
-                        const uint4 o = make_uint4(*reinterpret_cast<const uint32_t*>(&o0), *reinterpret_cast<const uint32_t*>(&o1),
-                                                   *reinterpret_cast<const uint32_t*>(&o2), *reinterpret_cast<const uint32_t*>(&o3));
-                        *reinterpret_cast<uint4*>(ys + (c * TOKS + tk[j]) * xp + ci[j] * 16) = st_permute8(o);
-                    }
+                for (int t = 0; t < 4; ++t) {
+                    bl[s][t] = on ? ldg32(src + 2 * t * p.r) : 0u;
+                    bh[s][t] = on && p.r > 8 ? ldg32(src + 2 * t * p.r + 8) : 0u;
                 }
             }
-            if (ps == 0 && fused) {                        // the down-projection's MMAs, with the slice's loads behind them
-                float ag[NT][4];
-#pragma unroll
-                for (int tt = 0; tt < NT; ++tt) ag[tt][0] = ag[tt][1] = ag[tt][2] = ag[tt][3] = 0.f;
-                for (int nn = h_n0;;) {
-#pragma unroll
-                    for (int h = 0; h < ST_HSTEPS; ++h) {
-                        const uint32_t a0 = st_movm(ha[h][0]), a1 = st_movm(ha[h][1]), a2 = st_movm(ha[h][2]), a3 = st_movm(ha[h][3]);
-#pragma unroll
-                        for (int tt = 0; tt < NT; ++tt) st_mma(ag[tt], a0, a1, a2, a3, hb[h][tt][0], hb[h][tt][1]);
-                    }
-                    nn += 16 * nw * ST_HSTEPS;
-                    if (nn >= n_hi_cta) break;
-                    h_load(nn);
-                }
-                st_store_hp<NT>(ag, hp, warp, g, q);
+            if (!staged) {                                 // (with the first loads on their way: every warp comes here once)
+                st_stage_lup<true>(p, smem + sp.lup, hfull, c_lo);
+                cp_wait_all();
+                __syncthreads();                           // the group parameters are staged
+                staged = true;
             }
-            __syncthreads();
-            if (ps == 0 && fused) {
-                for (int e = tid; e < 256; e += nthr) {
-                    float h = 0.f;
-                    for (int w = 0; w < nw; ++w) h += hp[w * 256 + e];
-                    hs[e] = h;
-                }
-            }
-            // zero-point term: sum_n dYs[m, n] (OFF + z[G, n]) as one MMA row; the warps of a part share its 32-column units
-            const int un_end = ((min(pb1 << LSW, p.N) - (pb0 << LSW)) + 31) >> 5;
-            for (int c = 0; c < p.copies; ++c) {
-                const int gk = gk0 + c;
-                float za[NT][4];
 #pragma unroll
-                for (int tt = 0; tt < NT; ++tt) za[tt][0] = za[tt][1] = za[tt][2] = za[tt][3] = 0.f;
-                for (int un = fw; un < un_end; un += p.wc) {
-                    const int n = (pb0 << LSW) + 32 * un + 8 * q;
-                    uint32_t zr[4] = {0u, 0u, 0u, 0u};     // (z0,z4) (z1,z5) (z2,z6) (z3,z7) as bf16 of OFF + z
-                    if (g == 0 && n < p.N && gk < ngroups) {
-                        const uint4 z8 = *reinterpret_cast<const uint4*>(p.zeros + (size_t)gk * p.N + n);
-                        const float2 z0 = __half22float2(*reinterpret_cast<const __half2*>(&z8.x)), z1 = __half22float2(*reinterpret_cast<const __half2*>(&z8.y));
-                        const float2 z2 = __half22float2(*reinterpret_cast<const __half2*>(&z8.z)), z3 = __half22float2(*reinterpret_cast<const __half2*>(&z8.w));
-                        const __nv_bfloat162 r0 = __floats2bfloat162_rn(F::OFF + z0.x, F::OFF + z2.x), r1 = __floats2bfloat162_rn(F::OFF + z0.y, F::OFF + z2.y);
-                        const __nv_bfloat162 r2 = __floats2bfloat162_rn(F::OFF + z1.x, F::OFF + z3.x), r3 = __floats2bfloat162_rn(F::OFF + z1.y, F::OFF + z3.y);
-                        zr[0] = *reinterpret_cast<const uint32_t*>(&r0); zr[1] = *reinterpret_cast<const uint32_t*>(&r1);
-                        zr[2] = *reinterpret_cast<const uint32_t*>(&r2); zr[3] = *reinterpret_cast<const uint32_t*>(&r3);
-                    }
+            for (int s = 0; s < SB; ++s) {
+                const int sl = s0 + s * ST_WARPS;
+                if (sl >= nu) break;
+                if (p.fused) {
+                    uint32_t a[4], b[4];
+#pragma unroll
+                    for (int t = 0; t < 4; ++t) { a[t] = st_movm(bl[s][t]); b[t] = p.r > 8 ? st_movm(bh[s][t]) : 0u; }
 #pragma unroll
                     for (int tt = 0; tt < NT; ++tt) {
-                        const uint4 xv = *reinterpret_cast<const uint4*>(ys + (c * TOKS + g + 8 * tt) * xp + (((kh << lcpp) + un * 4 + q) << 4));
-                        st_mma(za[tt], zr[0], 0u, zr[1], 0u, xv.x, xv.y);
-                        st_mma(za[tt], zr[2], 0u, zr[3], 0u, xv.z, xv.w);
+                        st_mma(hacc[tt], a[0], b[0], a[1], b[1], yv[s][tt].x, yv[s][tt].y);
+                        st_mma(hacc[tt], a[2], b[2], a[3], b[3], yv[s][tt].z, yv[s][tt].w);
                     }
                 }
-                if (g == 0) {
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    if (c >= p.ngl) break;
+                    const uint4 s8 = *reinterpret_cast<const uint4*>(sz + (2 * c) * p.range + 32 * sl + 8 * q);
+                    const uint4 z8 = *reinterpret_cast<const uint4*>(sz + (2 * c + 1) * p.range + 32 * sl + 8 * q);
 #pragma unroll
                     for (int tt = 0; tt < NT; ++tt) {
-                        zp[warp * 32 + c * 16 + 8 * tt + 2 * q] += za[tt][0];
-                        zp[warp * 32 + c * 16 + 8 * tt + 2 * q + 1] += za[tt][1];
-                    }
-                }
-            }
-            if (ps == 0) {
-                st_cluster_wait();                         // every CTA of the cluster is running: its shared memory may be written
-                if (fused) {
-                    __syncthreads();                       // hs is complete
-                    st_push_h(rl, hs, rank, p.ks);
-                }
-            }
-        }
-        if (live) {
-            const uint8_t* yw = ys + (copy * TOKS + g) * xp + (((kh << lcpp) + q) << 4);
-#pragma unroll 2
-            for (int stg = pb0; stg < pb1; ++stg) {
-                cp_wait<F::BNS - 1>();
-                __syncwarp();
-                const uint8_t* slot = ring + c_slot * F::BSLOT;
-#pragma unroll
-                for (int su = 0; su < F::SU; ++su) {
-                    const int ul = (stg - pb0) * F::SU + su;   // 32-column unit inside this part's staged slice
-                    uint32_t mx[4][F::BPAIR];                  // [column i of the lane's four][pair], transposed
-                    if constexpr (BITS == 2) {
-                        const uint4 w = *reinterpret_cast<const uint4*>(slot + su * 128 + g * 16);
-#pragma unroll
-                        for (int i = 0; i < 4; ++i)
-#pragma unroll
-                            for (int j = 0; j < 2; ++j)
-                                mx[i][j] = st_movm(((st_comp(w, i) >> (2 * (2 * q + j))) & 0x00030003u) | 0x43004300u);
-                    } else {
-                        uint4 w[F::NLD];
-                        st_load_words<BITS>(slot, g, q, w);
+                        const uint4 v = yv[s][tt];
+                        uint32_t o[4];
+                        float zs = 0.f;
 #pragma unroll
                         for (int i = 0; i < 4; ++i) {
-                            uint32_t pr[4];
-                            st_unpack<BITS>(st_comp(w[0], i), F::NLD > 1 ? st_comp(w[F::NLD - 1], i) : 0u, q, pr);
-#pragma unroll
-                            for (int t = 0; t < 4; ++t) mx[i][t] = st_movm(pr[t]);
+                            const uint32_t vi = st_comp(v, i), si = st_comp(s8, i), zi = st_comp(z8, i);
+                            const float2 sf = __half22float2(*reinterpret_cast<const __half2*>(&si)), zf = __half22float2(*reinterpret_cast<const __half2*>(&zi));
+                            o[i] = st_pack(bf16_lo(vi) * sf.x, bf16_hi(vi) * sf.y);
+                            zs = fmaf(bf16_lo(o[i]), F::OFF + zf.x, zs);
+                            zs = fmaf(bf16_hi(o[i]), F::OFF + zf.y, zs);
                         }
-                    }
-#pragma unroll
-                    for (int tt = 0; tt < NT; ++tt) {
-                        const uint4 xv = *reinterpret_cast<const uint4*>(yw + 8 * tt * xp + (ul << 6));
-#pragma unroll
-                        for (int t = 0; t < NTILE; ++t) {
-                            st_mma(acc[t][tt], mx[0][2 * t], mx[0][2 * t + 1], mx[1][2 * t], mx[1][2 * t + 1], xv.x, xv.y);
-                            st_mma(acc[t][tt], mx[2][2 * t], mx[2][2 * t + 1], mx[3][2 * t], mx[3][2 * t + 1], xv.z, xv.w);
-                        }
+                        zacc[c][tt] += zs;
+                        if (tok_ok[tt])
+                            *reinterpret_cast<uint4*>(ys + (size_t)(c * p.M + g + 8 * tt) * p.pitch + sl * 64 + q * 16) = make_uint4(o[0], o[1], o[2], o[3]);
                     }
                 }
-                if (++c_slot == F::BNS) c_slot = 0;
-                __syncwarp();
-                issue();
             }
         }
-        __syncthreads();
-    }
-    if (tid < 32) {                                        // zero-point sums of the whole range, warps added in order
-        float z = 0.f;
-        for (int w = 0; w < nw; ++w) z += zp[w * 32 + tid];
-        zc[tid] = z;
+        if (p.fused) st_store_hp<NT>(p, hacc, hp, warp, g, q);
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+#pragma unroll
+            for (int tt = 0; tt < 2; ++tt) {
+                const float z = tt < NT ? st_quad_sum(zacc[c][tt < NT ? tt : 0]) : 0.f;
+                if (q == 0) zp[warp * 32 + c * 16 + 8 * tt + g] = z;
+            }
     }
     __syncthreads();
-    // accumulator element (t, tt, e): MMA row g + 8 (e >> 1) of tile t = matrix 2t + (e >> 1), column g of it; token
-    // 2q + (e & 1) + 8 tt.  The zero-point sum covers the CTA's whole range, so part 0 alone subtracts it.  Each pair of
-    // tokens goes to the CTA that finishes that feature.
+    const uint32_t recv_h_addr = s_u32(smem + sp.recv_h);
+    if (p.ks > 1) st_cluster_wait();                       // every CTA of the cluster is running: its shared memory may be written
+    if (p.fused) st_share_h(p, hp, recv_h_addr, rank);
+    // zero-point sums of the CTA's whole range, warps added in order; part 0 alone subtracts them
+    float z_sub[NT][2];
 #pragma unroll
-    for (int t = 0; t < NTILE; ++t)
+    for (int tt = 0; tt < NT; ++tt) z_sub[tt][0] = z_sub[tt][1] = 0.f;
+    if (part == 0) {
 #pragma unroll
         for (int tt = 0; tt < NT; ++tt)
 #pragma unroll
-            for (int hh = 0; hh < 2; ++hh) {
-                const int m = 2 * t + hh;                  // pair index of the matrix
-                int f;                                     // feature of matrix m, column g (lane q' = g >> 1 supplied half g & 1)
-                if constexpr (BITS == 2) f = 2 * (g >> 1) + m + 8 * (g & 1);
-                else if constexpr (BITS == 8) f = 16 * (m >> 1) + 4 * (g >> 1) + 2 * (m & 1) + (g & 1);
-                else f = 8 * (g >> 1) + m + 4 * (g & 1);
-                const int tok = 2 * q + 8 * tt;
-                const float z0 = kh == 0 ? zc[copy * 16 + tok] : 0.f, z1 = kh == 0 ? zc[copy * 16 + tok + 1] : 0.f;
-                st_push2(rl, rank, kh, F::FW * fw + f, tok, acc[t][tt][2 * hh] - z0, acc[t][tt][2 * hh + 1] - z1);
+            for (int wv = 0; wv < ST_WARPS; ++wv) {
+                const float2 z = *reinterpret_cast<const float2*>(zp + wv * 32 + copy * 16 + 8 * tt + 2 * q);
+                z_sub[tt][0] += z.x; z_sub[tt][1] += z.y;
             }
-    st_finish<true, TOKS>(p, recv_part, recv_h, hfull, lup, tile_c, rank);
-}
-
-template <typename Kern>
-bool st_configure(Kern kern, size_t smem_bytes, size_t (&done)[ST_MAX_DEVICES], std::mutex& mu) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return false;
-    std::lock_guard<std::mutex> lock(mu);
-    if (dev >= 0 && dev < ST_MAX_DEVICES && done[dev] >= smem_bytes) return true;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes) != cudaSuccess) return false;
-    if (dev >= 0 && dev < ST_MAX_DEVICES) done[dev] = smem_bytes;
-    return true;
-}
-
-template <int BITS, int NT, bool TRANSPOSED>
-int st_launch(const StreamParams& p, int W, int tiles, size_t smem_bytes, cudaStream_t st) {
-    static std::mutex mu;
-    static size_t done[ST_MAX_DEVICES] = {};
-    cudaError_t err;
-    const dim3 grid((unsigned)p.ks, (unsigned)tiles), block((unsigned)(32 * W));
-    if (TRANSPOSED) {
-        auto kern = stream_bwd_kernel<BITS, NT>;
-        if (!st_configure(kern, smem_bytes, done, mu)) return QLORA_ERR_CUDA;
-        err = launch_pdl(kern, grid, block, smem_bytes, st, (unsigned)p.ks, p);
-    } else {
-        auto kern = stream_fwd_kernel<BITS, NT>;
-        if (!st_configure(kern, smem_bytes, done, mu)) return QLORA_ERR_CUDA;
-        err = launch_pdl(kern, grid, block, smem_bytes, st, (unsigned)p.ks, p);
     }
-    return err == cudaSuccess ? QLORA_OK : QLORA_ERR_CUDA;
+
+    // ---- main loop ----
+    float acc[FL / 2][NT][4];
+#pragma unroll
+    for (int i = 0; i < FL / 2; ++i)
+#pragma unroll
+        for (int tt = 0; tt < NT; ++tt) acc[i][tt][0] = acc[i][tt][1] = acc[i][tt][2] = acc[i][tt][3] = 0.f;
+    const uint32_t yl = s_u32(ys) + (uint32_t)((copy * p.M + g) * p.pitch + 8 * q);
+    uint32_t xv[NT][2];
+#pragma unroll
+    for (int tt = 0; tt < NT; ++tt) xv[tt][0] = xv[tt][1] = 0u;            // (stays zero for tokens that do not exist)
+#pragma unroll 1
+    for (int un = w0; un < w1; un += BF::DEPTH) {
+#pragma unroll
+        for (int d = 0; d < BF::DEPTH; ++d) {
+            if (un + d < w1) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const uint4& wa = w[d][h * BF::NLD];
+                    const uint4& wb = w[d][h * BF::NLD + BF::NLD - 1];
+                    uint32_t p0[FL], p1[FL];
+                    st_bwd_pairs<BITS, FL>(wa.x, wb.x, wa.y, wb.y, sh, sel, p0);
+                    st_bwd_pairs<BITS, FL>(wa.z, wb.z, wa.w, wb.w, sh, sel, p1);
+#pragma unroll
+                    for (int tt = 0; tt < NT; ++tt) {
+                        lds8(xv[tt][0], xv[tt][1], yl + (uint32_t)(8 * tt * p.pitch + (un + d - u0) * 64 + 32 * h), tok_ok[tt]);
+#pragma unroll
+                        for (int i = 0; i < FL / 2; ++i) st_mma(acc[i][tt], p0[2 * i], p0[2 * i + 1], p1[2 * i], p1[2 * i + 1], xv[tt][0], xv[tt][1]);
+                    }
+                }
+                load_unit(w[d], un + d + BF::DEPTH);
+            }
+        }
+    }
+    // accumulator element (i, tt, e): feature FL g + 2 i + (e >> 1) of the warp's, token 2q + (e & 1) + 8 tt
+    float* mine = reinterpret_cast<float*>(smem + sp.part) + part * p.M * tile_c + 8 * FL * fw + FL * g;
+#pragma unroll
+    for (int tt = 0; tt < NT; ++tt)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const int tok = 8 * tt + 2 * q + e;
+            if (tok < p.M) {
+#pragma unroll
+                for (int j = 0; j < FL / 4; ++j)
+                    *reinterpret_cast<float4*>(mine + tok * tile_c + 4 * j) = make_float4(acc[2 * j][tt][e] - z_sub[tt][e], acc[2 * j][tt][2 + e] - z_sub[tt][e],
+                                                                                        acc[2 * j + 1][tt][e] - z_sub[tt][e], acc[2 * j + 1][tt][2 + e] - z_sub[tt][e]);
+            }
+        }
+    st_finish<true>(p, smem, sp, c_lo, rank, blockIdx.y == 0 && rank == 0);
 }
 
-// Dynamic shared memory of a launch: the carve-up at the top of the two kernels, in the same order.
-template <int BITS>
-size_t st_smem_bytes(bool transposed, int nw, int toks, int xc, int copies, int KH, int ks, int tile_c) {
-    using F = Fmt<BITS>;
-    const size_t tail = (size_t)(256 + 1024) * 4 + ST_LUP_BYTES + (size_t)nw * 1024 + (size_t)ks * 1024 + (size_t)KH * tile_c * 64;
-    if (transposed)
-        return (size_t)nw * F::BNS * F::BSLOT + (size_t)copies * toks * (xc * 2 + 64) + (size_t)(nw * 32 + 32) * 4 + tail;
-    return (size_t)nw * F::NS * F::SLOT + (size_t)toks * (xc * 2 + F::XPAD) + (size_t)(toks * (xc / 8) + KH * (xc / F::KB / KH + 1) * toks) * 4 + tail;
-}
-
-// Warps per CTA of the backward kernel: the features of a CTA must lie in one group or span exactly two.
-int bwd_warps(int bits, int g) {
-    const int fw = bits == 2 ? 16 : 32;
-    const int order[4] = {4, 8, 2, 1};                     // four side by side leave room for four parts of the contraction
-    for (int i = 0; i < 4; ++i)
-        if (g % (order[i] * fw) == 0 || order[i] * fw == 2 * g) return order[i];
-    return 0;
+template <int BITS, int NT, int V, bool TRANSPOSED>          // V: GPC forward, FL backward
+int st_launch(const StreamParams& p, int tiles, size_t smem_bytes, cudaStream_t st) {
+    static SmemLimit limit;
+    const dim3 grid((unsigned)p.ks, (unsigned)tiles);
+    void (*kern)(const StreamParams);
+    if constexpr (TRANSPOSED) kern = stream_bwd_kernel<BITS, NT, V>;
+    else kern = stream_fwd_kernel<BITS, NT, V>;
+    if (!limit.raise(kern, 227 * 1024)) return QLORA_ERR_CUDA;
+    return launch_pdl(kern, grid, dim3(ST_THREADS), smem_bytes, st, (unsigned)p.ks, p) == cudaSuccess ? QLORA_OK : QLORA_ERR_CUDA;
 }
 
 int fwd_kb(int bits) { return bits == 2 ? 64 : 32; }
 
-__global__ void __launch_bounds__(512, 1) st_probe_kernel() {}
+constexpr int ST_MAX_DEVICES = kMaxDevices;
+__global__ void __launch_bounds__(ST_THREADS, 2) st_probe_kernel() {}
 
+// SM count, and how many clusters of 2 / 4 / 8 CTAs that share an SM two by two can run at once, per device ordinal.
 struct DeviceFacts { int sms = 0; int clusters[9] = {}; };
 
-// SM count and how many clusters of 2 / 4 / 8 CTAs that own an SM each can run at once, per device ordinal.
 const DeviceFacts& device_facts() {
     static std::mutex mu;
     static DeviceFacts facts[ST_MAX_DEVICES];
-    static DeviceFacts fallback;
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= ST_MAX_DEVICES) { fallback.sms = 148; fallback.clusters[2] = 74; fallback.clusters[4] = 32; fallback.clusters[8] = 14; return fallback; }
+    static const DeviceFacts fallback{148, {0, 296, 148, 0, 72, 0, 0, 0, 34}};
+    const int dev = device_ordinal();
+    if (dev < 0) return fallback;
     std::lock_guard<std::mutex> lock(mu);
     DeviceFacts& f = facts[dev];
     if (f.sms == 0) {
-        int v = 0;
-        f.sms = (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0) ? v : 148;
-        (void)cudaFuncSetAttribute(st_probe_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+        const int sms = sm_count();
+        f.clusters[1] = 2 * sms;
+        (void)cudaFuncSetAttribute(st_probe_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
         for (int cs = 2; cs <= 8; cs *= 2) {
             cudaLaunchConfig_t cfg{};
-            cfg.gridDim = dim3((unsigned)cs, (unsigned)f.sms);
-            cfg.blockDim = dim3(512);
-            cfg.dynamicSmemBytes = 200 * 1024;         // one CTA per SM, as the streaming kernels are
+            cfg.gridDim = dim3((unsigned)cs, (unsigned)sms);
+            cfg.blockDim = dim3(ST_THREADS);
+            cfg.dynamicSmemBytes = 100 * 1024;
             cudaLaunchAttribute attr;
             attr.id = cudaLaunchAttributeClusterDimension;
             attr.val.clusterDim.x = (unsigned)cs; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
             cfg.attrs = &attr;
             cfg.numAttrs = 1;
             int n = 0;
-            if (cudaOccupancyMaxActiveClusters(&n, st_probe_kernel, &cfg) != cudaSuccess || n <= 0) { (void)cudaGetLastError(); n = f.sms / cs * 3 / 4; }
+            if (cudaOccupancyMaxActiveClusters(&n, st_probe_kernel, &cfg) != cudaSuccess || n <= 0) { (void)cudaGetLastError(); n = 2 * sms / cs; }
             f.clusters[cs] = n;
         }
+        f.sms = sms;
     }
     return f;
 }
-int max_clusters(int cs) { return cs <= 1 ? device_facts().sms : device_facts().clusters[cs > 8 ? 8 : cs]; }
-int sm_count_here() { return device_facts().sms; }
+
+// How a shape is cut: warps side by side (wc), CTAs per cluster (ks).  Every candidate that fits is costed in cycles, with the times
+// read off stamped kernels (4096 x 4096 and the MLP shapes, 1 and 16 tokens):
+//   products  a warp's own units of the contraction, 1400 cycles per chunk forward and 650 per unit backward whatever else the SM
+//             does, up to a fifth more when a second CTA shares it: the chain of one warp, not the SM's throughput, sets the pace, so
+//             the best cut is usually the one with about 256 CTAs;
+//   staging   a warp's slices of the CTA's range, two in flight per round trip to L2;
+//   exchange  the cluster barriers and the adding up;
+// and the whole repeats when the CTAs exceed what the GPU holds at once (two per SM up to half an SM's shared memory).
+// (4096 x 4096, INT4, one token: 128 columns x 8 CTAs 6.3 us, 64 x 4 6.7, 32 x 2 8.2, 256 x 8 8.7, 128 x 4 9.3, 64 x 8 9.5.)
+struct StreamPlan { StreamParams p; int tiles, tile_c; SmemPlan sm; bool ok; };
+
+StreamPlan st_cut(StreamParams p, int bits, bool transposed) {
+    StreamPlan best{};
+    best.ok = false;
+    float best_cost = 0.f;
+    const DeviceFacts& gpu = device_facts();
+    const int toks = p.M > 8 ? 16 : 8, nt = toks / 8, sms = gpu.sms;
+    const int fl = p.g % 64 == 0 ? 8 : 4;
+    p.gd = p.g / 32;
+    p.gm = (uint32_t)(((1ull << 32) + p.gd - 1) / p.gd);
+    const int T = transposed ? p.N : p.K;
+    const int unit = transposed ? 32 : ST_CHUNK, units = (T + unit - 1) / unit;
+    for (int lwc = 0; lwc <= 3; ++lwc) {
+        p.wc = 1 << lwc; p.lwc = lwc; p.lwp = 3 - lwc;
+        const int tile_c = (transposed ? 8 * fl : 32) * p.wc, tiles = (p.C + tile_c - 1) / tile_c;
+        if (lwc > 0 && tile_c / 2 >= p.C) break;                       // (half the warps would have no column)
+        if (tiles > 65535) continue;
+        int groups = 1;                                                // backward: groups the features of a CTA span
+        if (transposed && p.g % tile_c != 0) groups = tile_c % p.g == 0 ? tile_c / p.g : (tile_c - 1) / p.g + 2;
+        if (groups > 2) continue;
+        for (int lks = 0; lks <= 3; ++lks) {
+            p.ks = 1 << lks; p.lks = lks;
+            const int sl = tile_c >> lks;
+            if (sl < 8) break;
+            p.lsl = 0;
+            while ((1 << p.lsl) < sl) ++p.lsl;
+            const int per_cta = (units + p.ks - 1) / p.ks, parts = 1 << p.lwp;
+            p.range = per_cta * unit;
+            p.ngl = transposed ? groups : (p.range + p.g - 1) / p.g + 1;
+            // rows far enough apart that the fragment loads of neighbouring tokens meet different banks
+            const int want = transposed ? 32 : (bits == 2 ? 16 : (bits == 8 ? 32 : 64));
+            p.pitch = p.range * 2;
+            p.pitch += (want - p.pitch % 128 + 128) % 128;
+            const SmemPlan sm = st_plan(p, transposed, toks, tile_c);
+            if (sm.total > 227 * 1024 - 1024) continue;
+            const int occ = sm.total <= 113 * 1024 ? 2 : 1;
+            const float fill = (float)(tiles * 2) / (float)(gpu.clusters[p.ks] * occ);     // of what the GPU holds at once
+            const float waves = fill <= 1.f ? 1.f : 0.5f * (fill + ceilf(fill));
+            const int per_warp = (per_cta + parts - 1) / parts;
+            const float step = (transposed ? 650.f + 150.f * (nt - 1) : 1400.f + 450.f * (nt - 1)) * (bits == 8 ? 1.3f : 1.f) * (tiles * p.ks > sms ? 1.2f : 1.f);
+            const float rounds = (float)((per_cta * (unit / 32) + 2 * ST_WARPS - 1) / (2 * ST_WARPS));
+            const float round = transposed ? 2500.f * nt : 900.f + 1100.f * nt;
+            const float cost = waves * ((float)per_warp * step + rounds * round + 1500.f + 500.f * (float)lks);
+            if (!best.ok || cost < best_cost) { best = StreamPlan{p, tiles, tile_c, sm, true}; best_cost = cost; }
+        }
+    }
+    return best;
+}
 
 }  // namespace
 
 bool stream_supported(const qlora_desc& d, int M, bool transposed) {
     if (M < 1 || M > 16) return false;
-    if (d.K < 32 || d.N < 8) return false;
-    if (transposed) return bwd_warps(d.bits, d.group_size) > 0;
-    return d.group_size % fwd_kb(d.bits) == 0;
+    if (d.K < 32 || d.N < 8 || d.K > (1 << 20)) return false;   // (the group index's reciprocal is exact up to there)
+    if (!transposed && d.group_size % fwd_kb(d.bits) != 0) return false;
+    if ((transposed ? d.N : d.K) <= 16384) return true;    // eight ways split, such a range always fits the shared memory
+    StreamParams p{};
+    p.M = M; p.K = d.K; p.N = d.N; p.g = d.group_size; p.r = d.r; p.C = transposed ? d.K : d.N;
+    p.fused = d.r > 0 && d.r <= 16 ? 1 : 0;
+    return st_cut(p, d.bits, transposed).ok;
 }
 
 int launch_stream_gemm(const qlora_desc& d, int M, bool transposed, const void* In, const int32_t* Q, const void* scales,
@@ -1006,70 +929,24 @@ int launch_stream_gemm(const qlora_desc& d, int M, bool transposed, const void* 
     p.Ldown = (const __nv_bfloat16*)Ldown; p.Lup = (const __nv_bfloat16*)Lup; p.P = P; p.Out = (__nv_bfloat16*)Out;
     p.fused = (d.r > 0 && !p_is_input) ? 1 : 0;
     if (p.fused && d.r > 16) return QLORA_ERR_INVALID_ARG;
-    const int nt = M > 8 ? 2 : 1, toks = 8 * nt;
-    int wc, tile_c, units;                                 // warps side by side, output columns per CTA, contraction stages
-    if (transposed) {
-        wc = bwd_warps(d.bits, d.group_size);
-        if (wc == 0) return QLORA_ERR_UNSUPPORTED;
-        tile_c = wc * (d.bits == 2 ? 16 : 32);
-        p.copies = tile_c > d.group_size ? 2 : 1;
-        units = (d.N + (d.bits == 2 ? 128 : 32) - 1) / (d.bits == 2 ? 128 : 32);
-    } else {
-        if (d.group_size % fwd_kb(d.bits) != 0) return QLORA_ERR_UNSUPPORTED;
-        wc = d.N >= 128 ? 4 : (d.N >= 64 ? 2 : 1);
-        tile_c = 32 * wc;
-        p.copies = 1;
-        units = (d.K + fwd_kb(d.bits) - 1) / fwd_kb(d.bits);
-    }
-    p.wc = wc;
-    p.lwc = 0;
-    while ((1 << p.lwc) < wc) ++p.lwc;
-    const int tiles = (p.C + tile_c - 1) / tile_c;
-    // split the contraction over a cluster until the grid covers the GPU: one CTA per SM, and no more clusters than can
-    // run at once (the clusters of a launch that come later would wait for whole earlier ones to finish)
-    int ks = 1;
-    while (ks < 8 && tiles * 2 * ks <= max_clusters(2 * ks) * 2 * ks && tiles * 2 * ks <= sm_count_here() && units / (2 * ks) >= 4 &&
-           tile_c / (2 * ks) >= 1)
-        ks *= 2;
-    p.ks = ks;
-    p.lks = 0;
-    while ((1 << p.lks) < ks) ++p.lks;
-    // ... and inside a CTA until it has sixteen warps, while a warp keeps at least two stages
-    p.khs = 0;
-    while ((wc << (p.khs + 1)) <= 16 && p.khs < 2 && units / (ks << (p.khs + 1)) >= 2) ++p.khs;
-    const int nw = wc << p.khs, KH = 1 << p.khs;
-    const int sl = tile_c / ks;
-    p.sls = 0;
-    while ((1 << p.sls) < sl) ++p.sls;
-    // the activations staged per pass (all parts of a CTA together): the CTA's whole range when that fits (one pass, two
-    // barriers), else 512 at a time; a power of two, and at least one stage per part
-    {
-        const int unit = transposed ? (d.bits == 2 ? 128 : 32) : fwd_kb(d.bits);
-        const int range = ((units + ks - 1) / ks + KH - 1) / KH * KH * unit;
-        const int cap = (transposed && p.copies * toks > 16) ? 512 : 1024;
-        p.xc = 128;
-        while (p.xc < range && p.xc < cap) p.xc *= 2;
-        if (p.xc < unit * KH) p.xc = unit * KH;
-    }
-    p.lup_staged = (sl * d.r * 2 <= ST_LUP_BYTES) ? 1 : 0;
-    size_t smem = 0;
-    switch (d.bits) {
-        case 2: smem = st_smem_bytes<2>(transposed, nw, toks, p.xc, p.copies, KH, ks, tile_c); break;
-        case 3: smem = st_smem_bytes<3>(transposed, nw, toks, p.xc, p.copies, KH, ks, tile_c); break;
-        case 4: smem = st_smem_bytes<4>(transposed, nw, toks, p.xc, p.copies, KH, ks, tile_c); break;
-        case 8: smem = st_smem_bytes<8>(transposed, nw, toks, p.xc, p.copies, KH, ks, tile_c); break;
-    }
-    if (smem > 227 * 1024) return QLORA_ERR_UNSUPPORTED;
-#define QLORA_ST(B, NT)                                                                                   \
-    return transposed ? st_launch<B, NT, true>(p, nw, tiles, smem, st) : st_launch<B, NT, false>(p, nw, tiles, smem, st)
+    const StreamPlan plan = st_cut(p, d.bits, transposed);
+    if (!plan.ok) return QLORA_ERR_UNSUPPORTED;
+#define QLORA_ST(B, NT)                                                                                                          \
+    if (transposed)                                                                                                              \
+        return d.group_size % 64 == 0 ? st_launch<B, NT, 8, true>(plan.p, plan.tiles, plan.sm.total, st)                         \
+                                      : st_launch<B, NT, 4, true>(plan.p, plan.tiles, plan.sm.total, st);                        \
+    if (d.group_size % 128 == 0) return st_launch<B, NT, 1, false>(plan.p, plan.tiles, plan.sm.total, st);                       \
+    if (d.group_size % 64 == 0) return st_launch<B, NT, 2, false>(plan.p, plan.tiles, plan.sm.total, st);                        \
+    if constexpr (B != 2) return st_launch<B, NT, 4, false>(plan.p, plan.tiles, plan.sm.total, st);                              \
+    else return QLORA_ERR_UNSUPPORTED
 #define QLORA_ST_BITS(NT)           \
     switch (d.bits) {               \
-        case 2: QLORA_ST(2, NT);    \
-        case 3: QLORA_ST(3, NT);    \
-        case 4: QLORA_ST(4, NT);    \
-        case 8: QLORA_ST(8, NT);    \
+        case 2: { QLORA_ST(2, NT); }    \
+        case 3: { QLORA_ST(3, NT); }    \
+        case 4: { QLORA_ST(4, NT); }    \
+        case 8: { QLORA_ST(8, NT); }    \
     }
-    if (nt == 1) { QLORA_ST_BITS(1) } else { QLORA_ST_BITS(2) }
+    if (M <= 8) { QLORA_ST_BITS(1) } else { QLORA_ST_BITS(2) }
 #undef QLORA_ST_BITS
 #undef QLORA_ST
     return QLORA_ERR_UNSUPPORTED;
