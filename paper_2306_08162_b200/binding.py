@@ -1,5 +1,6 @@
-"""ctypes binding of the C ABI in include/qlora.h.  Same names, same argument order; tensors are passed as their
-device pointers and `stream=None` means torch's current CUDA stream.  No arithmetic happens here."""
+"""Binding of the C ABI in include/qlora.h.  Same names, same argument order; tensors are passed as their device pointers and
+`stream=None` means torch's current CUDA stream.  No arithmetic happens here.  The calls of a training or generation loop go
+through the C extension of csrc/pycall.cpp, the others through ctypes."""
 from __future__ import annotations
 
 import ctypes
@@ -8,6 +9,7 @@ import os
 _PKG_DIR = os.path.dirname(os.path.abspath(__file__))
 _LIB_PATH = os.path.join(_PKG_DIR, "libqlora_b200.so")
 _lib = None
+_calls = None
 
 
 class QloraError(RuntimeError):
@@ -71,6 +73,17 @@ def library() -> ctypes.CDLL:
     return lib
 
 
+def _native():
+    """The C extension with the calls of the hot path (built in-tree together with the library)."""
+    global _calls
+    if _calls is None:
+        library()
+        from . import _pycall
+        _pycall.set_desc_type(_Desc)
+        _calls = _pycall
+    return _calls
+
+
 def _ptr(t):
     """Device pointer of a torch tensor; None -> NULL; an int is passed through (tests of the error paths)."""
     if t is None:
@@ -80,10 +93,6 @@ def _ptr(t):
     if not t.is_contiguous():
         raise ValueError("tensors must be contiguous (dense row-major)")
     return ctypes.c_void_p(t.data_ptr())
-
-
-def _nbytes(t) -> int:
-    return 0 if t is None else t.numel() * t.element_size()
 
 
 def _stream(stream):
@@ -111,23 +120,21 @@ def qlora_workspace_bytes(d: _Desc, M: int) -> int:
 
 
 def qlora_fwd(d, M, X, Q, scales, zeros, A, B, Y, H_out, workspace, stream=None, workspace_bytes=None):
-    wb = _nbytes(workspace) if workspace_bytes is None else int(workspace_bytes)
-    _check(library().qlora_fwd(ctypes.byref(d), int(M), _ptr(X), _ptr(Q), _ptr(scales), _ptr(zeros), _ptr(A), _ptr(B),
-                               _ptr(Y), _ptr(H_out), _ptr(workspace), wb, _stream(stream)), "qlora_fwd")
+    rc = _native().qlora_fwd(d, M, X, Q, scales, zeros, A, B, Y, H_out, workspace, workspace_bytes, stream)
+    if rc != 0:
+        raise QloraError(rc, "qlora_fwd")
 
 
 def qlora_bwd_input(d, M, dY, Q, scales, zeros, A, B, dX, G_out, workspace, stream=None, workspace_bytes=None):
-    wb = _nbytes(workspace) if workspace_bytes is None else int(workspace_bytes)
-    _check(library().qlora_bwd_input(ctypes.byref(d), int(M), _ptr(dY), _ptr(Q), _ptr(scales), _ptr(zeros), _ptr(A),
-                                     _ptr(B), _ptr(dX), _ptr(G_out), _ptr(workspace), wb, _stream(stream)),
-           "qlora_bwd_input")
+    rc = _native().qlora_bwd_input(d, M, dY, Q, scales, zeros, A, B, dX, G_out, workspace, workspace_bytes, stream)
+    if rc != 0:
+        raise QloraError(rc, "qlora_bwd_input")
 
 
 def qlora_bwd_input_db(d, M, dY, Q, scales, zeros, A, B, H, dX, G_out, dB, accumulate, workspace, stream=None, workspace_bytes=None):
-    wb = _nbytes(workspace) if workspace_bytes is None else int(workspace_bytes)
-    _check(library().qlora_bwd_input_db(ctypes.byref(d), int(M), _ptr(dY), _ptr(Q), _ptr(scales), _ptr(zeros), _ptr(A),
-                                        _ptr(B), _ptr(H), _ptr(dX), _ptr(G_out), _ptr(dB), int(accumulate), _ptr(workspace), wb,
-                                        _stream(stream)), "qlora_bwd_input_db")
+    rc = _native().qlora_bwd_input_db(d, M, dY, Q, scales, zeros, A, B, H, dX, G_out, dB, accumulate, workspace, workspace_bytes, stream)
+    if rc != 0:
+        raise QloraError(rc, "qlora_bwd_input_db")
 
 
 def qlora_bwd_input_db_on_producers(d, M) -> bool:
@@ -138,33 +145,29 @@ def qlora_bwd_input_db_on_producers(d, M) -> bool:
 
 
 def qlora_bwd_lora(d, M, X, dY, A, B, H, G, dA, dB, accumulate, workspace, stream=None, workspace_bytes=None):
-    wb = _nbytes(workspace) if workspace_bytes is None else int(workspace_bytes)
-    _check(library().qlora_bwd_lora(ctypes.byref(d), int(M), _ptr(X), _ptr(dY), _ptr(A), _ptr(B), _ptr(H), _ptr(G),
-                                    _ptr(dA), _ptr(dB), int(accumulate), _ptr(workspace), wb, _stream(stream)),
-           "qlora_bwd_lora")
+    rc = _native().qlora_bwd_lora(d, M, X, dY, A, B, H, G, dA, dB, accumulate, workspace, workspace_bytes, stream)
+    if rc != 0:
+        raise QloraError(rc, "qlora_bwd_lora")
 
 
 def qlora_fwd_dropout(d, M, X, mask, keep_scale, Q, scales, zeros, A, B, Y, H_out, workspace, stream=None, workspace_bytes=None):
-    wb = _nbytes(workspace) if workspace_bytes is None else int(workspace_bytes)
-    _check(library().qlora_fwd_dropout(ctypes.byref(d), int(M), _ptr(X), _ptr(mask), float(keep_scale), _ptr(Q), _ptr(scales),
-                                       _ptr(zeros), _ptr(A), _ptr(B), _ptr(Y), _ptr(H_out), _ptr(workspace), wb, _stream(stream)),
-           "qlora_fwd_dropout")
+    rc = _native().qlora_fwd_dropout(d, M, X, mask, keep_scale, Q, scales, zeros, A, B, Y, H_out, workspace, workspace_bytes, stream)
+    if rc != 0:
+        raise QloraError(rc, "qlora_fwd_dropout")
 
 
 def qlora_bwd_input_dropout(d, M, dY, mask, keep_scale, Q, scales, zeros, A, B, dX, G_out, workspace, stream=None,
                             workspace_bytes=None):
-    wb = _nbytes(workspace) if workspace_bytes is None else int(workspace_bytes)
-    _check(library().qlora_bwd_input_dropout(ctypes.byref(d), int(M), _ptr(dY), _ptr(mask), float(keep_scale), _ptr(Q), _ptr(scales),
-                                             _ptr(zeros), _ptr(A), _ptr(B), _ptr(dX), _ptr(G_out), _ptr(workspace), wb,
-                                             _stream(stream)), "qlora_bwd_input_dropout")
+    rc = _native().qlora_bwd_input_dropout(d, M, dY, mask, keep_scale, Q, scales, zeros, A, B, dX, G_out, workspace, workspace_bytes, stream)
+    if rc != 0:
+        raise QloraError(rc, "qlora_bwd_input_dropout")
 
 
 def qlora_bwd_lora_dropout(d, M, X, mask, keep_scale, dY, A, B, H, G, dA, dB, accumulate, workspace, stream=None,
                            workspace_bytes=None):
-    wb = _nbytes(workspace) if workspace_bytes is None else int(workspace_bytes)
-    _check(library().qlora_bwd_lora_dropout(ctypes.byref(d), int(M), _ptr(X), _ptr(mask), float(keep_scale), _ptr(dY), _ptr(A),
-                                            _ptr(B), _ptr(H), _ptr(G), _ptr(dA), _ptr(dB), int(accumulate), _ptr(workspace), wb,
-                                            _stream(stream)), "qlora_bwd_lora_dropout")
+    rc = _native().qlora_bwd_lora_dropout(d, M, X, mask, keep_scale, dY, A, B, H, G, dA, dB, accumulate, workspace, workspace_bytes, stream)
+    if rc != 0:
+        raise QloraError(rc, "qlora_bwd_lora_dropout")
 
 
 STATIC_SCRATCH_BYTES = 16 << 20   # QLORA_STATIC_SCRATCH_BYTES
@@ -189,16 +192,17 @@ def qlora_unpack(bits, K, N, Q, codes, stream=None):
 def qlora_lrec_loss(student_logits, teacher_logits, labels, lambda_kl, lambda_ce, grad_scale, loss_tokens, dlogits, stream=None):
     """Fused KL + cross-entropy loss of the error-correction objective and its gradient; logits bf16 [T, V]."""
     T, V = student_logits.shape
-    _check(library().qlora_lrec_loss(int(T), int(V), _ptr(student_logits), _ptr(teacher_logits), _ptr(labels), float(lambda_kl),
-                                     float(lambda_ce), float(grad_scale), _ptr(loss_tokens), _ptr(dlogits), _stream(stream)),
-           "qlora_lrec_loss")
+    rc = _native().qlora_lrec_loss(T, V, student_logits, teacher_logits, labels, lambda_kl, lambda_ce, grad_scale, loss_tokens, dlogits, stream)
+    if rc != 0:
+        raise QloraError(rc, "qlora_lrec_loss")
 
 
 def qlora_gather_columns(inp, perm, out, stream=None):
     """out[m, j] = inp[m, perm[j]] for 2-D bf16 / fp16 / fp32 tensors; perm int32 [cols]."""
     rows, cols = inp.shape
-    _check(library().qlora_gather_columns(inp.element_size(), int(rows), int(cols), _ptr(inp), _ptr(perm), _ptr(out),
-                                          _stream(stream)), "qlora_gather_columns")
+    rc = _native().qlora_gather_columns(inp.element_size(), rows, cols, inp, perm, out, stream)
+    if rc != 0:
+        raise QloraError(rc, "qlora_gather_columns")
 
 
 def qlora_dequant(d, Q, scales, zeros, W, stream=None):
@@ -208,8 +212,9 @@ def qlora_dequant(d, Q, scales, zeros, W, stream=None):
 
 def qlora_quantize_rtn(d, W, Q, scales, zeros, stream=None):
     """Min-max round-to-nearest quantization of W fp32 [N, K] into packed Q, fp16 scales and zeros [K/g, N]."""
-    _check(library().qlora_quantize_rtn(ctypes.byref(d), _ptr(W), _ptr(Q), _ptr(scales), _ptr(zeros), _stream(stream)),
-           "qlora_quantize_rtn")
+    rc = _native().qlora_quantize_rtn(d, W, Q, scales, zeros, stream)
+    if rc != 0:
+        raise QloraError(rc, "qlora_quantize_rtn")
 
 
 def qlora_selftest_bounded_wait(limit_us: int, stream=None):

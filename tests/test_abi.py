@@ -170,3 +170,32 @@ def test_which_way_db_goes_is_a_host_side_plan(ql):
     assert ql.qlora_workspace_bytes(gate, 2048) >= 24 * 512 * 1024      # 24 split tiles of the forward
     with pytest.raises(ql.QloraError):
         ql.qlora_bwd_input_db_on_producers(ql.desc(5, 64, 4096, 4096, 8, 16.0), 2048)
+
+
+def test_argument_conversion_of_the_call_extension(ql):
+    """The calls that go through the C extension take what the binding always took: ints and objects with __index__ or __int__ for
+    sizes, None or an address or a contiguous tensor for pointers -- and refuse the rest with the same exceptions."""
+    import numpy as np
+    import torch
+    d = ql.desc(4, 128, 256, 256, 8, 16.0)
+    ok, need = 0x1000, ql.qlora_workspace_bytes(ql.desc(4, 128, 256, 256, 8, 16.0), 4)
+
+    def status(*args, **kw):
+        with pytest.raises(ql.QloraError) as e:
+            ql.qlora_fwd(*args, **kw)
+        return e.value.status
+    assert status(d, np.int64(4), ok + 2, ok, ok, ok, ok, ok, ok, None, ok, stream=0, workspace_bytes=need) == -3
+    assert status(d, 4.0, ok, ok, ok, ok, ok, ok, ok, None, ok, stream=0, workspace_bytes=np.int32(need - 1)) == -4
+    ws = torch.empty(need - 1, dtype=torch.uint8)                         # sized from the tensor: one byte too few
+    assert status(d, 4, ok, ok, ok, ok, ok, ok, ok, None, ws, stream=0) == -4
+    assert status(d, 4, ok, ok, ok, ok, ok, ok, ok, None, None, stream=0) == -4
+    with pytest.raises(ValueError, match="contiguous"):
+        ql.qlora_fwd(d, 4, torch.empty((4, 512))[:, ::2], ok, ok, ok, ok, ok, ok, None, ok, stream=0, workspace_bytes=need)
+    with pytest.raises(TypeError):
+        ql.qlora_fwd(None, 4, ok, ok, ok, ok, ok, ok, ok, None, ok, stream=0, workspace_bytes=need)
+    with pytest.raises(AttributeError):
+        ql.qlora_fwd(d, 4, "x", ok, ok, ok, ok, ok, ok, None, ok, stream=0, workspace_bytes=need)
+
+    class Stream:
+        cuda_stream = 0
+    assert status(d, 4, None, ok, ok, ok, ok, ok, ok, None, ok, stream=Stream(), workspace_bytes=need) == -1
