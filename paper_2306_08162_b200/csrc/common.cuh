@@ -111,9 +111,14 @@ __device__ __forceinline__ void dequant32(const uint32_t (&w)[BITS], const Group
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const int bitpos = (j + h) * BITS, wi = bitpos >> 5, sh = bitpos & 31;
-                uint32_t q = w[wi] >> sh;
-                if (sh + BITS > 32) q |= w[(wi + 1) % BITS] << (32 - sh);   // only the 3-bit format straddles words
-                q = (q & mask) | 0x4B000000u;
+                uint32_t q;
+                if constexpr (BITS == 8) {                                    // one byte permute: the code below the exponent of 2^23
+                    q = __byte_perm(w[wi], 0x4B000000u, 0x7540 + (j + h) % 4);
+                } else {
+                    q = w[wi] >> sh;
+                    if (sh + BITS > 32) q |= w[(wi + 1) % BITS] << (32 - sh);   // only the 3-bit format straddles words
+                    q = (q & mask) | 0x4B000000u;
+                }
                 f[h] = (__uint_as_float(q) - gp.bias) * gp.scale;
             }
             const __nv_bfloat162 pr = __floats2bfloat162_rn(f[0], f[1]);

@@ -205,19 +205,20 @@ __device__ __forceinline__ bool wait_counter(const unsigned* ctr, unsigned targe
 
 #include "lora_down_stream.cuh"
 
-// Eight of s * P as bf16 (the LoRA operand), or -- low != 0 -- what that rounding left over, again as bf16.
-__device__ __forceinline__ uint4 lora_p_chunk(const float4& a, const float4& b, float s, bool low) {
+// Eight of s * P as bf16 (the LoRA operand), and in `low` what that rounding left over, again as bf16.
+__device__ __forceinline__ uint4 lora_p_chunk(const float4& a, const float4& b, float s, uint4& low) {
     const float f[8] = {s * a.x, s * a.y, s * a.z, s * a.w, s * b.x, s * b.y, s * b.z, s * b.w};
-    uint32_t o[4];
+    uint32_t o[4], l[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        __nv_bfloat162 h = __floats2bfloat162_rn(f[2 * i], f[2 * i + 1]);
-        if (low) {                       // (nothing is left of a value that became infinite or was no number)
-            const float l0 = f[2 * i] - __low2float(h), l1 = f[2 * i + 1] - __high2float(h);
-            h = __floats2bfloat162_rn(fabsf(l0) < INFINITY ? l0 : 0.f, fabsf(l1) < INFINITY ? l1 : 0.f);
-        }
+        const __nv_bfloat162 h = __floats2bfloat162_rn(f[2 * i], f[2 * i + 1]);
+        // (nothing is left of a value that became infinite or was no number)
+        const float l0 = f[2 * i] - __low2float(h), l1 = f[2 * i + 1] - __high2float(h);
+        const __nv_bfloat162 r = __floats2bfloat162_rn(fabsf(l0) < INFINITY ? l0 : 0.f, fabsf(l1) < INFINITY ? l1 : 0.f);
         o[i] = *reinterpret_cast<const uint32_t*>(&h);
+        l[i] = *reinterpret_cast<const uint32_t*>(&r);
     }
+    low = make_uint4(l[0], l[1], l[2], l[3]);
     return make_uint4(o[0], o[1], o[2], o[3]);
 }
 
@@ -430,34 +431,38 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
                 uint8_t* la = smem_gen + p.off_lora_a;
                 uint8_t* lp = smem_gen + p.off_lora_p;
                 const int row = et, wrow = w0 + row;
+                const int n8 = p.r >> 3;                      // chunks of eight ranks; the low pieces' chunks follow, then padding
                 for (int jc = 0; jc < p.r_pad / 8; ++jc) {
+                    if (p.lora_lo && jc >= n8) break;         // (no padding then: r_pad == 2 r)
                     uint4 v = make_uint4(0, 0, 0, 0);
-                    const int js = p.lora_lo && jc * 8 >= p.r ? jc * 8 - p.r : jc * 8;   // first rank of the chunk
-                    if (js < p.r && wrow < p.C) {
+                    if (jc < n8 && wrow < p.C) {
                         if (!TRANSPOSED) {
-                            v = __ldg(reinterpret_cast<const uint4*>(p.L + (size_t)wrow * p.r + js));      // B[n, j..j+7]
+                            v = __ldg(reinterpret_cast<const uint4*>(p.L + (size_t)wrow * p.r + jc * 8));      // B[n, j..j+7]
                         } else {
                             uint32_t e[8];
 #pragma unroll
                             for (int j = 0; j < 8; ++j)
-                                e[j] = __bfloat16_as_ushort(__ldg(p.L + (size_t)(js + j) * p.K + wrow));     // A[j, k]
+                                e[j] = __bfloat16_as_ushort(__ldg(p.L + (size_t)(jc * 8 + j) * p.K + wrow));     // A[j, k]
                             v = make_uint4(e[0] | (e[1] << 16), e[2] | (e[3] << 16), e[4] | (e[5] << 16), e[6] | (e[7] << 16));
                         }
                     }
-                    *reinterpret_cast<uint4*>(la + jc * (kWRows * 16) + (row >> 3) * 128 + (row & 7) * 16) = v;
+                    uint8_t* dst = la + jc * (kWRows * 16) + (row >> 3) * 128 + (row & 7) * 16;
+                    *reinterpret_cast<uint4*>(dst) = v;
+                    if (p.lora_lo) *reinterpret_cast<uint4*>(dst + n8 * (kWRows * 16)) = v;
                 }
                 for (int row_t = et; row_t < p.BT; row_t += 128) {
                     const int m = m0 + row_t;
                     for (int jc = 0; jc < p.r_pad / 8; ++jc) {
-                        uint4 v = make_uint4(0, 0, 0, 0);
-                        const bool low = p.lora_lo && jc * 8 >= p.r;
-                        const int js = low ? jc * 8 - p.r : jc * 8;
-                        if (js < p.r && m < p.M) {
+                        if (p.lora_lo && jc >= n8) break;
+                        uint4 v = make_uint4(0, 0, 0, 0), low = v;
+                        if (jc < n8 && m < p.M) {
                             // (not the read-only path: P may have been written by this launch's producer clusters)
-                            const float4* src = reinterpret_cast<const float4*>(p.Pmat + (size_t)m * p.r + js);
+                            const float4* src = reinterpret_cast<const float4*>(p.Pmat + (size_t)m * p.r + jc * 8);
                             v = lora_p_chunk(__ldcg(src), __ldcg(src + 1), p.s, low);
                         }
-                        *reinterpret_cast<uint4*>(lp + jc * (p.BT * 16) + (row_t >> 3) * 128 + (row_t & 7) * 16) = v;
+                        uint8_t* dst = lp + jc * (p.BT * 16) + (row_t >> 3) * 128 + (row_t & 7) * 16;
+                        *reinterpret_cast<uint4*>(dst) = v;
+                        if (p.lora_lo) *reinterpret_cast<uint4*>(dst + n8 * (p.BT * 16)) = low;
                     }
                 }
                 fence_proxy_async();

@@ -403,38 +403,42 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
                 // (the previous tile's LoRA MMA has completed: its accumulator-full barrier was observed below)
                 uint8_t* ll = smem_gen + p.off_lora_l;
                 uint8_t* lp = smem_gen + p.off_lora_p;
+                const int n8 = p.r >> 3;                  // chunks of eight ranks; the low pieces' chunks follow, then padding
                 {   // this CTA's 128 weight rows of B (forward) / columns of A (backward)
                     const int row = et, wrow = w0 + (int)cta * kPairW + row;
                     for (int jc = 0; jc < p.r_pad / 8; ++jc) {
+                        if (p.lora_lo && jc >= n8) break;     // (no padding then: r_pad == 2 r)
                         uint4 v = make_uint4(0, 0, 0, 0);
-                        const int js = p.lora_lo && jc * 8 >= p.r ? jc * 8 - p.r : jc * 8;   // first rank of the chunk
-                        if (js < p.r && wrow < p.C) {
+                        if (jc < n8 && wrow < p.C) {
                             if (!TRANSPOSED) {
-                                v = __ldg(reinterpret_cast<const uint4*>(p.L + (size_t)wrow * p.r + js));      // B[n, j..j+7]
+                                v = __ldg(reinterpret_cast<const uint4*>(p.L + (size_t)wrow * p.r + jc * 8));      // B[n, j..j+7]
                             } else {
                                 uint32_t e[8];
 #pragma unroll
                                 for (int j = 0; j < 8; ++j)
-                                    e[j] = __bfloat16_as_ushort(__ldg(p.L + (size_t)(js + j) * p.K + wrow));     // A[j, k]
+                                    e[j] = __bfloat16_as_ushort(__ldg(p.L + (size_t)(jc * 8 + j) * p.K + wrow));     // A[j, k]
                                 v = make_uint4(e[0] | (e[1] << 16), e[2] | (e[3] << 16), e[4] | (e[5] << 16), e[6] | (e[7] << 16));
                             }
                         }
-                        *reinterpret_cast<uint4*>(ll + jc * (kPairW * 16) + (row >> 3) * 128 + (row & 7) * 16) = v;
+                        uint8_t* dst = ll + jc * (kPairW * 16) + (row >> 3) * 128 + (row & 7) * 16;
+                        *reinterpret_cast<uint4*>(dst) = v;
+                        if (p.lora_lo) *reinterpret_cast<uint4*>(dst + n8 * (kPairW * 16)) = v;
                     }
                 }
 #pragma unroll
                 for (int a = 0; a < 2; ++a) {   // this CTA's token rows of s * H (or s * G) for both accumulators
                     const int m = m0 + a * (2 * kPairTok) + et;
                     for (int jc = 0; jc < p.r_pad / 8; ++jc) {
-                        uint4 v = make_uint4(0, 0, 0, 0);
-                        const bool low = p.lora_lo && jc * 8 >= p.r;
-                        const int js = low ? jc * 8 - p.r : jc * 8;
-                        if (js < p.r && m < p.M) {
+                        if (p.lora_lo && jc >= n8) break;
+                        uint4 v = make_uint4(0, 0, 0, 0), low = v;
+                        if (jc < n8 && m < p.M) {
                             // (not the read-only path: P may have been written by this launch's producer clusters)
-                            const float4* src = reinterpret_cast<const float4*>(p.Pmat + (size_t)m * p.r + js);
+                            const float4* src = reinterpret_cast<const float4*>(p.Pmat + (size_t)m * p.r + jc * 8);
                             v = lora_p_chunk(__ldcg(src), __ldcg(src + 1), p.s, low);
                         }
-                        *reinterpret_cast<uint4*>(lp + a * (kPairTok * p.r_pad * 2) + jc * (kPairTok * 16) + (et >> 3) * 128 + (et & 7) * 16) = v;
+                        uint8_t* dst = lp + a * (kPairTok * p.r_pad * 2) + jc * (kPairTok * 16) + (et >> 3) * 128 + (et & 7) * 16;
+                        *reinterpret_cast<uint4*>(dst) = v;
+                        if (p.lora_lo) *reinterpret_cast<uint4*>(dst + n8 * (kPairTok * 16)) = low;
                     }
                 }
                 fence_proxy_async();
