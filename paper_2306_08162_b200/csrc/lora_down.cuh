@@ -1,6 +1,6 @@
 // LoRA down-projection of one block of 16 token rows, as a device function shared by the stand-alone kernel
 // (simt_kernels.cu) and by the CTA-pair tensor-core kernel, whose idle SM pairs run it beside the main tiles.
-//   P[m, j] = out_scale * sum_t In[m, t] * L(j, t)     l_is_A: L = A [r, T] (contraction-contiguous), else L = B [T, r].
+//   P[m, j] = sum_t In[m, t] * L(j, t)     l_is_A: L = A [r, T] (contraction-contiguous), else L = B [T, r].
 // mma.sync m16n8k16 (bf16 in, fp32 accumulate) fed straight from 16-byte row loads: the warps of the block stride over
 // the contraction in steps of 32 and keep LD_UNROLL steps of loads in flight.  The 32 contraction indices of a step are
 // assigned to the fragments in a permuted order (lane q of a quad owns indices 8q..8q+7); activation and adapter fragments
@@ -40,8 +40,7 @@ __device__ __forceinline__ uint32_t movmatrix_trans(uint32_t a) {
 // `red` is shared memory for nwarps * NT * 128 floats.  In and L are read through the read-only path.
 template <bool L_IS_A, int NT>
 __device__ __forceinline__ void lora_down_rows(int M, int T, int r, const __nv_bfloat16* __restrict__ In,
-                                               const __nv_bfloat16* __restrict__ L, float* __restrict__ P,
-                                               const uint8_t* __restrict__ mask, float out_scale, int m_base, int nwarps,
+                                               const __nv_bfloat16* __restrict__ L, float* __restrict__ P, int m_base, int nwarps,
                                                float* red) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, q = lane & 3;
@@ -61,10 +60,6 @@ __device__ __forceinline__ void lora_down_rows(int M, int T, int r, const __nv_b
             const int k = kk + u * wstride + q * 8;            // T is a multiple of 8: 8 elements are all-in or all-out
             xlo[u] = (v0 && k < T) ? __ldg(reinterpret_cast<const uint4*>(row0 + k)) : zero4;
             xhi[u] = (v1 && k < T) ? __ldg(reinterpret_cast<const uint4*>(row1 + k)) : zero4;
-            if (mask != nullptr) {   // dropout on the branch input: dropped elements contribute nothing
-                if (v0 && k < T) xlo[u] = mask_eight(xlo[u], __ldg(reinterpret_cast<const uint2*>(mask + (size_t)r0 * T + k)));
-                if (v1 && k < T) xhi[u] = mask_eight(xhi[u], __ldg(reinterpret_cast<const uint2*>(mask + (size_t)r1 * T + k)));
-            }
         }
 #pragma unroll
         for (int u = 0; u < LD_UNROLL; ++u) {
@@ -107,7 +102,7 @@ __device__ __forceinline__ void lora_down_rows(int M, int T, int r, const __nv_b
         for (int w = 0; w < nwarps; ++w) v += red[((w * NT + nt) * 4 + c) * 32 + ln];
         const int row = m_base + (ln >> 2) + ((c & 2) ? 8 : 0);
         const int col = nt * 8 + (ln & 3) * 2 + (c & 1);
-        if (row < M && col < r) P[(size_t)row * r + col] = v * out_scale;
+        if (row < M && col < r) P[(size_t)row * r + col] = v;
     }
     __syncthreads();   // `red` may be rewritten by the next call
 }

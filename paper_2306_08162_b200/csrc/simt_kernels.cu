@@ -113,39 +113,190 @@ int launch_simt_gemm(const qlora_desc& d, int M, bool transposed, const void* In
 
 // ------------------------------------------------------------------------------------------------------------
 // LoRA down-projections: H = X A^T (contraction over K) and G = dY B (contraction over N), fp32 [M, r].
-// Skinny products bound by reading the activations once: a block owns 16 token rows (lora_down.cuh has the method).
+// Skinny products bound by reading the activations once.  Few rows, ranks up to 16, no mask: a block owns 16 token rows
+// (lora_down.cuh has the method).
 // ------------------------------------------------------------------------------------------------------------
 template <bool L_IS_A, int NT, int WARPS>
 __global__ void __launch_bounds__(WARPS * 32)
-lora_down_kernel(int M, int T, int r, const __nv_bfloat16* __restrict__ In, const __nv_bfloat16* __restrict__ L,
-                 float* __restrict__ P, const uint8_t* __restrict__ mask, float out_scale) {
+lora_down_kernel(int M, int T, int r, const __nv_bfloat16* __restrict__ In, const __nv_bfloat16* __restrict__ L, float* __restrict__ P) {
     __shared__ float red[WARPS * NT * 128];
     pdl_launch_dependents();
     pdl_wait();
-    lora_down_rows<L_IS_A, NT>(M, T, r, In, L, P, mask, out_scale, (int)blockIdx.x * 16, WARPS, red);
+    lora_down_rows<L_IS_A, NT>(M, T, r, In, L, P, (int)blockIdx.x * 16, WARPS, red);
+}
+
+// thread-block cluster helpers
+__device__ __forceinline__ uint32_t lg_map_to_cta(const void* smem_ptr, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(smem_ptr)), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ float4 lg_ld_cluster_f32x4(uint32_t cluster_addr) {
+    float4 v;
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(cluster_addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ void lg_cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// Ranks above 16, or a dropout mask: 16 token rows per cluster, the contraction split over its 1 << lcs CTAs and their eight warps.
+// Bound by the latency of the adapter and activation loads (the adapter's share of the loads grows with the rank), so a warp issues
+// all loads of DEPTH 32-wide steps together, and the cluster is as wide as keeps two CTAs per SM: 2048 tokens x 4096, rank 32,
+// inputs from DRAM: 18 -> 10 us (blocks of eight warps that waited for every step's adapter words before).
+// Fragments as in lora_down.cuh, except that a lane reads its 2 NT neighbouring ranks of a row of B in 16-byte pieces where the rank
+// fills the tiles: column c of tile i is then rank 2 NT (c / 2) + 2 i + c % 2.  Partial tiles: the warps' in order, then the CTAs' in
+// order, each CTA for a part of the elements: the same bits on every run.
+constexpr int LS_WARPS = 8;
+
+template <bool L_IS_A, int NT, bool MASKED>
+__global__ void __launch_bounds__(LS_WARPS * 32, 2)
+lora_down_split_kernel(int M, int T, int r, int lcs, const __nv_bfloat16* __restrict__ In, const __nv_bfloat16* __restrict__ L,
+                       float* __restrict__ P, const uint8_t* __restrict__ mask, float out_scale) {
+    constexpr int DEPTH = NT <= 2 ? 4 : (NT <= 4 ? 2 : 1), ELEMS = NT * 128;
+    __shared__ float red[LS_WARPS * ELEMS];
+    __shared__ float recv[ELEMS];                              // [CTA of the cluster][this CTA's share of the elements]
+    pdl_launch_dependents();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
+    const int cs = 1 << lcs, rank = (int)blockIdx.x & (cs - 1), m_base = ((int)blockIdx.x >> lcs) * 16;
+    const int steps = (T + 31) >> 5, s0 = (steps * rank) >> lcs, s1 = (steps * (rank + 1)) >> lcs;
+    const int r0 = m_base + g, r1 = r0 + 8;
+    const bool v0 = r0 < M, v1 = r1 < M, packed = r == 8 * NT;
+    const __nv_bfloat16* row0 = In + (size_t)r0 * T;
+    const __nv_bfloat16* row1 = In + (size_t)r1 * T;
+    float acc[NT][4];
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
+    const uint4 zero4 = make_uint4(0, 0, 0, 0);
+    pdl_wait();
+#pragma unroll 1
+    for (int st = s0 + warp; st < s1; st += LS_WARPS * DEPTH) {
+        uint4 xlo[DEPTH], xhi[DEPTH], l[DEPTH][NT];            // B: l[u][i] = tile i's words of the four 8 x 8 row tiles
+        uint2 mlo[DEPTH], mhi[DEPTH];
+#pragma unroll
+        for (int u = 0; u < DEPTH; ++u) {
+            const int k0 = (st + u * LS_WARPS) * 32, k = k0 + q * 8;
+            const bool in = st + u * LS_WARPS < s1 && k < T;   // T is a multiple of 8: 8 elements are all-in or all-out
+            xlo[u] = v0 && in ? __ldg(reinterpret_cast<const uint4*>(row0 + k)) : zero4;
+            xhi[u] = v1 && in ? __ldg(reinterpret_cast<const uint4*>(row1 + k)) : zero4;
+            if constexpr (MASKED) {
+                mlo[u] = v0 && in ? __ldg(reinterpret_cast<const uint2*>(mask + (size_t)r0 * T + k)) : make_uint2(0, 0);
+                mhi[u] = v1 && in ? __ldg(reinterpret_cast<const uint2*>(mask + (size_t)r1 * T + k)) : make_uint2(0, 0);
+            }
+            if constexpr (L_IS_A) {
+#pragma unroll
+                for (int nt = 0; nt < NT; ++nt)
+                    l[u][nt] = in && nt * 8 + g < r ? __ldg(reinterpret_cast<const uint4*>(L + (size_t)(nt * 8 + g) * T + k)) : zero4;
+            } else {
+                const int nb = k0 + 8 * (g >> 1) + (g & 1);    // tile t's row g <-> contraction index nb + 2 t
+                const bool on = st + u * LS_WARPS < s1 && nb < T;   // (T a multiple of 8: the four rows are all-in or all-out)
+                const __nv_bfloat16* src = L + (size_t)nb * r;
+#pragma unroll
+                for (int nt = 0; nt < NT; ++nt) l[u][nt] = zero4;
+                if (on) {
+                    if (packed && NT % 4 == 0) {
+#pragma unroll
+                        for (int h = 0; h < NT / 4; ++h) {
+                            const uint4 t0 = __ldg(reinterpret_cast<const uint4*>(src + 2 * NT * q + 8 * h));
+                            const uint4 t1 = __ldg(reinterpret_cast<const uint4*>(src + 2 * r + 2 * NT * q + 8 * h));
+                            const uint4 t2 = __ldg(reinterpret_cast<const uint4*>(src + 4 * r + 2 * NT * q + 8 * h));
+                            const uint4 t3 = __ldg(reinterpret_cast<const uint4*>(src + 6 * r + 2 * NT * q + 8 * h));
+                            l[u][(4 * h) % NT] = make_uint4(t0.x, t1.x, t2.x, t3.x);
+                            l[u][(4 * h + 1) % NT] = make_uint4(t0.y, t1.y, t2.y, t3.y);
+                            l[u][(4 * h + 2) % NT] = make_uint4(t0.z, t1.z, t2.z, t3.z);
+                            l[u][(4 * h + 3) % NT] = make_uint4(t0.w, t1.w, t2.w, t3.w);
+                        }
+                    } else {
+                        const int lane_r = packed ? 2 * NT * q : 2 * q, tile_r = packed ? 2 : 8;
+#pragma unroll
+                        for (int nt = 0; nt < NT; ++nt)
+                            if (nt * 8 < r) {
+                                const __nv_bfloat16* t = src + lane_r + tile_r * nt;
+                                l[u][nt] = make_uint4(__ldg(reinterpret_cast<const uint32_t*>(t)), __ldg(reinterpret_cast<const uint32_t*>(t + 2 * r)),
+                                                      __ldg(reinterpret_cast<const uint32_t*>(t + 4 * r)), __ldg(reinterpret_cast<const uint32_t*>(t + 6 * r)));
+                            }
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < DEPTH; ++u) {
+            if (st + u * LS_WARPS >= s1) break;                // warp-uniform
+            if constexpr (MASKED) { xlo[u] = mask_eight(xlo[u], mlo[u]); xhi[u] = mask_eight(xhi[u], mhi[u]); }
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt) {
+                uint4 lv = l[u][nt];
+                if constexpr (!L_IS_A) lv = make_uint4(movmatrix_trans(lv.x), movmatrix_trans(lv.y), movmatrix_trans(lv.z), movmatrix_trans(lv.w));
+                mma_bf16_16816(acc[nt], xlo[u].x, xhi[u].x, xlo[u].y, xhi[u].y, lv.x, lv.y);
+                mma_bf16_16816(acc[nt], xlo[u].z, xhi[u].z, xlo[u].w, xhi[u].w, lv.z, lv.w);
+            }
+        }
+    }
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) red[warp * ELEMS + (nt * 4 + c) * 32 + lane] = acc[nt][c];
+    __syncthreads();
+    const int share = ELEMS >> lcs;                            // elements a CTA finishes (a multiple of 16)
+    if (lcs > 0) lg_cluster_sync();                            // every CTA of the cluster is running: its shared memory may be written
+    for (int e = threadIdx.x; e < ELEMS; e += LS_WARPS * 32) {
+        float v = 0.f;
+#pragma unroll
+        for (int w = 0; w < LS_WARPS; ++w) v += red[w * ELEMS + e];
+        const int owner = e / share;
+        asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(lg_map_to_cta(recv + rank * share + (e - owner * share), (uint32_t)owner)), "f"(v) : "memory");
+    }
+    if (lcs > 0) lg_cluster_sync();                            // everyone's sums for this CTA's elements have arrived
+    else __syncthreads();
+    for (int i = threadIdx.x; i < share; i += LS_WARPS * 32) {
+        float v = 0.f;
+        for (int rk = 0; rk < cs; ++rk) v += recv[rk * share + i];
+        const int e = rank * share + i, nt = e >> 7, c = (e >> 5) & 3, ln = e & 31;
+        const int row = m_base + (ln >> 2) + ((c & 2) ? 8 : 0);
+        const int col = !L_IS_A && packed ? 2 * NT * (ln & 3) + 2 * nt + (c & 1) : nt * 8 + (ln & 3) * 2 + (c & 1);
+        if (row < M && col < r) P[(size_t)row * r + col] = v * out_scale;
+    }
 }
 
 int launch_lora_down(int M, int T, int r, bool l_is_A, const void* In, const void* L, float* P, cudaStream_t st,
                      const uint8_t* mask, float out_scale) {
     if (M == 0 || r == 0) return QLORA_OK;
+    const bool plain = mask == nullptr && out_scale == 1.0f && r <= 16;
     // Many rows, low rank: the streaming kernel (also the form that runs inside the CTA-pair kernel, so H / G have the
     // same bits whichever call produced them).
-    if (mask == nullptr && out_scale == 1.0f && M > 256 && r <= 16) return launch_lora_down_stream(M, T, r, l_is_A, In, L, P, st);
-    const unsigned grid = (unsigned)((M + 15) / 16);
+    if (plain && M > 256) return launch_lora_down_stream(M, T, r, l_is_A, In, L, P, st);
+    const unsigned blocks = (unsigned)((M + 15) / 16);
     const __nv_bfloat16* in = (const __nv_bfloat16*)In;
     const __nv_bfloat16* l = (const __nv_bfloat16*)L;
     const int nt = (r + 7) / 8;
     cudaError_t err = cudaSuccess;
-#define QLORA_LD(NTV, W)                                                                              \
+    if (plain) {
+#define QLORA_LD(NTV)                                                                                 \
     do {                                                                                              \
-        if (l_is_A) err = launch_pdl(lora_down_kernel<true, NTV, W>, dim3(grid), dim3(W * 32), 0, st, 1, M, T, r, in, l, P, mask, out_scale);   \
-        else        err = launch_pdl(lora_down_kernel<false, NTV, W>, dim3(grid), dim3(W * 32), 0, st, 1, M, T, r, in, l, P, mask, out_scale);  \
+        if (l_is_A) err = launch_pdl(lora_down_kernel<true, NTV, 32>, dim3(blocks), dim3(1024), 0, st, 1, M, T, r, in, l, P);   \
+        else        err = launch_pdl(lora_down_kernel<false, NTV, 32>, dim3(blocks), dim3(1024), 0, st, 1, M, T, r, in, l, P);  \
     } while (0)
-    if (nt <= 1) QLORA_LD(1, 32);
-    else if (nt <= 2) QLORA_LD(2, 32);
-    else if (nt <= 4) QLORA_LD(4, 8);
-    else QLORA_LD(8, 8);
+        if (nt <= 1) QLORA_LD(1);
+        else QLORA_LD(2);
 #undef QLORA_LD
+        return err == cudaSuccess ? QLORA_OK : QLORA_ERR_CUDA;
+    }
+    // clusters as wide as leave two CTAs per SM, while a CTA keeps a step for each of its warps
+    int lcs = 0;
+    while (lcs < 3 && (blocks << (lcs + 1)) <= 2u * (unsigned)sm_count() && (T >> (lcs + 1)) >= 32 * LS_WARPS) ++lcs;
+    const dim3 grid(blocks << lcs), block(LS_WARPS * 32);
+#define QLORA_LS(NTV)                                                                                                             \
+    do {                                                                                                                          \
+        if (!l_is_A)      err = launch_pdl(lora_down_split_kernel<false, NTV, false>, grid, block, 0, st, 1u << lcs, M, T, r, lcs, in, l, P, (const uint8_t*)nullptr, out_scale); \
+        else if (mask)    err = launch_pdl(lora_down_split_kernel<true, NTV, true>, grid, block, 0, st, 1u << lcs, M, T, r, lcs, in, l, P, mask, out_scale);   \
+        else              err = launch_pdl(lora_down_split_kernel<true, NTV, false>, grid, block, 0, st, 1u << lcs, M, T, r, lcs, in, l, P, mask, out_scale);  \
+    } while (0)
+    if (!l_is_A && mask != nullptr) return QLORA_ERR_INVALID_ARG;   // (a mask is on the input of the first adapter only)
+    if (nt <= 1) QLORA_LS(1);
+    else if (nt <= 2) QLORA_LS(2);
+    else if (nt <= 4) QLORA_LS(4);
+    else QLORA_LS(8);
+#undef QLORA_LS
     return err == cudaSuccess ? QLORA_OK : QLORA_ERR_CUDA;
 }
 
@@ -197,21 +348,6 @@ struct GradSide {
     float scale;               // s (times the dropout keep scale on the masked side)
     int out_is_dB;             // Out is dB [C, r] (else dA [r, C])
 };
-
-// thread-block cluster helpers of the one-launch form below
-__device__ __forceinline__ uint32_t lg_map_to_cta(const void* smem_ptr, uint32_t rank) {
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(smem_ptr)), "r"(rank));
-    return r;
-}
-__device__ __forceinline__ float4 lg_ld_cluster_f32x4(uint32_t cluster_addr) {
-    float4 v;
-    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(cluster_addr) : "memory");
-    return v;
-}
-__device__ __forceinline__ void lg_cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 
 // CL == 0: grid (column blocks, slices, 2 sides); the block writes its partial tile to scratch for lora_grad_reduce_kernel.
 // CL >= 1: one launch does it all.  grid (column blocks * CL, 1, 2 sides) in clusters of CL CTAs along x; the CTAs of a

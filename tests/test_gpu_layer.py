@@ -399,3 +399,16 @@ def test_infinite_branch_values_stay_infinite(M, g):
     Y = torch.empty((M, gl.N), dtype=torch.bfloat16, device="cuda")
     ql.qlora_fwd(gl.desc, M, X, gl.Q, gl.scales, gl.zeros, gl.A, gl.B, Y, None, gl.ws)
     assert torch.isinf(Y).all() and (Y[0::2] > 0).all() and (Y[1::2] < 0).all()
+
+
+@pytest.mark.parametrize("r", [24, 32, 40, 64])
+@pytest.mark.parametrize("M,K,N", [(1, 96, 40), (16, 4096, 1032), (17, 352, 264), (300, 1024, 192), (2500, 256, 128)])
+def test_ranks_above_16_split_down_projection(M, K, N, r):
+    """Ranks above 16: H and G from clusters of one to eight CTAs per 16 token rows (a short contraction is not split, the last
+    step of 32 may be ragged: N = 40, 1032, 264), ranks that fill the register tiles (32, 64) and ranks that do not (24, 40)."""
+    g = 32 if K % 64 else 64
+    layer = qi.random_codes_layer(K=K, N=N, bits=4, group_size=g, r=r, alpha=2.0 * r, M=M, seed=M + r)
+    errs, saved, gl = check_layer(layer, rows=sample_rows(M, seed=r), tol=2e-2)
+    assert errs["H"] < 1e-4 and errs["G"] < 1e-4             # fp32 sums of exact products
+    again = gl.run(save_hg=False)
+    assert torch.equal(saved["dA"], again["dA"]) and torch.equal(saved["dB"], again["dB"])
