@@ -354,7 +354,9 @@ struct GradSide {
 //   cluster take the CL row slices of one column block, leave their partial tiles in shared memory, and after a cluster
 //   barrier CTA i adds them in slice order (distributed shared memory, fixed order) for its 256 / CL columns, scales
 //   and writes (or adds to) dA / dB.
-template <int RT, int CL>   // rank tiles of 16; cluster width (0 = two-launch form)
+// MASKED: side 1 (dA) has a dropout mask on its activations; the mask bytes travel with the loads of their round and are applied when
+// the round's turn comes (applied as they were loaded they made every round wait for memory: 29 against 13.7 us at 1800 tokens).
+template <int RT, int CL, bool MASKED>   // rank tiles of 16; cluster width (0 = two-launch form)
 __global__ void __launch_bounds__(LG_WARPS * 32)
 lora_grad_partial_kernel(int M, int r, int rows_per_slice, GradSide side0, GradSide side1, int accumulate) {
     extern __shared__ __align__(16) uint8_t lg_smem[];
@@ -392,15 +394,19 @@ lora_grad_partial_kernel(int M, int r, int rows_per_slice, GradSide side0, GradS
     const int m_stop = min(M, m_begin + rows_per_slice);
     // two register sets: the loads of the next round of 16-row steps are in flight while this round is transposed and multiplied
     uint4 n0[LG_UNROLL], n1[LG_UNROLL];
+    uint2 k0[MASKED ? LG_UNROLL : 1], k1[MASKED ? LG_UNROLL : 1];
+    const bool masked = MASKED && sd.mask != nullptr;
     auto load_round = [&](int mm) {
 #pragma unroll
         for (int u = 0; u < LG_UNROLL; ++u) {
             const int ma = mm + 16 * u + g, mb = ma + 8;
             n0[u] = (live && ma < m_stop) ? *reinterpret_cast<const uint4*>(src + (size_t)ma * C) : zero4;
             n1[u] = (live && mb < m_stop) ? *reinterpret_cast<const uint4*>(src + (size_t)mb * C) : zero4;
-            if (sd.mask != nullptr) {
-                if (live && ma < m_stop) n0[u] = mask_eight(n0[u], __ldg(reinterpret_cast<const uint2*>(sd.mask + (size_t)ma * C + c0)));
-                if (live && mb < m_stop) n1[u] = mask_eight(n1[u], __ldg(reinterpret_cast<const uint2*>(sd.mask + (size_t)mb * C + c0)));
+            if constexpr (MASKED) {
+                if (masked) {
+                    if (live && ma < m_stop) k0[u] = __ldg(reinterpret_cast<const uint2*>(sd.mask + (size_t)ma * C + c0));
+                    if (live && mb < m_stop) k1[u] = __ldg(reinterpret_cast<const uint2*>(sd.mask + (size_t)mb * C + c0));
+                }
             }
         }
     };
@@ -408,7 +414,12 @@ lora_grad_partial_kernel(int M, int r, int rows_per_slice, GradSide side0, GradS
     for (int mm = m_begin; mm < m_stop; mm += 16 * LG_UNROLL) {
         uint4 x0[LG_UNROLL], x1[LG_UNROLL];
 #pragma unroll
-        for (int u = 0; u < LG_UNROLL; ++u) { x0[u] = n0[u]; x1[u] = n1[u]; }
+        for (int u = 0; u < LG_UNROLL; ++u) {
+            x0[u] = n0[u]; x1[u] = n1[u];
+            if constexpr (MASKED) {
+                if (masked) { x0[u] = mask_eight(x0[u], k0[u]); x1[u] = mask_eight(x1[u], k1[u]); }   // (rows beyond the last are zero anyway)
+            }
+        }
         if (mm + 16 * LG_UNROLL < m_stop) load_round(mm + 16 * LG_UNROLL);
 #pragma unroll
         for (int u = 0; u < LG_UNROLL; ++u) {
@@ -528,6 +539,7 @@ int launch_lora_grads(int M, int K, int N, int r, float s, const void* X, const 
     const int cols = want_dB && want_dA ? (N > K ? N : K) : (want_dB ? N : K);
     const int col_blocks = (cols + LG_COLS - 1) / LG_COLS;
     const int rt = (r + 15) / 16;
+    const bool masked = want_dA && x_mask != nullptr;
     cudaError_t err = cudaSuccess;
     // Up to 256 tokens: one launch; the (at most four) 64-row slices of a column block form a cluster and reduce through
     // distributed shared memory.  (With more tokens, clusters of eight slices measured slower than free-floating blocks
@@ -542,12 +554,14 @@ int launch_lora_grads(int M, int K, int N, int r, float s, const void* X, const 
         const size_t pt_bytes = (size_t)rt * 16 * (rows_cl + 8) * sizeof(__nv_bfloat16), tile_bytes = (size_t)LG_COLS * rt * 16 * sizeof(float);
         const size_t smem = pt_bytes > tile_bytes ? pt_bytes : tile_bytes;
         const dim3 grid((unsigned)(col_blocks * cl), 1, (unsigned)n_sides);
-#define QLORA_LGC(RTV, CLV)                                                                                    \
+#define QLORA_LGC_M(RTV, CLV, MK)                                                                              \
     do {                                                                                                       \
         static SmemLimit limit;                                                                                \
-        if (!limit.raise(lora_grad_partial_kernel<RTV, CLV>, (size_t)RTV * 16 * (1024 + 8) * 2)) return QLORA_ERR_CUDA; \
-        err = launch_pdl(lora_grad_partial_kernel<RTV, CLV>, grid, dim3(LG_WARPS * 32), smem, st, CLV, M, r, rows_cl, sB, sA, accumulate); \
+        if (!limit.raise(lora_grad_partial_kernel<RTV, CLV, MK>, (size_t)RTV * 16 * (1024 + 8) * 2)) return QLORA_ERR_CUDA; \
+        err = launch_pdl(lora_grad_partial_kernel<RTV, CLV, MK>, grid, dim3(LG_WARPS * 32), smem, st, CLV, M, r, rows_cl, sB, sA, accumulate); \
     } while (0)
+#define QLORA_LGC(RTV, CLV)                                                                                    \
+    do { if (masked) QLORA_LGC_M(RTV, CLV, true); else QLORA_LGC_M(RTV, CLV, false); } while (0)
 #define QLORA_LGC_RT(CLV)                                                                                      \
     switch (rt) {                                                                                              \
         case 1: QLORA_LGC(1, CLV); break;                                                                      \
@@ -562,6 +576,7 @@ int launch_lora_grads(int M, int K, int N, int r, float s, const void* X, const 
         }
 #undef QLORA_LGC_RT
 #undef QLORA_LGC
+#undef QLORA_LGC_M
         return err == cudaSuccess ? QLORA_OK : QLORA_ERR_CUDA;
     }
     // More tokens: partial sums per row slice to scratch, then a reduction launch.
@@ -586,12 +601,14 @@ int launch_lora_grads(int M, int K, int N, int r, float s, const void* X, const 
     if (!want_dB) sB = sA;
     dim3 grid(col_blocks, plan.slices, (unsigned)n_sides);
     const size_t smem = (size_t)rt * 16 * (plan.rows_per_slice + 8) * sizeof(__nv_bfloat16);
-#define QLORA_LG(RTV)                                                                                          \
+#define QLORA_LG_M(RTV, MK)                                                                                    \
     do {                                                                                                       \
         static SmemLimit limit;                                                                                \
-        if (!limit.raise(lora_grad_partial_kernel<RTV, 0>, (size_t)RTV * 16 * (1024 + 8) * 2)) return QLORA_ERR_CUDA; \
-        err = launch_pdl(lora_grad_partial_kernel<RTV, 0>, grid, dim3(LG_WARPS * 32), smem, st, 1, M, r, plan.rows_per_slice, sB, sA, accumulate); \
+        if (!limit.raise(lora_grad_partial_kernel<RTV, 0, MK>, (size_t)RTV * 16 * (1024 + 8) * 2)) return QLORA_ERR_CUDA; \
+        err = launch_pdl(lora_grad_partial_kernel<RTV, 0, MK>, grid, dim3(LG_WARPS * 32), smem, st, 1, M, r, plan.rows_per_slice, sB, sA, accumulate); \
     } while (0)
+#define QLORA_LG(RTV)                                                                                          \
+    do { if (masked) QLORA_LG_M(RTV, true); else QLORA_LG_M(RTV, false); } while (0)
     switch (rt) {
         case 1: QLORA_LG(1); break;
         case 2: QLORA_LG(2); break;
@@ -599,6 +616,7 @@ int launch_lora_grads(int M, int K, int N, int r, float s, const void* X, const 
         default: QLORA_LG(4); break;
     }
 #undef QLORA_LG
+#undef QLORA_LG_M
     if (err != cudaSuccess) return QLORA_ERR_CUDA;
     const GradSide& rB = want_dB ? sB : none;
     const GradSide& rA = want_dA ? sA : none;
@@ -611,50 +629,73 @@ int launch_lora_grads(int M, int K, int N, int r, float s, const void* X, const 
 // LoRA dropout, backward through the branch input: dX[m, k] += mask[m, k] * c * sum_j G[m, j] A[j, k]   (c = s * keep scale).
 // The tensor-core kernels add the LoRA term inside the accumulator, where a per-element mask cannot be applied, so with
 // dropout they run without the branch and this elementwise pass adds the masked term (dX is read and rounded once more).
-// One thread = 8 consecutive k of one token row.
+// Bound by reading and writing dX and reading the mask (5 bytes per element).  One thread = 8 consecutive k of LU_ROWS token rows: A is
+// read once for all of them (row by row it came from L2 64 KB at a time, 118 MB in all at 1800 tokens x 4096, rank 8: 16 us; now
+// 12 us), and the loads of dX and the mask are all under way before the products.
 // ------------------------------------------------------------------------------------------------------------
+constexpr int LU_ROWS = 4;
+
 __global__ void __launch_bounds__(256)
 lora_masked_update_kernel(int M, int K, int r, float c, const float* __restrict__ G, const __nv_bfloat16* __restrict__ A,
                           const uint8_t* __restrict__ mask, __nv_bfloat16* __restrict__ dX) {
     pdl_launch_dependents();
     pdl_wait();
-    const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int kchunks = K / 8;
-    if (idx >= (size_t)M * kchunks) return;
-    const int m = (int)(idx / kchunks), k = (int)(idx % kchunks) * 8;
-    const uint2 mb = __ldg(reinterpret_cast<const uint2*>(mask + (size_t)m * K + k));
-    if ((mb.x | mb.y) == 0u) return;
-    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    for (int j = 0; j < r; ++j) {
-        const float gj = __ldg(G + (size_t)m * r + j);
-        const uint4 av = __ldg(reinterpret_cast<const uint4*>(A + (size_t)j * K + k));
-        acc[0] = fmaf(gj, bf16_lo(av.x), acc[0]); acc[1] = fmaf(gj, bf16_hi(av.x), acc[1]);
-        acc[2] = fmaf(gj, bf16_lo(av.y), acc[2]); acc[3] = fmaf(gj, bf16_hi(av.y), acc[3]);
-        acc[4] = fmaf(gj, bf16_lo(av.z), acc[4]); acc[5] = fmaf(gj, bf16_hi(av.z), acc[5]);
-        acc[6] = fmaf(gj, bf16_lo(av.w), acc[6]); acc[7] = fmaf(gj, bf16_hi(av.w), acc[7]);
-    }
-    uint4* px = reinterpret_cast<uint4*>(dX + (size_t)m * K + k);
-    const uint4 xv = *px;
-    const uint32_t xin[4] = {xv.x, xv.y, xv.z, xv.w};
-    const uint32_t mbytes[2] = {mb.x, mb.y};
-    uint32_t o[4];
+    const int kc = (int)(blockIdx.x * blockDim.x + threadIdx.x), k = kc * 8, m0 = (int)blockIdx.y * LU_ROWS;
+    if (k >= K) return;
+    uint4 xv[LU_ROWS];
+    uint2 mb[LU_ROWS];
+    float acc[LU_ROWS][8];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const uint32_t m2 = mbytes[i >> 1] >> (16 * (i & 1));
-        const float lo = bf16_lo(xin[i]) + ((m2 & 0xFFu) ? c * acc[2 * i] : 0.f);
-        const float hi = bf16_hi(xin[i]) + ((m2 & 0xFF00u) ? c * acc[2 * i + 1] : 0.f);
-        const __nv_bfloat162 pr = __floats2bfloat162_rn(lo, hi);
-        o[i] = *reinterpret_cast<const uint32_t*>(&pr);
+    for (int i = 0; i < LU_ROWS; ++i) {
+        const bool in = m0 + i < M;
+        xv[i] = in ? *reinterpret_cast<const uint4*>(dX + (size_t)(m0 + i) * K + k) : make_uint4(0, 0, 0, 0);
+        mb[i] = in ? __ldg(reinterpret_cast<const uint2*>(mask + (size_t)(m0 + i) * K + k)) : make_uint2(0, 0);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) acc[i][e] = 0.f;
     }
-    *px = make_uint4(o[0], o[1], o[2], o[3]);
+    for (int j = 0; j < r; j += 4) {                           // (r is a multiple of 8)
+        uint4 av[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) av[t] = __ldg(reinterpret_cast<const uint4*>(A + (size_t)(j + t) * K + k));
+#pragma unroll
+        for (int i = 0; i < LU_ROWS; ++i) {
+            const float4 g4 = __ldg(reinterpret_cast<const float4*>(G + (size_t)min(m0 + i, M - 1) * r + j));
+            const float g[4] = {g4.x, g4.y, g4.z, g4.w};
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                acc[i][0] = fmaf(g[t], bf16_lo(av[t].x), acc[i][0]); acc[i][1] = fmaf(g[t], bf16_hi(av[t].x), acc[i][1]);
+                acc[i][2] = fmaf(g[t], bf16_lo(av[t].y), acc[i][2]); acc[i][3] = fmaf(g[t], bf16_hi(av[t].y), acc[i][3]);
+                acc[i][4] = fmaf(g[t], bf16_lo(av[t].z), acc[i][4]); acc[i][5] = fmaf(g[t], bf16_hi(av[t].z), acc[i][5]);
+                acc[i][6] = fmaf(g[t], bf16_lo(av[t].w), acc[i][6]); acc[i][7] = fmaf(g[t], bf16_hi(av[t].w), acc[i][7]);
+            }
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < LU_ROWS; ++i) {
+        if (m0 + i >= M || (mb[i].x | mb[i].y) == 0u) continue;
+        const uint32_t xin[4] = {xv[i].x, xv[i].y, xv[i].z, xv[i].w}, mbytes[2] = {mb[i].x, mb[i].y};
+        uint32_t o[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const uint32_t m2 = mbytes[e >> 1] >> (16 * (e & 1));
+            const float lo = bf16_lo(xin[e]) + ((m2 & 0xFFu) ? c * acc[i][2 * e] : 0.f);
+            const float hi = bf16_hi(xin[e]) + ((m2 & 0xFF00u) ? c * acc[i][2 * e + 1] : 0.f);
+            const __nv_bfloat162 pr = __floats2bfloat162_rn(lo, hi);
+            o[e] = *reinterpret_cast<const uint32_t*>(&pr);
+        }
+        *reinterpret_cast<uint4*>(dX + (size_t)(m0 + i) * K + k) = make_uint4(o[0], o[1], o[2], o[3]);
+    }
 }
 
 int launch_lora_masked_update(int M, int K, int r, float c, const float* G, const void* A, const uint8_t* mask, void* dX,
                               cudaStream_t st) {
     if (M == 0 || K == 0 || r == 0) return QLORA_OK;
-    const size_t total = (size_t)M * (K / 8);
-    const cudaError_t err = launch_pdl(lora_masked_update_kernel, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, st, 1, M, K, r,
-                                       c, G, (const __nv_bfloat16*)A, mask, (__nv_bfloat16*)dX);
+    cudaError_t err = cudaSuccess;
+    for (int m = 0; m < M && err == cudaSuccess; m += 65535 * LU_ROWS) {       // (the grid's height has a limit)
+        const int rows = M - m < 65535 * LU_ROWS ? M - m : 65535 * LU_ROWS;
+        err = launch_pdl(lora_masked_update_kernel, dim3((unsigned)((K / 8 + 255) / 256), (unsigned)((rows + LU_ROWS - 1) / LU_ROWS)), dim3(256), 0, st, 1,
+                         rows, K, r, c, G + (size_t)m * r, (const __nv_bfloat16*)A, mask + (size_t)m * K, (__nv_bfloat16*)dX + (size_t)m * K);
+    }
     return err == cudaSuccess ? QLORA_OK : QLORA_ERR_CUDA;
 }
 

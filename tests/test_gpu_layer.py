@@ -412,3 +412,31 @@ def test_ranks_above_16_split_down_projection(M, K, N, r):
     assert errs["H"] < 1e-4 and errs["G"] < 1e-4             # fp32 sums of exact products
     again = gl.run(save_hg=False)
     assert torch.equal(saved["dA"], again["dA"]) and torch.equal(saved["dB"], again["dB"])
+
+
+@pytest.mark.parametrize("M,K,N,r", [(1, 32, 8, 8), (5, 96, 72, 16), (333, 2080, 264, 8), (1801, 256, 128, 16), (260, 128, 64, 64)])
+def test_lora_dropout_ragged_rows(M, K, N, r):
+    """The masked paths at row counts that are no multiple of anything: masked down-projection, masked gradient, masked update."""
+    import paper_2306_08162_b200 as ql
+    g = 32
+    layer = qi.random_codes_layer(K=K, N=N, bits=4, group_size=g, r=r, alpha=2.0 * r, M=M, seed=700 + M)
+    gl = GpuLayer(layer)
+    p = 0.25
+    mask_np = (np.random.default_rng(M).random((M, K)) >= p).astype(np.uint8) * 255
+    mask = torch.from_numpy(mask_np).cuda()
+    Y = torch.empty((M, N), dtype=torch.bfloat16, device="cuda"); dX = torch.empty((M, K), dtype=torch.bfloat16, device="cuda")
+    H = torch.empty((M, r), dtype=torch.float32, device="cuda"); G = torch.empty_like(H)
+    dA = torch.empty((r, K), dtype=torch.float32, device="cuda"); dB = torch.empty((N, r), dtype=torch.float32, device="cuda")
+    keep = 1.0 / (1.0 - p)
+    ql.qlora_fwd_dropout(gl.desc, M, gl.X, mask, keep, gl.Q, gl.scales, gl.zeros, gl.A, gl.B, Y, H, gl.ws)
+    ql.qlora_bwd_input_dropout(gl.desc, M, gl.dY, mask, keep, gl.Q, gl.scales, gl.zeros, gl.A, gl.B, dX, G, gl.ws)
+    ql.qlora_bwd_lora_dropout(gl.desc, M, gl.X, mask, keep, gl.dY, gl.A, gl.B, H, G, dA, dB, 0, gl.ws)
+    assert ql.qlora_device_status() == 0
+    f64 = orc.bf16_bits_to_f64
+    W = orc.dequant(orc.pack(layer["codes"], 4), layer["scales"], layer["zeros"], 4, g)
+    Xr, dYr, Ar, Br = f64(layer["X"]), f64(layer["dY"]), f64(layer["A"]), f64(layer["B"])
+    Yo, Ho = orc.forward_dropout(Xr, W, Ar, Br, layer["alpha"], (mask_np != 0).astype(np.uint8), p)
+    dXo, dAo, dBo, Go = orc.backward_dropout(Xr, dYr, W, Ar, Br, layer["alpha"], (mask_np != 0).astype(np.uint8), p)
+    # few terms (K = 32, 96; N = 8) leave the rounding of single weights visible; H and G are fp32 sums of exact products
+    for name, got, want, tol in (("Y", Y, Yo, 3e-2), ("H", H, Ho, 1e-4), ("dX", dX, dXo, 3e-2), ("G", G, Go, 1e-4), ("dA", dA, dAo, REL_TOL), ("dB", dB, dBo, REL_TOL)):
+        assert rel_err(to_f64(got), want) <= tol, name
