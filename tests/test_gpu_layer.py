@@ -440,3 +440,16 @@ def test_lora_dropout_ragged_rows(M, K, N, r):
     # few terms (K = 32, 96; N = 8) leave the rounding of single weights visible; H and G are fp32 sums of exact products
     for name, got, want, tol in (("Y", Y, Yo, 3e-2), ("H", H, Ho, 1e-4), ("dX", dX, dXo, 3e-2), ("G", G, Go, 1e-4), ("dA", dA, dAo, REL_TOL), ("dB", dB, dBo, REL_TOL)):
         assert rel_err(to_f64(got), want) <= tol, name
+
+
+@pytest.mark.parametrize("rows,cols,dtype", [(1, 8, torch.bfloat16), (63, 11008, torch.bfloat16), (64, 11008, torch.bfloat16), (333, 11008, torch.bfloat16),
+                                             (65, 1004, torch.bfloat16), (200, 4096, torch.float32), (64, 16000, torch.float32), (70, 6, torch.float32)])
+def test_gather_columns_both_forms(rows, cols, dtype):
+    """Whole rows through shared memory (from 64 rows, rows of whole 16-byte pieces that fit) and element by element otherwise."""
+    import paper_2306_08162_b200 as ql
+    x = torch.randn((rows, cols), device="cuda").to(dtype)
+    perm = torch.randperm(cols, device="cuda")
+    perm[0] = perm[-1]                                       # not a permutation: any column may be read more than once
+    out = torch.full_like(x, float("nan"))
+    ql.qlora_gather_columns(x, perm.int(), out)
+    assert torch.equal(out, x[:, perm])
