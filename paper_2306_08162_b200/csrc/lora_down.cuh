@@ -2,7 +2,7 @@
 // (simt_kernels.cu) and by the CTA-pair tensor-core kernel, whose idle SM pairs run it beside the main tiles.
 //   P[m, j] = sum_t In[m, t] * L(j, t)     l_is_A: L = A [r, T] (contraction-contiguous), else L = B [T, r].
 // mma.sync m16n8k16 (bf16 in, fp32 accumulate) fed straight from 16-byte row loads: the warps of the block stride over
-// the contraction in steps of 32 and keep LD_UNROLL steps of loads in flight.  The 32 contraction indices of a step are
+// the contraction in steps of 32 and keep LD_UNROLL steps of loads in flight, the adapter's among them.  The 32 contraction indices of a step are
 // assigned to the fragments in a permuted order (lane q of a quad owns indices 8q..8q+7); activation and adapter fragments
 // use the same permutation, so the sum is unchanged.  A is contraction-contiguous and loads directly; B is rank-contiguous,
 // so its 8 x 8 fragment tiles are loaded row-wise and transposed across the warp with movmatrix.  The per-warp partial
@@ -36,71 +36,81 @@ __device__ __forceinline__ uint32_t movmatrix_trans(uint32_t a) {
     return d;
 }
 
-// Rows m_base .. m_base + 15.  Called by all `nwarps` warps of a block (it synchronises the block twice);
-// `red` is shared memory for nwarps * NT * 128 floats.  In and L are read through the read-only path.
-template <bool L_IS_A, int NT>
+// Rows m_base .. m_base + 15 and, with NB = 2, the block of rows `block_stride` further on (beside the first: the same adapter words serve
+// both).  Called by all `nwarps` warps of a block (it synchronises the block twice); `red` is shared memory for nwarps * NB * NT * 128
+// floats.  L is read through the read-only path, and so is In.
+template <bool L_IS_A, int NT, int NB = 1>
 __device__ __forceinline__ void lora_down_rows(int M, int T, int r, const __nv_bfloat16* __restrict__ In,
-                                               const __nv_bfloat16* __restrict__ L, float* __restrict__ P, int m_base, int nwarps,
+                                               const __nv_bfloat16* __restrict__ L, float* __restrict__ P, int m_base, int block_stride, int nwarps,
                                                float* red) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, q = lane & 3;
-    const int r0 = m_base + g, r1 = r0 + 8;
-    const __nv_bfloat16* row0 = In + (size_t)r0 * T;
-    const __nv_bfloat16* row1 = In + (size_t)r1 * T;
-    const bool v0 = r0 < M, v1 = r1 < M;
-    float acc[NT][4];
+    float acc[NB][NT][4];
 #pragma unroll
-    for (int nt = 0; nt < NT; ++nt) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
+    for (int b = 0; b < NB; ++b)
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt) acc[b][nt][0] = acc[b][nt][1] = acc[b][nt][2] = acc[b][nt][3] = 0.f;
     const uint4 zero4 = make_uint4(0, 0, 0, 0);
     const int wstride = nwarps * 32;
+#pragma unroll 1
     for (int kk = warp * 32; kk < T; kk += wstride * LD_UNROLL) {
-        uint4 xlo[LD_UNROLL], xhi[LD_UNROLL];
+        uint4 xlo[NB][LD_UNROLL], xhi[NB][LD_UNROLL], l[LD_UNROLL][NT];
 #pragma unroll
-        for (int u = 0; u < LD_UNROLL; ++u) {                 // all activation loads of the unrolled steps first
-            const int k = kk + u * wstride + q * 8;            // T is a multiple of 8: 8 elements are all-in or all-out
-            xlo[u] = (v0 && k < T) ? __ldg(reinterpret_cast<const uint4*>(row0 + k)) : zero4;
-            xhi[u] = (v1 && k < T) ? __ldg(reinterpret_cast<const uint4*>(row1 + k)) : zero4;
-        }
+        for (int u = 0; u < LD_UNROLL; ++u) {                 // all loads of the unrolled steps first
+            const int k0 = kk + u * wstride, k = k0 + q * 8;  // T is a multiple of 8: 8 elements are all-in or all-out
 #pragma unroll
-        for (int u = 0; u < LD_UNROLL; ++u) {
-            const int k0 = kk + u * wstride;                   // warp-uniform
-            if (k0 >= T) break;
-            const int k = k0 + q * 8;
+            for (int b = 0; b < NB; ++b) {
+                const int r0 = m_base + b * block_stride + g, r1 = r0 + 8;
+                xlo[b][u] = (r0 < M && k < T) ? __ldg(reinterpret_cast<const uint4*>(In + (size_t)r0 * T + k)) : zero4;
+                xhi[b][u] = (r1 < M && k < T) ? __ldg(reinterpret_cast<const uint4*>(In + (size_t)r1 * T + k)) : zero4;
+            }
 #pragma unroll
             for (int nt = 0; nt < NT; ++nt) {
                 uint4 lv = zero4;
                 if (L_IS_A) {
                     const int j = nt * 8 + g;                  // rank index of this lane's adapter fragment
                     if (k < T && j < r) lv = __ldg(reinterpret_cast<const uint4*>(L + (size_t)j * T + k));   // A[j, k..k+7]
-                } else {
-                    // tile t: row rho (0..7) <-> n = k0 + 8 (rho / 2) + (rho % 2) + 2 t, columns = ranks 8 nt .. 8 nt + 7;
-                    // after the transpose lane (g, q) holds B[k0 + 8q + 2t, 8nt + g], B[k0 + 8q + 2t + 1, 8nt + g]
-                    uint32_t w[4];
-#pragma unroll
-                    for (int t = 0; t < 4; ++t) {
-                        const int n = k0 + 8 * (g >> 1) + (g & 1) + 2 * t;
-                        uint32_t v = 0;
-                        if (n < T && nt * 8 < r) v = __ldg(reinterpret_cast<const uint32_t*>(L + (size_t)n * r + nt * 8 + 2 * q));
-                        w[t] = movmatrix_trans(v);
+                } else if (nt * 8 < r) {
+                    // tile t: row rho (0..7) <-> n = k0 + 8 (rho / 2) + (rho % 2) + 2 t, columns = ranks 8 nt .. 8 nt + 7
+                    const int n = k0 + 8 * (g >> 1) + (g & 1);
+                    if (n < T) {
+                        const __nv_bfloat16* src = L + (size_t)n * r + nt * 8 + 2 * q;
+                        lv = make_uint4(__ldg(reinterpret_cast<const uint32_t*>(src)), __ldg(reinterpret_cast<const uint32_t*>(src + 2 * r)),
+                                        __ldg(reinterpret_cast<const uint32_t*>(src + 4 * r)), __ldg(reinterpret_cast<const uint32_t*>(src + 6 * r)));
                     }
-                    lv = make_uint4(w[0], w[1], w[2], w[3]);
                 }
-                mma_bf16_16816(acc[nt], xlo[u].x, xhi[u].x, xlo[u].y, xhi[u].y, lv.x, lv.y);
-                mma_bf16_16816(acc[nt], xlo[u].z, xhi[u].z, xlo[u].w, xhi[u].w, lv.z, lv.w);
+                l[u][nt] = lv;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < LD_UNROLL; ++u) {
+            if (kk + u * wstride >= T) break;                  // warp-uniform
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt) {
+                uint4 lv = l[u][nt];
+                // after the transpose lane (g, q) holds B[k0 + 8q + 2t, 8nt + g], B[k0 + 8q + 2t + 1, 8nt + g]
+                if (!L_IS_A) lv = make_uint4(movmatrix_trans(lv.x), movmatrix_trans(lv.y), movmatrix_trans(lv.z), movmatrix_trans(lv.w));
+#pragma unroll
+                for (int b = 0; b < NB; ++b) {
+                    mma_bf16_16816(acc[b][nt], xlo[b][u].x, xhi[b][u].x, xlo[b][u].y, xhi[b][u].y, lv.x, lv.y);
+                    mma_bf16_16816(acc[b][nt], xlo[b][u].z, xhi[b][u].z, xlo[b][u].w, xhi[b][u].w, lv.z, lv.w);
+                }
             }
         }
     }
-    // red[warp][nt][c][lane]
+    // red[warp][b][nt][c][lane]
 #pragma unroll
-    for (int nt = 0; nt < NT; ++nt)
+    for (int b = 0; b < NB; ++b)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) red[((warp * NT + nt) * 4 + c) * 32 + lane] = acc[nt][c];
+        for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) red[(((warp * NB + b) * NT + nt) * 4 + c) * 32 + lane] = acc[b][nt][c];
     __syncthreads();
-    for (int idx = threadIdx.x; idx < NT * 128; idx += wstride) {
-        const int nt = idx >> 7, c = (idx >> 5) & 3, ln = idx & 31;
+    for (int idx = threadIdx.x; idx < NB * NT * 128; idx += wstride) {
+        const int b = idx / (NT * 128), nt = (idx >> 7) % NT, c = (idx >> 5) & 3, ln = idx & 31;
         float v = 0.f;
-        for (int w = 0; w < nwarps; ++w) v += red[((w * NT + nt) * 4 + c) * 32 + ln];
-        const int row = m_base + (ln >> 2) + ((c & 2) ? 8 : 0);
+        for (int w = 0; w < nwarps; ++w) v += red[(((w * NB + b) * NT + nt) * 4 + c) * 32 + ln];
+        const int row = m_base + b * block_stride + (ln >> 2) + ((c & 2) ? 8 : 0);
         const int col = nt * 8 + (ln & 3) * 2 + (c & 1);
         if (row < M && col < r) P[(size_t)row * r + col] = v;
     }

@@ -122,7 +122,7 @@ lora_down_kernel(int M, int T, int r, const __nv_bfloat16* __restrict__ In, cons
     __shared__ float red[WARPS * NT * 128];
     pdl_launch_dependents();
     pdl_wait();
-    lora_down_rows<L_IS_A, NT>(M, T, r, In, L, P, (int)blockIdx.x * 16, WARPS, red);
+    lora_down_rows<L_IS_A, NT>(M, T, r, In, L, P, (int)blockIdx.x * 16, 0, WARPS, red);
 }
 
 // thread-block cluster helpers

@@ -306,8 +306,16 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
         // the tiles leave idle (one CTA per row block or more; lowest block indices, so they wait for nobody)
         const int n_ctas = p.n_prod * p.split;
         pdl_wait();
-        if (p.r <= 8) lora_down_stream<!TRANSPOSED, 1>(p.M, p.T, p.r, p.In, p.Ldown, p.Pout, (int)blockIdx.x, n_ctas, smem_gen, p.lds_stages, abort_flag);
-        else          lora_down_stream<!TRANSPOSED, 2>(p.M, p.T, p.r, p.In, p.Ldown, p.Pout, (int)blockIdx.x, n_ctas, smem_gen, p.lds_stages, abort_flag);
+        if (p.M <= 256) {
+            // few row blocks (two per CTA at most) and a short main loop: 16-byte row loads, 120 KB of them in flight (the bulk copies of the
+            // streaming form bring 10 - 30 GB/s per SM: P came 5000 cycles after the main loops at 128 tokens, 4096 x 4096)
+            float* red = reinterpret_cast<float*>(smem_gen);
+            if (p.r <= 8) lora_down_rows<!TRANSPOSED, 1, 2>(p.M, p.T, p.r, p.In, p.Ldown, p.Pout, (int)blockIdx.x * 16, n_ctas * 16, kThreads / 32, red);
+            else          lora_down_rows<!TRANSPOSED, 2, 2>(p.M, p.T, p.r, p.In, p.Ldown, p.Pout, (int)blockIdx.x * 16, n_ctas * 16, kThreads / 32, red);
+        } else {
+            if (p.r <= 8) lora_down_stream<!TRANSPOSED, 1>(p.M, p.T, p.r, p.In, p.Ldown, p.Pout, (int)blockIdx.x, n_ctas, smem_gen, p.lds_stages, abort_flag);
+            else          lora_down_stream<!TRANSPOSED, 2>(p.M, p.T, p.r, p.In, p.Ldown, p.Pout, (int)blockIdx.x, n_ctas, smem_gen, p.lds_stages, abort_flag);
+        }
         __threadfence();       // every thread's rows of P are visible device-wide before the CTA is counted
         __syncthreads();
         if (threadIdx.x == 0) atomicAdd(&p.sync[0], 1u);
@@ -473,20 +481,7 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
             tc_fence_after();
             const int c = w0 + q * 32 + lane;                 // output column owned by this thread
             const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + buf * kAccStride;
-            if (p.split > 1) {
-                // this rank's part of the tile, fp32 [token][128 weight rows], over the (now idle) operand ring
-                float* part = reinterpret_cast<float*>(smem_gen);
-#pragma unroll 1
-                for (int cb = 0; cb < p.BT; cb += 16) {
-                    uint32_t v[16];
-                    tc_ld16(taddr + cb, v);
-                    tc_wait_ld();
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) part[(cb + j) * kWRows + q * 32 + lane] = __uint_as_float(v[j]);
-                }
-                tc_fence_before();
-                break;
-            }
+            if (p.split > 1) break;                           // (the parts of a split tile: below, with the dequant warps' help)
 #pragma unroll 1
             for (int cb = 0; cb < p.BT; cb += 16) {
                 uint32_t v[16];
@@ -571,6 +566,25 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
     }
 
 done:
+    if (p.split > 1 && warp >= kEpiWarp0 && first_tile >= 0 && first_tile < p.n_tiles) {
+        // This rank's part of the tile, fp32 [token][128 weight rows], over the (now idle) operand ring: the epilogue and the dequant
+        // warps, three per lane quarter, take 16 tokens at a time in turn.
+        __syncwarp();
+        if (warp_wait(bar_acc_full, 0u, abort_flag, lane)) {
+            tc_fence_after();
+            const int quarter = warp & 3;
+            float* part = reinterpret_cast<float*>(smem_gen) + quarter * 32 + lane;
+            const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16);
+#pragma unroll 1
+            for (int cb = 16 * ((warp - kEpiWarp0) >> 2); cb < p.BT; cb += 48) {
+                uint32_t v[16];
+                tc_ld16(taddr + cb, v);
+                tc_wait_ld();
+#pragma unroll
+                for (int j = 0; j < 16; ++j) part[(cb + j) * kWRows] = __uint_as_float(v[j]);
+            }
+        }
+    }
     // ---------------------------------------------------------------------- teardown
     tc_fence_before();
     __syncthreads();
@@ -590,14 +604,27 @@ done:
             const uint32_t part_addr = smem0;
             uint32_t peer[4];
             for (int rk = 0; rk < 4; ++rk) peer[rk] = map_to_cta(part_addr, (uint32_t)(rk < p.split ? rk : 0));
-            for (int e = threadIdx.x; e < tok_per_rank * (kWRows / 4); e += kThreads) {   // four weight rows (output columns) at a time
-                const int t = rank * tok_per_rank + e / (kWRows / 4), cw = (e % (kWRows / 4)) * 4;
-                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                for (int rk = 0; rk < p.split; ++rk) {
-                    const float4 x = ld_cluster_f32x4(peer[rk] + (uint32_t)((t * kWRows + cw) * 4));
-                    v.x += x.x; v.y += x.y; v.z += x.z; v.w += x.w;
+            // Four weight rows (output columns) at a time, two such pieces per turn: all reads of the peers are under way together (one
+            // after the other they took 4900 cycles at 128 tokens).  kThreads is a multiple of 32, so a thread's columns stay the same.
+            const int n_e = tok_per_rank * (kWRows / 4), cw = (threadIdx.x % (kWRows / 4)) * 4;
+#pragma unroll 1
+            for (int e0 = threadIdx.x; e0 < n_e; e0 += 2 * kThreads) {
+                float4 x[2][4];
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const int e = e0 + u * kThreads, t = rank * tok_per_rank + e / (kWRows / 4);
+#pragma unroll
+                    for (int rk = 0; rk < 4; ++rk)
+                        if (rk < p.split && e < n_e) x[u][rk] = ld_cluster_f32x4(peer[rk] + (uint32_t)((t * kWRows + cw) * 4));
                 }
-                if (m0 + t < p.M && w0 + cw < p.C) {     // C is a multiple of 8: four columns are all-in or all-out
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const int e = e0 + u * kThreads, t = rank * tok_per_rank + e / (kWRows / 4);
+                    if (e >= n_e || m0 + t >= p.M || w0 + cw >= p.C) continue;     // C is a multiple of 8: four columns are all-in or all-out
+                    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                    for (int rk = 0; rk < 4; ++rk)
+                        if (rk < p.split) { v.x += x[u][rk].x; v.y += x[u][rk].y; v.z += x[u][rk].z; v.w += x[u][rk].w; }
                     const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
                     *reinterpret_cast<uint2*>(p.Out + (size_t)(m0 + t) * p.C + w0 + cw) =
                         make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
