@@ -57,7 +57,7 @@ struct Params {
     // (r == 8, half an MMA's contraction is padding) and for groups of 32 (whose products the CUDA-core kernel gave in fp32).
     int lora_lo;
     int C;               // output columns (N forward, K backward)
-    int BT;              // token rows per tile (MMA N): 32, 64, 128 or 256
+    int BT;              // token rows per tile (MMA N): a multiple of 16, 32 .. 256
     int n_tok_tiles, n_tiles, steps;
     int split;           // CTAs per cluster sharing one tile, each taking `steps` consecutive steps of the contraction (1 = no cluster)
     int S, P;            // stages of the activation/weight ring and of the packed ring
@@ -942,7 +942,11 @@ int launch_umma_gemm(const qlora_desc& d, int M, bool transposed, const void* In
     p.M = M; p.N = d.N; p.K = d.K; p.bits = d.bits; p.g = d.group_size; p.r = d.r; p.lora_lo = keep_lora_low(d); p.r_pad = ((p.lora_lo ? 2 : 1) * d.r + 15) / 16 * 16;
     p.C = transposed ? d.K : d.N;
     const int T = transposed ? d.N : d.K;
-    p.BT = M > 128 ? 256 : (M > 64 ? 128 : (M > 32 ? 64 : 32));
+    // The tokens in as few tiles as 256 columns allow, cut evenly: a multiple of 16 (the MMA's N), not the next power of two, so that
+    // neither products nor the exchange between the ranks are made for tokens that do not exist (333: two tiles of 176, not 256).
+    p.n_tok_tiles = (M + 255) / 256;
+    p.BT = ((M + p.n_tok_tiles - 1) / p.n_tok_tiles + 15) / 16 * 16;
+    if (p.BT < 32) p.BT = 32;
     p.n_tok_tiles = (M + p.BT - 1) / p.BT;
     const int n_w_tiles = (p.C + kWRows - 1) / kWRows;
     p.n_tiles = p.n_tok_tiles * n_w_tiles;

@@ -453,3 +453,15 @@ def test_gather_columns_both_forms(rows, cols, dtype):
     out = torch.full_like(x, float("nan"))
     ql.qlora_gather_columns(x, perm.int(), out)
     assert torch.equal(out, x[:, perm])
+
+
+@pytest.mark.parametrize("M", [33, 47, 81, 145, 250, 257, 333, 520])
+@pytest.mark.parametrize("bits,K,N,r", [(4, 1024, 192, 8), (8, 512, 320, 16), (2, 2048, 64, 32)])
+def test_token_tiles_that_are_no_power_of_two(M, bits, K, N, r):
+    """Token tiles of the single-CTA kernel are cut evenly in multiples of 16 (81 -> 96, 145 -> 160, 333 -> two of 176), alone and
+    split over clusters whose ranks then finish odd numbers of tokens; producers with one and two row blocks, and none (rank 32)."""
+    layer = qi.random_codes_layer(K=K, N=N, bits=bits, group_size=64, r=r, alpha=2.0 * r, M=M, seed=M + bits)
+    _, out, gl = check_layer(layer)
+    again = gl.run()
+    for key in ("Y", "dX"):
+        assert torch.equal(out[key].view(torch.int16), again[key].view(torch.int16)), key
