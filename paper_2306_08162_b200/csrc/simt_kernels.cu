@@ -349,6 +349,11 @@ struct GradSide {
     int out_is_dB;             // Out is dB [C, r] (else dA [r, C])
 };
 
+// A 16-byte load that stays where it is written: ahead of the products of the round before.
+__device__ __forceinline__ void lg_load(uint4& v, const void* p) {
+    asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+}
+
 // CL == 0: grid (column blocks, slices, 2 sides); the block writes its partial tile to scratch for lora_grad_reduce_kernel.
 // CL >= 1: one launch does it all.  grid (column blocks * CL, 1, 2 sides) in clusters of CL CTAs along x; the CTAs of a
 //   cluster take the CL row slices of one column block, leave their partial tiles in shared memory, and after a cluster
@@ -356,8 +361,9 @@ struct GradSide {
 //   and writes (or adds to) dA / dB.
 // MASKED: side 1 (dA) has a dropout mask on its activations; the mask bytes travel with the loads of their round and are applied when
 // the round's turn comes (applied as they were loaded they made every round wait for memory: 29 against 13.7 us at 1800 tokens).
+// (Two blocks per SM for ranks up to 32; with 104 registers, up to 16, they leave room for a block of the reduction launch, which starts early.)
 template <int RT, int CL, bool MASKED>   // rank tiles of 16; cluster width (0 = two-launch form)
-__global__ void __launch_bounds__(LG_WARPS * 32)
+__global__ void __launch_bounds__(LG_WARPS * 32) __maxnreg__(RT == 1 && !MASKED ? 104 : (RT <= 2 ? 128 : 168))
 lora_grad_partial_kernel(int M, int r, int rows_per_slice, GradSide side0, GradSide side1, int accumulate) {
     extern __shared__ __align__(16) uint8_t lg_smem[];
     pdl_launch_dependents();
@@ -400,8 +406,9 @@ lora_grad_partial_kernel(int M, int r, int rows_per_slice, GradSide side0, GradS
 #pragma unroll
         for (int u = 0; u < LG_UNROLL; ++u) {
             const int ma = mm + 16 * u + g, mb = ma + 8;
-            n0[u] = (live && ma < m_stop) ? *reinterpret_cast<const uint4*>(src + (size_t)ma * C) : zero4;
-            n1[u] = (live && mb < m_stop) ? *reinterpret_cast<const uint4*>(src + (size_t)mb * C) : zero4;
+            n0[u] = zero4; n1[u] = zero4;
+            if (live && ma < m_stop) lg_load(n0[u], src + (size_t)ma * C);
+            if (live && mb < m_stop) lg_load(n1[u], src + (size_t)mb * C);
             if constexpr (MASKED) {
                 if (masked) {
                     if (live && ma < m_stop) k0[u] = __ldg(reinterpret_cast<const uint2*>(sd.mask + (size_t)ma * C + c0));
@@ -497,29 +504,42 @@ lora_grad_partial_kernel(int M, int r, int rows_per_slice, GradSide side0, GradS
             }
 }
 
-__global__ void lora_grad_reduce_kernel(int r, int slices, int accumulate, GradSide dB_side, GradSide dA_side) {
-    // elements [0, N*r): dB[n, j]; elements [N*r, N*r + K*r): dA (stored [r, K])
+// Adds the slices' partial sums in slice order.  A thread takes four ranks of one column: neighbouring threads the next ranks of dB [N, r]
+// (stored as it lies in scratch), the next columns of dA [r, K] (so that each of its four stores is contiguous across the warp; element
+// by element they were 4-byte stores K apart).
+__global__ void __launch_bounds__(256) lora_grad_reduce_kernel(int r, int slices, int accumulate, GradSide dB_side, GradSide dA_side) {
     pdl_launch_dependents();
-    pdl_wait();
-    const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const size_t nb = (size_t)dB_side.C * r, na = (size_t)dA_side.C * r;
-    if (idx >= nb + na) return;
+    const int r4 = r >> 2, nb = dB_side.C * r4, na = dA_side.C * r4;
+    const int idx = (int)(blockIdx.x * blockDim.x + threadIdx.x);
     const bool is_dB = idx < nb;
+    const int e = is_dB ? idx : idx - nb;
     const GradSide& sd = is_dB ? dB_side : dA_side;
-    const size_t e = is_dB ? idx : idx - nb;          // index into [C][r]
-    const size_t step = (size_t)sd.C * r;
-    float v = 0.f;
+    int c = 0, j = 0;
+    if (is_dB) { c = e / r4; j = 4 * (e - c * r4); }
+    else if (e < na) { j = e / sd.C; c = e - j * sd.C; j *= 4; }
+    pdl_wait();
+    if (idx >= nb + na) return;
+    const float4* src = reinterpret_cast<const float4*>(sd.partial + (size_t)c * r + j);
+    const size_t step = (size_t)sd.C * r / 4;
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
     int sl = 0;
     for (; sl + 4 <= slices; sl += 4) {               // four independent loads in flight, added in slice order
-        const float p0 = sd.partial[(size_t)sl * step + e], p1 = sd.partial[(size_t)(sl + 1) * step + e];
-        const float p2 = sd.partial[(size_t)(sl + 2) * step + e], p3 = sd.partial[(size_t)(sl + 3) * step + e];
-        v = (((v + p0) + p1) + p2) + p3;
+        const float4 p0 = src[sl * step], p1 = src[(sl + 1) * step], p2 = src[(sl + 2) * step], p3 = src[(sl + 3) * step];
+        v.x = (((v.x + p0.x) + p1.x) + p2.x) + p3.x; v.y = (((v.y + p0.y) + p1.y) + p2.y) + p3.y;
+        v.z = (((v.z + p0.z) + p1.z) + p2.z) + p3.z; v.w = (((v.w + p0.w) + p1.w) + p2.w) + p3.w;
     }
-    for (; sl < slices; ++sl) v += sd.partial[(size_t)sl * step + e];
-    v *= sd.scale;
-    const int c = (int)(e / r), j = (int)(e % r);
-    float* dst = is_dB ? sd.Out + e : sd.Out + (size_t)j * sd.C + c;
-    *dst = accumulate ? (*dst + v) : v;
+    for (; sl < slices; ++sl) { const float4 x = src[sl * step]; v.x += x.x; v.y += x.y; v.z += x.z; v.w += x.w; }
+    v.x *= sd.scale; v.y *= sd.scale; v.z *= sd.scale; v.w *= sd.scale;
+    if (is_dB) {
+        float4* dst = reinterpret_cast<float4*>(sd.Out + (size_t)c * r + j);
+        if (accumulate) { const float4 o = *dst; v.x = o.x + v.x; v.y = o.y + v.y; v.z = o.z + v.z; v.w = o.w + v.w; }
+        *dst = v;
+    } else {
+        float* dst = sd.Out + (size_t)j * sd.C + c;
+        const size_t C = (size_t)sd.C;
+        if (accumulate) { v.x = dst[0] + v.x; v.y = dst[C] + v.y; v.z = dst[2 * C] + v.z; v.w = dst[3 * C] + v.w; }
+        dst[0] = v.x; dst[C] = v.y; dst[2 * C] = v.z; dst[3 * C] = v.w;
+    }
 }
 
 int launch_lora_grads(int M, int K, int N, int r, float s, const void* X, const void* dY, const float* H, const float* G,
@@ -620,7 +640,7 @@ int launch_lora_grads(int M, int K, int N, int r, float s, const void* X, const 
     if (err != cudaSuccess) return QLORA_ERR_CUDA;
     const GradSide& rB = want_dB ? sB : none;
     const GradSide& rA = want_dA ? sA : none;
-    const size_t total = (size_t)(rB.C + rA.C) * r;
+    const size_t total = (size_t)(rB.C + rA.C) * r / 4;                 // (r is a multiple of 8; K, N and r fit 31 bits together: scratch is sized for them)
     err = launch_pdl(lora_grad_reduce_kernel, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, st, 1, r, plan.slices, accumulate, rB, rA);
     return err == cudaSuccess ? QLORA_OK : QLORA_ERR_CUDA;
 }
