@@ -205,20 +205,25 @@ __device__ __forceinline__ bool wait_counter(const unsigned* ctr, unsigned targe
 
 #include "lora_down_stream.cuh"
 
-// Eight of s * P as bf16 (the LoRA operand), and in `low` what that rounding left over, again as bf16.
-__device__ __forceinline__ uint4 lora_p_chunk(const float4& a, const float4& b, float s, uint4& low) {
+// Eight of s * P as bf16 (the LoRA operand), and -- where it is wanted -- in `low` what that rounding left over, again as bf16.
+__device__ __forceinline__ uint4 lora_p_chunk(const float4& a, const float4& b, float s, bool want_low, uint4& low) {
     const float f[8] = {s * a.x, s * a.y, s * a.z, s * a.w, s * b.x, s * b.y, s * b.z, s * b.w};
-    uint32_t o[4], l[4];
+    uint32_t o[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const __nv_bfloat162 h = __floats2bfloat162_rn(f[2 * i], f[2 * i + 1]);
-        // (nothing is left of a value that became infinite or was no number)
-        const float l0 = f[2 * i] - __low2float(h), l1 = f[2 * i + 1] - __high2float(h);
-        const __nv_bfloat162 r = __floats2bfloat162_rn(fabsf(l0) < INFINITY ? l0 : 0.f, fabsf(l1) < INFINITY ? l1 : 0.f);
         o[i] = *reinterpret_cast<const uint32_t*>(&h);
-        l[i] = *reinterpret_cast<const uint32_t*>(&r);
     }
-    low = make_uint4(l[0], l[1], l[2], l[3]);
+    if (want_low) {
+        uint32_t l[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {    // (nothing is left of a value that became infinite or was no number)
+            const float l0 = f[2 * i] - bf16_lo(o[i]), l1 = f[2 * i + 1] - bf16_hi(o[i]);
+            const __nv_bfloat162 r = __floats2bfloat162_rn(fabsf(l0) < INFINITY ? l0 : 0.f, fabsf(l1) < INFINITY ? l1 : 0.f);
+            l[i] = *reinterpret_cast<const uint32_t*>(&r);
+        }
+        low = make_uint4(l[0], l[1], l[2], l[3]);
+    }
     return make_uint4(o[0], o[1], o[2], o[3]);
 }
 
@@ -466,7 +471,7 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
                         if (jc < n8 && m < p.M) {
                             // (not the read-only path: P may have been written by this launch's producer clusters)
                             const float4* src = reinterpret_cast<const float4*>(p.Pmat + (size_t)m * p.r + jc * 8);
-                            v = lora_p_chunk(__ldcg(src), __ldcg(src + 1), p.s, low);
+                            v = lora_p_chunk(__ldcg(src), __ldcg(src + 1), p.s, p.lora_lo != 0, low);
                         }
                         uint8_t* dst = lp + jc * (p.BT * 16) + (row_t >> 3) * 128 + (row_t & 7) * 16;
                         *reinterpret_cast<uint4*>(dst) = v;
@@ -513,13 +518,13 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
         const int kb_stride = TRANSPOSED ? 2 : 1;                 // the thread's two code blocks are kb0 and kb0 + kb_stride
         const uint32_t row_base = (uint32_t)(col >> 3) * 1024u + (uint32_t)(col & 7) * 128u;   // row `col` of a swizzled tile
         const uint32_t sw = (uint32_t)(col & 7);
-        uint32_t w_off[2], chunk0[2], srow[2];
+        uint32_t w_off[2], chunk0[2], soff[2];
 #pragma unroll
         for (int b = 0; b < 2; ++b) {
             const int kb = kb0 + b * kb_stride;                   // 32-code block along k: 0..1 forward, 0..3 backward
             w_off[b] = row_base + (TRANSPOSED ? (uint32_t)(kb >> 1) * 8192u : 0u);
             chunk0[b] = (uint32_t)((TRANSPOSED ? (kb & 1) : kb) * 4);
-            srow[b] = (uint32_t)(((kb * 32) / p.g) % p.scale_rows);   // (a stage holds several group rows when groups are short)
+            soff[b] = (uint32_t)((((kb * 32) / p.g) % p.scale_rows) * p.packed_cols + col);   // (a stage holds several group rows when groups are short)
         }
         const uint32_t pcols = (uint32_t)p.packed_cols;
         const int my_tiles = first_tile < p.n_tiles ? (p.n_tiles - first_tile + tile_stride - 1) / tile_stride : 0;
@@ -539,8 +544,8 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
                 const uint32_t kb = (uint32_t)(kb0 + b * kb_stride);
 #pragma unroll
                 for (int i = 0; i < BITS; ++i) w[b][i] = pw[(kb * BITS + i) * pcols + col];
-                sc[b] = ps[srow[b] * pcols + col];
-                zp[b] = pz[srow[b] * pcols + col];
+                sc[b] = ps[soff[b]];
+                zp[b] = pz[soff[b]];
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_empty_p + 8 * ring_p.slot);

@@ -434,7 +434,7 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
                         if (jc < n8 && m < p.M) {
                             // (not the read-only path: P may have been written by this launch's producer clusters)
                             const float4* src = reinterpret_cast<const float4*>(p.Pmat + (size_t)m * p.r + jc * 8);
-                            v = lora_p_chunk(__ldcg(src), __ldcg(src + 1), p.s, low);
+                            v = lora_p_chunk(__ldcg(src), __ldcg(src + 1), p.s, p.lora_lo != 0, low);
                         }
                         uint8_t* dst = lp + a * (kPairTok * p.r_pad * 2) + jc * (kPairTok * 16) + (et >> 3) * 128 + (et & 7) * 16;
                         *reinterpret_cast<uint4*>(dst) = v;
@@ -571,13 +571,13 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
         const int kb_stride = TRANSPOSED ? 2 : 1;                 // the thread's two code blocks are kb0 and kb0 + kb_stride
         const uint32_t row_base = (uint32_t)(col >> 3) * 1024u + (uint32_t)(col & 7) * 128u;   // row `col` of a swizzled tile
         const uint32_t sw = (uint32_t)(col & 7);
-        uint32_t w_off[2], chunk0[2], srow[2];
+        uint32_t w_off[2], chunk0[2], soff[2];
 #pragma unroll
         for (int b = 0; b < 2; ++b) {
             const int kb = kb0 + b * kb_stride;                   // 32-code block along k: 0..1 forward, 0..3 backward
             w_off[b] = row_base + (TRANSPOSED ? (uint32_t)(kb >> 1) * 8192u : 0u);
             chunk0[b] = (uint32_t)((TRANSPOSED ? (kb & 1) : kb) * 4);
-            srow[b] = (uint32_t)(((kb * 32) / p.g) % p.scale_rows);   // (a stage holds several group rows when groups are short)
+            soff[b] = (uint32_t)((((kb * 32) / p.g) % p.scale_rows) * p.packed_cols + col);   // (a stage holds several group rows when groups are short)
         }
         const uint32_t pcols = (uint32_t)p.packed_cols;
         const uint32_t leader_full_w = map_to_cta(bar_full_w, 0);
@@ -601,8 +601,8 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
                 const uint32_t kb = (uint32_t)(kb0 + b * kb_stride);
 #pragma unroll
                 for (int i = 0; i < BITS; ++i) w[b][i] = pw[(kb * BITS + i) * pcols + col];
-                sc[b] = ps[srow[b] * pcols + col];
-                zp[b] = pz[srow[b] * pcols + col];
+                sc[b] = ps[soff[b]];
+                zp[b] = pz[soff[b]];
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_empty_p + 8 * ring_p.slot);
