@@ -313,8 +313,8 @@ __device__ __forceinline__ void st_finish(const StreamParams& p, uint8_t* smem, 
 // Warp (cg, part): 32 columns and its share of the chunks.  GPC: scale segments per chunk -- 1 for groups that are multiples of
 // 128, 2 for multiples of 64, 4 for multiples of 32 (the segment, not the group, is what one accumulator spans).
 // ------------------------------------------------------------------------------------------------------------
-template <int BITS, int NT, int GPC>
-__global__ void __launch_bounds__(ST_THREADS, 2) stream_fwd_kernel(const StreamParams p) {
+template <int BITS, int NT, int GPC, int PER_SM>
+__global__ void __launch_bounds__(ST_THREADS, PER_SM) stream_fwd_kernel(const StreamParams p) {
     using F = Fmt<BITS>;
     constexpr int TOKS = 8 * NT, SB = 2;                   // SB: slices of the staging pass whose loads a warp has in flight
     pdl_launch_dependents();
@@ -573,8 +573,8 @@ __device__ __forceinline__ void st_bwd_pairs(uint32_t a0, uint32_t a1, uint32_t 
     }
 }
 
-template <int BITS, int NT, int FL>
-__global__ void __launch_bounds__(ST_THREADS, 2) stream_bwd_kernel(const StreamParams p) {
+template <int BITS, int NT, int FL, int PER_SM>
+__global__ void __launch_bounds__(ST_THREADS, PER_SM) stream_bwd_kernel(const StreamParams p) {
     using F = Fmt<BITS>;
     using BF = BFmt<BITS, FL>;
     constexpr int TOKS = 8 * NT, SB = 2;
@@ -796,16 +796,8 @@ __global__ void __launch_bounds__(ST_THREADS, 2) stream_bwd_kernel(const StreamP
     st_finish<true>(p, smem, sp, c_lo, rank, blockIdx.y == 0 && rank == 0);
 }
 
-template <int BITS, int NT, int V, bool TRANSPOSED>          // V: GPC forward, FL backward
-int st_launch(const StreamParams& p, int tiles, size_t smem_bytes, cudaStream_t st) {
-    static SmemLimit limit;
-    const dim3 grid((unsigned)p.ks, (unsigned)tiles);
-    void (*kern)(const StreamParams);
-    if constexpr (TRANSPOSED) kern = stream_bwd_kernel<BITS, NT, V>;
-    else kern = stream_fwd_kernel<BITS, NT, V>;
-    if (!limit.raise(kern, 227 * 1024)) return QLORA_ERR_CUDA;
-    return launch_pdl(kern, grid, dim3(ST_THREADS), smem_bytes, st, (unsigned)p.ks, p) == cudaSuccess ? QLORA_OK : QLORA_ERR_CUDA;
-}
+// Three CTAs per SM (80 registers) exist where the kernels spill 24 bytes at most: up to 8 tokens, 4 bits, and 2 bits backward.
+constexpr bool st_has_three(int bits, int nt, bool transposed) { return nt == 1 && (bits == 4 || (bits == 2 && transposed)); }
 
 int fwd_kb(int bits) { return bits == 2 ? 64 : 32; }
 
@@ -853,9 +845,29 @@ const DeviceFacts& device_facts() {
 //             the best cut is usually the one with about 256 CTAs;
 //   staging   a warp's slices of the CTA's range, two in flight per round trip to L2;
 //   exchange  the cluster barriers and the adding up;
-// and the whole repeats when the CTAs exceed what the GPU holds at once (two per SM up to half an SM's shared memory).
+// and the whole repeats when the CTAs exceed what the GPU holds at once (two per SM up to half an SM's shared memory).  Three per SM, with
+// 80 registers, take 1.28 times as long for the same cut (4096 x 4096: 8.1 against 6.3 us) and are for cuts that two would need a second
+// wave for: 4096 -> 11008 forward, 344 CTAs, 15.9 -> 13.1 us; 4096 -> 11008 backward 17.4 -> 14.7.
 // (4096 x 4096, INT4, one token: 128 columns x 8 CTAs 6.3 us, 64 x 4 6.7, 32 x 2 8.2, 256 x 8 8.7, 128 x 4 9.3, 64 x 8 9.5.)
-struct StreamPlan { StreamParams p; int tiles, tile_c; SmemPlan sm; bool ok; };
+struct StreamPlan { StreamParams p; int tiles, tile_c, per_sm; SmemPlan sm; bool ok; };
+
+template <int BITS, int NT, int V, bool TRANSPOSED, int PER_SM>   // V: GPC forward, FL backward
+int st_launch_as(const StreamPlan& plan, cudaStream_t st) {
+    static SmemLimit limit;
+    const dim3 grid((unsigned)plan.p.ks, (unsigned)plan.tiles);
+    void (*kern)(const StreamParams);
+    if constexpr (TRANSPOSED) kern = stream_bwd_kernel<BITS, NT, V, PER_SM>;
+    else kern = stream_fwd_kernel<BITS, NT, V, PER_SM>;
+    if (!limit.raise(kern, 227 * 1024)) return QLORA_ERR_CUDA;
+    return launch_pdl(kern, grid, dim3(ST_THREADS), plan.sm.total, st, (unsigned)plan.p.ks, plan.p) == cudaSuccess ? QLORA_OK : QLORA_ERR_CUDA;
+}
+
+template <int BITS, int NT, int V, bool TRANSPOSED>
+int st_launch(const StreamPlan& plan, cudaStream_t st) {
+    if constexpr (st_has_three(BITS, NT, TRANSPOSED))
+        if (plan.per_sm == 3) return st_launch_as<BITS, NT, V, TRANSPOSED, 3>(plan, st);
+    return st_launch_as<BITS, NT, V, TRANSPOSED, 2>(plan, st);
+}
 
 StreamPlan st_cut(StreamParams p, int bits, bool transposed) {
     StreamPlan best{};
@@ -891,15 +903,18 @@ StreamPlan st_cut(StreamParams p, int bits, bool transposed) {
             p.pitch += (want - p.pitch % 128 + 128) % 128;
             const SmemPlan sm = st_plan(p, transposed, toks, tile_c);
             if (sm.total > 227 * 1024 - 1024) continue;
-            const int occ = sm.total <= 113 * 1024 ? 2 : 1;
-            const float fill = (float)(tiles * 2) / (float)(gpu.clusters[p.ks] * occ);     // of what the GPU holds at once
-            const float waves = fill <= 1.f ? 1.f : 0.5f * (fill + ceilf(fill));
             const int per_warp = (per_cta + parts - 1) / parts;
             const float step = (transposed ? 650.f + 150.f * (nt - 1) : 1400.f + 450.f * (nt - 1)) * (bits == 8 ? 1.3f : 1.f) * (tiles * p.ks > sms ? 1.2f : 1.f);
             const float rounds = (float)((per_cta * (unit / 32) + 2 * ST_WARPS - 1) / (2 * ST_WARPS));
             const float round = transposed ? 2500.f * nt : 900.f + 1100.f * nt;
-            const float cost = waves * ((float)per_warp * step + rounds * round + 1500.f + 500.f * (float)lks);
-            if (!best.ok || cost < best_cost) { best = StreamPlan{p, tiles, tile_c, sm, true}; best_cost = cost; }
+            const float once = (float)per_warp * step + rounds * round + 1500.f + 500.f * (float)lks;
+            for (int per_sm = 2; per_sm <= (st_has_three(bits, nt, transposed) && sm.total <= 74 * 1024 ? 3 : 2); ++per_sm) {
+                const int occ = sm.total <= 113 * 1024 ? per_sm : 1;
+                const float fill = (float)(tiles * 2) / (float)(gpu.clusters[p.ks] * occ);     // of what the GPU holds at once
+                const float waves = fill <= 1.f ? 1.f : 0.5f * (fill + ceilf(fill));
+                const float cost = waves * once * (per_sm == 3 ? 1.28f : 1.f);
+                if (!best.ok || cost < best_cost) { best = StreamPlan{p, tiles, tile_c, per_sm, sm, true}; best_cost = cost; }
+            }
         }
     }
     return best;
@@ -933,11 +948,11 @@ int launch_stream_gemm(const qlora_desc& d, int M, bool transposed, const void* 
     if (!plan.ok) return QLORA_ERR_UNSUPPORTED;
 #define QLORA_ST(B, NT)                                                                                                          \
     if (transposed)                                                                                                              \
-        return d.group_size % 64 == 0 ? st_launch<B, NT, 8, true>(plan.p, plan.tiles, plan.sm.total, st)                         \
-                                      : st_launch<B, NT, 4, true>(plan.p, plan.tiles, plan.sm.total, st);                        \
-    if (d.group_size % 128 == 0) return st_launch<B, NT, 1, false>(plan.p, plan.tiles, plan.sm.total, st);                       \
-    if (d.group_size % 64 == 0) return st_launch<B, NT, 2, false>(plan.p, plan.tiles, plan.sm.total, st);                        \
-    if constexpr (B != 2) return st_launch<B, NT, 4, false>(plan.p, plan.tiles, plan.sm.total, st);                              \
+        return d.group_size % 64 == 0 ? st_launch<B, NT, 8, true>(plan, st)                                                      \
+                                      : st_launch<B, NT, 4, true>(plan, st);                                                     \
+    if (d.group_size % 128 == 0) return st_launch<B, NT, 1, false>(plan, st);                                                    \
+    if (d.group_size % 64 == 0) return st_launch<B, NT, 2, false>(plan, st);                                                     \
+    if constexpr (B != 2) return st_launch<B, NT, 4, false>(plan, st);                                                           \
     else return QLORA_ERR_UNSUPPORTED
 #define QLORA_ST_BITS(NT)           \
     switch (d.bits) {               \

@@ -42,6 +42,19 @@ def test_llama_q_proj_shape(bits, M):
     assert errs["Y"] < 1e-2 and errs["dX"] < 1e-2
 
 
+@pytest.mark.parametrize("K,N", [(4096, 11008), (11008, 4096)])
+@pytest.mark.parametrize("bits,g,M", [(4, 32, 1), (4, 64, 8), (4, 128, 3), (2, 128, 8)])
+def test_wide_layers_with_three_ctas_per_sm(bits, g, M, K, N):
+    """Cuts whose CTAs two per SM could not hold at once: the 80-register builds, in the direction whose output is the wide side."""
+    check_layer(qi.random_codes_layer(K=K, N=N, bits=bits, group_size=g, r=8, alpha=16.0, M=M, seed=bits + g + M))
+
+
+@pytest.mark.parametrize("bits,g", [(4, 96), (3, 160), (8, 192), (2, 192)])
+def test_groups_no_power_of_two_and_a_contraction_beyond_16384(bits, g):
+    check_layer(qi.random_codes_layer(K=g * 96, N=104, bits=bits, group_size=g, r=16, alpha=32.0, M=6, seed=g))
+    check_layer(qi.random_codes_layer(K=g, N=17408, bits=bits, group_size=g, r=16, alpha=32.0, M=6, seed=g + 1))
+
+
 @pytest.mark.parametrize("bits", [2, 3, 4, 8])
 def test_activations_that_do_not_cancel(bits):
     """All-positive activations of very different magnitudes per token: sum_k X (128 + q) and (128 + z) sum_k X are then
