@@ -168,7 +168,7 @@ __global__ void __launch_bounds__(256) quantize_rtn_kernel(int g, int K, int N, 
 }
 
 // The same quantizer for groups of 32, 64 and 128 in one pass over W.  Bound by reading W (fp32) once; the kernel above reads it
-// twice, one dependent load -> reduce -> divide chain per row.  Here a block of 16 warps owns 64 output rows x 128 k: a warp holds its
+// twice, one dependent load -> reduce -> divide chain per row.  Here a block of 8 warps owns 32 output rows x 128 k: a warp holds its
 // four rows in registers (a float4 per lane and row, all four loads in flight together), so a group is 8, 16 or 32 neighbouring
 // lanes.
 //   - min and max of the four rows (max(w, 0) and max(-w, 0)) are eight values per lane: three halving exchanges (4 + 2 + 1
@@ -180,25 +180,24 @@ __global__ void __launch_bounds__(256) quantize_rtn_kernel(int g, int K, int N, 
 //   - four consecutive codes of a lane are one piece of 4 BITS bits, stored to shared memory by row and read back by column as words
 //     (odd pitch: no bank conflicts), so the word stores cover 32 neighbouring columns.
 // Consecutive blocks walk along k, i.e. along the rows of W in memory.
-// 4096 x 11008, 4 bits, group 128: 131 -> 47 us with 32 rows per block, 45 with 64 (4.5 TB/s of W + Q, 0.69 of the measured copy
-// bandwidth).
-constexpr int QF_K = 128, QF_ROWS = 64, QF_THREADS = 8 * QF_ROWS;
+// 4096 x 11008, 4 bits, group 128: 131 -> 47 us (4.3 TB/s of W + Q, 0.66 of the measured copy bandwidth).
+constexpr int QF_K = 128;
 
 template <int BITS> struct QfPiece { using type = uint16_t; };
 template <> struct QfPiece<2> { using type = uint8_t; };
 template <> struct QfPiece<8> { using type = uint32_t; };
 
 template <int BITS, int GL>   // GL: lanes per group (group size / 4)
-__global__ void __launch_bounds__(QF_THREADS) quantize_rtn_fast_kernel(int K, int N, const float* __restrict__ W, uint32_t* __restrict__ Q,
+__global__ void __launch_bounds__(256) quantize_rtn_fast_kernel(int K, int N, const float* __restrict__ W, uint32_t* __restrict__ Q,
                                                                 __half* __restrict__ scales, __half* __restrict__ zeros) {
     using Piece = typename QfPiece<BITS>::type;
     constexpr int PITCH = 8 * (int)sizeof(Piece) + 1;             // 32-bit words per row of pieces
     constexpr int GROUPS = 32 / GL;
     constexpr float QMAX = (float)((1 << BITS) - 1);
-    __shared__ uint32_t s_piece[QF_ROWS * PITCH];
-    __shared__ uint32_t s_sz[GROUPS][QF_ROWS];                    // scale | zero << 16, fp16 bits
+    __shared__ uint32_t s_piece[QZ_ROWS * PITCH];
+    __shared__ uint32_t s_sz[GROUPS][QZ_ROWS];                    // scale | zero << 16, fp16 bits
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int k0 = blockIdx.x * QF_K, n0 = blockIdx.y * QF_ROWS;
+    const int k0 = blockIdx.x * QF_K, n0 = blockIdx.y * QZ_ROWS;
     const int k = k0 + 4 * lane;                                  // (K is a multiple of the group: a group's lanes are all in or all out)
     float4 w[4];
 #pragma unroll
@@ -269,10 +268,10 @@ __global__ void __launch_bounds__(QF_THREADS) quantize_rtn_fast_kernel(int K, in
         pieces[(4 * warp + j) * PITCH * (4 / (int)sizeof(Piece)) + lane] = (Piece)piece;
     }
     __syncthreads();
-    const int r = 32 * (warp & 1) + lane, n = n0 + r;
+    const int r = lane, n = n0 + r;
     if (n < N) {
 #pragma unroll
-        for (int i = warp >> 1; i < 4 * BITS; i += 8) {                // word i of the 128 k: 32-code block i / BITS
+        for (int i = warp; i < 4 * BITS; i += 8) {                // word i of the 128 k: 32-code block i / BITS
             const uint32_t* row = s_piece + r * PITCH;
             uint32_t word;
             if constexpr (BITS == 3) {
@@ -286,10 +285,9 @@ __global__ void __launch_bounds__(QF_THREADS) quantize_rtn_fast_kernel(int K, in
             }
             if (k0 + 32 * (i / BITS) < K) Q[(size_t)(k0 / 32 * BITS + i) * N + n] = word;
         }
-        const int gr = warp >> 1;                                 // group of the strip
-        if (gr < GROUPS && k0 + gr * 4 * GL < K) {
-            const uint32_t sz = s_sz[gr][r];
-            const size_t gi = (size_t)(k0 / (4 * GL) + gr) * N + n;
+        if (warp < GROUPS && k0 + warp * 4 * GL < K) {
+            const uint32_t sz = s_sz[warp][r];
+            const size_t gi = (size_t)(k0 / (4 * GL) + warp) * N + n;
             scales[gi] = __ushort_as_half((unsigned short)(sz & 0xFFFFu));
             zeros[gi] = __ushort_as_half((unsigned short)(sz >> 16));
         }
@@ -298,10 +296,10 @@ __global__ void __launch_bounds__(QF_THREADS) quantize_rtn_fast_kernel(int K, in
 
 template <int BITS>
 static void launch_quantize_fast(const qlora_desc& d, const float* W, uint32_t* q, __half* s, __half* z, cudaStream_t st) {
-    const dim3 grid((unsigned)((d.K + QF_K - 1) / QF_K), (unsigned)((d.N + QF_ROWS - 1) / QF_ROWS));
-    if (d.group_size == 32) quantize_rtn_fast_kernel<BITS, 8><<<grid, QF_THREADS, 0, st>>>(d.K, d.N, W, q, s, z);
-    else if (d.group_size == 64) quantize_rtn_fast_kernel<BITS, 16><<<grid, QF_THREADS, 0, st>>>(d.K, d.N, W, q, s, z);
-    else quantize_rtn_fast_kernel<BITS, 32><<<grid, QF_THREADS, 0, st>>>(d.K, d.N, W, q, s, z);
+    const dim3 grid((unsigned)((d.K + QF_K - 1) / QF_K), (unsigned)((d.N + QZ_ROWS - 1) / QZ_ROWS));
+    if (d.group_size == 32) quantize_rtn_fast_kernel<BITS, 8><<<grid, 256, 0, st>>>(d.K, d.N, W, q, s, z);
+    else if (d.group_size == 64) quantize_rtn_fast_kernel<BITS, 16><<<grid, 256, 0, st>>>(d.K, d.N, W, q, s, z);
+    else quantize_rtn_fast_kernel<BITS, 32><<<grid, 256, 0, st>>>(d.K, d.N, W, q, s, z);
 }
 
 int launch_quantize_rtn(const qlora_desc& d, const float* W, int32_t* Q, void* scales, void* zeros, cudaStream_t st) {
@@ -311,7 +309,7 @@ int launch_quantize_rtn(const qlora_desc& d, const float* W, int32_t* Q, void* s
     __half* s = (__half*)scales;
     __half* z = (__half*)zeros;
     // groups that are whole lanes of one 128-wide strip: one pass; other sizes (96, 256, K, ...) reduce in a loop, in the first kernel
-    if ((d.group_size == 32 || d.group_size == 64 || d.group_size == 128) && (d.N + QF_ROWS - 1) / QF_ROWS <= 65535) {
+    if ((d.group_size == 32 || d.group_size == 64 || d.group_size == 128) && (d.N + QZ_ROWS - 1) / QZ_ROWS <= 65535) {
         switch (d.bits) {
             case 2: launch_quantize_fast<2>(d, W, q, s, z, st); break;
             case 3: launch_quantize_fast<3>(d, W, q, s, z, st); break;
