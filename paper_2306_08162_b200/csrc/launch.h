@@ -74,7 +74,7 @@ int launch_umma_gemm(const qlora_desc& d, int M, bool transposed, const void* In
 size_t umma_split_scratch_bytes(const qlora_desc& d, int M);
 // api.cu -- the workspace a layer call needs at least (qlora_workspace_bytes less the optional exchange area above)
 size_t required_workspace_bytes(const qlora_desc& d, int M);
-// stream_kernel.cu -- few tokens (M <= 16): cp.async-fed mma.sync kernels on raw codes, the contraction split over a
+// stream_kernel.cu -- few tokens (M <= 16): register-fed mma.sync kernels on raw codes, the contraction split over a
 // cluster.  Ldown / Lup: the adapter applied first / second (forward A, B; backward B, A).  P = H or G, fp32 [M, r]: read
 // when p_is_input, otherwise computed inside the kernel (ranks up to 16) and written out.
 bool stream_supported(const qlora_desc& d, int M, bool transposed);

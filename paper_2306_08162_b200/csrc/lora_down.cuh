@@ -1,5 +1,5 @@
-// LoRA down-projection of one block of 16 token rows, as a device function shared by the stand-alone kernel
-// (simt_kernels.cu) and by the CTA-pair tensor-core kernel, whose idle SM pairs run it beside the main tiles.
+// LoRA down-projection of one or two blocks of 16 token rows, as a device function shared by the stand-alone kernel for up to 256
+// rows (simt_kernels.cu) and by the single-CTA tensor-core kernel, whose spare clusters run it beside the main tiles.
 //   P[m, j] = sum_t In[m, t] * L(j, t)     l_is_A: L = A [r, T] (contraction-contiguous), else L = B [T, r].
 // mma.sync m16n8k16 (bf16 in, fp32 accumulate) fed straight from 16-byte row loads: the warps of the block stride over
 // the contraction in steps of 32 and keep LD_UNROLL steps of loads in flight, the adapter's among them.  The 32 contraction indices of a step are
