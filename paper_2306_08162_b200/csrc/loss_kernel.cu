@@ -97,9 +97,14 @@ lrec_loss_kernel(int T, int V, const __nv_bfloat16* __restrict__ Z, const __nv_b
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    constexpr float kLog2e = 1.4426950408889634f;
-    const f2 log2e2 = make_f2(kLog2e, kLog2e), minus1 = make_f2(-1.f, -1.f);
+    constexpr float kLog2e = 1.4426950408889634f, kAzScale = 0x1p-40f;
+    const f2 log2e2 = make_f2(kLog2e, kLog2e), scale2 = make_f2(kAzScale, kAzScale), minus1 = make_f2(-1.f, -1.f);
     if ((int)blockIdx.x < T) prefetch(blockIdx.x);
+    // Gradient: what grad_scale * lambda_kl has above 1 goes into the exponent of p_j as a power of two; on a masked logit's z - t it would
+    // overflow, and p_j = 0 must give 0.
+    const float g_all = grad_scale * lambda_kl;
+    const int n_up = fabsf(g_all) > 1.f ? min(ilogbf(g_all), 125) + 1 : 0;
+    const float up_inv = __uint_as_float((uint32_t)(127 - n_up) << 23), gkl = g_all * up_inv;
     int buf = 0;
     for (int row = blockIdx.x; row < T; row += gridDim.x, buf ^= 1) {
         uint4 zc[CH], tc[CH];
@@ -131,8 +136,13 @@ lrec_loss_kernel(int T, int V, const __nv_bfloat16* __restrict__ Z, const __nv_b
         // One pass gives both exp-sums and the KL numerator: with e_j = exp(z_j - mz) and sz = sum e_j,
         //   KL = sum_j (e_j / sz) ((z_j - lz) - (t_j - lt)) = (sum_j e_j (z_j - t_j)) / sz - lz + lt        (lz = mz + log sz, ...)
         // (padding: z = t = -inf would give 0 * nan, so padded chunks are skipped rather than relied on to vanish)
-        const float rz = mz_w == -INFINITY ? 0.f : -mz_w * kLog2e, rt = mt_w == -INFINITY ? 0.f : -mt_w * kLog2e;   // (a warp with nothing finite)
-        const f2 rz2 = make_f2(rz, rz), rt2 = make_f2(rt, rt);
+        // Masked logits (finfo.min, -1e30) can be all that a warp holds.  From 2^16 on two different bf16 lie 256 or more apart, so
+        // exp(z - mz) is 1 or 0 in any base, and in base 2 the difference is exact, where mz log2(e) would be rounded by more than 2^-8 or
+        // overflow.  Their z - t times a weight of 1 (relative to the warp's own maximum) is summed scaled, so that it stays finite.
+        // (No branch for them: one in this place kept the gradient's first steps from moving up between the shuffles, 86 -> 88 us.)
+        const float kz = fabsf(mz_w) < 65536.f ? kLog2e : 1.f, kt = fabsf(mt_w) < 65536.f ? kLog2e : 1.f;
+        const float rz = mz_w == -INFINITY ? 0.f : -mz_w * kz, rt = mt_w == -INFINITY ? 0.f : -mt_w * kt;   // (a warp with nothing finite)
+        const f2 kz2 = make_f2(kz, kz), kt2 = make_f2(kt, kt), rz2 = make_f2(rz, rz), rt2 = make_f2(rt, rt);
         f2 sz2 = make_f2(0.f, 0.f), st2 = sz2, az2 = sz2;
 #pragma unroll
         for (int c = 0; c < CH; ++c) {
@@ -141,10 +151,10 @@ lrec_loss_kernel(int T, int V, const __nv_bfloat16* __restrict__ Z, const __nv_b
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     const f2 z = unpack_bf16(zw[i]), t = unpack_bf16(tw[i]);
-                    const f2 e = exp2_2(fma2(z, log2e2, rz2));
+                    const f2 e = exp2_2(fma2(z, kz2, rz2));
                     sz2 = add2(sz2, e);
-                    az2 = fma2(e, fma2(t, minus1, z), az2);
-                    st2 = add2(st2, exp2_2(fma2(t, log2e2, rt2)));
+                    az2 = fma2(mul2(e, scale2), fma2(t, minus1, z), az2);
+                    st2 = add2(st2, exp2_2(fma2(t, kt2, rt2)));
                 }
             }
         }
@@ -162,14 +172,14 @@ lrec_loss_kernel(int T, int V, const __nv_bfloat16* __restrict__ Z, const __nv_b
         const float sz = warp_sum(has ? part[buf][2][lane] * fz : 0.f), st = warp_sum(has ? part[buf][3][lane] * ft : 0.f);
         const float az = warp_sum(has ? part[buf][4][lane] * fz : 0.f);
         const float lz = mz + logf(sz), lt = mt + logf(st);       // log-partition functions: log p_j = z_j - lz
-        const float kl = az / sz - lz + lt;
+        const float kl = az / sz * (1.f / kAzScale) - lz + lt;
         const bool has_label = label >= 0 && label < V;
         const int label_chunk = has_label ? label >> 3 : -1;
         if (!has_label && threadIdx.x == 0) loss_tokens[row] = lambda_kl * kl;
         uint4* dr = dZ != nullptr ? reinterpret_cast<uint4*>(dZ + (size_t)row * V) : nullptr;
         // g_j = p_j (lambda_kl ((z_j - t_j) - (lz - lt) - KL) + lambda_ce) - lambda_ce [j == label], times grad_scale
-        const float nshift = -((lz - lt) + kl), nlz = -lz * kLog2e, gkl = grad_scale * lambda_kl, gce = has_label ? grad_scale * lambda_ce : 0.f;
-        const f2 nshift2 = make_f2(nshift, nshift), nlz2 = make_f2(nlz, nlz), gkl2 = make_f2(gkl, gkl), gce2 = make_f2(gce, gce);
+        const float nshift = -((lz - lt) + kl), nlz = fmaf(-lz, kLog2e, (float)n_up), gce = has_label ? grad_scale * lambda_ce : 0.f, gce_n = gce * up_inv;
+        const f2 nshift2 = make_f2(nshift, nshift), nlz2 = make_f2(nlz, nlz), gkl2 = make_f2(gkl, gkl), gce2 = make_f2(gce_n, gce_n);
 #pragma unroll
         for (int c = 0; c < CH; ++c) {
             const int ci = c * threads + threadIdx.x;

@@ -56,6 +56,33 @@ def test_rows_with_infinitely_unlikely_teacher_tokens():
     assert torch.isinf(loss[1]) and loss[1] > 0 and loss[0].abs() < 1e-5 and loss[2].abs() < 1e-5
 
 
+@pytest.mark.parametrize("mask", [-3.3895313892515355e38, -1e30, -1e10, -65504.0])
+@pytest.mark.parametrize("student,teacher", [(True, True), (True, False), (False, True)])
+def test_rows_with_masked_vocabulary_entries(mask, student, teacher):
+    """Entries masked by a large negative logit (finfo.min among them), in stretches that fill whole warps and in single places, on
+    either side: a masked student entry has probability zero and adds nothing; a masked teacher entry beside an unmasked
+    student one is as expensive as the formula says.  With loss scaling: a probability of zero stays zero."""
+    T, V, scale = 5, 8192, 1024.0
+    z_bits, t_bits = qi.normal_bf16(91, 0, (T, V), 2.0), qi.normal_bf16(91, 1, (T, V), 2.0)
+    z, t = bf16_from_bits(z_bits), bf16_from_bits(t_bits)
+    for x, on in ((z, student), (t, teacher)):
+        if on:
+            x[1, 4096:] = mask
+            x[2, :256] = mask
+            x[3, 1::3] = mask
+            x[4, 8:] = mask
+    labels = torch.tensor([5, 7, 300, 0, 3], dtype=torch.int32, device="cuda")
+    loss, grad = torch.empty(T, dtype=torch.float32, device="cuda"), torch.empty_like(z)
+    ql.qlora_lrec_loss(z, t, labels, 0.9, 0.6, scale, loss, grad)
+    want_loss, want_grad = orc.lrec_loss(to_f64(z), to_f64(t), labels.cpu().numpy(), 0.9, 0.6)
+    assert np.allclose(loss.cpu().numpy(), want_loss, rtol=2e-4, atol=2e-5)
+    if student or mask > -1e38:                                          # (finfo.min in the teacher alone: the scaled gradient leaves bf16's range)
+        for row in range(T):
+            assert rel_err(to_f64(grad[row]), scale * want_grad[row]) <= REL_TOL, row
+    if student and teacher:
+        assert torch.equal(grad[1, 4096:], torch.zeros_like(grad[1, 4096:]))
+
+
 def test_loss_only_and_pure_terms_and_determinism():
     a = run_case(16, 32000, 1.0, 0.0, seed=1, with_grad=False)
     run_case(16, 32000, 0.0, 1.0, seed=2)
