@@ -11,7 +11,7 @@ ROOT = os.path.dirname(PKG_DIR)
 CSRC = os.path.join(PKG_DIR, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 LIB_PATH = os.path.join(PKG_DIR, "libqlora_b200.so")
-CALL_PATH = os.path.join(PKG_DIR, "_pycall.so")
+CALL_PATH = os.path.join(PKG_DIR, "_pycall" + sysconfig.get_config_var("EXT_SUFFIX"))   # (tagged: another interpreter builds its own)
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-shared"]

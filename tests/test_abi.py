@@ -172,6 +172,18 @@ def test_which_way_db_goes_is_a_host_side_plan(ql):
         ql.qlora_bwd_input_db_on_producers(ql.desc(5, 64, 4096, 4096, 8, 16.0), 2048)
 
 
+def test_call_extension_belongs_to_one_interpreter(ql, monkeypatch, tmp_path):
+    """The extension's file carries the tag of the interpreter whose headers it was built with: another interpreter finds none and
+    builds its own."""
+    import sysconfig
+    from importlib.machinery import EXTENSION_SUFFIXES
+    ql.binding._native()
+    assert ql.binding._calls.__file__ == qbuild.CALL_PATH and qbuild.CALL_PATH.endswith(sysconfig.get_config_var("EXT_SUFFIX"))
+    assert sysconfig.get_config_var("SOABI") in os.path.basename(qbuild.CALL_PATH) and EXTENSION_SUFFIXES[0] == sysconfig.get_config_var("EXT_SUFFIX")
+    monkeypatch.setattr(qbuild, "CALL_PATH", str(tmp_path / "_pycall.cpython-399-x86_64-linux-gnu.so"))
+    assert qbuild._stale()
+
+
 def test_argument_conversion_of_the_call_extension(ql):
     """The calls that go through the C extension take what the binding always took: ints and objects with __index__ or __int__ for
     sizes, None or an address or a contiguous tensor for pointers -- and refuse the rest with the same exceptions."""
