@@ -52,9 +52,10 @@ constexpr int kWaitLimitUs = 250000;   // default limit of a wait, a launch para
 
 struct Params {
     int M, N, K, bits, g, r, r_pad;
-    // r_pad: columns of the LoRA operands, a multiple of 16.  lora_lo: ranks [r, 2r) hold, beside the same adapter rows again,
-    // what the rounding of s * P to bf16 left over, so the update keeps P's fp32 bits: where the second r columns cost nothing
-    // (r == 8, half an MMA's contraction is padding) and for groups of 32 (whose products the CUDA-core kernel gave in fp32).
+    // r_pad: columns of the LoRA operands, a multiple of 16.  lora_lo: ranks [r, 2r) hold, beside the finite ones of the same adapter
+    // elements again, what the rounding of s * P to bf16 left over, so that the update has 16 significant bits of P's 24: for r == 8,
+    // where half an MMA's contraction is padding otherwise, and for groups of 32, whose products the CUDA-core kernel gave from fp32
+    // (the error of Y and dX against 64 bits is the same with it: that of the weights' and outputs' bf16).
     int lora_lo;
     int C;               // output columns (N forward, K backward)
     int BT;              // token rows per tile (MMA N): a multiple of 16, 32 .. 256
@@ -225,6 +226,18 @@ __device__ __forceinline__ uint4 lora_p_chunk(const float4& a, const float4& b, 
         low = make_uint4(l[0], l[1], l[2], l[3]);
     }
     return make_uint4(o[0], o[1], o[2], o[3]);
+}
+
+// Eight bf16 with 0 in the place of infinities and NaN: the adapter rows that meet the low pieces.  (An infinite element has had its say
+// in the product with the high piece; times a low piece that is zero, or of the other sign, it would make the sum a NaN.)
+__device__ __forceinline__ uint4 finite_only(uint4 v) {
+    uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        if ((w[i] & 0x7F80u) == 0x7F80u) w[i] &= 0xFFFF0000u;
+        if ((w[i] & 0x7F800000u) == 0x7F800000u) w[i] &= 0xFFFFu;
+    }
+    return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
 // Shared-memory matrix descriptor (version 1).  Offsets in bytes; layout 0 = no swizzle, 2 = 128-byte swizzle.
@@ -462,7 +475,7 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
                     }
                     uint8_t* dst = la + jc * (kWRows * 16) + (row >> 3) * 128 + (row & 7) * 16;
                     *reinterpret_cast<uint4*>(dst) = v;
-                    if (p.lora_lo) *reinterpret_cast<uint4*>(dst + n8 * (kWRows * 16)) = v;
+                    if (p.lora_lo) *reinterpret_cast<uint4*>(dst + n8 * (kWRows * 16)) = finite_only(v);
                 }
                 for (int row_t = et; row_t < p.BT; row_t += 128) {
                     const int m = m0 + row_t;

@@ -422,7 +422,7 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
                         }
                         uint8_t* dst = ll + jc * (kPairW * 16) + (row >> 3) * 128 + (row & 7) * 16;
                         *reinterpret_cast<uint4*>(dst) = v;
-                        if (p.lora_lo) *reinterpret_cast<uint4*>(dst + n8 * (kPairW * 16)) = v;
+                        if (p.lora_lo) *reinterpret_cast<uint4*>(dst + n8 * (kPairW * 16)) = finite_only(v);
                     }
                 }
 #pragma unroll

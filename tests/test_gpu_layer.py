@@ -401,6 +401,26 @@ def test_infinite_branch_values_stay_infinite(M, g):
     assert torch.isinf(Y).all() and (Y[0::2] > 0).all() and (Y[1::2] < 0).all()
 
 
+@pytest.mark.parametrize("M,g,r", [(200, 32, 8), (200, 128, 8), (600, 32, 8), (600, 128, 8), (200, 32, 24), (600, 32, 24)])
+def test_infinite_adapter_elements_give_infinities(M, g, r):
+    """An infinite element of B makes its column of Y infinite with the sign of s * H, an infinite element of A its column of dX with
+    the sign of s * G; no other column changes a bit."""
+    import paper_2306_08162_b200 as ql
+    layer = qi.random_codes_layer(K=256, N=128, bits=4, group_size=g, r=r, alpha=16.0, M=M, seed=M + g + r)
+    gl = GpuLayer(layer)
+    clean = gl.run()
+    A, B = gl.A.clone(), gl.B.clone()
+    A[3, 70], B[100, 5] = float("-inf"), float("inf")
+    Y, dX = torch.empty_like(clean["Y"]), torch.empty_like(clean["dX"])
+    H, G = torch.empty_like(clean["H"]), torch.empty_like(clean["G"])
+    ql.qlora_fwd(gl.desc, M, gl.X, gl.Q, gl.scales, gl.zeros, gl.A, B, Y, H, gl.ws)
+    ql.qlora_bwd_input(gl.desc, M, gl.dY, gl.Q, gl.scales, gl.zeros, A, gl.B, dX, G, gl.ws)
+    for got, was, col, want in ((Y, clean["Y"], 100, torch.sign(H[:, 5])), (dX, clean["dX"], 70, -torch.sign(G[:, 3]))):
+        assert torch.isinf(got[:, col]).all() and torch.equal(torch.sign(got[:, col].float()), want)
+        rest = torch.arange(got.shape[1], device="cuda") != col
+        assert torch.equal(got[:, rest], was[:, rest])
+
+
 @pytest.mark.parametrize("r", [24, 32, 40, 64])
 @pytest.mark.parametrize("M,K,N", [(1, 96, 40), (16, 4096, 1032), (17, 352, 264), (300, 1024, 192), (2500, 256, 128)])
 def test_ranks_above_16_split_down_projection(M, K, N, r):
