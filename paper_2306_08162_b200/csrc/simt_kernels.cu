@@ -320,7 +320,8 @@ constexpr int LG_MAX_SLICES = 64;
 struct GradPlan { int slices, rows_per_slice; };
 
 static GradPlan lora_grad_plan(int M, int K, int N) {
-    const int col_blocks = (K + LG_COLS - 1) / LG_COLS + (N + LG_COLS - 1) / LG_COLS;
+    int col_blocks = (K + LG_COLS - 1) / LG_COLS + (N + LG_COLS - 1) / LG_COLS;
+    if (col_blocks < 1) col_blocks = 1;                          // (K = N = 0: a layer without elements)
     int slices = (2 * 148) / col_blocks;                         // two blocks fit an SM (registers): aim for one wave of a 148-SM part
     if (slices > LG_MAX_SLICES) slices = LG_MAX_SLICES;
     if (slices < 1) slices = 1;
@@ -546,7 +547,7 @@ int launch_lora_grads(int M, int K, int N, int r, float s, const void* X, const 
                       float* dA, float* dB, int accumulate, void* scratch, cudaStream_t st, const uint8_t* x_mask, float keep_scale,
                       int sides) {
     if (r == 0) return QLORA_OK;
-    const bool want_dB = (sides & 1) != 0, want_dA = (sides & 2) != 0;
+    const bool want_dB = (sides & 1) != 0 && N > 0, want_dA = (sides & 2) != 0 && K > 0;   // (a gradient without elements: nothing to do)
     if (!want_dB && !want_dA) return QLORA_OK;
     if (M == 0) {   // empty sums: dA = dB = 0 unless accumulating
         if (!accumulate) {

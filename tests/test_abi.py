@@ -125,6 +125,20 @@ def test_calls_reject_bad_arguments_before_launch(ql):
     assert lib.qlora_gather_columns(2, 4, 8, ok, ok, ok, 0) == -1
 
 
+def test_layers_without_elements(ql):
+    """K = 0 or N = 0 passes the descriptor check: the workspace query answers, and a gradient that has no elements is done at once
+    (nothing is launched: this runs without a GPU)."""
+    ok = 0x1000
+    for K, N in ((0, 0), (0, 256), (256, 0)):
+        for M in (0, 4, 300):
+            assert ql.qlora_workspace_bytes(ql.desc(4, 32, K, N, 8, 16.0), M) > 0
+    for M in (4, 300):
+        d = ql.desc(4, 32, 0, 0, 8, 16.0)
+        ql.qlora_bwd_lora(d, M, ok, ok, ok, ok, ok, ok, ok, ok, 0, ok, stream=0, workspace_bytes=ql.qlora_workspace_bytes(d, M))
+        d = ql.desc(4, 32, 0, 256, 8, 16.0)
+        ql.qlora_bwd_lora(d, M, ok, None, ok, ok, None, ok, ok, None, 0, ok, stream=0, workspace_bytes=ql.qlora_workspace_bytes(d, M))
+
+
 def test_missing_library_fails_loudly(ql, monkeypatch, tmp_path):
     from paper_2306_08162_b200 import binding
     monkeypatch.setattr(binding, "_lib", None)
