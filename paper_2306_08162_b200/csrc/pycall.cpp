@@ -104,9 +104,10 @@ bool to_arg(PyObject* const* args, size_t i, size_t n, T* out) {
         *out = static_cast<T>(p);
         return true;
     } else if constexpr (std::is_same_v<T, float>) {
-        const double v = PyFloat_AsDouble(a);
-        if (v == -1.0 && PyErr_Occurred()) return false;
-        *out = (float)v;
+        PyObject* f = PyNumber_Float(a);                              // (what float() takes, as the binding always did)
+        if (f == nullptr) return false;
+        *out = (float)PyFloat_AS_DOUBLE(f);
+        Py_DECREF(f);
         return true;
     } else if constexpr (std::is_same_v<T, size_t>) {
         unsigned long long v = 0, e = 0;

@@ -221,6 +221,11 @@ def test_argument_conversion_of_the_call_extension(ql):
         ql.qlora_fwd(None, 4, ok, ok, ok, ok, ok, ok, ok, None, ok, stream=0, workspace_bytes=need)
     with pytest.raises(AttributeError):
         ql.qlora_fwd(d, 4, "x", ok, ok, ok, ok, ok, ok, None, ok, stream=0, workspace_bytes=need)
+    with pytest.raises(ql.QloraError) as e:                               # a keep scale in any form that float() takes: 0.5 is refused by the library
+        ql.qlora_fwd_dropout(d, 4, ok, ok, "0.5", ok, ok, ok, ok, ok, ok, None, ok, stream=0, workspace_bytes=need)
+    assert e.value.status == -1
+    with pytest.raises(ValueError):
+        ql.qlora_fwd_dropout(d, 4, ok, ok, "half", ok, ok, ok, ok, ok, ok, None, ok, stream=0, workspace_bytes=need)
 
     class Stream:
         cuda_stream = 0
