@@ -457,8 +457,9 @@ def test_lora_dropout_ragged_rows(M, K, N, r):
     Xr, dYr, Ar, Br = f64(layer["X"]), f64(layer["dY"]), f64(layer["A"]), f64(layer["B"])
     Yo, Ho = orc.forward_dropout(Xr, W, Ar, Br, layer["alpha"], (mask_np != 0).astype(np.uint8), p)
     dXo, dAo, dBo, Go = orc.backward_dropout(Xr, dYr, W, Ar, Br, layer["alpha"], (mask_np != 0).astype(np.uint8), p)
-    # few terms (K = 32, 96; N = 8) leave the rounding of single weights visible; H and G are fp32 sums of exact products
-    for name, got, want, tol in (("Y", Y, Yo, 3e-2), ("H", H, Ho, 1e-4), ("dX", dX, dXo, 3e-2), ("G", G, Go, 1e-4), ("dA", dA, dAo, REL_TOL), ("dB", dB, dBo, REL_TOL)):
+    # weights, s * H and outputs rounded to bf16 (dX twice) in otherwise exact arithmetic give 1.15e-2 on Y and 1.3e-2 on dX at most
+    # over these shapes; H and G are fp32 sums of exact products
+    for name, got, want, tol in (("Y", Y, Yo, REL_TOL), ("H", H, Ho, 1e-4), ("dX", dX, dXo, REL_TOL), ("G", G, Go, 1e-4), ("dA", dA, dAo, REL_TOL), ("dB", dB, dBo, REL_TOL)):
         assert rel_err(to_f64(got), want) <= tol, name
 
 
