@@ -2,7 +2,7 @@
 // rows (simt_kernels.cu) and by the single-CTA tensor-core kernel, whose spare clusters run it beside the main tiles.
 //   P[m, j] = sum_t In[m, t] * L(j, t)     l_is_A: L = A [r, T] (contraction-contiguous), else L = B [T, r].
 // mma.sync m16n8k16 (bf16 in, fp32 accumulate) fed straight from 16-byte row loads: the warps of the block stride over
-// the contraction in steps of 32 and keep LD_UNROLL steps of loads in flight, the adapter's among them.  The 32 contraction indices of a step are
+// the contraction in steps of 32 and keep UNROLL steps of loads in flight, the adapter's among them.  The 32 contraction indices of a step are
 // assigned to the fragments in a permuted order (lane q of a quad owns indices 8q..8q+7); activation and adapter fragments
 // use the same permutation, so the sum is unchanged.  A is contraction-contiguous and loads directly; B is rank-contiguous,
 // so its 8 x 8 fragment tiles are loaded row-wise and transposed across the warp with movmatrix.  The per-warp partial
@@ -12,8 +12,6 @@
 #include <stdint.h>
 
 namespace qlora {
-
-constexpr int LD_UNROLL = 4;
 
 __device__ __forceinline__ void mma_bf16_16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
                                                uint32_t b0, uint32_t b1) {
@@ -38,8 +36,9 @@ __device__ __forceinline__ uint32_t movmatrix_trans(uint32_t a) {
 
 // Rows m_base .. m_base + 15 and, with NB = 2, the block of rows `block_stride` further on (beside the first: the same adapter words serve
 // both).  Called by all `nwarps` warps of a block (it synchronises the block twice); `red` is shared memory for nwarps * NB * NT * 128
-// floats.  L is read through the read-only path, and so is In.
-template <bool L_IS_A, int NT, int NB = 1>
+// floats.  L is read through the read-only path, and so is In.  UNROLL: as many steps as the registers hold, 8 NB + 4 NT of them each
+// (with 1024 threads, four steps at NT = 2 spilled 150 bytes and took 1.3 to 1.8 times as long).
+template <bool L_IS_A, int NT, int NB, int UNROLL>
 __device__ __forceinline__ void lora_down_rows(int M, int T, int r, const __nv_bfloat16* __restrict__ In,
                                                const __nv_bfloat16* __restrict__ L, float* __restrict__ P, int m_base, int block_stride, int nwarps,
                                                float* red) {
@@ -53,10 +52,10 @@ __device__ __forceinline__ void lora_down_rows(int M, int T, int r, const __nv_b
     const uint4 zero4 = make_uint4(0, 0, 0, 0);
     const int wstride = nwarps * 32;
 #pragma unroll 1
-    for (int kk = warp * 32; kk < T; kk += wstride * LD_UNROLL) {
-        uint4 xlo[NB][LD_UNROLL], xhi[NB][LD_UNROLL], l[LD_UNROLL][NT];
+    for (int kk = warp * 32; kk < T; kk += wstride * UNROLL) {
+        uint4 xlo[NB][UNROLL], xhi[NB][UNROLL], l[UNROLL][NT];
 #pragma unroll
-        for (int u = 0; u < LD_UNROLL; ++u) {                 // all loads of the unrolled steps first
+        for (int u = 0; u < UNROLL; ++u) {                 // all loads of the unrolled steps first
             const int k0 = kk + u * wstride, k = k0 + q * 8;  // T is a multiple of 8: 8 elements are all-in or all-out
 #pragma unroll
             for (int b = 0; b < NB; ++b) {
@@ -83,7 +82,7 @@ __device__ __forceinline__ void lora_down_rows(int M, int T, int r, const __nv_b
             }
         }
 #pragma unroll
-        for (int u = 0; u < LD_UNROLL; ++u) {
+        for (int u = 0; u < UNROLL; ++u) {
             if (kk + u * wstride >= T) break;                  // warp-uniform
 #pragma unroll
             for (int nt = 0; nt < NT; ++nt) {

@@ -329,8 +329,14 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
             // streaming form bring 10 - 30 GB/s per SM: P came 5000 cycles after the main loops at 128 tokens, 4096 x 4096).
             // INT8, 128 tokens, three calls one by one: 42.3 -> 39.2 us; a chain of forwards alone on activations from DRAM pays 17.7 -> 18.6.
             float* red = reinterpret_cast<float*>(smem_gen);
-            if (p.r <= 8) lora_down_rows<!TRANSPOSED, 1, 2>(p.M, p.T, p.r, p.In, p.Ldown, p.Pout, (int)blockIdx.x * 16, n_ctas * 16, kThreads / 32, red);
-            else          lora_down_rows<!TRANSPOSED, 2, 2>(p.M, p.T, p.r, p.In, p.Ldown, p.Pout, (int)blockIdx.x * 16, n_ctas * 16, kThreads / 32, red);
+            const bool one = (p.M + 15) / 16 <= n_ctas;           // one row block per CTA
+            if (p.r <= 8) {
+                if (one) lora_down_rows<!TRANSPOSED, 1, 1, 6>(p.M, p.T, p.r, p.In, p.Ldown, p.Pout, (int)blockIdx.x * 16, n_ctas * 16, kThreads / 32, red);
+                else     lora_down_rows<!TRANSPOSED, 1, 2, 4>(p.M, p.T, p.r, p.In, p.Ldown, p.Pout, (int)blockIdx.x * 16, n_ctas * 16, kThreads / 32, red);
+            } else {
+                if (one) lora_down_rows<!TRANSPOSED, 2, 1, 5>(p.M, p.T, p.r, p.In, p.Ldown, p.Pout, (int)blockIdx.x * 16, n_ctas * 16, kThreads / 32, red);
+                else     lora_down_rows<!TRANSPOSED, 2, 2, 2>(p.M, p.T, p.r, p.In, p.Ldown, p.Pout, (int)blockIdx.x * 16, n_ctas * 16, kThreads / 32, red);
+            }
         } else {
             if (p.r <= 8) lora_down_stream<!TRANSPOSED, 1>(p.M, p.T, p.r, p.In, p.Ldown, p.Pout, (int)blockIdx.x, n_ctas, smem_gen, p.lds_stages, abort_flag);
             else          lora_down_stream<!TRANSPOSED, 2>(p.M, p.T, p.r, p.In, p.Ldown, p.Pout, (int)blockIdx.x, n_ctas, smem_gen, p.lds_stages, abort_flag);

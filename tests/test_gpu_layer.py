@@ -434,6 +434,21 @@ def test_ranks_above_16_split_down_projection(M, K, N, r):
     assert torch.equal(saved["dA"], again["dA"]) and torch.equal(saved["dB"], again["dB"])
 
 
+@pytest.mark.parametrize("r", [8, 16])
+@pytest.mark.parametrize("M,K,N", [(17, 4096, 1024), (60, 128, 64), (144, 2112, 320), (200, 4096, 256), (256, 352, 264), (256, 6144, 4096)])
+def test_down_projection_of_few_rows(M, K, N, r):
+    """17 .. 256 tokens, ranks up to 16: H and G from spare clusters beside the tiles (one or two row blocks per CTA), from a launch ahead
+    of them where those cannot take all rows, and recomputed for the gradients; contractions shorter than one round of a block's warps
+    and longer than several."""
+    layer = qi.random_codes_layer(K=K, N=N, bits=4, group_size=32 if K % 64 else 64, r=r, alpha=2.0 * r, M=M, seed=M + K + r)
+    errs, saved, gl = check_layer(layer)
+    assert errs["H"] < 1e-4 and errs["G"] < 1e-4             # fp32 sums of exact products
+    again = gl.run(save_hg=False)
+    for key in ("dA", "dB"):
+        # (P is rounded to bf16 for the products: sums in another order may flip that, 2^-8 of a term in a sum of M)
+        assert rel_err(to_f64(again[key]), to_f64(saved[key])) <= 2**-8, key
+
+
 @pytest.mark.parametrize("M,K,N,r", [(1, 32, 8, 8), (5, 96, 72, 16), (333, 2080, 264, 8), (1801, 256, 128, 16), (260, 128, 64, 64)])
 def test_lora_dropout_ragged_rows(M, K, N, r):
     """The masked paths at row counts that are no multiple of anything: masked down-projection, masked gradient, masked update."""
