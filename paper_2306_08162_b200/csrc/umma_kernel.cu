@@ -204,6 +204,8 @@ __device__ __forceinline__ bool wait_counter(const unsigned* ctr, unsigned targe
     return false;
 }
 
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
 #include "lora_down_stream.cuh"
 
 // Eight of s * P as bf16 (the LoRA operand), and -- where it is wanted -- in `low` what that rounding left over, again as bf16.
@@ -323,11 +325,21 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
         // ------------------------------------------------------------------ producer cluster: LoRA down-projection on SMs
         // the tiles leave idle (one CTA per row block or more; lowest block indices, so they wait for nobody)
         const int n_ctas = p.n_prod * p.split;
+        if (p.M <= 256) {   // ask all lines this CTA will read (its share of the adapter) into L2 at once; nothing is read into the SM
+            const size_t row = (size_t)p.T * 2, share = (size_t)p.r * row / (size_t)n_ctas;
+            const char* l = reinterpret_cast<const char*>(p.Ldown) + (size_t)blockIdx.x * share;
+            for (size_t o = (size_t)threadIdx.x * 128; o < share; o += kThreads * 128) prefetch_l2(l + o);
+            for (int m = (int)blockIdx.x * 16; m < p.M; m += n_ctas * 16) {
+                const char* x = reinterpret_cast<const char*>(p.In) + (size_t)m * row;
+                const size_t n = (size_t)min(16, p.M - m) * row;
+                for (size_t o = (size_t)threadIdx.x * 128; o < n; o += kThreads * 128) prefetch_l2(x + o);
+            }
+        }
         pdl_wait();
         if (p.M <= 256) {
-            // few row blocks (two per CTA at most) and a short main loop: 16-byte row loads, 120 KB of them in flight (the bulk copies of the
-            // streaming form bring 10 - 30 GB/s per SM: P came 5000 cycles after the main loops at 128 tokens, 4096 x 4096).
-            // INT8, 128 tokens, three calls one by one: 42.3 -> 39.2 us; a chain of forwards alone on activations from DRAM pays 17.7 -> 18.6.
+            // few row blocks (two per CTA at most) and a short main loop: 16-byte row loads (the bulk copies of the streaming form bring
+            // 10 - 30 GB/s per SM: P came 5000 cycles after the main loops at 128 tokens, 4096 x 4096).  INT8, 128 tokens, forward:
+            // activations in L2 18.0 -> 15.6 us, from DRAM 18.2 -> 16.4 (without the request ahead 19.0: a round of loads is in flight at a time).
             float* red = reinterpret_cast<float*>(smem_gen);
             const bool one = (p.M + 15) / 16 <= n_ctas;           // one row block per CTA
             if (p.r <= 8) {
