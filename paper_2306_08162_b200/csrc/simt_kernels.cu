@@ -502,41 +502,86 @@ lora_grad_partial_kernel(int M, int r, int rows_per_slice, GradSide side0, GradS
             }
 }
 
-// Adds the slices' partial sums in slice order.  A thread takes four ranks of one column: neighbouring threads the next ranks of dB [N, r]
-// (stored as it lies in scratch), the next columns of dA [r, K] (so that each of its four stores is contiguous across the warp; element
-// by element they were 4-byte stores K apart).
-__global__ void __launch_bounds__(256) lora_grad_reduce_kernel(int r, int slices, int accumulate, GradSide dB_side, GradSide dA_side) {
-    pdl_launch_dependents();
-    const int r4 = r >> 2, nb = dB_side.C * r4, na = dA_side.C * r4;
-    const int idx = (int)(blockIdx.x * blockDim.x + threadIdx.x);
-    const bool is_dB = idx < nb;
-    const int e = is_dB ? idx : idx - nb;
-    const GradSide& sd = is_dB ? dB_side : dA_side;
-    int c = 0, j = 0;
-    if (is_dB) { c = e / r4; j = 4 * (e - c * r4); }
-    else if (e < na) { j = e / sd.C; c = e - j * sd.C; j *= 4; }
-    pdl_wait();
-    if (idx >= nb + na) return;
-    const float4* src = reinterpret_cast<const float4*>(sd.partial + (size_t)c * r + j);
-    const size_t step = (size_t)sd.C * r / 4;
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+// Adds the slices' partial sums in slice order.  Two forms; of the blocks the first are dB's, the others dA's.
+//   reduce4: a thread takes four ranks of one column, neighbouring threads the next ranks of dB [N, r] (stored as it lies in scratch), the
+//   next columns of dA [r, K] (its four stores are contiguous across the warp; its loads are not).
+//   reduce: one element per thread as it lies in scratch, dA stored through shared memory, a block's columns of one rank together.
+// The scattered loads are few at rank 8, where two threads share a sector, and at rank 16 while there are few slices; the line lies there.
+// Gradient call, reduce4 / reduce: 4096 x 4096, 2048 tokens, rank 8 12.65 / 12.97 us, rank 16 14.0 / 14.3, rank 32 19.0 / 16.7;
+// 1024 x 1024, 1024 tokens (16 slices), rank 16 8.5 / 6.2.
+constexpr int LR_THREADS = 256, LR4_MAX_SLICES = 9;
+
+__device__ __forceinline__ float4 lg_add(float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
+__device__ __forceinline__ float lg_add(float a, float b) { return a + b; }
+
+// The sum over the slices, eight independent loads in flight.
+template <typename V>
+__device__ __forceinline__ V lg_slice_sum(const V* src, size_t step, int slices) {
+    V v{};
     int sl = 0;
-    for (; sl + 4 <= slices; sl += 4) {               // four independent loads in flight, added in slice order
-        const float4 p0 = src[sl * step], p1 = src[(sl + 1) * step], p2 = src[(sl + 2) * step], p3 = src[(sl + 3) * step];
-        v.x = (((v.x + p0.x) + p1.x) + p2.x) + p3.x; v.y = (((v.y + p0.y) + p1.y) + p2.y) + p3.y;
-        v.z = (((v.z + p0.z) + p1.z) + p2.z) + p3.z; v.w = (((v.w + p0.w) + p1.w) + p2.w) + p3.w;
+    for (; sl + 8 <= slices; sl += 8) {
+        V x[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) x[i] = src[(sl + i) * step];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v = lg_add(v, x[i]);
     }
-    for (; sl < slices; ++sl) { const float4 x = src[sl * step]; v.x += x.x; v.y += x.y; v.z += x.z; v.w += x.w; }
+    if (sl + 4 <= slices) {
+        V x[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) x[i] = src[(sl + i) * step];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v = lg_add(v, x[i]);
+        sl += 4;
+    }
+    for (; sl < slices; ++sl) v = lg_add(v, src[sl * step]);
+    return v;
+}
+
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS) lora_grad_reduce4_kernel(int r, int slices, int accumulate, int blocks_dB, GradSide dB_side, GradSide dA_side) {
+    pdl_launch_dependents();
+    const bool is_dB = (int)blockIdx.x < blocks_dB;
+    const GradSide& sd = is_dB ? dB_side : dA_side;
+    const int e = ((int)blockIdx.x - (is_dB ? 0 : blocks_dB)) * THREADS + (int)threadIdx.x, r4 = r >> 2;
+    const int j = 4 * (is_dB ? e % r4 : e / sd.C), c = is_dB ? e / r4 : e % sd.C;
+    pdl_wait();
+    if (e >= sd.C * r4) return;
+    const size_t C = (size_t)sd.C;
+    float4 v = lg_slice_sum(reinterpret_cast<const float4*>(sd.partial + (size_t)c * r + j), C * r / 4, slices);
     v.x *= sd.scale; v.y *= sd.scale; v.z *= sd.scale; v.w *= sd.scale;
     if (is_dB) {
         float4* dst = reinterpret_cast<float4*>(sd.Out + (size_t)c * r + j);
-        if (accumulate) { const float4 o = *dst; v.x = o.x + v.x; v.y = o.y + v.y; v.z = o.z + v.z; v.w = o.w + v.w; }
+        if (accumulate) v = lg_add(*dst, v);
         *dst = v;
     } else {
-        float* dst = sd.Out + (size_t)j * sd.C + c;
-        const size_t C = (size_t)sd.C;
+        float* dst = sd.Out + (size_t)j * C + c;
         if (accumulate) { v.x = dst[0] + v.x; v.y = dst[C] + v.y; v.z = dst[2 * C] + v.z; v.w = dst[3 * C] + v.w; }
         dst[0] = v.x; dst[C] = v.y; dst[2 * C] = v.z; dst[3 * C] = v.w;
+    }
+}
+
+__global__ void __launch_bounds__(LR_THREADS) lora_grad_reduce_kernel(int r, int slices, int accumulate, int blocks_dB, GradSide dB_side, GradSide dA_side) {
+    __shared__ float tile[LR_THREADS];                         // dA: [column of the block][rank]
+    pdl_launch_dependents();
+    const bool is_dB = (int)blockIdx.x < blocks_dB;
+    const GradSide& sd = is_dB ? dB_side : dA_side;
+    const int cols = LR_THREADS / r, tid = threadIdx.x;        // columns of a block (threads beyond cols * r have no part)
+    const int c0 = ((int)blockIdx.x - (is_dB ? 0 : blocks_dB)) * cols, n = min(cols, sd.C - c0) * r;
+    const size_t e = (size_t)c0 * r + tid;
+    pdl_wait();
+    if (tid < n) {
+        const float v = lg_slice_sum((const float*)sd.partial + e, (size_t)sd.C * r, slices) * sd.scale;
+        if (is_dB) sd.Out[e] = accumulate ? sd.Out[e] + v : v;
+        else tile[tid] = v;
+    }
+    if (is_dB) return;
+    __syncthreads();
+    const int j = tid / cols, cl = tid - j * cols;
+    if (j < r && cl * r < n) {
+        float* dst = sd.Out + (size_t)j * sd.C + c0 + cl;
+        const float v = tile[cl * r + j];
+        *dst = accumulate ? *dst + v : v;
     }
 }
 
@@ -638,8 +683,13 @@ int launch_lora_grads(int M, int K, int N, int r, float s, const void* X, const 
     if (err != cudaSuccess) return QLORA_ERR_CUDA;
     const GradSide& rB = want_dB ? sB : none;
     const GradSide& rA = want_dA ? sA : none;
-    const size_t total = (size_t)(rB.C + rA.C) * r / 4;                 // (r is a multiple of 8; K, N and r fit 31 bits together: scratch is sized for them)
-    err = launch_pdl(lora_grad_reduce_kernel, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, st, 1, r, plan.slices, accumulate, rB, rA);
+    const int threads = r == 8 ? 64 : LR_THREADS, r4 = r / 4, red_cols = LR_THREADS / r;
+    const bool four = r == 8 || (r == 16 && plan.slices <= LR4_MAX_SLICES);
+    auto blocks = [&](int C) { return four ? (int)(((size_t)C * r4 + threads - 1) / threads) : (C + red_cols - 1) / red_cols; };
+    const dim3 red_grid((unsigned)(blocks(rB.C) + blocks(rA.C))), red_block((unsigned)threads);
+    if (four && r == 8) err = launch_pdl(lora_grad_reduce4_kernel<64>, red_grid, red_block, 0, st, 1, r, plan.slices, accumulate, blocks(rB.C), rB, rA);
+    else if (four)      err = launch_pdl(lora_grad_reduce4_kernel<LR_THREADS>, red_grid, red_block, 0, st, 1, r, plan.slices, accumulate, blocks(rB.C), rB, rA);
+    else                err = launch_pdl(lora_grad_reduce_kernel, red_grid, red_block, 0, st, 1, r, plan.slices, accumulate, blocks(rB.C), rB, rA);
     return err == cudaSuccess ? QLORA_OK : QLORA_ERR_CUDA;
 }
 

@@ -326,6 +326,28 @@ def test_seeded_sweep_across_the_dispatch_boundaries(seed):
     check_layer(layer)
 
 
+@pytest.mark.parametrize("r", [8, 16, 24, 40, 64])
+@pytest.mark.parametrize("M,K,N", [(300, 96, 40), (1030, 256, 72), (2100, 128, 2112), (600, 4128, 8)])
+def test_gradients_from_many_row_slices(M, K, N, r):
+    """Above 256 tokens partial sums per row slice are added by a second launch: one slice to 34 of them, widths that leave the last block
+    partly filled, ranks that do not divide a block's threads; overwritten, accumulated (exact additions), and dA alone."""
+    import paper_2306_08162_b200 as ql
+    layer = qi.random_codes_layer(K=K, N=N, bits=4, group_size=32, r=r, alpha=2.0 * r, M=M, seed=M + r)
+    gl = GpuLayer(layer)
+    out = gl.run()
+    f64 = orc.bf16_bits_to_f64
+    s, bf = layer["alpha"] / r, lambda t: t.bfloat16().double().cpu().numpy()        # (H and G are rounded to bf16 for the products)
+    want = {"dA": s * bf(out["G"]).T @ f64(layer["X"]), "dB": s * f64(layer["dY"]).T @ bf(out["H"])}
+    for key in want:
+        assert rel_err(to_f64(out[key]), want[key]) <= 2e-5, key                     # fp32 sums of M exact products: M 2^-24 a term at most
+    dA0, dB0 = torch.full_like(out["dA"], 0.5), torch.full_like(out["dB"], -0.25)
+    more = gl.run(accumulate=1, dA=dA0.clone(), dB=dB0.clone())
+    assert torch.equal(more["dA"], dA0 + out["dA"]) and torch.equal(more["dB"], dB0 + out["dB"])
+    alone = torch.full_like(out["dA"], float("nan"))
+    ql.qlora_bwd_lora(gl.desc, M, gl.X, None, gl.A, gl.B, None, out["G"], alone, None, 0, gl.ws)
+    assert rel_err(to_f64(alone), want["dA"]) <= 2e-5
+
+
 def test_accumulate_adds_to_existing_gradients():
     layer = qi.random_codes_layer(K=256, N=256, bits=4, group_size=128, r=8, alpha=16.0, M=96, seed=4)
     gl = GpuLayer(layer)
