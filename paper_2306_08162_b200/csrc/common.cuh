@@ -28,7 +28,8 @@ __device__ __forceinline__ __nv_bfloat16 dequant_one(uint32_t q, __half scale, _
 // Programmatic dependent launch.  Every layer kernel is launched with the programmatic-stream-serialization attribute:
 // it may be scheduled while its predecessor in the stream is still running, does its own set-up (barriers, tensor memory,
 // descriptor fetches), and then blocks in pdl_wait() until the predecessor has completed and its writes are visible.
-// Nothing may read or write global memory before pdl_wait().  pdl_launch_dependents() at the top lets the successor be
+// Before pdl_wait() a kernel may read Q, scales and zeros, which are frozen, and ask other operands into L2 (a prefetch reads nothing
+// into the SM); every other access to global memory comes after it.  pdl_launch_dependents() at the top lets the successor be
 // scheduled as soon as every CTA of this grid has started.  This hides the launch latency between the kernels of a step.
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
@@ -47,8 +48,8 @@ __device__ __forceinline__ float bf16_hi(uint32_t packed) { return __uint_as_flo
 // The code is ORed into the mantissa of the bf16 constant 128 (ulp 1), so u = 128 + q and d = u - (128 + zero) = q - zero
 // exactly.  |d| <= 15 has <= 4 significant bits, hence p = s_lo * d (<= 7 bits) is exact in bf16, s_hi * d (<= 12 bits)
 // is exact inside the fused multiply-add, and fma(s_hi, d, p) rounds the exact value s * d once, to nearest even.
-// 3- and 8-bit path: the code is ORed into the mantissa of the fp32 constant 2^23, 2^23 + zero is subtracted (exact),
-// the fp32 product with the scale is exact and the pair is rounded once by the packed convert.
+// 3- and 8-bit path: the code is placed in the mantissa of the fp32 constant 2^23 (3 bits: shift, mask and OR; 8 bits: one byte
+// permute), 2^23 + zero is subtracted (exact), the fp32 product with the scale is exact and the pair is rounded once by the packed convert.
 // ------------------------------------------------------------------------------------------------------------
 struct GroupParams {
     uint32_t s_hi2, s_lo2, c2;   // bf16x2 constants of the 2/4-bit path

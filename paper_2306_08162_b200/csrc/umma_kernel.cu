@@ -792,8 +792,8 @@ bool umma_supported(const qlora_desc& d, int M) {
     if (M < 1) return false;
     if (d.K % 64 != 0 || d.N % 64 != 0) return false;              // contraction steps of 64 in both directions
     // a stage's 64 (forward) or 128 (backward) rows along k hold whole groups, or lie inside one: every 32-code block then has
-    // its scale row at the same place in every stage.  (Groups of 32 on the CUDA cores instead: 4130 us for a step of 333 tokens
-    // on 11008 -> 4096, against 153 here.)
+    // its scale row at the same place in every stage.  (Groups of 32 on the CUDA cores instead: 4210 us for a step of 333 tokens
+    // on 11008 -> 4096, against 126 here.)
     if (!(d.group_size == 32 || d.group_size == 64 || d.group_size % 128 == 0)) return false;
     if (d.r > 64) return false;
     return true;
@@ -944,6 +944,8 @@ static int launch_umma_pair(const qlora_desc& d, int M, bool transposed, const v
 // weight rows) leave most SM pairs without one on a 4096-wide layer (42 us against 23 at 512 tokens), but fill a wave
 // exactly where the single-CTA kernel's 128 x 256 tiles need two (11008 outputs: 45 against 68 us).  The choice follows
 // a small cost model fitted to measurements: waves of tiles times (steps x time per step + fixed part) for each kernel.
+// (The constants date from before the single-CTA kernel cut its token tiles in 16s; it has become faster since, so the border lies a
+// little too low for it.)
 static bool prefer_pair_kernel(const qlora_desc& d, int M, bool transposed) {
     if (M <= 256) return false;
     if (M > 1024) return true;
