@@ -45,6 +45,7 @@ namespace qlora {
 namespace {
 
 constexpr int ST_WARPS = 8, ST_THREADS = 32 * ST_WARPS;
+constexpr int ST_LONG = 16384;                               // contractions up to here are staged whole
 constexpr int ST_CHUNK = 128;                                // forward: contraction elements per step of a warp
 
 template <int BITS>
@@ -68,6 +69,7 @@ struct StreamParams {
     int lwp;                     // log2 of the parts the warps of a CTA split its range of the contraction into (wc << lwp == ST_WARPS)
     int lsl;                     // log2 of the columns a CTA of the cluster finishes
     int pitch;                   // bytes of a staged activation row
+    int pass;                    // units of the contraction (128 elements forward, 32 columns backward) a CTA stages at a time
     int range;                   // contraction elements a CTA stages at most
     int ngl;                     // forward: group rows of a CTA's range at most; backward: groups its features span (1 or 2)
     int gd;                      // g / 32, and ceil(2^32 / gd): a group index is a multiplication
@@ -200,15 +202,19 @@ __host__ __device__ inline SmemPlan st_plan(const StreamParams& p, bool transpos
 }
 
 // A warp's partial H / G tile (MMA accumulator layout: rows = ranks, columns = tokens) -> its slot of hp.
+// `add`: on top of what the slot holds (a later pass).
 template <int NT>
-__device__ __forceinline__ void st_store_hp(const StreamParams& p, const float (&ah)[NT][4], float* hp, int warp, int g, int q) {
+__device__ __forceinline__ void st_store_hp(const StreamParams& p, const float (&ah)[NT][4], float* hp, int warp, int g, int q, bool add) {
     float* mine = hp + warp * 16 * p.M + g;
 #pragma unroll
     for (int tt = 0; tt < NT; ++tt)
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
             const int tok = 8 * tt + 2 * q + e;
-            if (tok < p.M) { mine[tok * 16] = ah[tt][e]; mine[tok * 16 + 8] = ah[tt][2 + e]; }
+            if (tok < p.M) {
+                mine[tok * 16] = ah[tt][e] + (add ? mine[tok * 16] : 0.f);
+                mine[tok * 16 + 8] = ah[tt][2 + e] + (add ? mine[tok * 16 + 8] : 0.f);
+            }
         }
 }
 
@@ -312,8 +318,9 @@ __device__ __forceinline__ void st_finish(const StreamParams& p, uint8_t* smem, 
 // Forward: Y = X W^T + s H B^T.  CTA (rank, tile): columns [32 wc tile, + 32 wc), contraction chunks [c0, c1) of 128 elements.
 // Warp (cg, part): 32 columns and its share of the chunks.  GPC: scale segments per chunk -- 1 for groups that are multiples of
 // 128, 2 for multiples of 64, 4 for multiples of 32 (the segment, not the group, is what one accumulator spans).
+// MULTI: a contraction whose activations do not fit the shared memory; staging and products take p.pass chunks at a time in turn.
 // ------------------------------------------------------------------------------------------------------------
-template <int BITS, int NT, int GPC, int PER_SM>
+template <int BITS, int NT, int GPC, int PER_SM, bool MULTI>
 __global__ void __launch_bounds__(ST_THREADS, PER_SM) stream_fwd_kernel(const StreamParams p) {
     using F = Fmt<BITS>;
     constexpr int TOKS = 8 * NT, SB = 2;                   // SB: slices of the staging pass whose loads a warp has in flight
@@ -326,7 +333,8 @@ __global__ void __launch_bounds__(ST_THREADS, PER_SM) stream_fwd_kernel(const St
     const int tile_c0 = (int)blockIdx.y * tile_c, c_lo = tile_c0 + (rank << p.lsl);
     const int nch = (p.K + ST_CHUNK - 1) / ST_CHUNK;
     const int c0 = (nch * rank) >> p.lks, c1 = (nch * (rank + 1)) >> p.lks;
-    const int w0 = c0 + (((c1 - c0) * part) >> p.lwp), w1 = c0 + (((c1 - c0) * (part + 1)) >> p.lwp);
+    int p0 = c0, p1 = MULTI ? min(c1, c0 + p.pass) : c1;   // the chunks of this pass, and this warp's share of them
+    int w0 = p0 + (((p1 - p0) * part) >> p.lwp), w1 = p0 + (((p1 - p0) * (part + 1)) >> p.lwp);
     const SmemPlan sp = st_plan(p, false, TOKS, tile_c);
     uint8_t* xs = smem;                                    // [M][pitch] activations in fragment order
     const __half* sz = reinterpret_cast<const __half*>(smem + sp.sz);       // [group][scales, zeros][tile_c]
@@ -358,22 +366,30 @@ __global__ void __launch_bounds__(ST_THREADS, PER_SM) stream_fwd_kernel(const St
     uint4 w[F::DEPTH][F::LPC];
 #pragma unroll
     for (int d = 0; d < F::DEPTH; ++d) load_chunk(w[d], w0 + d);
-    const int g_first = st_group(p, c0 * (ST_CHUNK / 32));
-    {
-        const int g_last = c1 > c0 ? st_group(p, min(c1 * (ST_CHUNK / 32), p.K >> 5) - 1) : g_first - 1;
+    int g_first = 0;
+    auto load_sz = [&]() {
+        g_first = st_group(p, p0 * (ST_CHUNK / 32));
+        const int g_last = p1 > p0 ? st_group(p, min(p1 * (ST_CHUNK / 32), p.K >> 5) - 1) : g_first - 1;
         const int lper = p.lwc + 2, n = (g_last - g_first + 1) << (lper + 1);             // 16-byte pieces
         for (int e = tid; e < n; e += ST_THREADS) {
             const int row = e >> lper, c = tile_c0 + 8 * (e & ((1 << lper) - 1));
             const __half* src = ((row & 1) ? p.zeros : p.scales) + (size_t)(g_first + (row >> 1)) * p.N + c;
             cp16(s_u32(sz) + e * 16, c < p.N ? src : p.scales, c < p.N ? 16 : 0);
         }
-    }
+    };
+    load_sz();
     constexpr int SEG_K = ST_CHUNK / GPC, SEG_B = F::BPC / GPC;             // contraction elements and blocks of a segment
     const int spg = p.gd / (SEG_K / 32);                                    // segments per group
-    const int g_w0 = st_group(p, w0 * (ST_CHUNK / 32));
-    int gpos = w0 * GPC - g_w0 * spg;
-    const __half* sz_lane = sz + (g_w0 - g_first) * 2 * tile_c + 32 * cg + 4 * g;
-    const int k_lo = c0 * ST_CHUNK, n_slices = (c1 - c0) * (ST_CHUNK / 32), n_valid = min(n_slices, (p.K - k_lo) >> 5);
+    int gpos = 0;
+    const __half* sz_lane = nullptr;
+    int k_lo = 0, n_slices = 0, n_valid = 0;
+    auto set_pass = [&]() {
+        const int g_w0 = st_group(p, w0 * (ST_CHUNK / 32));
+        gpos = w0 * GPC - g_w0 * spg;
+        sz_lane = sz + (g_w0 - g_first) * 2 * tile_c + 32 * cg + 4 * g;
+        k_lo = p0 * ST_CHUNK; n_slices = (p1 - p0) * (ST_CHUNK / 32); n_valid = min(n_slices, (p.K - k_lo) >> 5);
+    };
+    set_pass();
     {   // ask the lines this CTA will read right after the wait into L2 (nothing is read into the SM): its slices of X, A and B
         const int rows = p.M + (p.fused ? p.r : 0);
         for (int j = warp; j < rows; j += ST_WARPS) {
@@ -385,10 +401,24 @@ __global__ void __launch_bounds__(ST_THREADS, PER_SM) stream_fwd_kernel(const St
 
     pdl_wait();
 
-    // ---- staging: activations into fragment order, their sums, and this CTA's part of H = X A^T ----
     const bool tok_ok[2] = {g < p.M, g + 8 < p.M};
+    const uint32_t recv_h_addr = s_u32(smem + sp.recv_h);
+    float acc[2][NT][4];
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int tt = 0; tt < NT; ++tt) acc[u][tt][0] = acc[u][tt][1] = acc[u][tt][2] = acc[u][tt][3] = 0.f;
+#pragma unroll 1
+    do {
+    // ---- staging: activations into fragment order, their sums, and this CTA's part of H = X A^T ----
+    const bool again = MULTI && p0 > c0;
+    if (again) {
+        __syncthreads();                                   // every warp is done with the pass before
+        load_sz();
+        set_pass();
+    }
     {
-        bool first = true;                                 // (every warp stages its share of the second adapter once)
+        bool first = !again;                               // (every warp stages its share of the second adapter once)
         float hacc[NT][4];
 #pragma unroll
         for (int tt = 0; tt < NT; ++tt) hacc[tt][0] = hacc[tt][1] = hacc[tt][2] = hacc[tt][3] = 0.f;
@@ -435,20 +465,16 @@ __global__ void __launch_bounds__(ST_THREADS, PER_SM) stream_fwd_kernel(const St
                 }
             }
         }
-        if (p.fused) st_store_hp<NT>(p, hacc, hp, warp, g, q);
+        if (p.fused) st_store_hp<NT>(p, hacc, hp, warp, g, q, again);
     }
     cp_wait_all();
     __syncthreads();
-    const uint32_t recv_h_addr = s_u32(smem + sp.recv_h);
-    if (p.ks > 1) st_cluster_wait();                       // every CTA of the cluster is running: its shared memory may be written
-    if (p.fused) st_share_h(p, hp, recv_h_addr, rank);
+    if (!MULTI || p1 == c1) {
+        if (p.ks > 1) st_cluster_wait();                   // every CTA of the cluster is running: its shared memory may be written
+        if (p.fused) st_share_h(p, hp, recv_h_addr, rank);
+    }
 
     // ---- main loop ----
-    float acc[2][NT][4];
-#pragma unroll
-    for (int u = 0; u < 2; ++u)
-#pragma unroll
-        for (int tt = 0; tt < NT; ++tt) acc[u][tt][0] = acc[u][tt][1] = acc[u][tt][2] = acc[u][tt][3] = 0.f;
     const uint32_t xl = s_u32(xs) + (uint32_t)(g * p.pitch + q * (BITS == 2 ? 32 : (BITS == 8 ? 8 : 16)));
     uint32_t xf[NT][F::NPAIR];                             // activation fragments: token g (+ 8), this lane's quarter of a block
 #pragma unroll
@@ -456,8 +482,8 @@ __global__ void __launch_bounds__(ST_THREADS, PER_SM) stream_fwd_kernel(const St
 #pragma unroll
         for (int i = 0; i < F::NPAIR; ++i) xf[tt][i] = 0u; // (stays zero for tokens that do not exist)
     auto compute = [&](const uint4 (&wd)[F::LPC], int ch) {
-        const uint32_t xc = xl + (uint32_t)(ch - c0) * (ST_CHUNK * 2);
-        const float* sumc = xsum + (ch - c0) * (ST_CHUNK / 32) * TOKS + 2 * q;
+        const uint32_t xc = xl + (uint32_t)(ch - p0) * (ST_CHUNK * 2);
+        const float* sumc = xsum + (ch - p0) * (ST_CHUNK / 32) * TOKS + 2 * q;
 #pragma unroll
         for (int sg = 0; sg < GPC; ++sg) {
             if (GPC > 1 && ch * ST_CHUNK + sg * SEG_K >= p.K) break;        // (a last chunk that is not full: no such group)
@@ -527,6 +553,12 @@ __global__ void __launch_bounds__(ST_THREADS, PER_SM) stream_fwd_kernel(const St
             }
         }
     }
+    if (!MULTI || p1 == c1) break;
+    p0 = p1; p1 = min(c1, p0 + p.pass);
+    w0 = p0 + (((p1 - p0) * part) >> p.lwp); w1 = p0 + (((p1 - p0) * (part + 1)) >> p.lwp);
+#pragma unroll
+    for (int d = 0; d < F::DEPTH; ++d) load_chunk(w[d], w0 + d);
+    } while (true);
     // accumulator element (u, tt, e): column 4g + 2u + (e >> 1) of this warp's 32, token 2q + (e & 1) + 8 tt
     float* mine = reinterpret_cast<float*>(smem + sp.part) + part * p.M * tile_c + 32 * cg + 4 * g;
 #pragma unroll
@@ -543,6 +575,7 @@ __global__ void __launch_bounds__(ST_THREADS, PER_SM) stream_fwd_kernel(const St
 // Backward: dX = dY W + s G A.  CTA (rank, tile): output features [8 FL wc tile, + 8 FL wc), contraction units [u0, u1) of 32
 // packed columns.  Warp (fw, part): 8 FL features (all inside one group) and its share of the units.  Lane (g, q) has features
 // FL g .. FL g + FL - 1 of the warp's, columns 4q .. 4q+3 (+ 16) of a unit.  FL = 8, or 4 where groups are not multiples of 64.
+// MULTI as forward.
 // ------------------------------------------------------------------------------------------------------------
 template <int BITS, int FL>
 struct BFmt {
@@ -573,11 +606,11 @@ __device__ __forceinline__ void st_bwd_pairs(uint32_t a0, uint32_t a1, uint32_t 
     }
 }
 
-template <int BITS, int NT, int FL, int PER_SM>
+template <int BITS, int NT, int FL, int PER_SM, bool MULTI>
 __global__ void __launch_bounds__(ST_THREADS, PER_SM) stream_bwd_kernel(const StreamParams p) {
     using F = Fmt<BITS>;
     using BF = BFmt<BITS, FL>;
-    constexpr int TOKS = 8 * NT, SB = 2;
+    constexpr int TOKS = 8 * NT, SB = MULTI && NT == 1 ? 4 : 2;   // SB: as forward
     pdl_launch_dependents();
     if (p.ks > 1) st_cluster_arrive_relaxed();             // waited for before the first store into a peer's shared memory
     extern __shared__ __align__(128) uint8_t smem[];
@@ -587,7 +620,8 @@ __global__ void __launch_bounds__(ST_THREADS, PER_SM) stream_bwd_kernel(const St
     const int tile_f0 = (int)blockIdx.y * tile_c, c_lo = tile_f0 + (rank << p.lsl), f0 = tile_f0 + 8 * FL * fw;
     const int nun = (p.N + 31) >> 5;
     const int u0 = (nun * rank) >> p.lks, u1 = (nun * (rank + 1)) >> p.lks;
-    const int w0 = u0 + (((u1 - u0) * part) >> p.lwp), w1 = u0 + (((u1 - u0) * (part + 1)) >> p.lwp);
+    int p0 = u0, p1 = MULTI ? min(u1, u0 + p.pass) : u1;   // the units of this pass, and this warp's share of them
+    int w0 = p0 + (((p1 - p0) * part) >> p.lwp), w1 = p0 + (((p1 - p0) * (part + 1)) >> p.lwp);
     const int gk0 = st_group(p, tile_f0 >> 5), ngroups = st_group(p, p.K >> 5);    // group of the CTA's first feature
     const int copy = min(st_group(p, f0 >> 5) - gk0, p.ngl - 1);
     const SmemPlan sp = st_plan(p, true, TOKS, tile_c);
@@ -619,8 +653,9 @@ __global__ void __launch_bounds__(ST_THREADS, PER_SM) stream_bwd_kernel(const St
     uint4 w[BF::DEPTH][2 * BF::NLD];
 #pragma unroll
     for (int d = 0; d < BF::DEPTH; ++d) load_unit(w[d], w0 + d);
-    const int n_lo = u0 << 5, nu = u1 - u0;
-    {
+    int n_lo = 0, nu = 0;
+    auto load_sz = [&]() {
+        n_lo = p0 << 5; nu = p1 - p0;
         const int per = nu * 4;                            // 16-byte pieces of a row
         for (int rr = 0; rr < 2 * p.ngl; ++rr) {
             const int gk = gk0 + (rr >> 1);
@@ -630,7 +665,8 @@ __global__ void __launch_bounds__(ST_THREADS, PER_SM) stream_bwd_kernel(const St
                 cp16(s_u32(sz) + (uint32_t)(rr * p.range + 8 * i) * 2u, src + min(c, p.N - 8), c < p.N ? 16 : 0);
             }
         }
-    }
+    };
+    load_sz();
     {   // ask the lines this CTA will read right after the wait into L2 (nothing is read into the SM): its slices of dY, B and A
         const int n = min(32 * nu, p.N - n_lo);
         for (int j = warp; j < p.M; j += ST_WARPS)
@@ -643,6 +679,19 @@ __global__ void __launch_bounds__(ST_THREADS, PER_SM) stream_bwd_kernel(const St
     pdl_wait();
 
     const bool tok_ok[2] = {g < p.M, g + 8 < p.M};
+    const uint32_t recv_h_addr = s_u32(smem + sp.recv_h);
+    float acc[FL / 2][NT][4], z_sub[NT][2];
+#pragma unroll
+    for (int i = 0; i < FL / 2; ++i)
+#pragma unroll
+        for (int tt = 0; tt < NT; ++tt) acc[i][tt][0] = acc[i][tt][1] = acc[i][tt][2] = acc[i][tt][3] = 0.f;
+#pragma unroll 1
+    do {
+    const bool again = MULTI && p0 > u0;
+    if (again) {
+        __syncthreads();                                   // every warp is done with the pass before
+        load_sz();
+    }
     // ---- staging: slices of dY, scaled by each group's scales (one rounding); the zero-point sums; this CTA's part of G = dY B ----
     {
         float hacc[NT][4], zacc[2][NT];
@@ -675,7 +724,7 @@ __global__ void __launch_bounds__(ST_THREADS, PER_SM) stream_bwd_kernel(const St
                 }
             }
             if (!staged) {                                 // (with the first loads on their way: every warp comes here once)
-                st_stage_lup<true>(p, smem + sp.lup, hfull, c_lo);
+                if (!again) st_stage_lup<true>(p, smem + sp.lup, hfull, c_lo);
                 cp_wait_all();
                 __syncthreads();                           // the group parameters are staged
                 staged = true;
@@ -719,39 +768,39 @@ __global__ void __launch_bounds__(ST_THREADS, PER_SM) stream_bwd_kernel(const St
                 }
             }
         }
-        if (p.fused) st_store_hp<NT>(p, hacc, hp, warp, g, q);
+        if (p.fused) st_store_hp<NT>(p, hacc, hp, warp, g, q, again);
 #pragma unroll
         for (int c = 0; c < 2; ++c)
 #pragma unroll
             for (int tt = 0; tt < 2; ++tt) {
                 const float z = tt < NT ? st_quad_sum(zacc[c][tt < NT ? tt : 0]) : 0.f;
-                if (q == 0) zp[warp * 32 + c * 16 + 8 * tt + g] = z;
+                if (q == 0) zp[warp * 32 + c * 16 + 8 * tt + g] = z + (again ? zp[warp * 32 + c * 16 + 8 * tt + g] : 0.f);
             }
     }
     __syncthreads();
-    const uint32_t recv_h_addr = s_u32(smem + sp.recv_h);
-    if (p.ks > 1) st_cluster_wait();                       // every CTA of the cluster is running: its shared memory may be written
-    if (p.fused) st_share_h(p, hp, recv_h_addr, rank);
-    // zero-point sums of the CTA's whole range, warps added in order; part 0 alone subtracts them
-    float z_sub[NT][2];
+    if (!MULTI || p1 == u1) {
+        if (p.ks > 1) st_cluster_wait();                   // every CTA of the cluster is running: its shared memory may be written
+        if (p.fused) st_share_h(p, hp, recv_h_addr, rank);
+        // zero-point sums of the CTA's whole range, warps added in order; part 0 alone subtracts them
 #pragma unroll
-    for (int tt = 0; tt < NT; ++tt) z_sub[tt][0] = z_sub[tt][1] = 0.f;
-    if (part == 0) {
+        for (int tt = 0; tt < NT; ++tt) z_sub[tt][0] = z_sub[tt][1] = 0.f;
+        if (part == 0) {
 #pragma unroll
-        for (int tt = 0; tt < NT; ++tt)
+            for (int tt = 0; tt < NT; ++tt)
 #pragma unroll
-            for (int wv = 0; wv < ST_WARPS; ++wv) {
-                const float2 z = *reinterpret_cast<const float2*>(zp + wv * 32 + copy * 16 + 8 * tt + 2 * q);
-                z_sub[tt][0] += z.x; z_sub[tt][1] += z.y;
-            }
+                for (int wv = 0; wv < ST_WARPS; ++wv) {
+                    const float2 z = *reinterpret_cast<const float2*>(zp + wv * 32 + copy * 16 + 8 * tt + 2 * q);
+                    z_sub[tt][0] += z.x; z_sub[tt][1] += z.y;
+                }
+        }
+    }
+
+    if (again) {                                           // (registers: they would lie idle during the staging)
+#pragma unroll
+        for (int d = 0; d < BF::DEPTH; ++d) load_unit(w[d], w0 + d);
     }
 
     // ---- main loop ----
-    float acc[FL / 2][NT][4];
-#pragma unroll
-    for (int i = 0; i < FL / 2; ++i)
-#pragma unroll
-        for (int tt = 0; tt < NT; ++tt) acc[i][tt][0] = acc[i][tt][1] = acc[i][tt][2] = acc[i][tt][3] = 0.f;
     const uint32_t yl = s_u32(ys) + (uint32_t)((copy * p.M + g) * p.pitch + 8 * q);
     uint32_t xv[NT][2];
 #pragma unroll
@@ -765,20 +814,24 @@ __global__ void __launch_bounds__(ST_THREADS, PER_SM) stream_bwd_kernel(const St
                 for (int h = 0; h < 2; ++h) {
                     const uint4& wa = w[d][h * BF::NLD];
                     const uint4& wb = w[d][h * BF::NLD + BF::NLD - 1];
-                    uint32_t p0[FL], p1[FL];
-                    st_bwd_pairs<BITS, FL>(wa.x, wb.x, wa.y, wb.y, sh, sel, p0);
-                    st_bwd_pairs<BITS, FL>(wa.z, wb.z, wa.w, wb.w, sh, sel, p1);
+                    uint32_t pa[FL], pb[FL];
+                    st_bwd_pairs<BITS, FL>(wa.x, wb.x, wa.y, wb.y, sh, sel, pa);
+                    st_bwd_pairs<BITS, FL>(wa.z, wb.z, wa.w, wb.w, sh, sel, pb);
 #pragma unroll
                     for (int tt = 0; tt < NT; ++tt) {
-                        lds8(xv[tt][0], xv[tt][1], yl + (uint32_t)(8 * tt * p.pitch + (un + d - u0) * 64 + 32 * h), tok_ok[tt]);
+                        lds8(xv[tt][0], xv[tt][1], yl + (uint32_t)(8 * tt * p.pitch + (un + d - p0) * 64 + 32 * h), tok_ok[tt]);
 #pragma unroll
-                        for (int i = 0; i < FL / 2; ++i) st_mma(acc[i][tt], p0[2 * i], p0[2 * i + 1], p1[2 * i], p1[2 * i + 1], xv[tt][0], xv[tt][1]);
+                        for (int i = 0; i < FL / 2; ++i) st_mma(acc[i][tt], pa[2 * i], pa[2 * i + 1], pb[2 * i], pb[2 * i + 1], xv[tt][0], xv[tt][1]);
                     }
                 }
                 load_unit(w[d], un + d + BF::DEPTH);
             }
         }
     }
+    if (!MULTI || p1 == u1) break;
+    p0 = p1; p1 = min(u1, p0 + p.pass);
+    w0 = p0 + (((p1 - p0) * part) >> p.lwp); w1 = p0 + (((p1 - p0) * (part + 1)) >> p.lwp);
+    } while (true);
     // accumulator element (i, tt, e): feature FL g + 2 i + (e >> 1) of the warp's, token 2q + (e & 1) + 8 tt
     float* mine = reinterpret_cast<float*>(smem + sp.part) + part * p.M * tile_c + 8 * FL * fw + FL * g;
 #pragma unroll
@@ -797,6 +850,8 @@ __global__ void __launch_bounds__(ST_THREADS, PER_SM) stream_bwd_kernel(const St
 }
 
 // Three CTAs per SM (80 registers) exist where the kernels spill 24 bytes at most: up to 8 tokens, 4 bits, and 2 bits backward.
+// (Of the builds with 128 registers, those for 9 .. 16 tokens spill up to 80 bytes at 3 bits and 72 at 8 bits, the others none; the multi-pass
+// ones up to 770, all of it around the staging.)
 constexpr bool st_has_three(int bits, int nt, bool transposed) { return nt == 1 && (bits == 4 || (bits == 2 && transposed)); }
 
 int fwd_kb(int bits) { return bits == 2 ? 64 : 32; }
@@ -847,17 +902,17 @@ const DeviceFacts& device_facts() {
 //   exchange  the cluster barriers and the adding up;
 // and the whole repeats when the CTAs exceed what the GPU holds at once (two per SM up to half an SM's shared memory).  Three per SM, with
 // 80 registers, take 1.28 times as long for the same cut (4096 x 4096: 8.1 against 6.3 us) and are for cuts that two would need a second
-// wave for: 4096 -> 11008 forward, 344 CTAs, 15.9 -> 13.1 us; 4096 -> 11008 backward 17.4 -> 14.7.
+// wave for, one INT4 token: K = 4096, N = 11008 forward, 344 CTAs, 15.9 -> 13.1 us; K = 11008, N = 4096 backward, 17.4 -> 14.7.
 // (4096 x 4096, INT4, one token: 128 columns x 8 CTAs 6.3 us, 64 x 4 6.7, 32 x 2 8.2, 256 x 8 8.7, 128 x 4 9.3, 64 x 8 9.5.)
-struct StreamPlan { StreamParams p; int tiles, tile_c, per_sm; SmemPlan sm; bool ok; };
+struct StreamPlan { StreamParams p; int tiles, tile_c, per_sm, nt; SmemPlan sm; bool multi, ok; };
 
-template <int BITS, int NT, int V, bool TRANSPOSED, int PER_SM>   // V: GPC forward, FL backward
+template <int BITS, int NT, int V, bool TRANSPOSED, int PER_SM, bool MULTI>   // V: GPC forward, FL backward
 int st_launch_as(const StreamPlan& plan, cudaStream_t st) {
     static SmemLimit limit;
     const dim3 grid((unsigned)plan.p.ks, (unsigned)plan.tiles);
     void (*kern)(const StreamParams);
-    if constexpr (TRANSPOSED) kern = stream_bwd_kernel<BITS, NT, V, PER_SM>;
-    else kern = stream_fwd_kernel<BITS, NT, V, PER_SM>;
+    if constexpr (TRANSPOSED) kern = stream_bwd_kernel<BITS, NT, V, PER_SM, MULTI>;
+    else kern = stream_fwd_kernel<BITS, NT, V, PER_SM, MULTI>;
     if (!limit.raise(kern, 227 * 1024)) return QLORA_ERR_CUDA;
     return launch_pdl(kern, grid, dim3(ST_THREADS), plan.sm.total, st, (unsigned)plan.p.ks, plan.p) == cudaSuccess ? QLORA_OK : QLORA_ERR_CUDA;
 }
@@ -865,8 +920,9 @@ int st_launch_as(const StreamPlan& plan, cudaStream_t st) {
 template <int BITS, int NT, int V, bool TRANSPOSED>
 int st_launch(const StreamPlan& plan, cudaStream_t st) {
     if constexpr (st_has_three(BITS, NT, TRANSPOSED))
-        if (plan.per_sm == 3) return st_launch_as<BITS, NT, V, TRANSPOSED, 3>(plan, st);
-    return st_launch_as<BITS, NT, V, TRANSPOSED, 2>(plan, st);
+        if (plan.per_sm == 3) return st_launch_as<BITS, NT, V, TRANSPOSED, 3, false>(plan, st);
+    if (plan.multi) return st_launch_as<BITS, NT, V, TRANSPOSED, 2, true>(plan, st);
+    return st_launch_as<BITS, NT, V, TRANSPOSED, 2, false>(plan, st);
 }
 
 StreamPlan st_cut(StreamParams p, int bits, bool transposed) {
@@ -874,7 +930,7 @@ StreamPlan st_cut(StreamParams p, int bits, bool transposed) {
     best.ok = false;
     float best_cost = 0.f;
     const DeviceFacts& gpu = device_facts();
-    const int toks = p.M > 8 ? 16 : 8, nt = toks / 8, sms = gpu.sms;
+    const int sms = gpu.sms;
     const int fl = p.g % 64 == 0 ? 8 : 4;
     p.gd = p.g / 32;
     p.gm = (uint32_t)(((1ull << 32) + p.gd - 1) / p.gd);
@@ -895,25 +951,34 @@ StreamPlan st_cut(StreamParams p, int bits, bool transposed) {
             p.lsl = 0;
             while ((1 << p.lsl) < sl) ++p.lsl;
             const int per_cta = (units + p.ks - 1) / p.ks, parts = 1 << p.lwp;
-            p.range = per_cta * unit;
-            p.ngl = transposed ? groups : (p.range + p.g - 1) / p.g + 1;
-            // rows far enough apart that the fragment loads of neighbouring tokens meet different banks
-            const int want = transposed ? 32 : (bits == 2 ? 16 : (bits == 8 ? 32 : 64));
-            p.pitch = p.range * 2;
-            p.pitch += (want - p.pitch % 128 + 128) % 128;
-            const SmemPlan sm = st_plan(p, transposed, toks, tile_c);
-            if (sm.total > 227 * 1024 - 1024) continue;
-            const int per_warp = (per_cta + parts - 1) / parts;
-            const float step = (transposed ? 650.f + 150.f * (nt - 1) : 1400.f + 450.f * (nt - 1)) * (bits == 8 ? 1.3f : 1.f) * (tiles * p.ks > sms ? 1.2f : 1.f);
-            const float rounds = (float)((per_cta * (unit / 32) + 2 * ST_WARPS - 1) / (2 * ST_WARPS));
-            const float round = transposed ? 2500.f * nt : 900.f + 1100.f * nt;
-            const float once = (float)per_warp * step + rounds * round + 1500.f + 500.f * (float)lks;
-            for (int per_sm = 2; per_sm <= (st_has_three(bits, nt, transposed) && sm.total <= 74 * 1024 ? 3 : 2); ++per_sm) {
-                const int occ = sm.total <= 113 * 1024 ? per_sm : 1;
-                const float fill = (float)(tiles * 2) / (float)(gpu.clusters[p.ks] * occ);     // of what the GPU holds at once
-                const float waves = fill <= 1.f ? 1.f : 0.5f * (fill + ceilf(fill));
-                const float cost = waves * once * (per_sm == 3 ? 1.28f : 1.f);
-                if (!best.ok || cost < best_cost) { best = StreamPlan{p, tiles, tile_c, per_sm, sm, true}; best_cost = cost; }
+            // the whole range in one pass, or in passes that leave room for two CTAs per SM, or for one
+            for (int mode = 0; mode < (T > ST_LONG ? 3 : 1); ++mode) {
+                const int nt = p.M > 8 ? 2 : 1, toks = 8 * nt;
+                SmemPlan sm{};
+                for (p.pass = per_cta;;) {
+                    p.range = p.pass * unit;
+                    p.ngl = transposed ? groups : (p.range + p.g - 1) / p.g + 1;
+                    // rows far enough apart that the fragment loads of neighbouring tokens meet different banks
+                    const int want = transposed ? 32 : (bits == 2 ? 16 : (bits == 8 ? 32 : 64));
+                    p.pitch = p.range * 2;
+                    p.pitch += (want - p.pitch % 128 + 128) % 128;
+                    sm = st_plan(p, transposed, toks, tile_c);
+                    if (mode == 0 || p.pass == 1 || sm.total <= (mode == 1 ? 113u * 1024 : 227u * 1024 - 1024)) break;
+                    p.pass = p.pass > 16 ? p.pass * 7 / 8 : p.pass - 1;
+                }
+                if (sm.total > 227 * 1024 - 1024 || (mode > 0 && p.pass == per_cta)) continue;
+                const int passes = (per_cta + p.pass - 1) / p.pass, per_warp = (p.pass + parts - 1) / parts * passes;
+                const float step = (transposed ? 650.f + 150.f * (nt - 1) : 1400.f + 450.f * (nt - 1)) * (bits == 8 ? 1.3f : 1.f) * (tiles * p.ks > sms ? 1.2f : 1.f);
+                const float rounds = (float)((p.pass * (unit / 32) + 2 * ST_WARPS - 1) / (2 * ST_WARPS) * passes);
+                const float round = transposed ? 2500.f * nt : 900.f + 1100.f * nt;
+                const float once = (float)per_warp * step + rounds * round + 1500.f + 500.f * (float)lks + 1000.f * (float)(passes - 1);
+                for (int per_sm = 2; per_sm <= (mode == 0 && st_has_three(bits, nt, transposed) && sm.total <= 74 * 1024 ? 3 : 2); ++per_sm) {
+                    const int occ = sm.total <= 113 * 1024 ? per_sm : 1;
+                    const float fill = (float)(tiles * 2) / (float)(gpu.clusters[p.ks] * occ);     // of what the GPU holds at once
+                    const float waves = fill <= 1.f ? 1.f : 0.5f * (fill + ceilf(fill));
+                    const float cost = waves * once * (per_sm == 3 ? 1.28f : 1.f);
+                    if (!best.ok || cost < best_cost) { best = StreamPlan{p, tiles, tile_c, per_sm, nt, sm, mode > 0, true}; best_cost = cost; }
+                }
             }
         }
     }
@@ -926,7 +991,11 @@ bool stream_supported(const qlora_desc& d, int M, bool transposed) {
     if (M < 1 || M > 16) return false;
     if (d.K < 32 || d.N < 8 || d.K > (1 << 20)) return false;   // (the group index's reciprocal is exact up to there)
     if (!transposed && d.group_size % fwd_kb(d.bits) != 0) return false;
-    if ((transposed ? d.N : d.K) <= 16384) return true;    // eight ways split, such a range always fits the shared memory
+    const int T = transposed ? d.N : d.K;
+    if (T <= ST_LONG) return true;                          // eight ways split, such a range always fits the shared memory
+    // More than 8 tokens on a longer one, backward: 16 scaled copies of it are staged, in as many passes as they need, and the tensor-core kernel
+    // is the faster one where it takes the shape (N = 128256: 206 against 302 us).
+    if (transposed && M > 8 && umma_supported(d, M)) return false;
     StreamParams p{};
     p.M = M; p.K = d.K; p.N = d.N; p.g = d.group_size; p.r = d.r; p.C = transposed ? d.K : d.N;
     p.fused = d.r > 0 && d.r <= 16 ? 1 : 0;
@@ -961,7 +1030,7 @@ int launch_stream_gemm(const qlora_desc& d, int M, bool transposed, const void* 
         case 4: { QLORA_ST(4, NT); }    \
         case 8: { QLORA_ST(8, NT); }    \
     }
-    if (M <= 8) { QLORA_ST_BITS(1) } else { QLORA_ST_BITS(2) }
+    if (plan.nt == 1) { QLORA_ST_BITS(1) } else { QLORA_ST_BITS(2) }
 #undef QLORA_ST_BITS
 #undef QLORA_ST
     return QLORA_ERR_UNSUPPORTED;

@@ -157,3 +157,18 @@ def test_weights_repacked_in_stream_right_before_the_call(M):
         assert rel_err(to_f64(dXg[rows_t]), ref["dX"]) <= REL_TOL, (M, step)
     # the two code matrices give different results, so a stale read would have shown
     assert rel_err(to_f64(outs[0][0][rows_t]), refs[1]["Y"]) > REL_TOL
+
+
+@pytest.mark.parametrize("M,r", [(16, 8), (13, 24), (8, 16), (3, 0)])
+@pytest.mark.parametrize("bits,g,K,N", [(2, 64, 131136, 40), (3, 32, 131136, 40), (4, 64, 131136, 40), (8, 32, 131136, 40),
+                                        (2, 64, 64, 131080), (3, 32, 96, 131080), (4, 32, 96, 131080), (8, 64, 64, 131080)])
+def test_contractions_longer_than_the_shared_memory_holds(M, r, bits, g, K, N):
+    """131136 input or 131080 output features: the activations of a CTA's range are staged in several passes (from 8 tokens on; with
+    fewer, in one or several), the last of them shorter; sums of H / G and of the zero-points run over all passes."""
+    layer = qi.random_codes_layer(K=K, N=N, bits=bits, group_size=g, r=r, alpha=2.0 * max(r, 1), M=M, seed=M + bits + r)
+    errs, out, gl = check_layer(layer)
+    if r:
+        assert errs["H"] < 1e-4 and errs["G"] < 1e-4             # fp32 sums of exact products
+    again = gl.run()
+    for key in ("Y", "dX"):
+        assert torch.equal(out[key].view(torch.int16), again[key].view(torch.int16)), key
