@@ -6,6 +6,8 @@
 #include "launch.h"
 #include "lora_down.cuh"
 
+#include <type_traits>
+
 namespace qlora {
 
 // ------------------------------------------------------------------------------------------------------------
@@ -505,14 +507,18 @@ lora_grad_partial_kernel(int M, int r, int rows_per_slice, GradSide side0, GradS
 // Adds the slices' partial sums in slice order.  Two forms; of the blocks the first are dB's, the others dA's.
 //   reduce4: a thread takes four ranks of one column, neighbouring threads the next ranks of dB [N, r] (stored as it lies in scratch), the
 //   next columns of dA [r, K] (its four stores are contiguous across the warp; its loads are not).
-//   reduce: one element per thread as it lies in scratch, dA stored through shared memory, a block's columns of one rank together.
+//   reduce: one element per thread as it lies in scratch, or four where there are plenty (2^18), dA stored through shared memory, a
+//   block's columns of one rank together.
 // The scattered loads are few at rank 8, where two threads share a sector, and at rank 16 while there are few slices; the line lies there.
-// Gradient call, reduce4 / reduce: 4096 x 4096, 2048 tokens, rank 8 12.65 / 12.97 us, rank 16 14.0 / 14.3, rank 32 19.0 / 16.7;
-// 1024 x 1024, 1024 tokens (16 slices), rank 16 8.5 / 6.2.
+// Gradient call, reduce4 / reduce by one / by four: 4096 x 4096, 2048 tokens, rank 8 12.65 / 12.97 / 13.7 us, rank 16 14.0 / 14.3 / 13.9,
+// rank 32 19.0 / 16.7 / 17.2, rank 64 38.9 / 36.3 / 36.0; 4096 x 11008, 512 tokens, rank 64 23.3 / 24.8 / 22.8; 1024 x 1024, 1024 tokens
+// (16 slices), rank 16 8.5 / 6.2 / 7.8.
 constexpr int LR_THREADS = 256, LR4_MAX_SLICES = 9;
 
 __device__ __forceinline__ float4 lg_add(float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
 __device__ __forceinline__ float lg_add(float a, float b) { return a + b; }
+__device__ __forceinline__ float4 lg_scaled(float4 a, float s) { return make_float4(a.x * s, a.y * s, a.z * s, a.w * s); }
+__device__ __forceinline__ float lg_scaled(float a, float s) { return a * s; }
 
 // The sum over the slices, eight independent loads in flight.
 template <typename V>
@@ -548,8 +554,7 @@ __global__ void __launch_bounds__(THREADS) lora_grad_reduce4_kernel(int r, int s
     pdl_wait();
     if (e >= sd.C * r4) return;
     const size_t C = (size_t)sd.C;
-    float4 v = lg_slice_sum(reinterpret_cast<const float4*>(sd.partial + (size_t)c * r + j), C * r / 4, slices);
-    v.x *= sd.scale; v.y *= sd.scale; v.z *= sd.scale; v.w *= sd.scale;
+    float4 v = lg_scaled(lg_slice_sum(reinterpret_cast<const float4*>(sd.partial + (size_t)c * r + j), C * r / 4, slices), sd.scale);
     if (is_dB) {
         float4* dst = reinterpret_cast<float4*>(sd.Out + (size_t)c * r + j);
         if (accumulate) v = lg_add(*dst, v);
@@ -561,27 +566,36 @@ __global__ void __launch_bounds__(THREADS) lora_grad_reduce4_kernel(int r, int s
     }
 }
 
-__global__ void __launch_bounds__(LR_THREADS) lora_grad_reduce_kernel(int r, int slices, int accumulate, int blocks_dB, GradSide dB_side, GradSide dA_side) {
-    __shared__ float tile[LR_THREADS];                         // dA: [column of the block][rank]
+template <int W>   // ranks per thread: 1 or 4
+__global__ void __launch_bounds__(LR_THREADS / W) lora_grad_reduce_kernel(int r, int slices, int accumulate, int blocks_dB, GradSide dB_side, GradSide dA_side) {
+    using V = std::conditional_t<W == 4, float4, float>;
+    __shared__ __align__(16) float tile[LR_THREADS];           // dA: [column of the block][rank]
     pdl_launch_dependents();
     const bool is_dB = (int)blockIdx.x < blocks_dB;
     const GradSide& sd = is_dB ? dB_side : dA_side;
     const int cols = LR_THREADS / r, tid = threadIdx.x;        // columns of a block (threads beyond cols * r have no part)
     const int c0 = ((int)blockIdx.x - (is_dB ? 0 : blocks_dB)) * cols, n = min(cols, sd.C - c0) * r;
-    const size_t e = (size_t)c0 * r + tid;
+    const size_t e = (size_t)c0 * r + W * tid;
     pdl_wait();
-    if (tid < n) {
-        const float v = lg_slice_sum((const float*)sd.partial + e, (size_t)sd.C * r, slices) * sd.scale;
-        if (is_dB) sd.Out[e] = accumulate ? sd.Out[e] + v : v;
-        else tile[tid] = v;
+    if (W * tid < n) {
+        V v = lg_scaled(lg_slice_sum(reinterpret_cast<const V*>(sd.partial + e), (size_t)sd.C * r / W, slices), sd.scale);
+        if (is_dB) {
+            V* dst = reinterpret_cast<V*>(sd.Out + e);
+            *dst = accumulate ? lg_add(*dst, v) : v;
+        } else {
+            *reinterpret_cast<V*>(tile + W * tid) = v;
+        }
     }
     if (is_dB) return;
     __syncthreads();
-    const int j = tid / cols, cl = tid - j * cols;
-    if (j < r && cl * r < n) {
-        float* dst = sd.Out + (size_t)j * sd.C + c0 + cl;
-        const float v = tile[cl * r + j];
-        *dst = accumulate ? *dst + v : v;
+#pragma unroll
+    for (int i = 0; i < W; ++i) {
+        const int t = tid + i * (LR_THREADS / W), j = t / cols, cl = t - j * cols;
+        if (j < r && cl * r < n) {
+            float* dst = sd.Out + (size_t)j * sd.C + c0 + cl;
+            const float v = tile[cl * r + j];
+            *dst = accumulate ? *dst + v : v;
+        }
     }
 }
 
@@ -683,13 +697,12 @@ int launch_lora_grads(int M, int K, int N, int r, float s, const void* X, const 
     if (err != cudaSuccess) return QLORA_ERR_CUDA;
     const GradSide& rB = want_dB ? sB : none;
     const GradSide& rA = want_dA ? sA : none;
-    const int threads = r == 8 ? 64 : LR_THREADS, r4 = r / 4, red_cols = LR_THREADS / r;
-    const bool four = r == 8 || (r == 16 && plan.slices <= LR4_MAX_SLICES);
-    auto blocks = [&](int C) { return four ? (int)(((size_t)C * r4 + threads - 1) / threads) : (C + red_cols - 1) / red_cols; };
+    const bool four = r == 8 || (r == 16 && plan.slices <= LR4_MAX_SLICES), wide = (size_t)(rB.C + rA.C) * r > (1u << 18);
+    const int threads = four ? (r == 8 ? 64 : LR_THREADS) : (wide ? LR_THREADS / 4 : LR_THREADS), per = LR_THREADS / r;
+    auto blocks = [&](int C) { return four ? (int)(((size_t)C * (r / 4) + threads - 1) / threads) : (C + per - 1) / per; };
     const dim3 red_grid((unsigned)(blocks(rB.C) + blocks(rA.C))), red_block((unsigned)threads);
-    if (four && r == 8) err = launch_pdl(lora_grad_reduce4_kernel<64>, red_grid, red_block, 0, st, 1, r, plan.slices, accumulate, blocks(rB.C), rB, rA);
-    else if (four)      err = launch_pdl(lora_grad_reduce4_kernel<LR_THREADS>, red_grid, red_block, 0, st, 1, r, plan.slices, accumulate, blocks(rB.C), rB, rA);
-    else                err = launch_pdl(lora_grad_reduce_kernel, red_grid, red_block, 0, st, 1, r, plan.slices, accumulate, blocks(rB.C), rB, rA);
+    auto reduce = four ? (r == 8 ? lora_grad_reduce4_kernel<64> : lora_grad_reduce4_kernel<LR_THREADS>) : (wide ? lora_grad_reduce_kernel<4> : lora_grad_reduce_kernel<1>);
+    err = launch_pdl(reduce, red_grid, red_block, 0, st, 1, r, plan.slices, accumulate, blocks(rB.C), rB, rA);
     return err == cudaSuccess ? QLORA_OK : QLORA_ERR_CUDA;
 }
 

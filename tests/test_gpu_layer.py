@@ -327,7 +327,7 @@ def test_seeded_sweep_across_the_dispatch_boundaries(seed):
 
 
 @pytest.mark.parametrize("r", [8, 16, 24, 40, 64])
-@pytest.mark.parametrize("M,K,N", [(300, 96, 40), (1030, 256, 72), (2100, 128, 2112), (600, 4128, 8)])
+@pytest.mark.parametrize("M,K,N", [(300, 96, 40), (1030, 256, 72), (2100, 128, 2112), (600, 4128, 8), (300, 8224, 40)])
 def test_gradients_from_many_row_slices(M, K, N, r):
     """Above 256 tokens partial sums per row slice are added by a second launch: one slice to 34 of them, widths that leave the last block
     partly filled, ranks that do not divide a block's threads; overwritten, accumulated (exact additions), and dA alone."""
