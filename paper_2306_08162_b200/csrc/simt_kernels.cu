@@ -379,14 +379,16 @@ lora_grad_partial_kernel(int M, int r, int rows_per_slice, GradSide side0, GradS
     const int m_begin = slice * rows_per_slice;
     const int stride = rows_per_slice + 8;                     // in bf16: (stride / 2) % 32 == 4 -> conflict-free fragment loads
     constexpr int RP = RT * 16;
-    // stage P^T (bf16) of this slice: rows beyond M and ranks beyond r are zero
-    for (int e = threadIdx.x; e < rows_per_slice * RP; e += LG_WARPS * 32) {
-        const int ml = e / RP, j = e % RP;
-        const int m = m_begin + ml;
-        const float v = (m < M && j < r) ? __ldg(sd.P + (size_t)m * r + j) : 0.f;
-        Pt[j * stride + ml] = __float2bfloat16_rn(v);
-    }
-    __syncthreads();
+    auto stage_p = [&]() {   // P^T (bf16) of this slice: rows beyond M and ranks beyond r are zero
+        for (int e = threadIdx.x; e < rows_per_slice * RP; e += LG_WARPS * 32) {
+            const int ml = e / RP, j = e % RP;
+            const int m = m_begin + ml;
+            const float v = (m < M && j < r) ? __ldg(sd.P + (size_t)m * r + j) : 0.f;
+            Pt[j * stride + ml] = __float2bfloat16_rn(v);
+        }
+        __syncthreads();
+    };
+    if constexpr (RT > 1) stage_p();
 
     const int c0 = cb + warp * 32 + q * 8;                     // this lane loads columns c0 .. c0 + 7
     const bool live = c0 < C;                                  // C is a multiple of 8
@@ -418,6 +420,9 @@ lora_grad_partial_kernel(int M, int r, int rows_per_slice, GradSide side0, GradS
         }
     };
     load_round(m_begin);
+    // One rank tile has the registers to keep the first round under way while P is staged: 64 tokens, 4096 x 4096, 3.28 -> 2.90 us (3.25
+    // before the loads were made volatile); 1024 tokens 8.8 -> 8.5.
+    if constexpr (RT == 1) stage_p();
     for (int mm = m_begin; mm < m_stop; mm += 16 * LG_UNROLL) {
         uint4 x0[LG_UNROLL], x1[LG_UNROLL];
 #pragma unroll
