@@ -361,9 +361,11 @@ __device__ __forceinline__ void lg_load(uint4& v, const void* p) {
 //   and writes (or adds to) dA / dB.
 // MASKED: side 1 (dA) has a dropout mask on its activations; the mask bytes travel with the loads of their round and are applied when
 // the round's turn comes (applied as they were loaded they made every round wait for memory: 29 against 13.7 us at 1800 tokens).
-// (Two blocks per SM for ranks up to 32; with 104 registers, up to 16, they leave room for a block of the reduction launch, which starts early.)
+// (Two blocks per SM for ranks up to 32; with 104 registers, up to 16, they leave room for a block of the reduction launch, which starts early.
+// The masked form with two rank tiles spills 48 bytes for it, and gains: 1800 tokens, rank 32, 21.7 us against 27.7 with 140 registers and one
+// block; in clusters, where there are few blocks anyway, it has the 140: 200 tokens 8.8 -> 7.4.)
 template <int RT, int CL, bool MASKED>   // rank tiles of 16; cluster width (0 = two-launch form)
-__global__ void __launch_bounds__(LG_WARPS * 32) __maxnreg__(RT == 1 && !MASKED ? 104 : (RT <= 2 ? 128 : 168))
+__global__ void __launch_bounds__(LG_WARPS * 32) __maxnreg__(RT == 1 && !MASKED ? 104 : (RT == 1 || (RT == 2 && !(MASKED && CL > 0)) ? 128 : 184))
 lora_grad_partial_kernel(int M, int r, int rows_per_slice, GradSide side0, GradSide side1, int accumulate) {
     extern __shared__ __align__(16) uint8_t lg_smem[];
     pdl_launch_dependents();
