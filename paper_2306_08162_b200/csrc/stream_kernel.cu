@@ -851,7 +851,7 @@ __global__ void __launch_bounds__(ST_THREADS, PER_SM) stream_bwd_kernel(const St
 
 // Three CTAs per SM (80 registers) exist where the kernels spill 24 bytes at most: up to 8 tokens, 4 bits, and 2 bits backward.
 // (Of the builds with 128 registers, those for 9 .. 16 tokens spill up to 80 bytes at 3 bits and 72 at 8 bits, the others none; the multi-pass
-// ones up to 770, all of it around the staging.)
+// ones up to 650, all of it around the staging.)
 constexpr bool st_has_three(int bits, int nt, bool transposed) { return nt == 1 && (bits == 4 || (bits == 2 && transposed)); }
 
 int fwd_kb(int bits) { return bits == 2 ? 64 : 32; }
