@@ -335,8 +335,9 @@ static cudaError_t launch_gather(int rows, int cols, const void* in, const int32
     // from 64 rows on the whole-row blocks cover enough SMs (below, an element per thread is the faster); two blocks fit an SM
     if (rows >= 64 && (size_t)cols * sizeof(T) % 16 == 0 && smem <= 100 * 1024) {
         const dim3 grid((unsigned)((rows + GC_ROWS - 1) / GC_ROWS));
-        // narrow rows: fewer threads, of which more have a piece (8192 rows of 256 floats: 9.5 us by elements, 11.4 with 512 threads, 5.4 now)
-        if ((size_t)cols * sizeof(T) <= GC_NARROW)
+        // narrow rows, more of them than the SMs hold at 512 threads a block: fewer threads, of which more have a piece (8192 rows of 256 floats:
+        // 9.5 us by elements, 11.4 with 512 threads, 5.6 with 128; 200 rows of 512 floats 1.9 with 512, 2.1 with 128)
+        if ((size_t)cols * sizeof(T) <= GC_NARROW && rows > GC_ROWS * 4 * sm_count())
             return launch_pdl(gather_rows_kernel<T, GC_NARROW_THREADS>, grid, dim3(GC_NARROW_THREADS), smem, st, 1, rows, cols, (const T*)in, perm, (T*)out);
         static SmemLimit limit;
         if (!limit.raise(gather_rows_kernel<T, GC_THREADS>, 100 * 1024)) return cudaErrorUnknown;

@@ -501,7 +501,7 @@ def test_lora_dropout_ragged_rows(M, K, N, r):
 
 
 @pytest.mark.parametrize("rows,cols,dtype", [(1, 8, torch.bfloat16), (63, 11008, torch.bfloat16), (64, 11008, torch.bfloat16), (333, 11008, torch.bfloat16),
-                                             (65, 1004, torch.bfloat16), (65, 8, torch.bfloat16), (333, 1024, torch.bfloat16), (200, 516, torch.float32), (200, 4096, torch.float32), (64, 16000, torch.float32), (70, 6, torch.float32)])
+                                             (65, 1004, torch.bfloat16), (65, 8, torch.bfloat16), (1301, 8, torch.bfloat16), (1300, 1024, torch.bfloat16), (2001, 516, torch.float32), (1301, 512, torch.float32), (200, 4096, torch.float32), (64, 16000, torch.float32), (70, 6, torch.float32)])
 def test_gather_columns_both_forms(rows, cols, dtype):
     """Whole rows through shared memory (from 64 rows, rows of whole 16-byte pieces that fit) and element by element otherwise."""
     import paper_2306_08162_b200 as ql
