@@ -135,6 +135,15 @@ __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatil
     if (ok) (void)mbar_try_wait(bar, parity);
     return ok != 0;
 }
+// One lane of a converged warp, the same one every time.  The roles that issue TMA copies and MMAs run as whole warps and elect a lane for
+// the instructions alone, so that ring positions, addresses and descriptors are warp-uniform values, which these instructions want: run by
+// lane 0 of a diverged warp they cost 75 to 150 cycles each (a trace of one CTA had the dequant warps 3000 cycles ahead of the MMAs).
+// INT4, rank 0, 64 tokens: 4096 -> 11008 29.3 -> 25.9, 4096 x 4096 13.3 -> 12.2 us; nothing from 257 tokens on, where the products are what takes the time.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t ok;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(ok) ::"memory");
+    return ok != 0;
+}
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y) {
     asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
                  ::"r"(dst), "l"(map), "r"(bar), "r"(x), "r"(y) : "memory");
@@ -358,95 +367,89 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
         if (threadIdx.x == 0) atomicAdd(&p.sync[0], 1u);
     } else if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer: activation tiles
-        if (lane == 0) {
-            pdl_wait();
-            Ring ring;
-            for (int tile = first_tile; tile < p.n_tiles; tile += tile_stride) {
-                const int m0 = (tile % p.n_tok_tiles) * p.BT;
-                for (int step = 0; step < p.steps; ++step) {
-                    if (!mbar_wait(bar_empty + 8 * ring.slot, ring.phase ^ 1u, abort_flag)) goto done;
-                    const uint32_t bar = bar_full_x + 8 * ring.slot;
+        pdl_wait();
+        Ring ring;
+        for (int tile = first_tile; tile < p.n_tiles; tile += tile_stride) {
+            const int m0 = (tile % p.n_tok_tiles) * p.BT;
+            for (int step = 0; step < p.steps; ++step) {
+                if (!warp_wait(bar_empty + 8 * ring.slot, ring.phase ^ 1u, abort_flag, lane)) goto done;
+                const uint32_t bar = bar_full_x + 8 * ring.slot, dst = smem0 + p.off_x + ring.slot * p.x_stage_bytes;
+                const int c0 = (step0 + step) * kStepC;
+                if (elect_one()) {
                     mbar_expect_tx(bar, p.x_stage_bytes);
-                    tma_load_2d(smem0 + p.off_x + ring.slot * p.x_stage_bytes, &tm_act, bar, (step0 + step) * kStepC, m0);
-                    ring.advance(S);
+                    tma_load_2d(dst, &tm_act, bar, c0, m0);
                 }
+                ring.advance(S);
             }
         }
     } else if (warp == 2) {
         // ------------------------------------------------------------------ TMA producer: packed codes, scales, zeros
-        if (lane == 0) {
-            Ring ring;
-            const uint32_t tx_bytes = p.words_bytes + 2 * p.scale_bytes;
-            for (int tile = first_tile; tile < p.n_tiles; tile += tile_stride) {
-                const int w0 = (tile / p.n_tok_tiles) * kWRows;
-                // forward: weight rows n = w0.., contraction k = c0..;  backward: weight rows k = w0.., contraction n = c0..
-                const int g_row = TRANSPOSED ? w0 / p.g : 0;
-                for (int step = 0; step < p.steps; ++step) {
-                    if (!mbar_wait(bar_empty_p + 8 * ring.slot, ring.phase ^ 1u, abort_flag)) goto done;
-                    const uint32_t dst = smem0 + p.off_p + ring.slot * p.packed_slot_bytes;
-                    const uint32_t bar = bar_full_p + 8 * ring.slot;
+        Ring ring;
+        const uint32_t tx_bytes = p.words_bytes + 2 * p.scale_bytes;
+        for (int tile = first_tile; tile < p.n_tiles; tile += tile_stride) {
+            // forward: weight rows n = w0.., contraction k = c0..;  backward: weight rows k = w0.., contraction n = c0..
+            const int w0 = (tile / p.n_tok_tiles) * kWRows;
+            for (int step = 0; step < p.steps; ++step) {
+                if (!warp_wait(bar_empty_p + 8 * ring.slot, ring.phase ^ 1u, abort_flag, lane)) goto done;
+                const uint32_t dst = smem0 + p.off_p + ring.slot * p.packed_slot_bytes, bar = bar_full_p + 8 * ring.slot;
+                const int c0 = (step0 + step) * kStepC, x = TRANSPOSED ? c0 : w0, k = TRANSPOSED ? w0 : c0, gr = k / p.g;
+                if (elect_one()) {
                     mbar_expect_tx(bar, tx_bytes);
-                    const int c0 = (step0 + step) * kStepC;
-                    if (!TRANSPOSED) {
-                        const int gr = c0 / p.g;
-                        tma_load_2d(dst, &tm_q, bar, w0, c0 * BITS / 32);
-                        tma_load_2d(dst + p.words_bytes, &tm_scales, bar, w0, gr);
-                        tma_load_2d(dst + p.words_bytes + p.scale_bytes, &tm_zeros, bar, w0, gr);
-                    } else {
-                        tma_load_2d(dst, &tm_q, bar, c0, w0 * BITS / 32);
-                        tma_load_2d(dst + p.words_bytes, &tm_scales, bar, c0, g_row);
-                        tma_load_2d(dst + p.words_bytes + p.scale_bytes, &tm_zeros, bar, c0, g_row);
-                    }
-                    ring.advance(P);
+                    tma_load_2d(dst, &tm_q, bar, x, k * BITS / 32);
+                    tma_load_2d(dst + p.words_bytes, &tm_scales, bar, x, gr);
+                    tma_load_2d(dst + p.words_bytes + p.scale_bytes, &tm_zeros, bar, x, gr);
                 }
+                ring.advance(P);
             }
         }
     } else if (warp == 1) {
-        // ------------------------------------------------------------------ MMA issuer (one thread)
-        if (lane == 0) {
-            const uint32_t idesc = instr_desc((uint32_t)p.BT, TRANSPOSED ? 1u : 0u, 0u);
-            const uint32_t idesc_lora = instr_desc((uint32_t)p.BT, 0u, 0u);
-            // Descriptors of slot 0; the start-address field (16-byte units) is advanced per slot and per 16-wide MMA step.
-            // activation tile: contraction-contiguous rows of 128 B, 128-byte swizzle, 8-row groups 1024 B apart.
-            // weight tile: forward = the same layout (rows n); backward = rows are the contraction (n) with 64 k contiguous:
-            //   MN-major, 64-element atoms 8192 B apart (LBO), 8-row contraction groups 1024 B apart (SBO).
-            const uint64_t b_desc0 = smem_desc(smem0 + p.off_x, 16, 1024, 2);
-            const uint64_t a_desc0 = TRANSPOSED ? smem_desc(smem0 + p.off_w, 8192, 1024, 2) : smem_desc(smem0 + p.off_w, 16, 1024, 2);
-            constexpr uint32_t a_k16 = TRANSPOSED ? (2048u >> 4) : (32u >> 4);
-            const uint32_t x_step = p.x_stage_bytes >> 4;
-            Ring ring;
-            uint32_t tile_it = 0;
-            for (int tile = first_tile; tile < p.n_tiles; tile += tile_stride, ++tile_it) {
-                const uint32_t buf = tile_it & 1u;
-                const uint32_t d_tmem = tmem_base + buf * kAccStride;
-                if (!mbar_wait(bar_acc_empty + 8 * buf, ((tile_it >> 1) & 1u) ^ 1u, abort_flag)) goto done;
+        // ------------------------------------------------------------------ MMA issuer (one elected thread)
+        const uint32_t idesc = instr_desc((uint32_t)p.BT, TRANSPOSED ? 1u : 0u, 0u);
+        const uint32_t idesc_lora = instr_desc((uint32_t)p.BT, 0u, 0u);
+        // Descriptors of slot 0; the start-address field (16-byte units) is advanced per slot and per 16-wide MMA step.
+        // activation tile: contraction-contiguous rows of 128 B, 128-byte swizzle, 8-row groups 1024 B apart.
+        // weight tile: forward = the same layout (rows n); backward = rows are the contraction (n) with 64 k contiguous:
+        //   MN-major, 64-element atoms 8192 B apart (LBO), 8-row contraction groups 1024 B apart (SBO).
+        const uint64_t b_desc0 = smem_desc(smem0 + p.off_x, 16, 1024, 2);
+        const uint64_t a_desc0 = TRANSPOSED ? smem_desc(smem0 + p.off_w, 8192, 1024, 2) : smem_desc(smem0 + p.off_w, 16, 1024, 2);
+        constexpr uint32_t a_k16 = TRANSPOSED ? (2048u >> 4) : (32u >> 4);
+        const uint32_t x_step = p.x_stage_bytes >> 4;
+        Ring ring;
+        uint32_t tile_it = 0;
+        for (int tile = first_tile; tile < p.n_tiles; tile += tile_stride, ++tile_it) {
+            const uint32_t buf = tile_it & 1u;
+            const uint32_t d_tmem = tmem_base + buf * kAccStride;
+            if (!warp_wait(bar_acc_empty + 8 * buf, ((tile_it >> 1) & 1u) ^ 1u, abort_flag, lane)) goto done;
+            tc_fence_after();
+            uint32_t acc = 0;
+            for (int step = 0; step < p.steps; ++step) {
+                if (!warp_wait(bar_full_x + 8 * ring.slot, ring.phase, abort_flag, lane)) goto done;
                 tc_fence_after();
-                uint32_t acc = 0;
-                for (int step = 0; step < p.steps; ++step) {
-                    if (!mbar_wait(bar_full_x + 8 * ring.slot, ring.phase, abort_flag)) goto done;
-                    tc_fence_after();
-                    const uint64_t b_desc = b_desc0 + ring.slot * x_step;
-                    const uint64_t a_desc = a_desc0 + ring.slot * (uint32_t)(kWStageBytes >> 4);
+                const uint64_t b_desc = b_desc0 + ring.slot * x_step;
+                const uint64_t a_desc = a_desc0 + ring.slot * (uint32_t)(kWStageBytes >> 4);
+                const uint32_t bar = bar_empty + 8 * ring.slot;
+                if (elect_one()) {
 #pragma unroll
-                    for (int k16 = 0; k16 < kStepC / 16; ++k16) {
-                        tc_mma(d_tmem, a_desc + k16 * a_k16, b_desc + k16 * 2, idesc, acc);
-                        acc = 1;
-                    }
-                    tc_commit(bar_empty + 8 * ring.slot);
-                    ring.advance(S);
+                    for (int k16 = 0; k16 < kStepC / 16; ++k16)
+                        tc_mma(d_tmem, a_desc + k16 * a_k16, b_desc + k16 * 2, idesc, acc | (uint32_t)(k16 > 0));
+                    tc_commit(bar);
                 }
-                if (p.r > 0 && rank == 0) {   // the LoRA update goes into one rank's part only
-                    if (!mbar_wait(bar_lora_full, tile_it & 1u, abort_flag)) goto done;
-                    tc_fence_after();
+                acc = 1;
+                ring.advance(S);
+            }
+            if (p.r > 0 && rank == 0) {   // the LoRA update goes into one rank's part only
+                if (!warp_wait(bar_lora_full, tile_it & 1u, abort_flag, lane)) goto done;
+                tc_fence_after();
+                if (elect_one())
                     for (int jb = 0; jb < p.r_pad / 16; ++jb) {
                         // un-swizzled operands: 8-row x 16-byte core matrices 128 B apart (SBO), contraction halves LBO apart
                         const uint64_t a_desc = smem_desc(smem0 + p.off_lora_a + jb * 2 * (kWRows * 16), kWRows * 16, 128, 0);
                         const uint64_t b_desc = smem_desc(smem0 + p.off_lora_p + jb * 2 * (p.BT * 16), p.BT * 16, 128, 0);
                         tc_mma(d_tmem, a_desc, b_desc, idesc_lora, 1u);
                     }
-                }
-                tc_commit(bar_acc_full + 8 * buf);
+                __syncwarp();
             }
+            if (elect_one()) tc_commit(bar_acc_full + 8 * buf);
         }
     } else if (warp >= kEpiWarp0 && warp < kDequantWarp0) {
         // ------------------------------------------------------------------ epilogue (+ LoRA operand staging)
