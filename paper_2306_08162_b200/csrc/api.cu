@@ -187,13 +187,13 @@ static int fwd_common(const qlora_desc* desc, int M, const void* X, const uint8_
         return launch_stream_gemm(d, M, false, X, Q, scales, zeros, A, B, H, !fused, Y, st);
     }
     // the tensor-core path computes H itself when given A (beside its tiles where SM pairs are idle, else ahead of them)
-    if (umma_supported(d, M) && mask == nullptr) return launch_umma_gemm(d, M, false, X, Q, scales, zeros, B, H, Y, st, A, sync, static_cast<char*>(workspace) + w.split_off,
-                                workspace_bytes - w.split_off);
+    const DownExtra dropout{mask, keep_scale, 0};
+    if (umma_supported(d, M)) return launch_umma_gemm(d, M, false, X, Q, scales, zeros, B, H, Y, st, d.r > 0 ? A : nullptr, sync, static_cast<char*>(workspace) + w.split_off,
+                                workspace_bytes - w.split_off, nullptr, mask != nullptr ? &dropout : nullptr);
     if (d.r > 0) {
         rc = launch_lora_down(M, d.K, d.r, true, X, A, H, st, mask, keep_scale);
         if (rc != QLORA_OK) return rc;
     }
-    if (umma_supported(d, M)) return launch_umma_gemm(d, M, false, X, Q, scales, zeros, B, H, Y, st);
     return launch_simt_gemm(d, M, false, X, Q, scales, zeros, B, H, Y, st);
 }
 
@@ -217,13 +217,17 @@ static int bwd_input_common(const qlora_desc* desc, int M, const void* dY, const
     cudaStream_t st = (cudaStream_t)cuda_stream;
     float* G = G_out ? G_out : reinterpret_cast<float*>(static_cast<char*>(workspace) + w.p0_off);
     if (mask != nullptr && d.r > 0) {
-        rc = launch_lora_down(M, d.N, d.r, false, dY, B, G, st);
-        if (rc != QLORA_OK) return rc;
         qlora_desc d0 = d;
         d0.r = 0;
-        if (stream_supported(d0, M, true)) rc = launch_stream_gemm(d0, M, true, dY, Q, scales, zeros, B, A, G, true, dX, st);
-        else if (umma_supported(d0, M)) rc = launch_umma_gemm(d0, M, true, dY, Q, scales, zeros, A, G, dX, st);
-        else rc = launch_simt_gemm(d0, M, true, dY, Q, scales, zeros, A, G, dX, st);
+        if (!stream_supported(d0, M, true) && umma_supported(d0, M)) {       // G beside the tiles where SM pairs are idle, else ahead of them
+            const DownExtra g_only{nullptr, 1.0f, d.r};
+            rc = launch_umma_gemm(d0, M, true, dY, Q, scales, zeros, A, G, dX, st, B, nullptr, nullptr, 0, nullptr, &g_only);
+        } else {
+            rc = launch_lora_down(M, d.N, d.r, false, dY, B, G, st);
+            if (rc != QLORA_OK) return rc;
+            rc = stream_supported(d0, M, true) ? launch_stream_gemm(d0, M, true, dY, Q, scales, zeros, B, A, G, true, dX, st)
+                                               : launch_simt_gemm(d0, M, true, dY, Q, scales, zeros, A, G, dX, st);
+        }
         if (rc != QLORA_OK) return rc;
         return launch_lora_masked_update(M, d.K, d.r, keep_scale * d.alpha / (float)d.r, G, A, mask, dX, st);
     }

@@ -30,9 +30,11 @@ int launch_simt_gemm(const qlora_desc& d, int M, bool transposed, const void* In
 // mask (optional, only with l_is_A): uint8 [M, T] dropout mask on In, non-zero = keep; the result is multiplied by out_scale.
 int launch_lora_down(int M, int T, int r, bool l_is_A, const void* In, const void* L, float* P, cudaStream_t st,
                      const uint8_t* mask = nullptr, float out_scale = 1.0f);
-// umma_kernel.cu -- the same product for many rows and r <= 16: activations streamed through shared memory by bulk
-// copies (launch_lora_down routes there above 256 rows; the CTA-pair kernel runs the same code on idle SM pairs).
-int launch_lora_down_stream(int M, int T, int r, bool l_is_A, const void* In, const void* L, float* P, cudaStream_t st);
+// umma_kernel.cu -- the same product for many rows: activations streamed through shared memory by bulk copies (launch_lora_down routes
+// there above 256 rows for r <= 16, and where lora_down_streams_wide says so; the CTA-pair kernel runs the same code on idle SM pairs).
+int launch_lora_down_stream(int M, int T, int r, bool l_is_A, const void* In, const void* L, float* P, cudaStream_t st, const uint8_t* mask = nullptr,
+                            float out_scale = 1.0f);
+bool lora_down_streams_wide(int M, int r, bool masked);
 // dB = s dY^T H [N, r] and dA = s G^T X [r, K] in one pair of launches (partial sums per row slice, then a fixed-order
 // reduction); scratch needs lora_grad_scratch_bytes().
 size_t lora_grad_scratch_bytes(int M, int K, int N, int r);
@@ -61,6 +63,14 @@ struct DbFuse {
     size_t part_bytes;
     bool done;
 };
+// Forms of the product that launch_umma_gemm computes on the way (Ldown != NULL) beyond the plain one: LoRA dropout's mask on In with a
+// scale of the result (forward), or -- with d.r == 0, only_r > 0 -- a product of that many ranks that the layer itself does not use
+// (backward under dropout: G, whose masked term a later pass adds).
+struct DownExtra {
+    const uint8_t* mask;
+    float out_scale;
+    int only_r;
+};
 // Workspace bytes with which any backward call of this shape can take dB on (0: none can).
 size_t umma_db_part_bytes(const qlora_desc& d, int M);
 // The number of producer pairs on which such a call, given its whole workspace, forms dB on the current device; else 0.
@@ -68,7 +78,7 @@ int umma_db_on_producers(const qlora_desc& d, int M);
 int launch_umma_gemm(const qlora_desc& d, int M, bool transposed, const void* In, const int32_t* Q,
                      const void* scales, const void* zeros, const void* L, float* P, void* Out,
                      cudaStream_t st, const void* Ldown = nullptr, unsigned int* sync = nullptr, void* split_buf = nullptr,
-                     size_t split_bytes = 0, DbFuse* db = nullptr);
+                     size_t split_bytes = 0, DbFuse* db = nullptr, const DownExtra* extra = nullptr);
 // Bytes of workspace (`split_buf`) with which the CTA-pair kernel splits the tiles of a partly filled last wave along the
 // contraction (two SM pairs per tile, exchanging halves of the result); 0 when it would not.  Needs `sync` as well.
 size_t umma_split_scratch_bytes(const qlora_desc& d, int M);

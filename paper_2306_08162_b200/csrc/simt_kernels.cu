@@ -269,7 +269,7 @@ int launch_lora_down(int M, int T, int r, bool l_is_A, const void* In, const voi
     const bool plain = mask == nullptr && out_scale == 1.0f && r <= 16;
     // Many rows, low rank: the streaming kernel (also the form that runs inside the CTA-pair kernel, so H / G have the
     // same bits whichever call produced them).
-    if (plain && M > 256) return launch_lora_down_stream(M, T, r, l_is_A, In, L, P, st);
+    if ((plain && M > 256) || lora_down_streams_wide(M, r, mask != nullptr)) return launch_lora_down_stream(M, T, r, l_is_A, In, L, P, st, mask, out_scale);
     const unsigned blocks = (unsigned)((M + 15) / 16);
     const __nv_bfloat16* in = (const __nv_bfloat16*)In;
     const __nv_bfloat16* l = (const __nv_bfloat16*)L;

@@ -779,9 +779,10 @@ int launch_impl(const CUtensorMap& ta, const CUtensorMap& tq, const CUtensorMap&
 
 }  // namespace
 
-int launch_lora_down_stream(int M, int T, int r, bool l_is_A, const void* In, const void* L, float* P, cudaStream_t st) {
-    return launch_lora_down_stream_impl(M, T, r, l_is_A, In, L, P, st);
+int launch_lora_down_stream(int M, int T, int r, bool l_is_A, const void* In, const void* L, float* P, cudaStream_t st, const uint8_t* mask, float out_scale) {
+    return launch_lora_down_stream_impl(M, T, r, l_is_A, In, L, P, st, mask, out_scale);
 }
+bool lora_down_streams_wide(int M, int r, bool masked) { return lds_wide(M, r, masked); }
 
 static int keep_lora_low(const qlora_desc& d) { return d.r == 8 || d.group_size == 32 ? 1 : 0; }
 
@@ -831,7 +832,8 @@ size_t umma_db_part_bytes(const qlora_desc& d, int M) {
 // CTA-pair kernel: 512 tokens x 256 weight rows per pair of SMs (see prefer_pair_kernel for when it is used).
 static int launch_umma_pair(const qlora_desc& d, int M, bool transposed, const void* In, const int32_t* Q, const void* scales,
                             const void* zeros, const void* L, float* Pmat, void* Out, cudaStream_t st, const void* Ldown,
-                            unsigned int* sync, void* split_buf, size_t split_bytes, DbFuse* db, bool plan_only = false) {
+                            unsigned int* sync, void* split_buf, size_t split_bytes, DbFuse* db, bool plan_only = false,
+                            const DownExtra* extra = nullptr) {
     // plan_only: nothing is launched and no pointer is looked at; the return value is the number of producer pairs when a
     // backward call with every optional workspace area would form dB on them, else 0
     PairParams p{};
@@ -873,12 +875,21 @@ static int launch_umma_pair(const qlora_desc& d, int M, bool transposed, const v
     const int pairs = sm_count() / 2;
     p.n_prod = 0; p.T = T; p.sync = nullptr; p.wait_limit_us = kWaitLimitUs;
     p.In = (const __nv_bfloat16*)In; p.Ldown = (const __nv_bfloat16*)Ldown; p.Pout = Pmat;
-    p.lds_stages = (int)((p.off_bar - LDS_BAR_BYTES) / LDS_STAGE_BYTES);
+    p.r_down = extra != nullptr && extra->only_r > 0 ? extra->only_r : d.r;
+    p.mask = extra != nullptr ? extra->mask : nullptr;
+    p.out_scale = extra != nullptr ? extra->out_scale : 1.0f;
+    const int lds_stage = p.mask != nullptr ? LDS_MASKED_STAGE_BYTES : LDS_STAGE_BYTES;
+    p.lds_stages = (int)((p.off_bar - LDS_BAR_BYTES) / lds_stage);
     if (p.lds_stages > 6) p.lds_stages = 6;
+    const bool ring_fits = p.lds_stages * lds_stage >= LDS_MIN_STAGES * LDS_STAGE_BYTES;    // (the ring also holds the reduction)
+    // row blocks per producer CTA (ranks above 16, backward: at seven the producers, which gather B's words, came after the tiles: 2048 tokens,
+    // 4096 x 4096, rank 32, 57.8 us against 56.6 with a launch ahead)
+    const int max_blocks = p.r_down > 16 ? (transposed ? LDS_WIDE_BLOCKS - 1 : LDS_WIDE_BLOCKS) : LDS_MAXB;
+    const bool r_fits = (p.mask == nullptr && p.r_down <= 16) || lds_wide(M, p.r_down, p.mask != nullptr);   // (the forms that a launch of its own takes too)
     // P = In * Ldown still to be computed (Ldown given): on SM pairs the tiles leave idle when those can take all row
     // blocks (they are then done well before the tiles' contractions are), else by a launch ahead of this one.  Both sum
     // in the same order.  producers(last) = how many pairs would do it when the last wave has `last` items (0: none can).
-    const bool want_p = (Ldown != nullptr || plan_only) && d.r > 0;
+    const bool want_p = (Ldown != nullptr || plan_only) && p.r_down > 0;
     if (plan_only) { sync = reinterpret_cast<unsigned int*>(sizeof(unsigned int)); split_buf = sync; split_bytes = ~(size_t)0; }   // (never dereferenced)
     const int n_blocks = (M + 15) / 16;
     auto producers = [&](int last) {
@@ -886,8 +897,7 @@ static int launch_umma_pair(const qlora_desc& d, int M, bool transposed, const v
         const int idle = p.n_tiles < pairs ? pairs - p.n_tiles : (last ? pairs - last : 0);
         int n_prod = (n_blocks + 3) / 4;                     // four row blocks per producer CTA pair when there is room
         if (n_prod > idle) n_prod = idle;
-        const bool fits = want_p && sync != nullptr && d.r <= 16 && n_prod > 0 && n_prod * 2 * LDS_MAXB >= n_blocks &&
-                          p.lds_stages >= LDS_MIN_STAGES;
+        const bool fits = want_p && (sync != nullptr || d.r == 0) && r_fits && n_prod > 0 && n_prod * 2 * max_blocks >= n_blocks && ring_fits;
         return fits ? n_prod : 0;
     };
     // A partly filled last wave (more tiles than pairs, at most half a wave left over): each left-over tile goes to two
@@ -904,7 +914,7 @@ static int launch_umma_pair(const qlora_desc& d, int M, bool transposed, const v
     // dB on the producers' pass over dY (backward, ranks up to 16): every producer CTA leaves its part in the workspace
     // -- where the producers have a whole tile's time to spare: with a split last wave they are only half a tile ahead of
     // the others, and the extra work then lengthens the kernel (down_proj backward, r = 16: 159 against 140 us)
-    const bool db_fits = transposed && p.n_prod > 0 && p.nsplit == 1 &&
+    const bool db_fits = transposed && p.n_prod > 0 && p.nsplit == 1 && d.r > 0 && d.r <= 16 &&
                          p.n_prod * 2 * (d.r <= 8 ? LDS_MAXB : 3) >= n_blocks;   // (two rank tiles: three row blocks per producer CTA at most)
     if (plan_only) return db_fits ? p.n_prod : 0;
     p.with_db = 0;
@@ -921,10 +931,10 @@ static int launch_umma_pair(const qlora_desc& d, int M, bool transposed, const v
         return QLORA_ERR_CUDA;
 
     if (want_p && p.n_prod == 0) {
-        const int rc = launch_lora_down(M, T, d.r, !transposed, In, Ldown, Pmat, st);
+        const int rc = launch_lora_down(M, T, p.r_down, !transposed, In, Ldown, Pmat, st, p.mask, p.out_scale);
         if (rc != QLORA_OK) return rc;
     }
-    if (p.n_prod > 0 || p.nsplit > 1) {                      // the counters in the workspace are in use: zero them in stream order
+    if ((p.n_prod > 0 && d.r > 0) || p.nsplit > 1) {         // the counters in the workspace are in use: zero them in stream order
         p.sync = sync;
         const int rc = zero_sync_pair(sync, st);
         if (rc != QLORA_OK) return rc;
@@ -977,9 +987,14 @@ int umma_db_on_producers(const qlora_desc& d, int M) {
 
 int launch_umma_gemm(const qlora_desc& d, int M, bool transposed, const void* In, const int32_t* Q, const void* scales,
                      const void* zeros, const void* L, float* Pmat, void* Out, cudaStream_t st, const void* Ldown,
-                     unsigned int* sync, void* split_buf, size_t split_bytes, DbFuse* db) {
+                     unsigned int* sync, void* split_buf, size_t split_bytes, DbFuse* db, const DownExtra* extra) {
     if (prefer_pair_kernel(d, M, transposed))
-        return launch_umma_pair(d, M, transposed, In, Q, scales, zeros, L, Pmat, Out, st, Ldown, sync, split_buf, split_bytes, db);
+        return launch_umma_pair(d, M, transposed, In, Q, scales, zeros, L, Pmat, Out, st, Ldown, sync, split_buf, split_bytes, db, false, extra);
+    if (extra != nullptr && Ldown != nullptr) {              // (not on the single-CTA kernel's spare clusters)
+        const int rc = launch_lora_down(M, transposed ? d.N : d.K, extra->only_r > 0 ? extra->only_r : d.r, !transposed, In, Ldown, Pmat, st, extra->mask, extra->out_scale);
+        if (rc != QLORA_OK) return rc;
+        Ldown = nullptr;
+    }
     Params p{};
     p.M = M; p.N = d.N; p.K = d.K; p.bits = d.bits; p.g = d.group_size; p.r = d.r; p.lora_lo = keep_lora_low(d); p.r_pad = ((p.lora_lo ? 2 : 1) * d.r + 15) / 16 * 16;
     p.C = transposed ? d.K : d.N;

@@ -56,6 +56,9 @@ struct PairParams {
     __nv_bfloat16* Out;
     // producer clusters (n_prod > 0): P = In * Ldown is computed by this launch and written to Pout (== Pmat)
     int n_prod, T, lds_stages;
+    int r_down;                  // ranks of that product: r, or (r == 0) those of a product that the tiles do not use and do not wait for
+    const uint8_t* mask;         // LoRA dropout, forward: mask on In (uint8 [M, T]), and the scale of the product
+    float out_scale;
     unsigned int* sync;          // the launch's counter pair (n_prod > 0)
     int wait_limit_us;           // every wait inside the kernel gives up after this long
     const __nv_bfloat16* In;     // [M, T]
@@ -221,22 +224,30 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
         // ------------------------------------------------------------------ producer cluster: LoRA down-projection first
         // (this CTA's row blocks: blockIdx.x, blockIdx.x + 2 n_prod, ...; the ring takes the operand area, below the barriers)
         pdl_wait();
-        bool db_here = false;                // (the parts are added up by the tile CTAs, see the epilogue)
+        bool done_here = false;
         if constexpr (TRANSPOSED) {
             if (p.with_db) {       // the same pass over dY also gives this CTA's part of dB
-                db_here = true;
+                done_here = true;            // (the parts are added up by the tile CTAs, see the epilogue)
                 float* part = p.db_part + (size_t)blockIdx.x * p.T * p.r;
                 if (p.r <= 8) lora_down_stream<false, 1, true>(p.M, p.T, p.r, p.In, p.Ldown, p.Pout, (int)blockIdx.x, 2 * p.n_prod, smem_gen, p.lds_stages, abort_flag, p.Hmat, part);
                 else          lora_down_stream<false, 2, true, 3>(p.M, p.T, p.r, p.In, p.Ldown, p.Pout, (int)blockIdx.x, 2 * p.n_prod, smem_gen, p.lds_stages, abort_flag, p.Hmat, part);   // (two rank tiles: registers for three row blocks per CTA only; the host sees to it)
             }
         }
-        if (!db_here) {
-            if (p.r <= 8) lora_down_stream<!TRANSPOSED, 1>(p.M, p.T, p.r, p.In, p.Ldown, p.Pout, (int)blockIdx.x, 2 * p.n_prod, smem_gen, p.lds_stages, abort_flag);
-            else          lora_down_stream<!TRANSPOSED, 2>(p.M, p.T, p.r, p.In, p.Ldown, p.Pout, (int)blockIdx.x, 2 * p.n_prod, smem_gen, p.lds_stages, abort_flag);
+        if constexpr (!TRANSPOSED) {
+            if (p.mask != nullptr) {
+                done_here = true;
+                if (p.r_down <= 8) lora_down_stream<true, 1, false, LDS_MAXB, 1, true>(p.M, p.T, p.r_down, p.In, p.Ldown, p.Pout, (int)blockIdx.x, 2 * p.n_prod, smem_gen, p.lds_stages, abort_flag, nullptr, nullptr, p.mask, p.out_scale);
+                else               lora_down_stream<true, 2, false, LDS_MAXB, 1, true>(p.M, p.T, p.r_down, p.In, p.Ldown, p.Pout, (int)blockIdx.x, 2 * p.n_prod, smem_gen, p.lds_stages, abort_flag, nullptr, nullptr, p.mask, p.out_scale);
+            }
+        }
+        if (!done_here) {
+            if (p.r_down <= 8)       lora_down_stream<!TRANSPOSED, 1>(p.M, p.T, p.r_down, p.In, p.Ldown, p.Pout, (int)blockIdx.x, 2 * p.n_prod, smem_gen, p.lds_stages, abort_flag);
+            else if (p.r_down <= 16) lora_down_stream<!TRANSPOSED, 2>(p.M, p.T, p.r_down, p.In, p.Ldown, p.Pout, (int)blockIdx.x, 2 * p.n_prod, smem_gen, p.lds_stages, abort_flag);
+            else                     lora_down_stream<!TRANSPOSED, 2, false, LDS_WIDE_BLOCKS, 2>(p.M, p.T, p.r_down, p.In, p.Ldown, p.Pout, (int)blockIdx.x, 2 * p.n_prod, smem_gen, p.lds_stages, abort_flag);
         }
         __threadfence();       // every thread's rows of P (and of its part of dB) are visible device-wide before the CTA is counted
         __syncthreads();
-        if (threadIdx.x == 0) atomicAdd(&p.sync[0], 1u);
+        if (threadIdx.x == 0 && p.r > 0) atomicAdd(&p.sync[0], 1u);
         fence_proxy_async();   // the shared memory just used goes to the TMA / tensor-core side for this cluster's tiles, if any
         __syncthreads();
     }
@@ -353,7 +364,7 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
             const int wt = tile / p.n_tok_tiles, tt = tile % p.n_tok_tiles;
             const int w0 = wt * (2 * kPairW);                          // first weight row (output column) of the pair tile
             const int m0 = tt * (4 * kPairTok) + (int)cta * kPairTok;  // this CTA's first token row of accumulator 0
-            if (p.n_prod > 0 && tile_it == 0) {
+            if (p.n_prod > 0 && p.r > 0 && tile_it == 0) {
                 // P is being computed by the producer clusters of this launch: one thread waits for all of their CTAs, is
                 // counted as done with the counter, and the last such CTA of the launch zeroes the pair for the next one.
                 if (et == 0 && wait_counter(&p.sync[0], 2u * (unsigned)p.n_prod, abort_flag)) {

@@ -1,0 +1,59 @@
+"""The down-projection forms of the CTA-pair kernel's producer clusters beyond plain ranks of up to 16: under a dropout mask (forward), for a
+product the tiles do not use (backward under dropout), and ranks 17 to 32 -- on pairs without a tile and on pairs that take tiles
+afterwards, with ragged rows and a last chunk that is not full."""
+import numpy as np
+import pytest
+import torch
+
+import qlora_inputs as qi
+from gpu_util import GpuLayer, to_f64
+from helpers import REL_TOL, rel_err
+from oracle import qlora_oracle as orc
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("M,K,N,r", [(1025, 1088, 512, 8), (1499, 512, 1088, 16), (1100, 256, 10240, 8), (1100, 10240, 256, 16), (1030, 512, 256, 24), (1040, 320, 256, 40)])
+def test_dropout_beside_the_tiles(M, K, N, r):
+    import paper_2306_08162_b200 as ql
+    layer = qi.random_codes_layer(K=K, N=N, bits=4, group_size=64, r=r, alpha=2.0 * r, M=M, seed=M + r)
+    gl = GpuLayer(layer)
+    p = 0.25
+    keep = 1.0 / (1.0 - p)
+    mask_np = (np.random.default_rng(M).random((M, K)) >= p).astype(np.uint8)
+    mask = torch.from_numpy(mask_np).cuda()
+    Y = torch.empty((M, N), dtype=torch.bfloat16, device="cuda")
+    dX = torch.empty((M, K), dtype=torch.bfloat16, device="cuda")
+    H = torch.empty((M, r), dtype=torch.float32, device="cuda")
+    G = torch.empty_like(H)
+    grads = [(torch.empty((r, K), device="cuda"), torch.empty((N, r), device="cuda")) for _ in range(2)]
+    ql.qlora_fwd_dropout(gl.desc, M, gl.X, mask, keep, gl.Q, gl.scales, gl.zeros, gl.A, gl.B, Y, H, gl.ws)
+    ql.qlora_bwd_input_dropout(gl.desc, M, gl.dY, mask, keep, gl.Q, gl.scales, gl.zeros, gl.A, gl.B, dX, G, gl.ws)
+    for (dA, dB), (h, g) in zip(grads, ((H, G), (None, None))):
+        ql.qlora_bwd_lora_dropout(gl.desc, M, gl.X, mask, keep, gl.dY, gl.A, gl.B, h, g, dA, dB, 0, gl.ws)
+    torch.cuda.synchronize()
+    assert ql.qlora_device_status() == 0
+    f64 = orc.bf16_bits_to_f64
+    W = orc.dequant(orc.pack(layer["codes"], 4), layer["scales"], layer["zeros"], 4, 64)
+    X, dY, A, B = f64(layer["X"]), f64(layer["dY"]), f64(layer["A"]), f64(layer["B"])
+    Yo, Ho = orc.forward_dropout(X, W, A, B, layer["alpha"], mask_np, p)
+    dXo, dAo, dBo, Go = orc.backward_dropout(X, dY, W, A, B, layer["alpha"], mask_np, p)
+    assert rel_err(to_f64(H), Ho) < 1e-4 and rel_err(to_f64(G), Go) < 1e-4          # fp32 sums of exact products
+    for name, got, want in (("Y", Y, Yo), ("dX", dX, dXo), ("dA", grads[0][0], dAo), ("dB", grads[0][1], dBo)):
+        assert rel_err(to_f64(got), want) <= REL_TOL, name
+    for a, b in zip(*grads):                                                        # recomputed H / G: the same bits wherever they are formed
+        assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("M,K,N,r", [(1100, 1088, 512, 24), (1100, 256, 10240, 32), (1100, 10240, 256, 32)])
+def test_ranks_17_to_32_beside_the_tiles(M, K, N, r):
+    layer = qi.random_codes_layer(K=K, N=N, bits=4, group_size=64, r=r, alpha=2.0 * r, M=M, seed=M + K + r)
+    gl = GpuLayer(layer)
+    saved = gl.run()
+    ref = orc.layer_reference(layer)
+    for name in ("H", "G"):
+        assert rel_err(to_f64(saved[name]), ref[name]) < 1e-4, name                 # fp32 sums of exact products
+    for name in ("Y", "dX", "dA", "dB"):
+        assert rel_err(to_f64(saved[name]), ref[name]) <= REL_TOL, name
+    again = gl.run(save_hg=False)
+    assert torch.equal(saved["dA"], again["dA"]) and torch.equal(saved["dB"], again["dB"])
