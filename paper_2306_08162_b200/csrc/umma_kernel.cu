@@ -47,6 +47,9 @@ constexpr int kWRows = 128;          // weight rows (MMA M) per tile: n in forwa
 constexpr int kStepC = 64;           // contraction elements per pipeline stage
 constexpr int kWStageBytes = kWRows * kStepC * 2;   // 16 KiB of bf16 per stage
 constexpr int kAccStride = 256;      // tensor-memory columns per accumulator buffer
+constexpr int kMinSplitSteps = 4;    // contraction steps that a rank of a split tile has at least
+constexpr int kMaxDownTokens = 128, kMaxDownSteps = 8;   // up to here a split tile's ranks form P themselves.  INT4, rank 8,
+// 64 tokens, forward: 512 x 512 8.3 -> 6.6 us, 1024 x 1024 8.6 -> 6.8; INT3 2048 x 2048 9.05 -> 8.1
 constexpr uint32_t kSpinLimit = 1u << 26;
 constexpr int kWaitLimitUs = 250000;   // default limit of a wait, a launch parameter: far beyond any healthy wait (microseconds), short for a hang
 
@@ -66,7 +69,8 @@ struct Params {
     int packed_rows;     // int32 rows per stage
     int scale_rows;      // group rows per stage
     uint32_t words_bytes, scale_bytes, packed_slot_bytes, x_stage_bytes;
-    uint32_t off_x, off_w, off_p, off_lora_a, off_lora_p, off_bar;   // offsets from the 1024-aligned smem base
+    uint32_t off_x, off_w, off_l, off_p, off_lora_a, off_lora_p, off_bar;   // offsets from the 1024-aligned smem base
+    uint32_t down_bytes;             // DOWN: bytes per stage of the adapter applied first (else 0)
     float s;
     const float* Pmat;               // H (forward) or G (backward), fp32 [M, r]
     const __nv_bfloat16* L;          // B [N, r] (forward) or A [r, K] (backward)
@@ -183,8 +187,13 @@ __device__ __forceinline__ uint32_t map_to_cta(uint32_t local_addr, uint32_t ran
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local_addr), "r"(rank));
     return r;
 }
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync_all() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void st_cluster_16(uint32_t cluster_addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(cluster_addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
 __device__ __forceinline__ float4 ld_cluster_f32x4(uint32_t cluster_addr) {
     float4 v;
@@ -256,10 +265,10 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint3
     return (uint64_t)((addr >> 4) & 0x3FFFu) | ((uint64_t)((lbo >> 4) & 0x3FFFu) << 16) |
            ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | (1ull << 46) | ((uint64_t)layout << 61);
 }
-// Instruction descriptor: bf16 x bf16 -> fp32, M = 128, N = n_mma; majors: 0 = contraction-contiguous, 1 = other.
-__device__ __forceinline__ uint32_t instr_desc(uint32_t n_mma, uint32_t a_mn_major, uint32_t b_mn_major) {
+// Instruction descriptor: bf16 x bf16 -> fp32, M = m_mma, N = n_mma; majors: 0 = contraction-contiguous, 1 = other.
+__device__ __forceinline__ uint32_t instr_desc(uint32_t n_mma, uint32_t a_mn_major, uint32_t b_mn_major, uint32_t m_mma = 128) {
     return (1u << 4) | (1u << 7) | (1u << 10) | (a_mn_major << 15) | (b_mn_major << 16) | ((n_mma >> 3) << 17) |
-           ((128u >> 4) << 24);
+           ((m_mma >> 4) << 24);
 }
 
 // Ring position: slot index plus the phase bit of the current lap (no division in the hot loops).
@@ -268,11 +277,29 @@ struct Ring {
     __device__ __forceinline__ void advance(uint32_t n) { if (++slot == n) { slot = 0; phase ^= 1u; } }
 };
 
-template <int BITS, bool TRANSPOSED>
+// Eight ranks of the adapter applied second, for one weight row (zero beyond the last).
+template <bool TRANSPOSED>
+__device__ __forceinline__ uint4 lora_up_chunk(const Params& p, int wrow, int jc) {
+    if (wrow >= p.C) return make_uint4(0, 0, 0, 0);
+    if constexpr (!TRANSPOSED) {
+        return __ldg(reinterpret_cast<const uint4*>(p.L + (size_t)wrow * p.r + jc * 8));      // B[n, j..j+7]
+    } else {
+        uint32_t e[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) e[j] = __bfloat16_as_ushort(__ldg(p.L + (size_t)(jc * 8 + j) * p.K + wrow));     // A[j, k]
+        return make_uint4(e[0] | (e[1] << 16), e[2] | (e[3] << 16), e[4] | (e[5] << 16), e[6] | (e[7] << 16));
+    }
+}
+
+// DOWN (split tiles of short contractions, ranks 8 and 16): no producer clusters.  Every rank forms its part of P = In * Ldown beside its
+// part of the tile, from the activation stages it has anyway -- four more MMAs per stage, the adapter as their 64-row operand -- and the
+// parts of P meet where the tile's parts do; s P L is added in fp32 there.  So nothing has to be counted in device memory, nor the counters
+// set to zero by a launch ahead, and a tile waits for no other.
+template <int BITS, bool TRANSPOSED, bool DOWN>
 __global__ void __launch_bounds__(kThreads, 1)
 umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_constant__ CUtensorMap tm_q,
                  const __grid_constant__ CUtensorMap tm_scales, const __grid_constant__ CUtensorMap tm_zeros,
-                 const Params p) {
+                 const __grid_constant__ CUtensorMap tm_down, const Params p) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag_s[2];   // [0] set when a wait gave up, [1] the launch's wait limit in microseconds
@@ -330,7 +357,8 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
     const int first_tile = (int)blockIdx.x / p.split - p.n_prod, tile_stride = (int)gridDim.x / p.split - p.n_prod;
     const int step0 = rank * p.steps;
 
-    if (first_tile < 0) {
+    if (!DOWN && first_tile < 0) {
+        if constexpr (!DOWN) {
         // ------------------------------------------------------------------ producer cluster: LoRA down-projection on SMs
         // the tiles leave idle (one CTA per row block or more; lowest block indices, so they wait for nobody)
         const int n_ctas = p.n_prod * p.split;
@@ -365,6 +393,7 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
         __threadfence();       // every thread's rows of P are visible device-wide before the CTA is counted
         __syncthreads();
         if (threadIdx.x == 0) atomicAdd(&p.sync[0], 1u);
+        }
     } else if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer: activation tiles
         pdl_wait();
@@ -375,9 +404,14 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
                 if (!warp_wait(bar_empty + 8 * ring.slot, ring.phase ^ 1u, abort_flag, lane)) goto done;
                 const uint32_t bar = bar_full_x + 8 * ring.slot, dst = smem0 + p.off_x + ring.slot * p.x_stage_bytes;
                 const int c0 = (step0 + step) * kStepC;
+                const uint32_t dst_l = smem0 + p.off_l + ring.slot * p.down_bytes;
                 if (elect_one()) {
-                    mbar_expect_tx(bar, p.x_stage_bytes);
+                    mbar_expect_tx(bar, p.x_stage_bytes + (DOWN ? p.down_bytes : 0u));
                     tma_load_2d(dst, &tm_act, bar, c0, m0);
+                    if constexpr (DOWN) {                    // the stage's part of the adapter: eight ranks in 1 KiB
+                        tma_load_2d(dst_l, &tm_down, bar, TRANSPOSED ? 0 : c0, TRANSPOSED ? c0 : 0);
+                        if (TRANSPOSED && p.r > 8) tma_load_2d(dst_l + 1024, &tm_down, bar, 8, c0);
+                    }
                 }
                 ring.advance(S);
             }
@@ -414,6 +448,13 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
         const uint64_t a_desc0 = TRANSPOSED ? smem_desc(smem0 + p.off_w, 8192, 1024, 2) : smem_desc(smem0 + p.off_w, 16, 1024, 2);
         constexpr uint32_t a_k16 = TRANSPOSED ? (2048u >> 4) : (32u >> 4);
         const uint32_t x_step = p.x_stage_bytes >> 4;
+        // DOWN: the adapter as the 64-row operand (rows beyond r are whatever lies there; their sums are not looked at); the sums go to the
+        // second accumulator, which a split tile does not use.
+        //   forward A [r, k]: rows of 128 B, 128-byte swizzle;  backward B [n, r]: 16-byte rows of eight ranks, so 8 x 8 core matrices
+        //   of 128 B, consecutive along the contraction, 1 KiB from one eight ranks to the next
+        const uint32_t idesc_down = instr_desc((uint32_t)p.BT, TRANSPOSED ? 1u : 0u, 0u, 64u);
+        const uint64_t l_desc0 = TRANSPOSED ? smem_desc(smem0 + p.off_l, 128, 1024, 0) : smem_desc(smem0 + p.off_l, 16, 1024, 2);
+        constexpr uint32_t l_k16 = TRANSPOSED ? (256u >> 4) : (32u >> 4);
         Ring ring;
         uint32_t tile_it = 0;
         for (int tile = first_tile; tile < p.n_tiles; tile += tile_stride, ++tile_it) {
@@ -427,17 +468,22 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
                 tc_fence_after();
                 const uint64_t b_desc = b_desc0 + ring.slot * x_step;
                 const uint64_t a_desc = a_desc0 + ring.slot * (uint32_t)(kWStageBytes >> 4);
+                const uint64_t l_desc = l_desc0 + ring.slot * (p.down_bytes >> 4);
                 const uint32_t bar = bar_empty + 8 * ring.slot;
                 if (elect_one()) {
 #pragma unroll
                     for (int k16 = 0; k16 < kStepC / 16; ++k16)
                         tc_mma(d_tmem, a_desc + k16 * a_k16, b_desc + k16 * 2, idesc, acc | (uint32_t)(k16 > 0));
+                    if constexpr (DOWN)
+#pragma unroll
+                        for (int k16 = 0; k16 < kStepC / 16; ++k16)
+                            tc_mma(tmem_base + kAccStride, l_desc + k16 * l_k16, b_desc + k16 * 2, idesc_down, acc | (uint32_t)(k16 > 0));
                     tc_commit(bar);
                 }
                 acc = 1;
                 ring.advance(S);
             }
-            if (p.r > 0 && rank == 0) {   // the LoRA update goes into one rank's part only
+            if (!DOWN && p.r > 0 && rank == 0) {   // the LoRA update goes into one rank's part only
                 if (!warp_wait(bar_lora_full, tile_it & 1u, abort_flag, lane)) goto done;
                 tc_fence_after();
                 if (elect_one())
@@ -461,7 +507,7 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
             const int wt = tile / p.n_tok_tiles, tt = tile % p.n_tok_tiles;
             const int w0 = wt * kWRows, m0 = tt * p.BT;
             const uint32_t buf = tile_it & 1u;
-            if (p.n_prod > 0 && tile_it == 0 && rank == 0) {
+            if (!DOWN && p.n_prod > 0 && tile_it == 0 && rank == 0) {
                 // P is being computed by this launch's producer clusters: one thread waits for all of their CTAs, is counted
                 // as done with the counter, and the last such CTA of the launch zeroes the pair for the next one.
                 if (et == 0 && wait_counter(&p.sync[0], (unsigned)(p.n_prod * p.split), abort_flag)) {
@@ -474,7 +520,10 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
                 asm volatile("bar.sync 2, %0;" ::"r"(kEpiWarps * 32) : "memory");
                 if (*abort_flag) break;
             }
-            if (p.r > 0 && rank == 0) {   // (the LoRA update goes into rank 0's part only)
+            if constexpr (DOWN) {         // the adapter applied second, [8 ranks][weight row]: every rank adds the update to its tokens below
+                uint8_t* la = smem_gen + p.off_lora_a;
+                for (int jc = 0; jc < p.r / 8; ++jc) *reinterpret_cast<uint4*>(la + (jc * kWRows + et) * 16) = lora_up_chunk<TRANSPOSED>(p, w0 + et, jc);
+            } else if (p.r > 0 && rank == 0) {   // (the LoRA update goes into rank 0's part only)
                 // (the previous tile's LoRA MMA has completed: its accumulator-full barrier was observed below)
                 uint8_t* la = smem_gen + p.off_lora_a;
                 uint8_t* lp = smem_gen + p.off_lora_p;
@@ -482,18 +531,7 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
                 const int n8 = p.r >> 3;                      // chunks of eight ranks; the low pieces' chunks follow, then padding
                 for (int jc = 0; jc < p.r_pad / 8; ++jc) {
                     if (p.lora_lo && jc >= n8) break;         // (no padding then: r_pad == 2 r)
-                    uint4 v = make_uint4(0, 0, 0, 0);
-                    if (jc < n8 && wrow < p.C) {
-                        if (!TRANSPOSED) {
-                            v = __ldg(reinterpret_cast<const uint4*>(p.L + (size_t)wrow * p.r + jc * 8));      // B[n, j..j+7]
-                        } else {
-                            uint32_t e[8];
-#pragma unroll
-                            for (int j = 0; j < 8; ++j)
-                                e[j] = __bfloat16_as_ushort(__ldg(p.L + (size_t)(jc * 8 + j) * p.K + wrow));     // A[j, k]
-                            v = make_uint4(e[0] | (e[1] << 16), e[2] | (e[3] << 16), e[4] | (e[5] << 16), e[6] | (e[7] << 16));
-                        }
-                    }
+                    const uint4 v = jc < n8 ? lora_up_chunk<TRANSPOSED>(p, wrow, jc) : make_uint4(0, 0, 0, 0);
                     uint8_t* dst = la + jc * (kWRows * 16) + (row >> 3) * 128 + (row & 7) * 16;
                     *reinterpret_cast<uint4*>(dst) = v;
                     if (p.lora_lo) *reinterpret_cast<uint4*>(dst + n8 * (kWRows * 16)) = finite_only(v);
@@ -606,7 +644,117 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
     }
 
 done:
-    if (p.split > 1 && warp >= kEpiWarp0 && first_tile >= 0 && first_tile < p.n_tiles) {
+    if constexpr (DOWN) {
+        // The parts meet at the ranks that finish them: rank i takes tokens i * BT / split ...  Every rank stores its fp32 sums from tensor
+        // memory straight into the owners' shared memory, over the operand ring, which is idle once every rank's products are
+        // through: that is what the first cluster barrier says; the second says that the parts have arrived, and after it nobody touches a
+        // peer's memory again.  Bound by what comes into an SM from its neighbours, about 13 bytes a cycle whichever way it is moved: the other
+        // form below (parts put down, read by their owners) is 0.2 - 0.3 us slower up to 64 tokens and 10 % faster at 256; st.async on the
+        // owners' mbarriers and bulk copies were 0.4 - 1.2 us slower.
+        // Layout: [rank][token / 4][128 weight rows][4 tokens], a warp's store is 512 contiguous bytes; behind it P's, [rank][token / 4][r][4 tokens].
+        __syncwarp();
+        bool mine = warp >= kEpiWarp0;                         // the epilogue and the dequant warps, three per lane quarter, 16 tokens in turn
+        if (mine) mine = warp_wait(bar_acc_full, 0u, abort_flag, lane);
+        tc_fence_after();
+        cluster_arrive();
+        const uint32_t quarter = (uint32_t)warp & 3u, tpr4 = (uint32_t)(p.BT / p.split) >> 2, r = (uint32_t)p.r;
+        const uint32_t taddr = tmem_base + ((quarter * 32u) << 16);
+        int cb = 16 * ((warp - kEpiWarp0) >> 2);
+        uint32_t v[16];
+        if (mine && cb < p.BT) { tc_ld16(taddr + cb, v); tc_wait_ld(); }
+        cluster_wait();
+        if (mine) {
+            const uint32_t row = quarter * 32u + (uint32_t)lane;
+            // (lane: the first lanes of P's accumulator are its ranks)
+            auto send = [&](uint32_t base, uint32_t width, uint32_t col) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const uint32_t t4 = (uint32_t)(cb >> 2) + j, owner = t4 / tpr4;
+                    const uint32_t off = base + (((uint32_t)rank * tpr4 + (t4 - owner * tpr4)) * width + col) * 16u;
+                    st_cluster_16(map_to_cta(smem0 + off, owner), v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+                }
+            };
+#pragma unroll 1
+            while (cb < p.BT) {
+                send(0u, kWRows, row);
+                if (quarter == 0) {
+                    tc_ld16(taddr + kAccStride + cb, v);
+                    tc_wait_ld();
+                    if (lane < p.r) send((uint32_t)p.BT * (kWRows * 4u), r, (uint32_t)lane);
+                    __syncwarp();
+                }
+                cb += 48;
+                if (cb < p.BT) { tc_ld16(taddr + cb, v); tc_wait_ld(); }
+            }
+        }
+        __syncwarp();
+        cluster_arrive();
+        cluster_wait();
+        pdl_wait();             // every thread stores part of the output
+        const bool go = __all_sync(0xFFFFFFFFu, !*abort_flag) != 0;
+        const int wt = first_tile / p.n_tok_tiles, tt = first_tile % p.n_tok_tiles;
+        const int m_own = tt * p.BT + rank * (p.BT / p.split), c = wt * kWRows;
+        const float4* parts = reinterpret_cast<const float4*>(smem_gen);
+        float4* sp = reinterpret_cast<float4*>(smem_gen + p.off_lora_p);     // s * P of this rank's tokens, [token / 4][r][4 tokens]
+        if (go)
+            for (uint32_t i = threadIdx.x; i < tpr4 * r; i += kThreads) {
+                const float4* part = parts + (uint32_t)p.BT * (kWRows / 4) + i;
+                float4 y = part[0];
+                for (uint32_t rk = 1; rk < (uint32_t)p.split; ++rk) {
+                    const float4 x = part[rk * tpr4 * r];
+                    y.x += x.x; y.y += x.y; y.z += x.z; y.w += x.w;
+                }
+                if (wt == 0) {                                 // one tile of a token's many writes P out
+                    const uint32_t t4 = i / r, j = i - t4 * r;
+                    const int m = m_own + 4 * (int)t4;
+                    float* out = p.Pout + (size_t)m * p.r + j;
+                    if (m < p.M) out[0] = y.x;
+                    if (m + 1 < p.M) out[p.r] = y.y;
+                    if (m + 2 < p.M) out[2 * p.r] = y.z;
+                    if (m + 3 < p.M) out[3 * p.r] = y.w;
+                }
+                sp[i] = make_float4(p.s * y.x, p.s * y.y, p.s * y.z, p.s * y.w);
+            }
+        __syncthreads();
+        if (go) {
+            const bool odd = (lane & 1) != 0;
+            // four tokens of one weight row (output column) at a time; the ranks' parts are added in rank order (the same bits on every run)
+#pragma unroll 1
+            for (uint32_t e = threadIdx.x; e < tpr4 * kWRows; e += kThreads) {
+                float4 x[4];
+#pragma unroll
+                for (int rk = 0; rk < 4; ++rk)
+                    if (rk < p.split) x[rk] = parts[(uint32_t)rk * tpr4 * kWRows + e];
+                float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int rk = 0; rk < 4; ++rk)
+                    if (rk < p.split) { y.x += x[rk].x; y.y += x[rk].y; y.z += x[rk].z; y.w += x[rk].w; }
+                const uint32_t t4 = e / kWRows, n = e % kWRows;
+                const uint4* up = reinterpret_cast<const uint4*>(smem_gen + p.off_lora_a) + n;
+#pragma unroll 1
+                for (uint32_t jc = 0; jc < r / 8; ++jc) {      // + s P L, in fp32
+                    const uint4 l = up[jc * kWRows];
+                    const float lf[8] = {bf16_lo(l.x), bf16_hi(l.x), bf16_lo(l.y), bf16_hi(l.y), bf16_lo(l.z), bf16_hi(l.z), bf16_lo(l.w), bf16_hi(l.w)};
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        const float4 q4 = sp[t4 * r + jc * 8 + j];
+                        y.x = fmaf(q4.x, lf[j], y.x); y.y = fmaf(q4.y, lf[j], y.y); y.z = fmaf(q4.z, lf[j], y.z); y.w = fmaf(q4.w, lf[j], y.w);
+                    }
+                }
+                // neighbouring lanes trade two tokens each, so that a lane stores two columns of two tokens
+                const float r0 = __shfl_xor_sync(0xFFFFFFFFu, odd ? y.x : y.z, 1), r1 = __shfl_xor_sync(0xFFFFFFFFu, odd ? y.y : y.w, 1);
+                const __nv_bfloat162 o0 = odd ? __floats2bfloat162_rn(r0, y.z) : __floats2bfloat162_rn(y.x, r0);
+                const __nv_bfloat162 o1 = odd ? __floats2bfloat162_rn(r1, y.w) : __floats2bfloat162_rn(y.y, r1);
+                const int m = m_own + (int)t4 * 4 + (odd ? 2 : 0), col = c + (int)(n & ~1u);
+                if (col < p.C) {                                  // C is a multiple of 64: both columns or none
+                    __nv_bfloat16* out = p.Out + (size_t)m * p.C + col;
+                    if (m < p.M) *reinterpret_cast<__nv_bfloat162*>(out) = o0;
+                    if (m + 1 < p.M) *reinterpret_cast<__nv_bfloat162*>(out + p.C) = o1;
+                }
+            }
+        }
+    }
+    if (!DOWN && p.split > 1 && warp >= kEpiWarp0 && first_tile >= 0 && first_tile < p.n_tiles) {
         // This rank's part of the tile, fp32 [token][128 weight rows], over the (now idle) operand ring: the epilogue and the dequant
         // warps, three per lane quarter, take 16 tokens at a time in turn.
         __syncwarp();
@@ -632,7 +780,7 @@ done:
         for (int i = 0; i < 200; ++i) __nanosleep(1000);
         __syncthreads();
     }
-    if (p.split > 1) {
+    if (!DOWN && p.split > 1) {
         // Add the ranks' parts in rank order (fixed order: deterministic); rank i finishes tokens i * BT / split ...
         __syncwarp();
         cluster_sync_all();
@@ -727,12 +875,19 @@ int zero_sync_pair(unsigned int* sync, cudaStream_t st) {
 // (cudaOccupancyMaxActiveClusters: 33 clusters of 4 fit on 148 SMs, 74 of 2), producer clusters in front of the grid do
 // it beside the tiles; else a down-projection launch goes ahead of the kernel.
 template <int BITS, bool TRANSPOSED>
-int launch_impl(const CUtensorMap& ta, const CUtensorMap& tq, const CUtensorMap& ts, const CUtensorMap& tz, const Params& p_in,
+int launch_impl(const CUtensorMap& ta, const CUtensorMap& tq, const CUtensorMap& ts, const CUtensorMap& tz, const CUtensorMap& tl, const Params& p_in,
                 size_t smem_bytes, int grid, cudaStream_t st, const void* Ldown, unsigned int* sync) {
+    if (p_in.down_bytes > 0) {
+        static SmemLimit down_limit;
+        auto down_kern = umma_gemm_kernel<BITS, TRANSPOSED, true>;
+        if (!down_limit.raise(down_kern, 232448 - 1024)) return QLORA_ERR_CUDA;
+        return launch_pdl(down_kern, dim3((unsigned)grid), dim3(kThreads), smem_bytes, st, (unsigned)p_in.split, ta, tq, ts, tz, tl, p_in) == cudaSuccess
+                   ? QLORA_OK : QLORA_ERR_CUDA;
+    }
     static SmemLimit limit;
     static std::mutex mu;
     static int max_clusters_dev[kMaxDevices][5] = {};   // per device, by cluster width
-    auto kern = umma_gemm_kernel<BITS, TRANSPOSED>;
+    auto kern = umma_gemm_kernel<BITS, TRANSPOSED, false>;
     if (!limit.raise(kern, 232448 - 1024)) return QLORA_ERR_CUDA;
     Params p = p_in;
     p.n_prod = 0; p.sync = nullptr; p.wait_limit_us = kWaitLimitUs;
@@ -771,7 +926,7 @@ int launch_impl(const CUtensorMap& ta, const CUtensorMap& tq, const CUtensorMap&
         }
     }
     // one cluster of p.split CTAs per tile when the contraction is split
-    return launch_pdl(kern, dim3((unsigned)grid), dim3(kThreads), smem_bytes, st, (unsigned)p.split, ta, tq, ts, tz, p) == cudaSuccess
+    return launch_pdl(kern, dim3((unsigned)grid), dim3(kThreads), smem_bytes, st, (unsigned)p.split, ta, tq, ts, tz, tl, p) == cudaSuccess
                ? QLORA_OK : QLORA_ERR_CUDA;
 }
 
@@ -1023,47 +1178,54 @@ int launch_umma_gemm(const qlora_desc& d, int M, bool transposed, const void* In
     const uint32_t budget = 232448 - 1024 /*alignment slack*/ - 2048 /*static, barriers, padding*/;
     // With few tokens the kernel is bound by the latency of streaming cold packed weights through a handful of CTAs,
     // so the packed ring is deep (bytes in flight), at the cost of one or two operand stages.
-    const uint32_t per_stage = p.x_stage_bytes + kWStageBytes;
-    int S = 0;
-    uint32_t fixed = 0;
-    for (p.P = p.BT <= 128 ? 16 : 8;; p.P -= p.P > 4 ? 4 : 1) {   // the packed ring gives way until three operand stages fit (two, below four slots)
-        fixed = lora_a + lora_p + p.P * p.packed_slot_bytes + 512;
-        S = budget > fixed ? (int)((budget - fixed) / per_stage) : 0;
-        if (S >= (p.P > 4 ? 3 : 2) || p.P == 2) break;
-    }
-    if (S > 8) S = 8;
-    if (S < 2) return QLORA_ERR_UNSUPPORTED;
-    p.S = S;
-    p.off_x = 0;
-    p.off_w = p.off_x + S * p.x_stage_bytes;
-    p.off_p = p.off_w + S * kWStageBytes;
-    p.off_lora_a = p.off_p + p.P * p.packed_slot_bytes;
-    p.off_lora_p = p.off_lora_a + lora_a;
-    p.off_bar = (p.off_lora_p + lora_p + 127u) / 128u * 128u;
+    auto plan = [&](int split) {
+        p.split = split;
+        p.down_bytes = split > 1 && Ldown != nullptr && (d.r == 8 || d.r == 16) && p.BT <= kMaxDownTokens && p.steps / split <= kMaxDownSteps ? (uint32_t)d.r * 128u : 0u;
+        const uint32_t per_stage = p.x_stage_bytes + kWStageBytes + p.down_bytes;
+        uint32_t S = 0;
+        for (p.P = p.BT <= 128 ? 16 : 8;; p.P -= p.P > 4 ? 4 : 1) {   // the packed ring gives way until three operand stages fit (two, below four slots)
+            const uint32_t fixed = lora_a + lora_p + p.P * p.packed_slot_bytes + 512;
+            S = budget > fixed ? (budget - fixed) / per_stage : 0;
+            if (S >= (p.P > 4 ? 3 : 2) || p.P == 2) break;
+        }
+        if (S > 8) S = 8;
+        p.S = (int)S;
+        p.off_x = 0;
+        p.off_w = p.off_x + S * p.x_stage_bytes;
+        p.off_l = p.off_w + S * kWStageBytes;
+        p.off_p = p.off_l + S * p.down_bytes;
+        p.off_lora_a = p.off_p + p.P * p.packed_slot_bytes;
+        p.off_lora_p = p.off_lora_a + lora_a;
+        p.off_bar = (p.off_lora_p + lora_p + 127u) / 128u * 128u;
+        return S >= 2 && (split == 1 || (uint32_t)(p.BT * (kWRows + (p.down_bytes ? d.r : 0)) * 4) <= p.off_p);
+    };
+    // Few tiles (few tokens): split each tile's contraction over a cluster of 2 or 4 CTAs so that the whole GPU streams
+    // the weights.  Needs one tile per cluster, an even split of the steps, and room for the fp32 parts in the operand ring.
+    int split = 1;
+    for (int sp = 4; sp >= 2 && split == 1; sp /= 2)
+        if (p.n_tiles * sp <= sm_count() && p.steps % sp == 0 && p.steps / sp >= kMinSplitSteps && p.BT % sp == 0 && plan(sp)) split = sp;
+    if (split == 1 && !plan(1)) return QLORA_ERR_UNSUPPORTED;
     const size_t smem_bytes = (size_t)p.off_bar + 512 + 1024;
 
-    CUtensorMap ta, tq, ts, tz;
+    CUtensorMap ta, tq, ts, tz, tl{};
     if (!make_map_2d(&ta, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, In, (uint64_t)T, (uint64_t)M, 64, (uint32_t)p.BT, CU_TENSOR_MAP_SWIZZLE_128B) ||
         !make_map_2d(&tq, CU_TENSOR_MAP_DATA_TYPE_INT32, 4, Q, (uint64_t)d.N, (uint64_t)(d.K * d.bits / 32), (uint32_t)p.packed_cols, (uint32_t)p.packed_rows, CU_TENSOR_MAP_SWIZZLE_NONE) ||
         !make_map_2d(&ts, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, scales, (uint64_t)d.N, (uint64_t)(d.K / d.group_size), (uint32_t)p.packed_cols, (uint32_t)p.scale_rows, CU_TENSOR_MAP_SWIZZLE_NONE) ||
         !make_map_2d(&tz, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, zeros, (uint64_t)d.N, (uint64_t)(d.K / d.group_size), (uint32_t)p.packed_cols, (uint32_t)p.scale_rows, CU_TENSOR_MAP_SWIZZLE_NONE))
         return QLORA_ERR_CUDA;
 
-    // Few tiles (few tokens): split each tile's contraction over a cluster of 2 or 4 CTAs so that the whole GPU streams
-    // the weights.  Needs one tile per cluster, an even split of the steps, and room for the fp32 part in the operand ring.
-    p.split = 1;
-    for (int sp = 4; sp >= 2; sp /= 2) {
-        if (p.n_tiles * sp <= sm_count() && p.steps % sp == 0 && p.steps / sp >= 4 && p.BT % sp == 0 &&
-            (uint32_t)(kWRows * p.BT * 4) <= p.off_p) { p.split = sp; break; }
-    }
     p.steps /= p.split;
     const int grid = p.split > 1 ? p.n_tiles * p.split : (p.n_tiles < sm_count() ? p.n_tiles : sm_count());
-    p.T = T; p.In = (const __nv_bfloat16*)In; p.Ldown = (const __nv_bfloat16*)Ldown; p.Pout = Pmat;
+    if (p.down_bytes != 0 &&
+        !(transposed ? make_map_2d(&tl, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Ldown, (uint64_t)d.r, (uint64_t)T, 8, 64, CU_TENSOR_MAP_SWIZZLE_NONE)
+                     : make_map_2d(&tl, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Ldown, (uint64_t)T, (uint64_t)d.r, 64, (uint32_t)d.r, CU_TENSOR_MAP_SWIZZLE_128B)))
+        return QLORA_ERR_CUDA;
+    p.T = T; p.In = (const __nv_bfloat16*)In; p.Ldown = (const __nv_bfloat16*)Ldown; p.Pout = Pmat; p.wait_limit_us = kWaitLimitUs;
     p.lds_stages = (int)((p.off_bar - LDS_BAR_BYTES) / LDS_STAGE_BYTES);
     if (p.lds_stages > 6) p.lds_stages = 6;
 #define QLORA_LAUNCH(B)                                                                              \
-    return transposed ? launch_impl<B, true>(ta, tq, ts, tz, p, smem_bytes, grid, st, Ldown, sync)  \
-                      : launch_impl<B, false>(ta, tq, ts, tz, p, smem_bytes, grid, st, Ldown, sync)
+    return transposed ? launch_impl<B, true>(ta, tq, ts, tz, tl, p, smem_bytes, grid, st, Ldown, sync)  \
+                      : launch_impl<B, false>(ta, tq, ts, tz, tl, p, smem_bytes, grid, st, Ldown, sync)
     switch (d.bits) {
         case 2: QLORA_LAUNCH(2);
         case 3: QLORA_LAUNCH(3);
