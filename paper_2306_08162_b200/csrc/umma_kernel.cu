@@ -47,9 +47,15 @@ constexpr int kWRows = 128;          // weight rows (MMA M) per tile: n in forwa
 constexpr int kStepC = 64;           // contraction elements per pipeline stage
 constexpr int kWStageBytes = kWRows * kStepC * 2;   // 16 KiB of bf16 per stage
 constexpr int kAccStride = 256;      // tensor-memory columns per accumulator buffer
-constexpr int kMinSplitSteps = 4;    // contraction steps that a rank of a split tile has at least
-constexpr int kMaxDownTokens = 128, kMaxDownSteps = 8;   // up to here a split tile's ranks form P themselves.  INT4, rank 8,
-// 64 tokens, forward: 512 x 512 8.3 -> 6.6 us, 1024 x 1024 8.6 -> 6.8; INT3 2048 x 2048 9.05 -> 8.1
+// contraction steps that a rank of a split tile has at least, up to 128 tokens and above (512 x 512, rank 8: four ranks of two steps against two
+// of four 5.1 / 5.7 us at 17 tokens, 7.6 / 8.3 at 128, but 11.8 / 10.6 at 256: what the ranks exchange grows with the tokens)
+constexpr int kMinSplitSteps = 2, kMinSplitSteps256 = 4;
+constexpr int kMaxDownTokens = 128;
+// Up to 128 tokens, where a split tile's ranks form P themselves.  Their MMAs cost some 250 cycles per step, the producer clusters a launch, a
+// counter and a chain that grows with the rank; two ranks have more of the tile to exchange and less room to gain.  INT4, forward, 64
+// tokens, rank 8: 512 x 512 8.3 -> 6.6 us, 1024 x 1024 8.6 -> 6.8, INT3 2048 x 2048 9.05 -> 8.1; 4096 x 4096, 16 steps, 128 tokens 16.3 -> 15.1;
+// 8192 -> 2048, 32 steps, 64 tokens 16.4 -> 16.9, but rank 16 19.3 -> 17.3; two ranks of 16 steps, 128 tokens 13.2 -> 14.9.
+static bool down_pays(int split, int steps, int r) { return steps <= 8 || (split == 4 && (r == 16 || steps <= 16)); }
 constexpr uint32_t kSpinLimit = 1u << 26;
 constexpr int kWaitLimitUs = 250000;   // default limit of a wait, a launch parameter: far beyond any healthy wait (microseconds), short for a hang
 
@@ -497,7 +503,7 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
             }
             if (elect_one()) tc_commit(bar_acc_full + 8 * buf);
         }
-    } else if (warp >= kEpiWarp0 && warp < kDequantWarp0) {
+    } else if (!DOWN && warp >= kEpiWarp0 && warp < kDequantWarp0) {
         // ------------------------------------------------------------------ epilogue (+ LoRA operand staging)
         const int q = warp & 3;                      // tensor-memory lane quarter this warp may read
         const int et = threadIdx.x - kEpiWarp0 * 32; // 0..127
@@ -520,10 +526,7 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
                 asm volatile("bar.sync 2, %0;" ::"r"(kEpiWarps * 32) : "memory");
                 if (*abort_flag) break;
             }
-            if constexpr (DOWN) {         // the adapter applied second, [8 ranks][weight row]: every rank adds the update to its tokens below
-                uint8_t* la = smem_gen + p.off_lora_a;
-                for (int jc = 0; jc < p.r / 8; ++jc) *reinterpret_cast<uint4*>(la + (jc * kWRows + et) * 16) = lora_up_chunk<TRANSPOSED>(p, w0 + et, jc);
-            } else if (p.r > 0 && rank == 0) {   // (the LoRA update goes into rank 0's part only)
+            if (p.r > 0 && rank == 0) {   // (the LoRA update goes into rank 0's part only)
                 // (the previous tile's LoRA MMA has completed: its accumulator-full barrier was observed below)
                 uint8_t* la = smem_gen + p.off_lora_a;
                 uint8_t* lp = smem_gen + p.off_lora_p;
@@ -579,13 +582,15 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_acc_empty + 8 * buf);
         }
-    } else if (warp >= kDequantWarp0) {
+    } else if (warp >= (DOWN ? kEpiWarp0 : kDequantWarp0)) {
         // ------------------------------------------------------------------ unpack + dequant
+        // (DOWN: one tile per CTA, so the epilogue's warps would be idle until the end; they are a third group.)
+        constexpr int kGroups = DOWN ? 3 : 2, kWarp0 = DOWN ? kEpiWarp0 : kDequantWarp0;
         // Two groups of four warps take alternate pipeline stages, so each group has two stage times for its serial chain
         // (wait, shared-memory loads, arithmetic, wait, stores, fence, arrive).  Inside a group a thread owns one column of
         // the packed tile and two blocks of 32 consecutive-k codes.
-        const int group = (warp - kDequantWarp0) / kGroupWarps;    // 0 or 1
-        const int gt = threadIdx.x - (kDequantWarp0 + group * kGroupWarps) * 32;   // 0..127 inside the group
+        const int group = (warp - kWarp0) / kGroupWarps;
+        const int gt = threadIdx.x - (kWarp0 + group * kGroupWarps) * 32;   // 0..127 inside the group
         const int col = gt % p.packed_cols;                       // column of the packed tile (n in both directions)
         const int kb0 = gt / p.packed_cols;                       // forward: 0; backward: 0..1
         const int kb_stride = TRANSPOSED ? 2 : 1;                 // the thread's two code blocks are kb0 and kb0 + kb_stride
@@ -603,8 +608,8 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
         const int my_tiles = first_tile < p.n_tiles ? (p.n_tiles - first_tile + tile_stride - 1) / tile_stride : 0;
         const int total = my_tiles * p.steps;
         Ring ring_w, ring_p;
-        if (group == 1) { ring_w.advance(S); ring_p.advance(P); }
-        for (int it = group; it < total; it += 2) {
+        for (int i = 0; i < group; ++i) { ring_w.advance(S); ring_p.advance(P); }
+        for (int it = group; it < total; it += kGroups) {
             if (!warp_wait(bar_full_p + 8 * ring_p.slot, ring_p.phase, abort_flag, lane)) break;
             const uint8_t* pk = smem_gen + p.off_p + ring_p.slot * p.packed_slot_bytes;
             const uint32_t* pw = reinterpret_cast<const uint32_t*>(pk);
@@ -638,8 +643,13 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
             fence_proxy_async();
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_full_w + 8 * ring_w.slot);
-            ring_w.advance(S); ring_w.advance(S);
-            ring_p.advance(P); ring_p.advance(P);
+#pragma unroll
+            for (int i = 0; i < kGroups; ++i) { ring_w.advance(S); ring_p.advance(P); }
+        }
+        if (DOWN && group == 0) {         // the adapter applied second, [8 ranks][weight row]: every rank adds the update to its tokens below
+            pdl_wait();
+            uint8_t* la = smem_gen + p.off_lora_a;
+            for (int jc = 0; jc < p.r / 8; ++jc) *reinterpret_cast<uint4*>(la + (jc * kWRows + gt) * 16) = lora_up_chunk<TRANSPOSED>(p, first_tile / p.n_tok_tiles * kWRows + gt, jc);
         }
     }
 
@@ -1180,7 +1190,7 @@ int launch_umma_gemm(const qlora_desc& d, int M, bool transposed, const void* In
     // so the packed ring is deep (bytes in flight), at the cost of one or two operand stages.
     auto plan = [&](int split) {
         p.split = split;
-        p.down_bytes = split > 1 && Ldown != nullptr && (d.r == 8 || d.r == 16) && p.BT <= kMaxDownTokens && p.steps / split <= kMaxDownSteps ? (uint32_t)d.r * 128u : 0u;
+        p.down_bytes = split > 1 && Ldown != nullptr && (d.r == 8 || d.r == 16) && p.BT <= kMaxDownTokens && down_pays(split, p.steps / split, d.r) ? (uint32_t)d.r * 128u : 0u;
         const uint32_t per_stage = p.x_stage_bytes + kWStageBytes + p.down_bytes;
         uint32_t S = 0;
         for (p.P = p.BT <= 128 ? 16 : 8;; p.P -= p.P > 4 ? 4 : 1) {   // the packed ring gives way until three operand stages fit (two, below four slots)
@@ -1203,7 +1213,7 @@ int launch_umma_gemm(const qlora_desc& d, int M, bool transposed, const void* In
     // the weights.  Needs one tile per cluster, an even split of the steps, and room for the fp32 parts in the operand ring.
     int split = 1;
     for (int sp = 4; sp >= 2 && split == 1; sp /= 2)
-        if (p.n_tiles * sp <= sm_count() && p.steps % sp == 0 && p.steps / sp >= kMinSplitSteps && p.BT % sp == 0 && plan(sp)) split = sp;
+        if (p.n_tiles * sp <= sm_count() && p.steps % sp == 0 && p.steps / sp >= (p.BT <= kMaxDownTokens ? kMinSplitSteps : kMinSplitSteps256) && p.BT % sp == 0 && plan(sp)) split = sp;
     if (split == 1 && !plan(1)) return QLORA_ERR_UNSUPPORTED;
     const size_t smem_bytes = (size_t)p.off_bar + 512 + 1024;
 
