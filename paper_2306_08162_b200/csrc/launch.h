@@ -31,10 +31,10 @@ int launch_simt_gemm(const qlora_desc& d, int M, bool transposed, const void* In
 int launch_lora_down(int M, int T, int r, bool l_is_A, const void* In, const void* L, float* P, cudaStream_t st,
                      const uint8_t* mask = nullptr, float out_scale = 1.0f);
 // umma_kernel.cu -- the same product for many rows: activations streamed through shared memory by bulk copies (launch_lora_down routes
-// there above 256 rows for r <= 16, and where lora_down_streams_wide says so; the CTA-pair kernel runs the same code on idle SM pairs).
+// there above 256 rows for r <= 16, under a mask where lora_down_streams_masked says so; the CTA-pair kernel runs the same code on idle SM pairs).
 int launch_lora_down_stream(int M, int T, int r, bool l_is_A, const void* In, const void* L, float* P, cudaStream_t st, const uint8_t* mask = nullptr,
                             float out_scale = 1.0f);
-bool lora_down_streams_wide(int M, int r, bool masked);
+bool lora_down_streams_masked(int M, int r);
 // dB = s dY^T H [N, r] and dA = s G^T X [r, K] in one pair of launches (partial sums per row slice, then a fixed-order
 // reduction); scratch needs lora_grad_scratch_bytes().
 size_t lora_grad_scratch_bytes(int M, int K, int N, int r);

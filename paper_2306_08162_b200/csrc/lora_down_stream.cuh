@@ -16,6 +16,7 @@ constexpr int LDS_ROW_BYTES = LDS_TC * 2 + 64;            // padded: rows 16 wor
 constexpr int LDS_STAGE_BYTES = 16 * LDS_ROW_BYTES;       // 33 KiB
 constexpr int LDS_MAXB = 8;                               // row blocks per CTA
 constexpr int LDS_CWARPS = 14;                            // consumer warps (warp 14 issues the copies)
+constexpr int LDS_STEPS = (LDS_TC / 32 + LDS_CWARPS - 1) / LDS_CWARPS;   // 32-wide contraction steps per warp and chunk
 constexpr int LDS_BAR_BYTES = 256;                        // full[S] + empty[S] barriers behind the ring (S <= 16)
 // Under dropout a stage carries the mask bytes of its rows behind them (rows 8 words apart (mod 32): conflict-free 8-byte loads).
 constexpr int LDS_MASK_ROW_BYTES = LDS_TC + 32;
@@ -38,18 +39,15 @@ constexpr int LDS_MIN_STAGES = (LDS_CWARPS * LDS_MAXB * 2 * 128 * 4 + LDS_STAGE_
 // transposed across the warp (movmatrix) into the 16-row operand and H supplies the 8-column one.  A warp owns the columns
 // n of its own contraction steps, so nothing is summed across warps; its accumulators live for one chunk and are then
 // written to dBpart [T, r] (fp32, this CTA's own: every n below T is written exactly once, provided the CTA has a row block).
-// RG = 2 (ranks 17 to 32): seven consumer warps take the first 16 ranks, seven the others; each reads all activation fragments, so the
-//   activations still pass through once.  (All ranks in every warp would need 64 more registers.)
 // MASKED: `mask` (uint8 [M, T], non-zero = keep) is applied to In, and P is multiplied by out_scale (LoRA dropout).
-template <bool L_IS_A, int NT, bool WITH_DB = false, int MAXB = LDS_MAXB, int RG = 1, bool MASKED = false>   // MAXB: row blocks this instantiation keeps accumulators for
+template <bool L_IS_A, int NT, bool WITH_DB = false, int MAXB = LDS_MAXB, bool MASKED = false>   // MAXB: row blocks this instantiation keeps accumulators for
 __device__ __forceinline__ void lora_down_stream(int M, int T, int r, const __nv_bfloat16* __restrict__ In,
                                                  const __nv_bfloat16* __restrict__ L, float* __restrict__ P, int first_block,
                                                  int block_stride, uint8_t* smem, int stages, volatile int* abort_flag,
                                                  const float* __restrict__ Hm = nullptr, float* __restrict__ dBpart = nullptr,
                                                  const uint8_t* __restrict__ mask = nullptr, float out_scale = 1.f) {
-    static_assert(!(WITH_DB && L_IS_A) && !(WITH_DB && RG > 1), "dB rides on the backward's pass over dY");
+    static_assert(!(WITH_DB && L_IS_A), "dB rides on the backward's pass over dY");
     constexpr int STAGE = MASKED ? LDS_MASKED_STAGE_BYTES : LDS_STAGE_BYTES;
-    constexpr int GW = LDS_CWARPS / RG, STEPS = (LDS_TC / 32 + GW - 1) / GW;       // warps per rank group; 32-wide contraction steps per warp and chunk
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, q = lane & 3;
     const uint32_t ring = smem_u32(smem);
@@ -105,24 +103,23 @@ __device__ __forceinline__ void lora_down_stream(int M, int T, int r, const __nv
     } else if (warp < LDS_CWARPS) {
         // ---------------------------------------------------------------- consumers (warps beyond the issuer's have no part)
         uint32_t slot = 0, phase = 0;
-        const int gw = warp % GW, j0 = warp / GW * 16;              // place in the rank group, its first rank
         const uint4 zero4 = make_uint4(0, 0, 0, 0);
         bool live = true;
         for (int c = 0; c < n_chunks && live; ++c) {
             const int t0 = c * LDS_TC;
             const int chunk_len = T - t0 < LDS_TC ? T - t0 : LDS_TC;
-            // this warp's adapter fragments of the chunk (steps gw, gw + GW, ...), reused for every row block
-            uint4 lf[STEPS][NT];
+            // this warp's adapter fragments of the chunk (steps warp, warp + 14, ...), reused for every row block
+            uint4 lf[LDS_STEPS][NT];
 #pragma unroll
-            for (int i = 0; i < STEPS; ++i) {
-                const int k0 = t0 + (gw + i * GW) * 32;                    // warp-uniform
+            for (int i = 0; i < LDS_STEPS; ++i) {
+                const int k0 = t0 + (warp + i * LDS_CWARPS) * 32;          // warp-uniform
                 const int k = k0 + q * 8;
 #pragma unroll
                 for (int nt = 0; nt < NT; ++nt) {
                     uint4 lv = zero4;
-                    if ((gw + i * GW) * 32 < chunk_len) {
+                    if ((warp + i * LDS_CWARPS) * 32 < chunk_len) {
                         if (L_IS_A) {
-                            const int j = j0 + nt * 8 + g;
+                            const int j = nt * 8 + g;
                             if (k < T && j < r) lv = __ldg(reinterpret_cast<const uint4*>(L + (size_t)j * T + k));
                         } else {
                             // 8 x 8 tiles of B loaded row-wise and transposed across the warp (see lora_down.cuh)
@@ -131,7 +128,7 @@ __device__ __forceinline__ void lora_down_stream(int M, int T, int r, const __nv
                             for (int t = 0; t < 4; ++t) {
                                 const int n = k0 + 8 * (g >> 1) + (g & 1) + 2 * t;
                                 uint32_t v = 0;
-                                if (n < T && j0 + nt * 8 < r) v = __ldg(reinterpret_cast<const uint32_t*>(L + (size_t)n * r + j0 + nt * 8 + 2 * q));
+                                if (n < T && nt * 8 < r) v = __ldg(reinterpret_cast<const uint32_t*>(L + (size_t)n * r + nt * 8 + 2 * q));
                                 w[t] = movmatrix_trans(v);
                             }
                             lv = make_uint4(w[0], w[1], w[2], w[3]);
@@ -140,10 +137,10 @@ __device__ __forceinline__ void lora_down_stream(int M, int T, int r, const __nv
                     lf[i][nt] = lv;
                 }
             }
-            float dbacc[WITH_DB ? STEPS : 1][2][NT][4];
+            float dbacc[WITH_DB ? LDS_STEPS : 1][2][NT][4];
             if constexpr (WITH_DB) {
 #pragma unroll
-                for (int i = 0; i < STEPS; ++i)
+                for (int i = 0; i < LDS_STEPS; ++i)
 #pragma unroll
                     for (int h = 0; h < 2; ++h)
 #pragma unroll
@@ -175,8 +172,8 @@ __device__ __forceinline__ void lora_down_stream(int M, int T, int r, const __nv
                     const bool v0 = m0 + g < M, v1 = m0 + g + 8 < M;       // rows beyond M were not copied
                     const uint8_t* st = smem + slot * STAGE;
 #pragma unroll
-                    for (int i = 0; i < STEPS; ++i) {
-                        const int kl = (gw + i * GW) * 32;       // warp-uniform
+                    for (int i = 0; i < LDS_STEPS; ++i) {
+                        const int kl = (warp + i * LDS_CWARPS) * 32;       // warp-uniform
                         if (kl < chunk_len) {
                             const int k = kl + q * 8;                      // chunk_len % 8 == 0: 8 elements are all-in or all-out
                             uint4 xlo = (v0 && k < chunk_len) ? *reinterpret_cast<const uint4*>(st + g * LDS_ROW_BYTES + k * 2) : zero4;
@@ -213,8 +210,8 @@ __device__ __forceinline__ void lora_down_stream(int M, int T, int r, const __nv
                 // accumulator (i, h, nt): rows g / g + 8 = columns n and n + 2, n = step base + 4 h + 8 (g >> 1) + (g & 1); ranks 2q, 2q + 1
                 if (live && nb > 0) {
 #pragma unroll
-                    for (int i = 0; i < STEPS; ++i) {
-                        const int kl = (gw + i * GW) * 32;
+                    for (int i = 0; i < LDS_STEPS; ++i) {
+                        const int kl = (warp + i * LDS_CWARPS) * 32;
                         if (kl < chunk_len) {
 #pragma unroll
                             for (int h = 0; h < 2; ++h)
@@ -245,24 +242,24 @@ __device__ __forceinline__ void lora_down_stream(int M, int T, int r, const __nv
                     for (int c = 0; c < 4; ++c) red[(((warp * LDS_MAXB + b) * NT + nt) * 4 + c) * 32 + lane] = acc[b][nt][c];
     }
     __syncthreads();
-    for (int idx = threadIdx.x; idx < nb * RG * NT * 128; idx += blockDim.x) {
-        const int b = idx / (RG * NT * 128), rg = idx / (NT * 128) % RG, nt = (idx >> 7) % NT, c = (idx >> 5) & 3, ln = idx & 31;
+    for (int idx = threadIdx.x; idx < nb * NT * 128; idx += blockDim.x) {
+        const int b = idx / (NT * 128), nt = (idx >> 7) % NT, c = (idx >> 5) & 3, ln = idx & 31;
         float v = 0.f;
-        for (int w = rg * GW; w < (rg + 1) * GW; ++w) v += red[(((w * LDS_MAXB + b) * NT + nt) * 4 + c) * 32 + ln];
+        for (int w = 0; w < LDS_CWARPS; ++w) v += red[(((w * LDS_MAXB + b) * NT + nt) * 4 + c) * 32 + ln];
         const int row = (first_block + b * block_stride) * 16 + (ln >> 2) + ((c & 2) ? 8 : 0);
-        const int col = rg * 16 + nt * 8 + (ln & 3) * 2 + (c & 1);
+        const int col = nt * 8 + (ln & 3) * 2 + (c & 1);
         if (row < M && col < r) P[(size_t)row * r + col] = MASKED ? v * out_scale : v;
     }
     __syncthreads();
 }
 
-// The streaming form beyond plain ranks of up to 16: ranks up to 32, and up to 16 under a mask, from this many tokens on -- wherever the
-// product is formed, so that saved and recomputed H / G have the same bits.  Against a launch of lora_down_split_kernel ahead of the layer (1800
-// tokens, 4096 x 4096, INT4): dropout forward 58.9 -> 51.5 us, backward 71.0 -> 58.0; rank 32 forward 56.7 -> 49.4, backward 55.9 -> 53.1.
-// Below, where the single-CTA kernel mostly runs and cannot host it, the split kernel is the shorter launch.
-constexpr int LDS_WIDE_TOKENS = 1025;
-static bool lds_wide(int M, int r, bool masked) { return M >= LDS_WIDE_TOKENS && r <= (masked ? 16 : 32); }
-constexpr int LDS_WIDE_BLOCKS = 7;                        // row blocks per CTA at ranks 17 to 32 (registers)
+// Under a dropout mask the streaming form is taken from this many tokens on -- wherever the product is formed, so that saved and recomputed H have
+// the same bits.  1800 tokens, 4096 x 4096, INT4, against a launch of lora_down_split_kernel ahead of the layer: dropout forward 58.9 -> 51.5 us
+// (and backward, G beside the tiles, 71.0 -> 58.0).  Below, where the single-CTA kernel mostly runs and cannot host it, the split kernel is
+// the shorter launch.  Ranks 17 to 32, seven warps per 16 of them, were timed and taken out: beside the tiles X A^T came to 57.9 -> 51.5 us at
+// rank 32, but as a launch of its own (H recomputed for the gradients, 33 -> 43 us) the form is slower than the split kernel.
+constexpr int LDS_MASKED_TOKENS = 1025;
+static bool lds_masked(int M, int r) { return M >= LDS_MASKED_TOKENS && r <= 16; }
 
 struct LdsParams {
     int M, T, r, stages, wait_limit_us;
@@ -284,14 +281,12 @@ __global__ void __launch_bounds__(kThreads, 1) lora_down_stream_kernel(const Lds
     pdl_wait();
     const int first = (int)blockIdx.x, stride = (int)gridDim.x;
     if (L_IS_A && p.mask != nullptr) {
-        if (p.r <= 8) lora_down_stream<true, 1, false, LDS_MAXB, 1, true>(p.M, p.T, p.r, p.In, p.L, p.P, first, stride, smem, p.stages, abort_flag_s, nullptr, nullptr, p.mask, p.out_scale);
-        else          lora_down_stream<true, 2, false, LDS_MAXB, 1, true>(p.M, p.T, p.r, p.In, p.L, p.P, first, stride, smem, p.stages, abort_flag_s, nullptr, nullptr, p.mask, p.out_scale);
+        if (p.r <= 8) lora_down_stream<true, 1, false, LDS_MAXB, true>(p.M, p.T, p.r, p.In, p.L, p.P, first, stride, smem, p.stages, abort_flag_s, nullptr, nullptr, p.mask, p.out_scale);
+        else          lora_down_stream<true, 2, false, LDS_MAXB, true>(p.M, p.T, p.r, p.In, p.L, p.P, first, stride, smem, p.stages, abort_flag_s, nullptr, nullptr, p.mask, p.out_scale);
     } else if (p.r <= 8) {
         lora_down_stream<L_IS_A, 1>(p.M, p.T, p.r, p.In, p.L, p.P, first, stride, smem, p.stages, abort_flag_s);
-    } else if (p.r <= 16) {
-        lora_down_stream<L_IS_A, 2>(p.M, p.T, p.r, p.In, p.L, p.P, first, stride, smem, p.stages, abort_flag_s);
     } else {
-        lora_down_stream<L_IS_A, 2, false, LDS_WIDE_BLOCKS, 2>(p.M, p.T, p.r, p.In, p.L, p.P, first, stride, smem, p.stages, abort_flag_s);
+        lora_down_stream<L_IS_A, 2>(p.M, p.T, p.r, p.In, p.L, p.P, first, stride, smem, p.stages, abort_flag_s);
     }
     if (abort_flag_s[0]) {   // give copies that may still be in flight time to land before the CTA's memory is released
         for (int i = 0; i < 200; ++i) __nanosleep(1000);
@@ -299,13 +294,13 @@ __global__ void __launch_bounds__(kThreads, 1) lora_down_stream_kernel(const Lds
     }
 }
 
-// Stand-alone launch: one CTA per SM at most, each with up to LDS_MAXB (LDS_WIDE_BLOCKS) row blocks.
+// Stand-alone launch (r <= 16): one CTA per SM at most, each with up to LDS_MAXB row blocks.
 int launch_lora_down_stream_impl(int M, int T, int r, bool l_is_A, const void* In, const void* L, float* P, cudaStream_t st, const uint8_t* mask,
                                  float out_scale) {
     if (M == 0 || r == 0) return QLORA_OK;
-    const int n_blocks = (M + 15) / 16, most = r > 16 ? LDS_WIDE_BLOCKS : LDS_MAXB;
+    const int n_blocks = (M + 15) / 16;
     int grid = n_blocks < sm_count() ? n_blocks : sm_count();
-    if ((n_blocks + grid - 1) / grid > most) grid = (n_blocks + most - 1) / most;   // several waves of CTAs
+    if ((n_blocks + grid - 1) / grid > LDS_MAXB) grid = (n_blocks + LDS_MAXB - 1) / LDS_MAXB;   // several waves of CTAs
     LdsParams p{};
     p.M = M; p.T = T; p.r = r; p.stages = mask != nullptr ? 4 : 6; p.wait_limit_us = kWaitLimitUs;
     p.In = (const __nv_bfloat16*)In; p.L = (const __nv_bfloat16*)L; p.P = P;

@@ -145,7 +145,7 @@ __device__ __forceinline__ void lg_cluster_sync() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// Ranks above 8 (above 16 with many rows), or a dropout mask: 16 token rows per cluster, the contraction split over its 1 << lcs CTAs and their eight warps.
+// Ranks above 8 (above 16 with many rows), or a dropout mask (with many rows, ranks above 16): 16 token rows per cluster, the contraction split over its 1 << lcs CTAs and their eight warps.
 // Bound by the latency of the adapter and activation loads (the adapter's share of the loads grows with the rank), so a warp issues
 // all loads of DEPTH 32-wide steps together, and the cluster is as wide as keeps two CTAs per SM: 2048 tokens x 4096, rank 32,
 // inputs from DRAM: 18 -> 10 us (blocks of eight warps that waited for every step's adapter words before).
@@ -269,7 +269,7 @@ int launch_lora_down(int M, int T, int r, bool l_is_A, const void* In, const voi
     const bool plain = mask == nullptr && out_scale == 1.0f && r <= 16;
     // Many rows, low rank: the streaming kernel (also the form that runs inside the CTA-pair kernel, so H / G have the
     // same bits whichever call produced them).
-    if ((plain && M > 256) || lora_down_streams_wide(M, r, mask != nullptr)) return launch_lora_down_stream(M, T, r, l_is_A, In, L, P, st, mask, out_scale);
+    if ((plain && M > 256) || (mask != nullptr && l_is_A && lora_down_streams_masked(M, r))) return launch_lora_down_stream(M, T, r, l_is_A, In, L, P, st, mask, out_scale);
     const unsigned blocks = (unsigned)((M + 15) / 16);
     const __nv_bfloat16* in = (const __nv_bfloat16*)In;
     const __nv_bfloat16* l = (const __nv_bfloat16*)L;

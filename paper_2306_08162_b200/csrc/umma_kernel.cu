@@ -947,7 +947,7 @@ int launch_impl(const CUtensorMap& ta, const CUtensorMap& tq, const CUtensorMap&
 int launch_lora_down_stream(int M, int T, int r, bool l_is_A, const void* In, const void* L, float* P, cudaStream_t st, const uint8_t* mask, float out_scale) {
     return launch_lora_down_stream_impl(M, T, r, l_is_A, In, L, P, st, mask, out_scale);
 }
-bool lora_down_streams_wide(int M, int r, bool masked) { return lds_wide(M, r, masked); }
+bool lora_down_streams_masked(int M, int r) { return lds_masked(M, r); }
 
 static int keep_lora_low(const qlora_desc& d) { return d.r == 8 || d.group_size == 32 ? 1 : 0; }
 
@@ -1047,10 +1047,7 @@ static int launch_umma_pair(const qlora_desc& d, int M, bool transposed, const v
     p.lds_stages = (int)((p.off_bar - LDS_BAR_BYTES) / lds_stage);
     if (p.lds_stages > 6) p.lds_stages = 6;
     const bool ring_fits = p.lds_stages * lds_stage >= LDS_MIN_STAGES * LDS_STAGE_BYTES;    // (the ring also holds the reduction)
-    // row blocks per producer CTA (ranks above 16, backward: at seven the producers, which gather B's words, came after the tiles: 2048 tokens,
-    // 4096 x 4096, rank 32, 57.8 us against 56.6 with a launch ahead)
-    const int max_blocks = p.r_down > 16 ? (transposed ? LDS_WIDE_BLOCKS - 1 : LDS_WIDE_BLOCKS) : LDS_MAXB;
-    const bool r_fits = (p.mask == nullptr && p.r_down <= 16) || lds_wide(M, p.r_down, p.mask != nullptr);   // (the forms that a launch of its own takes too)
+    const bool r_fits = p.mask != nullptr ? lds_masked(M, p.r_down) : p.r_down <= 16;       // (the forms that a launch of its own takes too)
     // P = In * Ldown still to be computed (Ldown given): on SM pairs the tiles leave idle when those can take all row
     // blocks (they are then done well before the tiles' contractions are), else by a launch ahead of this one.  Both sum
     // in the same order.  producers(last) = how many pairs would do it when the last wave has `last` items (0: none can).
@@ -1062,7 +1059,7 @@ static int launch_umma_pair(const qlora_desc& d, int M, bool transposed, const v
         const int idle = p.n_tiles < pairs ? pairs - p.n_tiles : (last ? pairs - last : 0);
         int n_prod = (n_blocks + 3) / 4;                     // four row blocks per producer CTA pair when there is room
         if (n_prod > idle) n_prod = idle;
-        const bool fits = want_p && (sync != nullptr || d.r == 0) && r_fits && n_prod > 0 && n_prod * 2 * max_blocks >= n_blocks && ring_fits;
+        const bool fits = want_p && (sync != nullptr || d.r == 0) && r_fits && n_prod > 0 && n_prod * 2 * LDS_MAXB >= n_blocks && ring_fits;
         return fits ? n_prod : 0;
     };
     // A partly filled last wave (more tiles than pairs, at most half a wave left over): each left-over tile goes to two

@@ -236,14 +236,13 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
         if constexpr (!TRANSPOSED) {
             if (p.mask != nullptr) {
                 done_here = true;
-                if (p.r_down <= 8) lora_down_stream<true, 1, false, LDS_MAXB, 1, true>(p.M, p.T, p.r_down, p.In, p.Ldown, p.Pout, (int)blockIdx.x, 2 * p.n_prod, smem_gen, p.lds_stages, abort_flag, nullptr, nullptr, p.mask, p.out_scale);
-                else               lora_down_stream<true, 2, false, LDS_MAXB, 1, true>(p.M, p.T, p.r_down, p.In, p.Ldown, p.Pout, (int)blockIdx.x, 2 * p.n_prod, smem_gen, p.lds_stages, abort_flag, nullptr, nullptr, p.mask, p.out_scale);
+                if (p.r_down <= 8) lora_down_stream<true, 1, false, LDS_MAXB, true>(p.M, p.T, p.r_down, p.In, p.Ldown, p.Pout, (int)blockIdx.x, 2 * p.n_prod, smem_gen, p.lds_stages, abort_flag, nullptr, nullptr, p.mask, p.out_scale);
+                else               lora_down_stream<true, 2, false, LDS_MAXB, true>(p.M, p.T, p.r_down, p.In, p.Ldown, p.Pout, (int)blockIdx.x, 2 * p.n_prod, smem_gen, p.lds_stages, abort_flag, nullptr, nullptr, p.mask, p.out_scale);
             }
         }
         if (!done_here) {
-            if (p.r_down <= 8)       lora_down_stream<!TRANSPOSED, 1>(p.M, p.T, p.r_down, p.In, p.Ldown, p.Pout, (int)blockIdx.x, 2 * p.n_prod, smem_gen, p.lds_stages, abort_flag);
-            else if (p.r_down <= 16) lora_down_stream<!TRANSPOSED, 2>(p.M, p.T, p.r_down, p.In, p.Ldown, p.Pout, (int)blockIdx.x, 2 * p.n_prod, smem_gen, p.lds_stages, abort_flag);
-            else                     lora_down_stream<!TRANSPOSED, 2, false, LDS_WIDE_BLOCKS, 2>(p.M, p.T, p.r_down, p.In, p.Ldown, p.Pout, (int)blockIdx.x, 2 * p.n_prod, smem_gen, p.lds_stages, abort_flag);
+            if (p.r_down <= 8) lora_down_stream<!TRANSPOSED, 1>(p.M, p.T, p.r_down, p.In, p.Ldown, p.Pout, (int)blockIdx.x, 2 * p.n_prod, smem_gen, p.lds_stages, abort_flag);
+            else               lora_down_stream<!TRANSPOSED, 2>(p.M, p.T, p.r_down, p.In, p.Ldown, p.Pout, (int)blockIdx.x, 2 * p.n_prod, smem_gen, p.lds_stages, abort_flag);
         }
         __threadfence();       // every thread's rows of P (and of its part of dB) are visible device-wide before the CTA is counted
         __syncthreads();

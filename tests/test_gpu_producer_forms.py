@@ -1,6 +1,6 @@
 """The down-projection forms of the CTA-pair kernel's producer clusters beyond plain ranks of up to 16: under a dropout mask (forward), for a
-product the tiles do not use (backward under dropout), and ranks 17 to 32 -- on pairs without a tile and on pairs that take tiles
-afterwards, with ragged rows and a last chunk that is not full."""
+product the tiles do not use (backward under dropout) -- on pairs without a tile and on pairs that take tiles
+afterwards, with ragged rows and a last chunk that is not full -- and ranks 17 to 32 at such sizes."""
 import numpy as np
 import pytest
 import torch
@@ -46,7 +46,7 @@ def test_dropout_beside_the_tiles(M, K, N, r):
 
 
 @pytest.mark.parametrize("M,K,N,r", [(1100, 1088, 512, 24), (1100, 256, 10240, 32), (1100, 10240, 256, 32)])
-def test_ranks_17_to_32_beside_the_tiles(M, K, N, r):
+def test_ranks_17_to_32_many_tokens(M, K, N, r):
     layer = qi.random_codes_layer(K=K, N=N, bits=4, group_size=64, r=r, alpha=2.0 * r, M=M, seed=M + K + r)
     gl = GpuLayer(layer)
     saved = gl.run()
