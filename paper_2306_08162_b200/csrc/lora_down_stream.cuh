@@ -256,7 +256,7 @@ __device__ __forceinline__ void lora_down_stream(int M, int T, int r, const __nv
 // Under a dropout mask the streaming form is taken from this many tokens on -- wherever the product is formed, so that saved and recomputed H have
 // the same bits.  1800 tokens, 4096 x 4096, INT4, against a launch of lora_down_split_kernel ahead of the layer: dropout forward 58.9 -> 51.5 us
 // (and backward, G beside the tiles, 71.0 -> 58.0).  Below, where the single-CTA kernel mostly runs and cannot host it, the split kernel is
-// the shorter launch.  Ranks 17 to 32, seven warps per 16 of them, were timed and taken out: beside the tiles X A^T came to 57.9 -> 51.5 us at
+// the shorter launch.  (Gradients that recompute H: 1100 tokens 29.0 -> 32.2 us, 1800 38.0 -> 36.3, 4096 63.8 -> 59.3.)  Ranks 17 to 32, seven warps per 16 of them, were timed and taken out: beside the tiles X A^T came to 57.9 -> 51.5 us at
 // rank 32, but as a launch of its own (H recomputed for the gradients, 33 -> 43 us) the form is slower than the split kernel.
 constexpr int LDS_MASKED_TOKENS = 1025;
 static bool lds_masked(int M, int r) { return M >= LDS_MASKED_TOKENS && r <= 16; }
