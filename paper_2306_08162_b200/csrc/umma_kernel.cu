@@ -16,7 +16,8 @@
 //
 // Warp roles (480 threads): warp 0 = TMA producer of activation tiles, warp 1 = MMA issuer (+ tensor-memory
 // allocation), warp 2 = TMA producer of packed codes + group parameters (its ring runs ahead of the activation ring),
-// warps 3-6 = epilogue (+ LoRA operand staging), warps 7-14 = unpack/dequant (two groups taking alternate stages).
+// warps 3-6 = epilogue (+ LoRA operand staging), warps 7-14 = unpack/dequant (two groups taking alternate stages).  In the DOWN
+// build warps 3-14 are three dequant groups, and all warps finish the tile.
 // Every mbarrier wait is bounded; on a timeout the kernel records a status word, drains and returns.
 #include <cuda.h>
 
