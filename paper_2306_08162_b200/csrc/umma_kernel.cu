@@ -27,6 +27,7 @@
 #include "device_state.h"
 #include "launch.h"
 #include "lora_down.cuh"
+#include "umma_plan.h"
 
 namespace qlora {
 
@@ -44,23 +45,11 @@ constexpr int kDequantWarp0 = 7, kGroupWarps = 4;   // two dequant groups of fou
 constexpr int kEpiWarp0 = 3, kEpiWarps = 4;
 constexpr int kSyncWords = 64;                       // counters in the workspace: [0], [1] producer clusters, [2 ..] one per split tile
 constexpr size_t kSplitTileBytes = 2 * 2 * 8 * 8 * 128 * 16;   // exchange area of one split tile: 2 halves x 2 CTAs x 8 chunks x 4 KiB
-constexpr int kWRows = 128;          // weight rows (MMA M) per tile: n in forward, k in backward
-constexpr int kStepC = 64;           // contraction elements per pipeline stage
-constexpr int kWStageBytes = kWRows * kStepC * 2;   // 16 KiB of bf16 per stage
 constexpr int kAccStride = 256;      // tensor-memory columns per accumulator buffer
-// contraction steps that a rank of a split tile has at least, up to 128 tokens and above (512 x 512, rank 8: four ranks of two steps against two
-// of four 5.1 / 5.7 us at 17 tokens, 7.6 / 8.3 at 128, but 11.8 / 10.6 at 256: what the ranks exchange grows with the tokens)
-constexpr int kMinSplitSteps = 2, kMinSplitSteps256 = 4;
-constexpr int kMaxDownTokens = 128;
-// Up to 128 tokens, where a split tile's ranks form P themselves.  Their MMAs cost some 250 cycles per step, the producer clusters a launch, a
-// counter and a chain that grows with the rank; two ranks have more of the tile to exchange and less room to gain.  INT4, forward, 64
-// tokens, rank 8: 512 x 512 8.3 -> 6.6 us, 1024 x 1024 8.6 -> 6.8, INT3 2048 x 2048 9.05 -> 8.1; 4096 x 4096, 16 steps, 128 tokens 16.3 -> 15.1;
-// 8192 -> 2048, 32 steps, 64 tokens 16.4 -> 16.9, but rank 16 19.3 -> 17.3; two ranks of 16 steps, 128 tokens 13.2 -> 14.9.
-static bool down_pays(int split, int steps, int r) { return steps <= 8 || (split == 4 && (r == 16 || steps <= 16)); }
 constexpr uint32_t kSpinLimit = 1u << 26;
 constexpr int kWaitLimitUs = 250000;   // default limit of a wait, a launch parameter: far beyond any healthy wait (microseconds), short for a hang
 
-struct Params {
+struct Params : TilePlan {
     int M, N, K, bits, g, r, r_pad;
     // r_pad: columns of the LoRA operands, a multiple of 16.  lora_lo: ranks [r, 2r) hold, beside the finite ones of the same adapter
     // elements again, what the rounding of s * P to bf16 left over, so that the update has 16 significant bits of P's 24: for r == 8,
@@ -68,16 +57,6 @@ struct Params {
     // (the error of Y and dX against 64 bits is the same with it: that of the weights' and outputs' bf16).
     int lora_lo;
     int C;               // output columns (N forward, K backward)
-    int BT;              // token rows per tile (MMA N): a multiple of 16, 32 .. 256
-    int n_tok_tiles, n_tiles, steps;
-    int split;           // CTAs per cluster sharing one tile, each taking `steps` consecutive steps of the contraction (1 = no cluster)
-    int S, P;            // stages of the activation/weight ring and of the packed ring
-    int packed_cols;     // 128 forward, 64 backward
-    int packed_rows;     // int32 rows per stage
-    int scale_rows;      // group rows per stage
-    uint32_t words_bytes, scale_bytes, packed_slot_bytes, x_stage_bytes;
-    uint32_t off_x, off_w, off_l, off_p, off_lora_a, off_lora_p, off_bar;   // offsets from the 1024-aligned smem base
-    uint32_t down_bytes;             // DOWN: bytes per stage of the adapter applied first (else 0)
     float s;
     const float* Pmat;               // H (forward) or G (backward), fp32 [M, r]
     const __nv_bfloat16* L;          // B [N, r] (forward) or A [r, K] (backward)
@@ -950,14 +929,6 @@ int launch_lora_down_stream(int M, int T, int r, bool l_is_A, const void* In, co
 }
 bool lora_down_streams_masked(int M, int r) { return lds_masked(M, r); }
 
-static int keep_lora_low(const qlora_desc& d) { return d.r == 8 || d.group_size == 32 ? 1 : 0; }
-
-// Rows of scales / zeros that go with the k range of one pipeline stage (64 rows of W forward, 128 backward).
-static int scale_rows_per_stage(const qlora_desc& d, bool transposed) {
-    const int k_rows = transposed ? kWRows : kStepC;
-    return d.group_size >= k_rows ? 1 : k_rows / d.group_size;
-}
-
 bool umma_supported(const qlora_desc& d, int M) {
     if (M < 1) return false;
     if (d.K % 64 != 0 || d.N % 64 != 0) return false;              // contraction steps of 64 in both directions
@@ -1003,36 +974,23 @@ static int launch_umma_pair(const qlora_desc& d, int M, bool transposed, const v
     // plan_only: nothing is launched and no pointer is looked at; the return value is the number of producer pairs when a
     // backward call with every optional workspace area would form dB on them, else 0
     PairParams p{};
-    p.M = M; p.N = d.N; p.K = d.K; p.bits = d.bits; p.g = d.group_size; p.r = d.r; p.lora_lo = keep_lora_low(d); p.r_pad = ((p.lora_lo ? 2 : 1) * d.r + 15) / 16 * 16;
+    p.M = M; p.N = d.N; p.K = d.K; p.bits = d.bits; p.g = d.group_size; p.r = d.r; p.lora_lo = keep_lora_low(d.r, d.group_size); p.r_pad = lora_columns(d.r, d.group_size);
     p.C = transposed ? d.K : d.N;
     const int T = transposed ? d.N : d.K;
     p.n_tok_tiles = (M + 4 * kPairTok - 1) / (4 * kPairTok);
     const int n_w_tiles = (p.C + 2 * kPairW - 1) / (2 * kPairW);
     p.n_tiles = p.n_tok_tiles * n_w_tiles;
     p.steps = T / kStepC;
-    p.packed_cols = transposed ? 64 : 128;
-    p.packed_rows = (transposed ? 128 : 64) * d.bits / 32;
-    p.scale_rows = scale_rows_per_stage(d, transposed);
-    p.words_bytes = (uint32_t)(p.packed_rows * p.packed_cols * 4);
-    p.scale_bytes = (uint32_t)(p.scale_rows * p.packed_cols * 2);
-    p.packed_slot_bytes = (p.words_bytes + 2 * p.scale_bytes + 127u) / 128u * 128u;
+    static_cast<PackedStage&>(p) = plan_packed_stage(d.bits, d.group_size, transposed);
     p.s = d.r > 0 ? d.alpha / (float)d.r : 0.f;
     p.Pmat = Pmat; p.L = (const __nv_bfloat16*)L; p.Out = (__nv_bfloat16*)Out;
 
     uint32_t lora_l = (uint32_t)(kPairW * p.r_pad * 2), lora_p = (uint32_t)(2 * kPairTok * p.r_pad * 2);
     if (lora_l + lora_p < 8192) lora_p = 8192 - lora_l;   // the area doubles as the epilogue's staging slices (4 warps x 2 KiB)
-    const uint32_t budget = 232448 - 1024 /*alignment slack*/ - 2048 /*static, barriers, padding*/;
-    const uint32_t per_stage = kPairXStage + kWStageBytes;
-    int S = 0;
-    for (p.P = 4; p.P >= 2 && S < 2; --p.P)                 // (the packed ring gives way where the LoRA operands are at their largest)
-        S = (int)((budget - (lora_l + lora_p + p.P * p.packed_slot_bytes + 512)) / per_stage);
-    ++p.P;
-    if (S > 8) S = 8;
-    if (S < 2) return QLORA_ERR_UNSUPPORTED;
-    p.S = S;
+    if (!plan_pair_rings(p.packed_slot_bytes, lora_l + lora_p, p.S, p.P)) return QLORA_ERR_UNSUPPORTED;
     p.off_x = 0;
-    p.off_w = p.off_x + S * kPairXStage;
-    p.off_p = p.off_w + S * kWStageBytes;
+    p.off_w = p.off_x + p.S * kPairXStage;
+    p.off_p = p.off_w + p.S * kWStageBytes;
     p.off_lora_l = p.off_p + p.P * p.packed_slot_bytes;
     p.off_lora_p = p.off_lora_l + lora_l;
     p.off_bar = (p.off_lora_p + lora_p + 127u) / 128u * 128u;
@@ -1159,60 +1117,13 @@ int launch_umma_gemm(const qlora_desc& d, int M, bool transposed, const void* In
         Ldown = nullptr;
     }
     Params p{};
-    p.M = M; p.N = d.N; p.K = d.K; p.bits = d.bits; p.g = d.group_size; p.r = d.r; p.lora_lo = keep_lora_low(d); p.r_pad = ((p.lora_lo ? 2 : 1) * d.r + 15) / 16 * 16;
+    p.M = M; p.N = d.N; p.K = d.K; p.bits = d.bits; p.g = d.group_size; p.r = d.r; p.lora_lo = keep_lora_low(d.r, d.group_size); p.r_pad = lora_columns(d.r, d.group_size);
     p.C = transposed ? d.K : d.N;
     const int T = transposed ? d.N : d.K;
-    // The tokens in as few tiles as 256 columns allow, cut evenly: a multiple of 16 (the MMA's N), not the next power of two, so that
-    // neither products nor the exchange between the ranks are made for tokens that do not exist (333: two tiles of 176, not 256).
-    p.n_tok_tiles = (M + 255) / 256;
-    p.BT = ((M + p.n_tok_tiles - 1) / p.n_tok_tiles + 15) / 16 * 16;
-    if (p.BT < 32) p.BT = 32;
-    p.n_tok_tiles = (M + p.BT - 1) / p.BT;
-    const int n_w_tiles = (p.C + kWRows - 1) / kWRows;
-    p.n_tiles = p.n_tok_tiles * n_w_tiles;
-    p.steps = T / kStepC;
-    p.packed_cols = transposed ? 64 : 128;
-    p.packed_rows = (transposed ? 128 : 64) * d.bits / 32;
-    p.scale_rows = scale_rows_per_stage(d, transposed);
-    p.words_bytes = (uint32_t)(p.packed_rows * p.packed_cols * 4);
-    p.scale_bytes = (uint32_t)(p.scale_rows * p.packed_cols * 2);
-    p.packed_slot_bytes = (p.words_bytes + 2 * p.scale_bytes + 127u) / 128u * 128u;
-    p.x_stage_bytes = (uint32_t)(p.BT * 128);
+    if (!plan_tiles(p, d.bits, d.group_size, d.r, p.r_pad, M, p.C, T, transposed, Ldown != nullptr, sm_count())) return QLORA_ERR_UNSUPPORTED;
     p.s = d.r > 0 ? d.alpha / (float)d.r : 0.f;
     p.Pmat = Pmat; p.L = (const __nv_bfloat16*)L; p.Out = (__nv_bfloat16*)Out;
 
-    // shared-memory plan (offsets from a 1024-byte aligned base)
-    const uint32_t lora_a = (uint32_t)(kWRows * p.r_pad * 2), lora_p = (uint32_t)(p.BT * p.r_pad * 2);
-    const uint32_t budget = 232448 - 1024 /*alignment slack*/ - 2048 /*static, barriers, padding*/;
-    // With few tokens the kernel is bound by the latency of streaming cold packed weights through a handful of CTAs,
-    // so the packed ring is deep (bytes in flight), at the cost of one or two operand stages.
-    auto plan = [&](int split) {
-        p.split = split;
-        p.down_bytes = split > 1 && Ldown != nullptr && (d.r == 8 || d.r == 16) && p.BT <= kMaxDownTokens && down_pays(split, p.steps / split, d.r) ? (uint32_t)d.r * 128u : 0u;
-        const uint32_t per_stage = p.x_stage_bytes + kWStageBytes + p.down_bytes;
-        uint32_t S = 0;
-        for (p.P = p.BT <= 128 ? 16 : 8;; p.P -= p.P > 4 ? 4 : 1) {   // the packed ring gives way until three operand stages fit (two, below four slots)
-            const uint32_t fixed = lora_a + lora_p + p.P * p.packed_slot_bytes + 512;
-            S = budget > fixed ? (budget - fixed) / per_stage : 0;
-            if (S >= (p.P > 4 ? 3 : 2) || p.P == 2) break;
-        }
-        if (S > 8) S = 8;
-        p.S = (int)S;
-        p.off_x = 0;
-        p.off_w = p.off_x + S * p.x_stage_bytes;
-        p.off_l = p.off_w + S * kWStageBytes;
-        p.off_p = p.off_l + S * p.down_bytes;
-        p.off_lora_a = p.off_p + p.P * p.packed_slot_bytes;
-        p.off_lora_p = p.off_lora_a + lora_a;
-        p.off_bar = (p.off_lora_p + lora_p + 127u) / 128u * 128u;
-        return S >= 2 && (split == 1 || (uint32_t)(p.BT * (kWRows + (p.down_bytes ? d.r : 0)) * 4) <= p.off_p);
-    };
-    // Few tiles (few tokens): split each tile's contraction over a cluster of 2 or 4 CTAs so that the whole GPU streams
-    // the weights.  Needs one tile per cluster, an even split of the steps, and room for the fp32 parts in the operand ring.
-    int split = 1;
-    for (int sp = 4; sp >= 2 && split == 1; sp /= 2)
-        if (p.n_tiles * sp <= sm_count() && p.steps % sp == 0 && p.steps / sp >= (p.BT <= kMaxDownTokens ? kMinSplitSteps : kMinSplitSteps256) && p.BT % sp == 0 && plan(sp)) split = sp;
-    if (split == 1 && !plan(1)) return QLORA_ERR_UNSUPPORTED;
     const size_t smem_bytes = (size_t)p.off_bar + 512 + 1024;
 
     CUtensorMap ta, tq, ts, tz, tl{};
@@ -1222,7 +1133,6 @@ int launch_umma_gemm(const qlora_desc& d, int M, bool transposed, const void* In
         !make_map_2d(&tz, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, zeros, (uint64_t)d.N, (uint64_t)(d.K / d.group_size), (uint32_t)p.packed_cols, (uint32_t)p.scale_rows, CU_TENSOR_MAP_SWIZZLE_NONE))
         return QLORA_ERR_CUDA;
 
-    p.steps /= p.split;
     const int grid = p.split > 1 ? p.n_tiles * p.split : (p.n_tiles < sm_count() ? p.n_tiles : sm_count());
     if (p.down_bytes != 0 &&
         !(transposed ? make_map_2d(&tl, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Ldown, (uint64_t)d.r, (uint64_t)T, 8, 64, CU_TENSOR_MAP_SWIZZLE_NONE)

@@ -1,0 +1,137 @@
+// How the tensor-core kernels cut a layer call: token tiles, ranks per tile, ring lengths and the layout of shared memory.  Host code without
+// CUDA, so that its rules can be checked over all shapes on the CPU.
+#pragma once
+#include <stdint.h>
+
+namespace qlora {
+
+constexpr int kWRows = 128;          // weight rows (MMA M) per tile: n in forward, k in backward
+constexpr int kStepC = 64;           // contraction elements per pipeline stage
+constexpr int kWStageBytes = kWRows * kStepC * 2;   // 16 KiB of bf16 per stage
+constexpr int kPairTok = 128;                          // CTA-pair kernel: token rows per CTA per accumulator
+constexpr int kPairW = 128;                            // weight rows per CTA (256 per pair tile)
+constexpr int kPairXSub = kPairTok * kStepC * 2;       // 16 KiB: one 128-token sub-tile of a stage
+constexpr int kPairXStage = 2 * kPairXSub;             // two accumulators' sub-tiles
+constexpr int kDequantGroups = 2, kDownGroups = 3;     // dequant groups, and in the DOWN build
+constexpr uint32_t kSmemBudget = 232448 - 1024 /*alignment slack*/ - 2048 /*static, barriers, padding*/;
+// contraction steps that a rank of a split tile has at least, up to 128 tokens and above (512 x 512, rank 8: four ranks of two steps against two
+// of four 5.1 / 5.7 us at 17 tokens, 7.6 / 8.3 at 128, but 11.8 / 10.6 at 256: what the ranks exchange grows with the tokens)
+constexpr int kMinSplitSteps = 2, kMinSplitSteps256 = 4;
+constexpr int kMaxDownTokens = 128;
+
+// Whether `groups` dequant groups that take the stages of a tile in turn may run on an operand ring of S stages and a packed ring of P slots.
+// A group tells the laps of a slot apart by one parity bit, so whoever waits for lap l must know that lap l - 1 is over.  A group that is about to
+// take step t has seen the MMAs of step t - groups - S through (it waited for that stage to be free), hence of all steps before it:
+//   - the stage of step t was last but one used by step t - 2 S, which is over when S >= groups;
+//   - the slot of step t was last filled for step t - P: over when P >= S + groups, or when that step was this very group's (P a multiple of groups).
+// Else a wait may return a lap early, on codes that have not landed.
+inline bool rings_sound(int S, int P, int groups) { return S >= groups && (P % groups == 0 || P >= S + groups); }
+
+// Rows of scales / zeros that go with the k range of one pipeline stage (64 rows of W forward, 128 backward).
+inline int scale_rows_per_stage(int g, bool transposed) {
+    const int k_rows = transposed ? kWRows : kStepC;
+    return g >= k_rows ? 1 : k_rows / g;
+}
+
+// Whether the LoRA operands carry what the rounding of s * P to bf16 left over (Params::lora_lo), and their columns, a multiple of 16.
+inline int keep_lora_low(int r, int g) { return r == 8 || g == 32 ? 1 : 0; }
+inline int lora_columns(int r, int g) { return ((keep_lora_low(r, g) ? 2 : 1) * r + 15) / 16 * 16; }
+
+struct PackedStage {
+    int packed_cols;     // 128 forward, 64 backward
+    int packed_rows;     // int32 rows per stage
+    int scale_rows;      // group rows per stage
+    uint32_t words_bytes, scale_bytes, packed_slot_bytes;
+};
+inline PackedStage plan_packed_stage(int bits, int g, bool transposed) {
+    PackedStage s;
+    s.packed_cols = transposed ? 64 : 128;
+    s.packed_rows = (transposed ? 128 : 64) * bits / 32;
+    s.scale_rows = scale_rows_per_stage(g, transposed);
+    s.words_bytes = (uint32_t)(s.packed_rows * s.packed_cols * 4);
+    s.scale_bytes = (uint32_t)(s.scale_rows * s.packed_cols * 2);
+    s.packed_slot_bytes = (s.words_bytes + 2 * s.scale_bytes + 127u) / 128u * 128u;
+    return s;
+}
+
+// Single-CTA kernel.  Offsets count from the 1024-byte aligned base of shared memory.
+struct TilePlan : PackedStage {
+    int BT;              // token rows per tile (MMA N): a multiple of 16, 32 .. 256
+    int n_tok_tiles, n_tiles, steps;   // steps: of one rank
+    int split;           // CTAs per cluster sharing one tile, each taking `steps` consecutive steps of the contraction (1 = no cluster)
+    int S, P;            // stages of the activation/weight ring and of the packed ring
+    uint32_t x_stage_bytes;
+    uint32_t off_x, off_w, off_l, off_p, off_lora_a, off_lora_p, off_bar;
+    uint32_t down_bytes;             // DOWN: bytes per stage of the adapter applied first (else 0)
+};
+
+// Up to 128 tokens, where a split tile's ranks form P themselves.  Their MMAs cost some 250 cycles per step, the producer clusters a launch, a
+// counter and a chain that grows with the rank; two ranks have more of the tile to exchange and less room to gain.  INT4, forward, 64
+// tokens, rank 8: 512 x 512 8.3 -> 6.6 us, 1024 x 1024 8.6 -> 6.8, INT3 2048 x 2048 9.05 -> 8.1; 4096 x 4096, 16 steps, 128 tokens 16.3 -> 15.1;
+// 8192 -> 2048, 32 steps, 64 tokens 16.4 -> 16.9, but rank 16 19.3 -> 17.3; two ranks of 16 steps, 128 tokens 13.2 -> 14.9.
+inline bool down_pays(int split, int steps, int r) { return steps <= 8 || (split == 4 && (r == 16 || steps <= 16)); }
+
+// Rings and layout for `split` ranks per tile, `total_steps` steps among them; with_down: the DOWN build.  False: does not fit.
+inline bool plan_rings(TilePlan& p, int split, int total_steps, int r, int r_pad, bool with_down) {
+    p.split = split;
+    p.steps = total_steps / split;
+    p.down_bytes = with_down ? (uint32_t)r * 128u : 0u;
+    const uint32_t lora_a = (uint32_t)(kWRows * r_pad * 2), lora_p = (uint32_t)(p.BT * r_pad * 2);
+    const uint32_t per_stage = p.x_stage_bytes + kWStageBytes + p.down_bytes;
+    // With few tokens the kernel is bound by the latency of streaming cold packed weights through a handful of CTAs, so the packed ring is
+    // deep (bytes in flight), at the cost of one or two operand stages; it gives way until three of those fit (two, at four slots and below).
+    // Lengths are even: three slots beside two stages are none that two groups may use (rings_sound).  Only INT8 with groups of 32 at rank 64 ever had them:
+    // with two, 250 tokens on 4096 x 4096 49.6 -> 52.7 us forward, 50.1 -> 55.6 backward, in the CTA-pair kernel nothing.
+    uint32_t S = 0;
+    for (p.P = p.BT <= 128 ? 16 : 8;; p.P -= p.P > 4 ? 4 : 2) {
+        const uint32_t fixed = lora_a + lora_p + p.P * p.packed_slot_bytes + 512;
+        S = kSmemBudget > fixed ? (kSmemBudget - fixed) / per_stage : 0;
+        if (S >= (p.P > 4 ? 3u : 2u) || p.P == 2) break;
+    }
+    if (S > 8) S = 8;
+    p.S = (int)S;
+    p.off_x = 0;
+    p.off_w = p.off_x + S * p.x_stage_bytes;
+    p.off_l = p.off_w + S * kWStageBytes;
+    p.off_p = p.off_l + S * p.down_bytes;
+    p.off_lora_a = p.off_p + p.P * p.packed_slot_bytes;
+    p.off_lora_p = p.off_lora_a + lora_a;
+    p.off_bar = (p.off_lora_p + lora_p + 127u) / 128u * 128u;
+    // a split tile's fp32 parts (and those of P) meet in the operand ring
+    return rings_sound(p.S, p.P, with_down ? kDownGroups : kDequantGroups) &&
+           (split == 1 || (uint32_t)(p.BT * (kWRows + (with_down ? r : 0)) * 4) <= p.off_p);
+}
+
+// M tokens, C output columns, T contraction elements.  wants_p: P = In * Ldown is still to be computed.  False: the shape does not fit.
+inline bool plan_tiles(TilePlan& p, int bits, int g, int r, int r_pad, int M, int C, int T, bool transposed, bool wants_p, int sms) {
+    static_cast<PackedStage&>(p) = plan_packed_stage(bits, g, transposed);
+    // The tokens in as few tiles as 256 columns allow, cut evenly: a multiple of 16 (the MMA's N), not the next power of two, so that
+    // neither products nor the exchange between the ranks are made for tokens that do not exist (333: two tiles of 176, not 256).
+    p.n_tok_tiles = (M + 255) / 256;
+    p.BT = ((M + p.n_tok_tiles - 1) / p.n_tok_tiles + 15) / 16 * 16;
+    if (p.BT < 32) p.BT = 32;
+    p.n_tok_tiles = (M + p.BT - 1) / p.BT;
+    p.n_tiles = p.n_tok_tiles * ((C + kWRows - 1) / kWRows);
+    p.x_stage_bytes = (uint32_t)(p.BT * 128);
+    // Few tiles (few tokens): split each tile's contraction over a cluster of 2 or 4 CTAs so that the whole GPU streams
+    // the weights.  Needs one tile per cluster, an even split of the steps, and room for the fp32 parts in the operand ring.
+    const int steps = T / kStepC;
+    for (int sp = 4; sp >= 2; sp /= 2) {
+        if (p.n_tiles * sp > sms || steps % sp != 0 || steps / sp < (p.BT <= kMaxDownTokens ? kMinSplitSteps : kMinSplitSteps256) || p.BT % sp != 0) continue;
+        if (wants_p && (r == 8 || r == 16) && p.BT <= kMaxDownTokens && down_pays(sp, steps / sp, r) && plan_rings(p, sp, steps, r, r_pad, true)) return true;
+        if (plan_rings(p, sp, steps, r, r_pad, false)) return true;
+    }
+    return plan_rings(p, 1, steps, r, r_pad, false);
+}
+
+// CTA-pair kernel: the lengths of its rings beside `lora_bytes` of LoRA operands.  False: does not fit.
+inline bool plan_pair_rings(uint32_t packed_slot_bytes, uint32_t lora_bytes, int& S, int& P) {
+    for (P = 4; P >= 2; P -= 2) {                              // (the packed ring gives way where the LoRA operands are at their largest)
+        S = (int)((kSmemBudget - (lora_bytes + P * packed_slot_bytes + 512)) / (kPairXStage + kWStageBytes));
+        if (S > 8) S = 8;
+        if (rings_sound(S, P, kDequantGroups)) return true;
+    }
+    return false;
+}
+
+}  // namespace qlora

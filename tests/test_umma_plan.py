@@ -1,0 +1,73 @@
+"""The host's plan for the tensor-core kernels (csrc/umma_plan.h), over all shapes, without a GPU: the header is compiled by itself."""
+import ctypes
+import os
+import shutil
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+SHIM = r"""
+#include "umma_plan.h"
+using namespace qlora;
+extern "C" int tiles(int bits, int g, int r, int M, int C, int T, int transposed, int wants_p, int* out) {
+    TilePlan p{};
+    const bool ok = plan_tiles(p, bits, g, r, lora_columns(r, g), M, C, T, transposed != 0, wants_p != 0, 148);
+    const int v[] = {p.S, p.P, p.split, p.steps, p.down_bytes != 0, p.BT, (int)p.off_bar, (int)p.x_stage_bytes};
+    for (int i = 0; i < 8; ++i) out[i] = v[i];
+    return ok;
+}
+extern "C" int pair(int bits, int g, int r, int transposed, int* out) {
+    const unsigned l = (unsigned)(kPairW * lora_columns(r, g) * 2), a = (unsigned)(2 * kPairTok * lora_columns(r, g) * 2);
+    return plan_pair_rings(plan_packed_stage(bits, g, transposed != 0).packed_slot_bytes, l + a < 8192 ? 8192 : l + a, out[0], out[1]);
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def plan(tmp_path_factory):
+    if shutil.which("g++") is None:
+        pytest.skip("no g++")
+    d = tmp_path_factory.mktemp("plan")
+    (d / "shim.cpp").write_text(SHIM)
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-I", os.path.join(ROOT, "paper_2306_08162_b200", "csrc"),
+                    str(d / "shim.cpp"), "-o", str(d / "plan.so")], check=True)
+    return ctypes.CDLL(str(d / "plan.so"))
+
+
+def early_wait(S, P, groups, n=60):
+    """A step at which a dequant group's wait may return a lap early: what it knows to be over before step t is every step whose products it has
+    seen through (up to t - groups - S: it waited for its previous stage to be free) and its own steps."""
+    for t in range(n):
+        seen = t - groups - S
+        if t - 2 * S >= 0 and t - 2 * S > seen:
+            return t
+        if t - P >= 0 and t - P > seen and (t - P) % groups != t % groups:
+            return t
+    return None
+
+
+SHAPES = [(bits, g, r, tr) for bits in (2, 3, 4, 8) for g in (32, 64, 128) for r in range(0, 65, 8) for tr in (0, 1)]
+
+
+def test_rings_of_the_single_cta_kernel(plan):
+    out = (ctypes.c_int * 8)()
+    seen_down = False
+    for bits, g, r, tr in SHAPES:
+        for M in list(range(1, 257, 15)) + [333, 512, 700, 1024]:
+            for C, T in ((256, 512), (2048, 768), (4096, 4096), (4096, 11008), (11008, 4096)):
+                for wants_p in (0, 1):
+                    assert plan.tiles(bits, g, r, M, C, T, tr, wants_p, out), (bits, g, r, tr, M, C, T)
+                    S, P, split, steps, down, BT, off_bar, _ = out
+                    assert split * steps == T // 64 and off_bar + 512 + 1024 + 1024 <= 232448
+                    assert early_wait(S, P, 3 if down else 2) is None, (bits, g, r, tr, M, C, T, S, P, down)
+                    seen_down |= bool(down)
+    assert seen_down
+
+
+def test_rings_of_the_pair_kernel(plan):
+    out = (ctypes.c_int * 2)()
+    for bits, g, r, tr in SHAPES:
+        assert plan.pair(bits, g, r, tr, out), (bits, g, r, tr)
+        assert early_wait(out[0], out[1], 2) is None, (bits, g, r, tr, list(out))
