@@ -50,13 +50,6 @@ constexpr uint32_t kSpinLimit = 1u << 26;
 constexpr int kWaitLimitUs = 250000;   // default limit of a wait, a launch parameter: far beyond any healthy wait (microseconds), short for a hang
 
 struct Params : TilePlan {
-    int M, N, K, bits, g, r, r_pad;
-    // r_pad: columns of the LoRA operands, a multiple of 16.  lora_lo: ranks [r, 2r) hold, beside the finite ones of the same adapter
-    // elements again, what the rounding of s * P to bf16 left over, so that the update has 16 significant bits of P's 24: for r == 8,
-    // where half an MMA's contraction is padding otherwise, and for groups of 32, whose products the CUDA-core kernel gave from fp32
-    // (the error of Y and dX against 64 bits is the same with it: that of the weights' and outputs' bf16).
-    int lora_lo;
-    int C;               // output columns (N forward, K backward)
     float s;
     const float* Pmat;               // H (forward) or G (backward), fp32 [M, r]
     const __nv_bfloat16* L;          // B [N, r] (forward) or A [r, K] (backward)
@@ -861,6 +854,36 @@ int zero_sync_pair(unsigned int* sync, cudaStream_t st) {
     return launch_pdl(sync_zero_kernel, dim3(1), dim3(kSyncWords), 0, st, 1, sync) == cudaSuccess ? QLORA_OK : QLORA_ERR_CUDA;
 }
 
+// Clusters of `width` CTAs, an SM each, that run at a time on the current device (the builds of the kernel differ in nothing that counts here).
+int fitting_clusters(int width) {
+    static std::mutex mu;
+    static int max_clusters_dev[kMaxDevices][5] = {};   // per device, by cluster width
+    static SmemLimit limit;
+    const int dev = device_ordinal();
+    std::lock_guard<std::mutex> lock(mu);
+    int& n = max_clusters_dev[dev < 0 ? 0 : dev][width];
+    if (n == 0) {
+        auto kern = umma_gemm_kernel<4, false, false>;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3((unsigned)(sm_count() / width * width));
+        cfg.blockDim = dim3(kThreads);
+        cfg.dynamicSmemBytes = 232448 - 1024;
+        cudaLaunchAttribute attr;
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = (unsigned)width; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        if (!limit.raise(kern, 232448 - 1024) || cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n <= 0) { (void)cudaGetLastError(); n = -1; }
+    }
+    return n;
+}
+
+// (a device that does not tell: its SMs by the cluster's width)
+GpuFit gpu_fit() {
+    const int sms = sm_count(), c2 = fitting_clusters(2), c4 = fitting_clusters(4);
+    return GpuFit{sms, c2 > 0 ? c2 : sms / 2, c4 > 0 ? c4 : sms / 4};
+}
+
 // Ldown != NULL: P = In * Ldown is still to be computed.  Where the tile clusters leave room for more clusters on the GPU
 // (cudaOccupancyMaxActiveClusters: 33 clusters of 4 fit on 148 SMs, 74 of 2), producer clusters in front of the grid do
 // it beside the tiles; else a down-projection launch goes ahead of the kernel.
@@ -875,32 +898,13 @@ int launch_impl(const CUtensorMap& ta, const CUtensorMap& tq, const CUtensorMap&
                    ? QLORA_OK : QLORA_ERR_CUDA;
     }
     static SmemLimit limit;
-    static std::mutex mu;
-    static int max_clusters_dev[kMaxDevices][5] = {};   // per device, by cluster width
     auto kern = umma_gemm_kernel<BITS, TRANSPOSED, false>;
     if (!limit.raise(kern, 232448 - 1024)) return QLORA_ERR_CUDA;
     Params p = p_in;
     p.n_prod = 0; p.sync = nullptr; p.wait_limit_us = kWaitLimitUs;
     if (Ldown != nullptr && p.r > 0) {
-        std::lock_guard<std::mutex> lock(mu);
-        const int dev = device_ordinal();
-        int* max_clusters = max_clusters_dev[dev < 0 ? 0 : dev];
-        if (max_clusters[p.split] == 0) {
-            cudaLaunchConfig_t cfg{};
-            cfg.gridDim = dim3((unsigned)(sm_count() / p.split * p.split));
-            cfg.blockDim = dim3(kThreads);
-            cfg.dynamicSmemBytes = 232448 - 1024;
-            cudaLaunchAttribute attr;
-            attr.id = cudaLaunchAttributeClusterDimension;
-            attr.val.clusterDim.x = (unsigned)p.split; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
-            cfg.attrs = &attr;
-            cfg.numAttrs = 1;
-            int n = 0;
-            if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n <= 0) { (void)cudaGetLastError(); n = -1; }
-            max_clusters[p.split] = n;
-        }
         const int n_blocks = (p.M + 15) / 16;
-        const int idle = max_clusters[p.split] - grid / p.split;
+        const int idle = fitting_clusters(p.split) - grid / p.split;
         int n_prod = (n_blocks + p.split - 1) / p.split;           // one row block per producer CTA when there is room
         if (n_prod > idle) n_prod = idle;
         const bool fits = p.r <= 16 && n_prod > 0 && n_prod * p.split * 2 >= n_blocks && p.lds_stages >= LDS_MIN_STAGES;
@@ -981,7 +985,7 @@ static int launch_umma_pair(const qlora_desc& d, int M, bool transposed, const v
     const int n_w_tiles = (p.C + 2 * kPairW - 1) / (2 * kPairW);
     p.n_tiles = p.n_tok_tiles * n_w_tiles;
     p.steps = T / kStepC;
-    static_cast<PackedStage&>(p) = plan_packed_stage(d.bits, d.group_size, transposed);
+    plan_packed_stage(p, d.bits, d.group_size, transposed);
     p.s = d.r > 0 ? d.alpha / (float)d.r : 0.f;
     p.Pmat = Pmat; p.L = (const __nv_bfloat16*)L; p.Out = (__nv_bfloat16*)Out;
 
@@ -1120,7 +1124,7 @@ int launch_umma_gemm(const qlora_desc& d, int M, bool transposed, const void* In
     p.M = M; p.N = d.N; p.K = d.K; p.bits = d.bits; p.g = d.group_size; p.r = d.r; p.lora_lo = keep_lora_low(d.r, d.group_size); p.r_pad = lora_columns(d.r, d.group_size);
     p.C = transposed ? d.K : d.N;
     const int T = transposed ? d.N : d.K;
-    if (!plan_tiles(p, d.bits, d.group_size, d.r, p.r_pad, M, p.C, T, transposed, Ldown != nullptr, sm_count())) return QLORA_ERR_UNSUPPORTED;
+    if (!plan_tiles(p, T, transposed, Ldown != nullptr, gpu_fit())) return QLORA_ERR_UNSUPPORTED;
     p.s = d.r > 0 ? d.alpha / (float)d.r : 0.f;
     p.Pmat = Pmat; p.L = (const __nv_bfloat16*)L; p.Out = (__nv_bfloat16*)Out;
 

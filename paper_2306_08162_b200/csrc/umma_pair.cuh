@@ -32,7 +32,7 @@
 // instead of a whole one.  Every wait in this kernel points from higher block indices to lower ones (tiles wait for producer
 // clusters, the finishing half of a split tile for the giving half), i.e. to CTAs that were dispatched earlier.
 
-struct PairParams : PackedStage {
+struct PairParams {
     int M, N, K, bits, g, r, r_pad;
     int lora_lo;                 // as in Params
     int C;                       // output columns (N forward, K backward)
@@ -42,6 +42,8 @@ struct PairParams : PackedStage {
     int n_full, nsplit;
     float4* split_buf;           // fp32 exchange area of the split tiles (workspace)
     int S, P;
+    int packed_cols, packed_rows, scale_rows;
+    uint32_t words_bytes, scale_bytes, packed_slot_bytes;
     uint32_t off_x, off_w, off_p, off_lora_l, off_lora_p, off_bar;
     float s;
     const float* Pmat;           // H (forward) or G (backward), fp32 [M, r]

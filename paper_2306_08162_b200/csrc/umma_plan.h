@@ -33,36 +33,49 @@ inline int scale_rows_per_stage(int g, bool transposed) {
     return g >= k_rows ? 1 : k_rows / g;
 }
 
-// Whether the LoRA operands carry what the rounding of s * P to bf16 left over (Params::lora_lo), and their columns, a multiple of 16.
+// lora_lo and r_pad (see TilePlan).
 inline int keep_lora_low(int r, int g) { return r == 8 || g == 32 ? 1 : 0; }
 inline int lora_columns(int r, int g) { return ((keep_lora_low(r, g) ? 2 : 1) * r + 15) / 16 * 16; }
 
-struct PackedStage {
-    int packed_cols;     // 128 forward, 64 backward
-    int packed_rows;     // int32 rows per stage
-    int scale_rows;      // group rows per stage
-    uint32_t words_bytes, scale_bytes, packed_slot_bytes;
-};
-inline PackedStage plan_packed_stage(int bits, int g, bool transposed) {
-    PackedStage s;
-    s.packed_cols = transposed ? 64 : 128;
-    s.packed_rows = (transposed ? 128 : 64) * bits / 32;
-    s.scale_rows = scale_rows_per_stage(g, transposed);
-    s.words_bytes = (uint32_t)(s.packed_rows * s.packed_cols * 4);
-    s.scale_bytes = (uint32_t)(s.scale_rows * s.packed_cols * 2);
-    s.packed_slot_bytes = (s.words_bytes + 2 * s.scale_bytes + 127u) / 128u * 128u;
-    return s;
+// A pipeline stage of packed codes and group parameters (Plan: TilePlan or the CTA-pair kernel's parameters).
+template <class Plan>
+inline void plan_packed_stage(Plan& p, int bits, int g, bool transposed) {
+    p.packed_cols = transposed ? 64 : 128;
+    p.packed_rows = (transposed ? 128 : 64) * bits / 32;
+    p.scale_rows = scale_rows_per_stage(g, transposed);
+    p.words_bytes = (uint32_t)(p.packed_rows * p.packed_cols * 4);
+    p.scale_bytes = (uint32_t)(p.scale_rows * p.packed_cols * 2);
+    p.packed_slot_bytes = (p.words_bytes + 2 * p.scale_bytes + 127u) / 128u * 128u;
 }
 
-// Single-CTA kernel.  Offsets count from the 1024-byte aligned base of shared memory.
-struct TilePlan : PackedStage {
+// Single-CTA kernel.  Offsets count from the 1024-byte aligned base of shared memory.  (The head of the kernel's parameters: their order
+// is that in which a CTA first reads them.)
+struct TilePlan {
+    int M, N, K, bits, g, r, r_pad;
+    // r_pad: columns of the LoRA operands, a multiple of 16.  lora_lo: ranks [r, 2r) hold, beside the finite ones of the same adapter
+    // elements again, what the rounding of s * P to bf16 left over, so that the update has 16 significant bits of P's 24: for r == 8,
+    // where half an MMA's contraction is padding otherwise, and for groups of 32, whose products the CUDA-core kernel gave from fp32
+    // (the error of Y and dX against 64 bits is the same with it: that of the weights' and outputs' bf16).
+    int lora_lo;
+    int C;               // output columns (N forward, K backward)
     int BT;              // token rows per tile (MMA N): a multiple of 16, 32 .. 256
     int n_tok_tiles, n_tiles, steps;   // steps: of one rank
     int split;           // CTAs per cluster sharing one tile, each taking `steps` consecutive steps of the contraction (1 = no cluster)
     int S, P;            // stages of the activation/weight ring and of the packed ring
-    uint32_t x_stage_bytes;
+    int packed_cols;     // 128 forward, 64 backward
+    int packed_rows;     // int32 rows per stage
+    int scale_rows;      // group rows per stage
+    uint32_t words_bytes, scale_bytes, packed_slot_bytes, x_stage_bytes;
     uint32_t off_x, off_w, off_l, off_p, off_lora_a, off_lora_p, off_bar;
     uint32_t down_bytes;             // DOWN: bytes per stage of the adapter applied first (else 0)
+};
+
+// What runs at a time: SMs, and clusters of two and of four CTAs with an SM to each (148 SMs: 74 and 33, not 37, as a cluster stays in one group of SMs).
+// 34 to 37 tiles on clusters of four are two waves: two ranks per tile instead are 20 to 50 % faster (4352 outputs, rank 8, 64 tokens, T = 512 11.5 -> 6.4 us,
+// 4096 20.6 -> 14.6; 4736, 256 tokens, 11008 long 60.6 -> 45.3).
+struct GpuFit {
+    int sms, clusters2, clusters4;
+    int clusters(int width) const { return width == 4 ? clusters4 : width == 2 ? clusters2 : sms; }
 };
 
 // Up to 128 tokens, where a split tile's ranks form P themselves.  Their MMAs cost some 250 cycles per step, the producer clusters a launch, a
@@ -72,11 +85,11 @@ struct TilePlan : PackedStage {
 inline bool down_pays(int split, int steps, int r) { return steps <= 8 || (split == 4 && (r == 16 || steps <= 16)); }
 
 // Rings and layout for `split` ranks per tile, `total_steps` steps among them; with_down: the DOWN build.  False: does not fit.
-inline bool plan_rings(TilePlan& p, int split, int total_steps, int r, int r_pad, bool with_down) {
+inline bool plan_rings(TilePlan& p, int split, int total_steps, bool with_down) {
     p.split = split;
     p.steps = total_steps / split;
-    p.down_bytes = with_down ? (uint32_t)r * 128u : 0u;
-    const uint32_t lora_a = (uint32_t)(kWRows * r_pad * 2), lora_p = (uint32_t)(p.BT * r_pad * 2);
+    p.down_bytes = with_down ? (uint32_t)p.r * 128u : 0u;
+    const uint32_t lora_a = (uint32_t)(kWRows * p.r_pad * 2), lora_p = (uint32_t)(p.BT * p.r_pad * 2);
     const uint32_t per_stage = p.x_stage_bytes + kWStageBytes + p.down_bytes;
     // With few tokens the kernel is bound by the latency of streaming cold packed weights through a handful of CTAs, so the packed ring is
     // deep (bytes in flight), at the cost of one or two operand stages; it gives way until three of those fit (two, at four slots and below).
@@ -99,29 +112,29 @@ inline bool plan_rings(TilePlan& p, int split, int total_steps, int r, int r_pad
     p.off_bar = (p.off_lora_p + lora_p + 127u) / 128u * 128u;
     // a split tile's fp32 parts (and those of P) meet in the operand ring
     return rings_sound(p.S, p.P, with_down ? kDownGroups : kDequantGroups) &&
-           (split == 1 || (uint32_t)(p.BT * (kWRows + (with_down ? r : 0)) * 4) <= p.off_p);
+           (split == 1 || (uint32_t)(p.BT * (kWRows + (with_down ? p.r : 0)) * 4) <= p.off_p);
 }
 
-// M tokens, C output columns, T contraction elements.  wants_p: P = In * Ldown is still to be computed.  False: the shape does not fit.
-inline bool plan_tiles(TilePlan& p, int bits, int g, int r, int r_pad, int M, int C, int T, bool transposed, bool wants_p, int sms) {
-    static_cast<PackedStage&>(p) = plan_packed_stage(bits, g, transposed);
+// For the shape in M .. C and a contraction of T elements.  wants_p: P = In * Ldown is still to be computed.  False: does not fit.
+inline bool plan_tiles(TilePlan& p, int T, bool transposed, bool wants_p, const GpuFit& fit) {
+    plan_packed_stage(p, p.bits, p.g, transposed);
     // The tokens in as few tiles as 256 columns allow, cut evenly: a multiple of 16 (the MMA's N), not the next power of two, so that
     // neither products nor the exchange between the ranks are made for tokens that do not exist (333: two tiles of 176, not 256).
-    p.n_tok_tiles = (M + 255) / 256;
-    p.BT = ((M + p.n_tok_tiles - 1) / p.n_tok_tiles + 15) / 16 * 16;
+    p.n_tok_tiles = (p.M + 255) / 256;
+    p.BT = ((p.M + p.n_tok_tiles - 1) / p.n_tok_tiles + 15) / 16 * 16;
     if (p.BT < 32) p.BT = 32;
-    p.n_tok_tiles = (M + p.BT - 1) / p.BT;
-    p.n_tiles = p.n_tok_tiles * ((C + kWRows - 1) / kWRows);
+    p.n_tok_tiles = (p.M + p.BT - 1) / p.BT;
+    p.n_tiles = p.n_tok_tiles * ((p.C + kWRows - 1) / kWRows);
     p.x_stage_bytes = (uint32_t)(p.BT * 128);
     // Few tiles (few tokens): split each tile's contraction over a cluster of 2 or 4 CTAs so that the whole GPU streams
     // the weights.  Needs one tile per cluster, an even split of the steps, and room for the fp32 parts in the operand ring.
     const int steps = T / kStepC;
     for (int sp = 4; sp >= 2; sp /= 2) {
-        if (p.n_tiles * sp > sms || steps % sp != 0 || steps / sp < (p.BT <= kMaxDownTokens ? kMinSplitSteps : kMinSplitSteps256) || p.BT % sp != 0) continue;
-        if (wants_p && (r == 8 || r == 16) && p.BT <= kMaxDownTokens && down_pays(sp, steps / sp, r) && plan_rings(p, sp, steps, r, r_pad, true)) return true;
-        if (plan_rings(p, sp, steps, r, r_pad, false)) return true;
+        if (p.n_tiles > fit.clusters(sp) || steps % sp != 0 || steps / sp < (p.BT <= kMaxDownTokens ? kMinSplitSteps : kMinSplitSteps256) || p.BT % sp != 0) continue;
+        if (wants_p && (p.r == 8 || p.r == 16) && p.BT <= kMaxDownTokens && down_pays(sp, steps / sp, p.r) && plan_rings(p, sp, steps, true)) return true;
+        if (plan_rings(p, sp, steps, false)) return true;
     }
-    return plan_rings(p, 1, steps, r, r_pad, false);
+    return plan_rings(p, 1, steps, false);
 }
 
 // CTA-pair kernel: the lengths of its rings beside `lora_bytes` of LoRA operands.  False: does not fit.

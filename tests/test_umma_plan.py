@@ -13,14 +13,17 @@ SHIM = r"""
 using namespace qlora;
 extern "C" int tiles(int bits, int g, int r, int M, int C, int T, int transposed, int wants_p, int* out) {
     TilePlan p{};
-    const bool ok = plan_tiles(p, bits, g, r, lora_columns(r, g), M, C, T, transposed != 0, wants_p != 0, 148);
+    p.M = M; p.C = C; p.bits = bits; p.g = g; p.r = r; p.r_pad = lora_columns(r, g);
+    const bool ok = plan_tiles(p, T, transposed != 0, wants_p != 0, GpuFit{148, 74, 33});
     const int v[] = {p.S, p.P, p.split, p.steps, p.down_bytes != 0, p.BT, (int)p.off_bar, (int)p.x_stage_bytes};
     for (int i = 0; i < 8; ++i) out[i] = v[i];
     return ok;
 }
 extern "C" int pair(int bits, int g, int r, int transposed, int* out) {
     const unsigned l = (unsigned)(kPairW * lora_columns(r, g) * 2), a = (unsigned)(2 * kPairTok * lora_columns(r, g) * 2);
-    return plan_pair_rings(plan_packed_stage(bits, g, transposed != 0).packed_slot_bytes, l + a < 8192 ? 8192 : l + a, out[0], out[1]);
+    TilePlan p{};
+    plan_packed_stage(p, bits, g, transposed != 0);
+    return plan_pair_rings(p.packed_slot_bytes, l + a < 8192 ? 8192 : l + a, out[0], out[1]);
 }
 """
 
@@ -71,3 +74,15 @@ def test_rings_of_the_pair_kernel(plan):
     for bits, g, r, tr in SHAPES:
         assert plan.pair(bits, g, r, tr, out), (bits, g, r, tr)
         assert early_wait(out[0], out[1], 2) is None, (bits, g, r, tr, list(out))
+
+
+@pytest.mark.parametrize("M,BT_tiles", [(17, 1), (128, 1), (200, 1), (333, 2)])
+def test_split_tiles_run_in_one_wave(plan, M, BT_tiles):
+    """33 clusters of four CTAs run at a time on 148 SMs, 74 of two."""
+    out = (ctypes.c_int * 8)()
+    for C in range(64, 12000, 64):
+        for T in (512, 768, 1024, 4096, 11008):
+            for wants_p in (0, 1):
+                assert plan.tiles(4, 128, 8, M, C, T, 0, wants_p, out)
+                tiles = BT_tiles * ((C + 127) // 128)
+                assert out[2] == 1 or tiles <= {4: 33, 2: 74}[out[2]], (M, C, T, list(out))
