@@ -1124,7 +1124,7 @@ int launch_umma_gemm(const qlora_desc& d, int M, bool transposed, const void* In
     p.M = M; p.N = d.N; p.K = d.K; p.bits = d.bits; p.g = d.group_size; p.r = d.r; p.lora_lo = keep_lora_low(d.r, d.group_size); p.r_pad = lora_columns(d.r, d.group_size);
     p.C = transposed ? d.K : d.N;
     const int T = transposed ? d.N : d.K;
-    if (!plan_tiles(p, T, transposed, Ldown != nullptr, gpu_fit())) return QLORA_ERR_UNSUPPORTED;
+    if (!plan_tiles(p, T, transposed, Ldown != nullptr, extra != nullptr, gpu_fit())) return QLORA_ERR_UNSUPPORTED;
     p.s = d.r > 0 ? d.alpha / (float)d.r : 0.f;
     p.Pmat = Pmat; p.L = (const __nv_bfloat16*)L; p.Out = (__nv_bfloat16*)Out;
 

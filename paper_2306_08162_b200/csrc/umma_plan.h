@@ -14,9 +14,6 @@ constexpr int kPairXSub = kPairTok * kStepC * 2;       // 16 KiB: one 128-token 
 constexpr int kPairXStage = 2 * kPairXSub;             // two accumulators' sub-tiles
 constexpr int kDequantGroups = 2, kDownGroups = 3;     // dequant groups, and in the DOWN build
 constexpr uint32_t kSmemBudget = 232448 - 1024 /*alignment slack*/ - 2048 /*static, barriers, padding*/;
-// contraction steps that a rank of a split tile has at least, up to 128 tokens and above (512 x 512, rank 8: four ranks of two steps against two
-// of four 5.1 / 5.7 us at 17 tokens, 7.6 / 8.3 at 128, but 11.8 / 10.6 at 256: what the ranks exchange grows with the tokens)
-constexpr int kMinSplitSteps = 2, kMinSplitSteps256 = 4;
 constexpr int kMaxDownTokens = 128;
 
 // Whether `groups` dequant groups that take the stages of a tile in turn may run on an operand ring of S stages and a packed ring of P slots.
@@ -84,6 +81,22 @@ struct GpuFit {
 // 8192 -> 2048, 32 steps, 64 tokens 16.4 -> 16.9, but rank 16 19.3 -> 17.3; two ranks of 16 steps, 128 tokens 13.2 -> 14.9.
 inline bool down_pays(int split, int steps, int r) { return steps <= 8 || (split == 4 && (r == 16 || steps <= 16)); }
 
+// Contraction steps that a rank of a split tile of this plan has at least.  Up to 128 tokens the DOWN build takes two (512 x 512, rank 8: four ranks of
+// two steps against two of four 5.1 / 5.7 us at 17 tokens; what the ranks exchange grows with the tokens: 11.8 / 10.6 at 256).  Without it there is
+// the chain of a down-projection or nothing to hide more ranks behind, and they pay up to 16 ranks only, with two steps up to 64 tokens, with three
+// up to 128, while the clusters leave room for the CTAs of the launch behind; under dropout (`dropout`: other launches of the call go before and
+// after) that matters less.  INT4, microseconds, four ranks of two or three steps / two of four or six: rank 0, 512 -> 2048, 64 tokens 5.51 / 5.81,
+// 128 tokens 6.83 / 6.65; 512 -> 4096, 64 tokens 6.83 / 5.89; 768 -> 2048, 17 tokens 5.12 / 5.77, 128 tokens 7.06 / 7.18; rank 32, 768 -> 2048,
+// 64 tokens 9.87 / 9.91, 128 tokens 11.49 / 10.81; dropout forward, rank 16, 512 -> 2048, 17 tokens 7.88 / 8.12, 128 tokens 9.98 / 9.54, rank 8,
+// 768 -> 4096, 64 tokens 8.45 / 9.26; dropout backward (rank 0 in this kernel), 512 long, 17 tokens, 4096 wide 8.64 / 9.74, 48 tokens 12.34 / 11.33 (3072 wide 9.25 / 9.74).
+inline int min_split_steps(const TilePlan& p, int split, bool down, bool dropout, const GpuFit& fit) {
+    if (p.BT > kMaxDownTokens) return 4;
+    if (down) return 2;
+    const int ctas = p.n_tiles * split, most = !dropout || p.BT > 64 ? fit.sms / 2 : p.BT > 32 ? fit.sms * 2 / 3 : fit.sms;
+    if (p.r > 16 || (p.r == 0 && ctas > most)) return 4;
+    return p.BT <= 64 ? 2 : 3;
+}
+
 // Rings and layout for `split` ranks per tile, `total_steps` steps among them; with_down: the DOWN build.  False: does not fit.
 inline bool plan_rings(TilePlan& p, int split, int total_steps, bool with_down) {
     p.split = split;
@@ -115,8 +128,8 @@ inline bool plan_rings(TilePlan& p, int split, int total_steps, bool with_down) 
            (split == 1 || (uint32_t)(p.BT * (kWRows + (with_down ? p.r : 0)) * 4) <= p.off_p);
 }
 
-// For the shape in M .. C and a contraction of T elements.  wants_p: P = In * Ldown is still to be computed.  False: does not fit.
-inline bool plan_tiles(TilePlan& p, int T, bool transposed, bool wants_p, const GpuFit& fit) {
+// For the shape in M .. C and a contraction of T elements.  wants_p: P = In * Ldown is still to be computed; dropout: see min_split_steps.  False: does not fit.
+inline bool plan_tiles(TilePlan& p, int T, bool transposed, bool wants_p, bool dropout, const GpuFit& fit) {
     plan_packed_stage(p, p.bits, p.g, transposed);
     // The tokens in as few tiles as 256 columns allow, cut evenly: a multiple of 16 (the MMA's N), not the next power of two, so that
     // neither products nor the exchange between the ranks are made for tokens that do not exist (333: two tiles of 176, not 256).
@@ -130,8 +143,10 @@ inline bool plan_tiles(TilePlan& p, int T, bool transposed, bool wants_p, const 
     // the weights.  Needs one tile per cluster, an even split of the steps, and room for the fp32 parts in the operand ring.
     const int steps = T / kStepC;
     for (int sp = 4; sp >= 2; sp /= 2) {
-        if (p.n_tiles > fit.clusters(sp) || steps % sp != 0 || steps / sp < (p.BT <= kMaxDownTokens ? kMinSplitSteps : kMinSplitSteps256) || p.BT % sp != 0) continue;
-        if (wants_p && (p.r == 8 || p.r == 16) && p.BT <= kMaxDownTokens && down_pays(sp, steps / sp, p.r) && plan_rings(p, sp, steps, true)) return true;
+        if (p.n_tiles > fit.clusters(sp) || steps % sp != 0 || p.BT % sp != 0) continue;
+        const bool down = wants_p && (p.r == 8 || p.r == 16) && p.BT <= kMaxDownTokens && down_pays(sp, steps / sp, p.r);
+        if (steps / sp < min_split_steps(p, sp, down, dropout, fit)) continue;
+        if (down && plan_rings(p, sp, steps, true)) return true;
         if (plan_rings(p, sp, steps, false)) return true;
     }
     return plan_rings(p, 1, steps, false);

@@ -11,10 +11,10 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 SHIM = r"""
 #include "umma_plan.h"
 using namespace qlora;
-extern "C" int tiles(int bits, int g, int r, int M, int C, int T, int transposed, int wants_p, int* out) {
+extern "C" int tiles(int bits, int g, int r, int M, int C, int T, int transposed, int wants_p /* 2: dropout, the product is there already */, int* out) {
     TilePlan p{};
     p.M = M; p.C = C; p.bits = bits; p.g = g; p.r = r; p.r_pad = lora_columns(r, g);
-    const bool ok = plan_tiles(p, T, transposed != 0, wants_p != 0, GpuFit{148, 74, 33});
+    const bool ok = plan_tiles(p, T, transposed != 0, wants_p == 1, wants_p == 2, GpuFit{148, 74, 33});
     const int v[] = {p.S, p.P, p.split, p.steps, p.down_bytes != 0, p.BT, (int)p.off_bar, (int)p.x_stage_bytes};
     for (int i = 0; i < 8; ++i) out[i] = v[i];
     return ok;
@@ -86,3 +86,15 @@ def test_split_tiles_run_in_one_wave(plan, M, BT_tiles):
                 assert plan.tiles(4, 128, 8, M, C, T, 0, wants_p, out)
                 tiles = BT_tiles * ((C + 127) // 128)
                 assert out[2] == 1 or tiles <= {4: 33, 2: 74}[out[2]], (M, C, T, list(out))
+
+
+@pytest.mark.parametrize("r,wants_p,M,T,C,split,steps", [
+    (32, 1, 17, 512, 512, 2, 4), (32, 1, 128, 768, 2048, 2, 6), (64, 1, 128, 512, 4096, 2, 4), (24, 2, 96, 512, 1024, 2, 4),     # ranks above 16
+    (0, 0, 64, 512, 4096, 2, 4), (0, 0, 17, 768, 3072, 2, 6), (0, 0, 128, 512, 2048, 2, 4), (0, 2, 48, 512, 4096, 2, 4),          # rank 0
+    (8, 2, 128, 512, 2048, 2, 4), (16, 2, 65, 512, 512, 2, 4),                                                                  # dropout, many tokens
+    (0, 0, 64, 512, 2048, 4, 2), (0, 0, 128, 768, 1024, 4, 3), (16, 2, 64, 512, 4096, 4, 2), (0, 2, 17, 512, 4096, 4, 2),        # where short ranks pay
+    (8, 1, 128, 512, 512, 4, 2), (16, 1, 17, 768, 4096, 4, 3)])
+def test_short_ranks_only_where_they_pay(plan, r, wants_p, M, T, C, split, steps):
+    out = (ctypes.c_int * 8)()
+    assert plan.tiles(4, 128, r, M, C, T, 0, wants_p, out)
+    assert (out[2], out[3]) == (split, steps)
