@@ -118,10 +118,29 @@ __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatil
     if (ok) (void)mbar_try_wait(bar, parity);
     return ok != 0;
 }
+// The same for the MMA issuer, whose wait ends a stage's chain: every lane polls, so no lane hands the outcome on and the phase is not read again.
+// INT4, rank 8, from warp_wait to this: 512 x 512, 64 tokens 6.0 -> 5.65 us; 11008 -> 4096, 256 tokens 33.8 -> 33.3, 200 tokens 31.2 -> 30.7; 4096 x 4096,
+// 700 tokens 33.2 -> 32.6; four ranks on 32 tiles up to 1 % slower.  (In the roles that issue copies it gives nothing: 2048 x 2048, 300 tokens 13.85 -> 14.0.)
+__device__ __forceinline__ bool warp_poll(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+    uint64_t t0 = 0;
+    for (uint32_t i = 0; i < kSpinLimit; ++i) {
+        if (__all_sync(0xFFFFFFFFu, mbar_try_wait(bar, parity) != 0u)) return true;
+        if ((i & 63u) == 63u) {
+            if (__any_sync(0xFFFFFFFFu, *abort_flag != 0)) return false;
+            const uint64_t now = __shfl_sync(0xFFFFFFFFu, global_ns(), 0);
+            if (t0 == 0) t0 = now;
+            else if (now - t0 > (uint64_t)abort_flag[1] * 1000ull) break;
+        }
+    }
+    *abort_flag = 1;
+    atomicOr(&g_device_status, 1u);
+    return false;
+}
 // One lane of a converged warp, the same one every time.  The roles that issue TMA copies and MMAs run as whole warps and elect a lane for
 // the instructions alone, so that ring positions, addresses and descriptors are warp-uniform values, which these instructions want: run by
 // lane 0 of a diverged warp they cost 75 to 150 cycles each (a trace of one CTA had the dequant warps 3000 cycles ahead of the MMAs).
-// INT4, rank 0, 64 tokens: 4096 -> 11008 29.3 -> 25.9, 4096 x 4096 13.3 -> 12.2 us; nothing from 257 tokens on, where the products are what takes the time.
+// INT4, rank 0, 64 tokens: 4096 -> 11008 29.3 -> 25.9, 4096 x 4096 13.3 -> 12.2 us; rank 8, 300 tokens, 11008 -> 4096 44.6 -> 41.3.  Tiles of
+// 200 to 256 tokens, which wait for their products, gain nothing (4096 -> 11008, 256 tokens 33.0 -> 32.9; 11008 -> 4096 33.1 -> 33.3).
 __device__ __forceinline__ bool elect_one() {
     uint32_t ok;
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(ok) ::"memory");
@@ -439,11 +458,11 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
         for (int tile = first_tile; tile < p.n_tiles; tile += tile_stride, ++tile_it) {
             const uint32_t buf = tile_it & 1u;
             const uint32_t d_tmem = tmem_base + buf * kAccStride;
-            if (!warp_wait(bar_acc_empty + 8 * buf, ((tile_it >> 1) & 1u) ^ 1u, abort_flag, lane)) goto done;
+            if (!warp_poll(bar_acc_empty + 8 * buf, ((tile_it >> 1) & 1u) ^ 1u, abort_flag)) goto done;
             tc_fence_after();
             uint32_t acc = 0;
             for (int step = 0; step < p.steps; ++step) {
-                if (!warp_wait(bar_full_x + 8 * ring.slot, ring.phase, abort_flag, lane)) goto done;
+                if (!warp_poll(bar_full_x + 8 * ring.slot, ring.phase, abort_flag)) goto done;
                 tc_fence_after();
                 const uint64_t b_desc = b_desc0 + ring.slot * x_step;
                 const uint64_t a_desc = a_desc0 + ring.slot * (uint32_t)(kWStageBytes >> 4);
@@ -463,7 +482,7 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
                 ring.advance(S);
             }
             if (!DOWN && p.r > 0 && rank == 0) {   // the LoRA update goes into one rank's part only
-                if (!warp_wait(bar_lora_full, tile_it & 1u, abort_flag, lane)) goto done;
+                if (!warp_poll(bar_lora_full, tile_it & 1u, abort_flag)) goto done;
                 tc_fence_after();
                 if (elect_one())
                     for (int jb = 0; jb < p.r_pad / 16; ++jb) {
