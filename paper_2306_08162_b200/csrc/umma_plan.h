@@ -75,11 +75,22 @@ struct GpuFit {
     int clusters(int width) const { return width == 4 ? clusters4 : width == 2 ? clusters2 : sms; }
 };
 
-// Up to 128 tokens, where a split tile's ranks form P themselves.  Their MMAs cost some 250 cycles per step, the producer clusters a launch, a
-// counter and a chain that grows with the rank; two ranks have more of the tile to exchange and less room to gain.  INT4, forward, 64
-// tokens, rank 8: 512 x 512 8.3 -> 6.6 us, 1024 x 1024 8.6 -> 6.8, INT3 2048 x 2048 9.05 -> 8.1; 4096 x 4096, 16 steps, 128 tokens 16.3 -> 15.1;
-// 8192 -> 2048, 32 steps, 64 tokens 16.4 -> 16.9, but rank 16 19.3 -> 17.3; two ranks of 16 steps, 128 tokens 13.2 -> 14.9.
-inline bool down_pays(int split, int steps, int r) { return steps <= 8 || (split == 4 && (r == 16 || steps <= 16)); }
+// Whether ranks of `steps` contraction steps form P themselves (DOWN; rank 8 or 16, up to 128 tokens).  Their MMAs cost some 250 cycles per step and P's
+// parts go through the exchange; the producer clusters cost a launch, a counter and a chain that grows with the rank and is longer in the
+// backward; and DOWN has a third dequant group, which INT3 gains the most from.  Two ranks have twice as much to exchange.  Microseconds without / with,
+// INT4, forward: two ranks of five steps, 128 tokens, 512 wide 8.88 / 8.20, 8192 wide 9.26 / 9.56; of seven, 6016 wide, 64 tokens 8.57 / 8.22, 128 tokens
+// 9.37 / 9.91.  Four ranks, rank 8, 2048 wide: eight steps, 64 tokens 9.04 / 8.00; 16 steps, 48 tokens 10.27 / 10.04, 64 tokens 10.50 / 10.89, backward
+// 96 tokens 12.19 / 11.79, 128 tokens 12.76 / 13.22, INT3, 96 tokens 13.00 / 12.12.  Rank 16: 14 steps, 128 tokens 13.32 / 12.64; 16 steps, 112
+// tokens 12.94 / 12.71, 128 tokens 13.32 / 13.67; 24 steps, 96 tokens 15.10 / 15.00, 128 tokens 15.59 / 16.62, backward 17.17 / 16.70; 32 steps, 32 tokens
+// 14.77 / 14.76, 64 tokens 15.52 / 16.72; 43 steps, 512 wide, 64 tokens 19.25 / 20.47.  Where the producers would take the last clusters or find none
+// (4096 wide: 32 tiles), 43 steps, 128 tokens 32.4 / 25.7; rank 8, 16 steps, 96 tokens 13.63 / 13.15.
+inline bool down_pays(const TilePlan& p, int split, int steps, bool transposed, const GpuFit& fit) {
+    if (split == 2) return steps <= 5 ? p.BT <= 96 || 4 * p.n_tiles * split <= 3 * fit.sms : steps <= 8 && p.BT <= 168 - 12 * steps;
+    if (p.r == 8 && steps > 16) return false;
+    if (p.bits == 3 || fit.clusters(split) - p.n_tiles <= ((p.M + 15) / 16 + split - 1) / split) return true;
+    const int most = p.r == 16 ? (steps <= 14 ? 128 : steps <= 20 ? 112 : steps <= 24 ? 96 : steps <= 32 ? 48 : 32) : (steps <= 14 ? 128 : 48);
+    return p.BT <= most + (transposed ? 48 : 0);
+}
 
 // Contraction steps that a rank of a split tile of this plan has at least.  Up to 128 tokens the DOWN build takes two (512 x 512, rank 8: four ranks of
 // two steps against two of four 5.1 / 5.7 us at 17 tokens; what the ranks exchange grows with the tokens: 11.8 / 10.6 at 256).  Without it there is
@@ -144,7 +155,7 @@ inline bool plan_tiles(TilePlan& p, int T, bool transposed, bool wants_p, bool d
     const int steps = T / kStepC;
     for (int sp = 4; sp >= 2; sp /= 2) {
         if (p.n_tiles > fit.clusters(sp) || steps % sp != 0 || p.BT % sp != 0) continue;
-        const bool down = wants_p && (p.r == 8 || p.r == 16) && p.BT <= kMaxDownTokens && down_pays(sp, steps / sp, p.r);
+        const bool down = wants_p && (p.r == 8 || p.r == 16) && p.BT <= kMaxDownTokens && down_pays(p, sp, steps / sp, transposed, fit);
         if (steps / sp < min_split_steps(p, sp, down, dropout, fit)) continue;
         if (down && plan_rings(p, sp, steps, true)) return true;
         if (plan_rings(p, sp, steps, false)) return true;

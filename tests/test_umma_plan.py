@@ -98,3 +98,16 @@ def test_short_ranks_only_where_they_pay(plan, r, wants_p, M, T, C, split, steps
     out = (ctypes.c_int * 8)()
     assert plan.tiles(4, 128, r, M, C, T, 0, wants_p, out)
     assert (out[2], out[3]) == (split, steps)
+
+
+@pytest.mark.parametrize("bits,r,M,T,C,tr,split,steps,down", [
+    (4, 8, 128, 1024, 8192, 0, 2, 8, 0), (4, 16, 80, 1024, 6016, 1, 2, 8, 0), (4, 16, 128, 896, 2048, 0, 2, 7, 0),       # two ranks, many tokens
+    (4, 8, 112, 640, 8192, 0, 2, 5, 0), (4, 8, 112, 640, 512, 0, 2, 5, 1), (4, 8, 64, 1024, 6016, 0, 2, 8, 1),
+    (4, 8, 64, 4096, 2048, 0, 4, 16, 0), (2, 8, 128, 4096, 512, 1, 4, 16, 0), (4, 8, 48, 4096, 2048, 0, 4, 16, 1),        # rank 8, long ranks
+    (4, 8, 96, 4096, 2048, 1, 4, 16, 1), (3, 8, 96, 4096, 2048, 0, 4, 16, 1), (4, 8, 96, 4096, 4096, 0, 4, 16, 1),
+    (4, 16, 128, 6144, 2048, 0, 4, 24, 0), (4, 16, 64, 8192, 512, 0, 4, 32, 0), (8, 16, 48, 11008, 512, 0, 4, 43, 0),     # rank 16
+    (4, 16, 128, 3584, 2048, 0, 4, 14, 1), (4, 16, 128, 6144, 2048, 1, 4, 24, 1), (4, 16, 128, 11008, 4096, 0, 4, 43, 1)])
+def test_ranks_form_their_part_of_the_down_projection_where_that_pays(plan, bits, r, M, T, C, tr, split, steps, down):
+    out = (ctypes.c_int * 8)()
+    assert plan.tiles(bits, 128, r, M, C, T, tr, 1, out)
+    assert (out[2], out[3], out[4]) == (split, steps, down)
