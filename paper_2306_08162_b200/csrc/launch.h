@@ -30,8 +30,9 @@ int launch_simt_gemm(const qlora_desc& d, int M, bool transposed, const void* In
 // mask (optional, only with l_is_A): uint8 [M, T] dropout mask on In, non-zero = keep; the result is multiplied by out_scale.
 int launch_lora_down(int M, int T, int r, bool l_is_A, const void* In, const void* L, float* P, cudaStream_t st,
                      const uint8_t* mask = nullptr, float out_scale = 1.0f);
-// umma_kernel.cu -- the same product for many rows: activations streamed through shared memory by bulk copies (launch_lora_down routes
-// there above 256 rows for r <= 16, under a mask where lora_down_streams_masked says so; the CTA-pair kernel runs the same code on idle SM pairs).
+// umma_kernel.cu -- the same product for many rows, in the order of the code that the CTA-pair kernel runs on idle SM pairs, so with its bits: activations
+// streamed through shared memory by bulk copies, under a mask loaded by rows (launch_lora_down routes there above 256 rows for r <= 16, under a mask
+// where lora_down_streams_masked says so).
 int launch_lora_down_stream(int M, int T, int r, bool l_is_A, const void* In, const void* L, float* P, cudaStream_t st, const uint8_t* mask = nullptr,
                             float out_scale = 1.0f);
 bool lora_down_streams_masked(int M, int r);

@@ -9,7 +9,7 @@
 // then the warps' partial tiles are added in warp order through shared memory.  The summation order of a row block
 // depends on nothing but T, so every launch shape gives the same bits.
 // Used (a) by the producer clusters of the CTA-pair kernel and (b) by lora_down_stream_kernel, the stand-alone launch
-// ahead of the tensor-core kernels when they cannot host it.
+// ahead of the tensor-core kernels when they cannot host it (under a mask: lora_down_masked_kernel).
 
 constexpr int LDS_TC = 1024;                              // contraction elements per ring stage
 constexpr int LDS_ROW_BYTES = LDS_TC * 2 + 64;            // padded: rows 16 words apart (mod 32) -> conflict-free 16-byte fragment loads
@@ -31,8 +31,9 @@ __device__ __forceinline__ void bulk_copy_g2s(uint32_t dst, const void* src, uin
 constexpr int LDS_MIN_STAGES = (LDS_CWARPS * LDS_MAXB * 2 * 128 * 4 + LDS_STAGE_BYTES - 1) / LDS_STAGE_BYTES;   // room for the reduction
 
 // Row blocks first_block, first_block + block_stride, ... (at most LDS_MAXB of them below ceil(M / 16)).
-// Called by all threads of the CTA (15 warps or more; the first 15 work); `smem` is 128-byte aligned with room for lds_smem_bytes(stages), stages >=
-// LDS_MIN_STAGES.  Returns with no copy in flight (every issued stage has been waited for) unless the kernel is aborting.
+// Called by all threads of the CTA (15 warps or more; the first 15 work); `smem` is 128-byte aligned and holds `stages` ring stages with LDS_BAR_BYTES behind
+// them; the ring is as large as LDS_MIN_STAGES plain stages at least.  Returns with no copy in flight (every issued stage has been waited for)
+// unless the kernel is aborting.
 // WITH_DB (backward only: In = dY [M, T = N], L = B): the rows that pass through for G = dY B also give this CTA's part of
 //   dB[n, j] = sum_m dY[m, n] H[m, j]   (H fp32 [M, r], the forward's down-projection; the scale s is applied by whoever adds the parts up)
 // as a second product per fragment: the tokens are now the contraction, so the 8 x 8 blocks of the dY fragments are
@@ -253,10 +254,10 @@ __device__ __forceinline__ void lora_down_stream(int M, int T, int r, const __nv
     __syncthreads();
 }
 
-// Under a dropout mask the streaming form is taken from this many tokens on -- wherever the product is formed, so that saved and recomputed H have
+// Under a dropout mask the streaming order is taken from this many tokens on -- wherever the product is formed, so that saved and recomputed H have
 // the same bits.  1800 tokens, 4096 x 4096, INT4, against a launch of lora_down_split_kernel ahead of the layer: dropout forward 58.9 -> 51.5 us
 // (and backward, G beside the tiles, 71.0 -> 58.0).  Below, where the single-CTA kernel mostly runs and cannot host it, the split kernel is
-// the shorter launch.  (Gradients that recompute H: 1100 tokens 29.0 -> 32.2 us, 1800 38.0 -> 36.3, 4096 63.8 -> 59.3.)  Ranks 17 to 32, seven warps per 16 of them, were timed and taken out: beside the tiles X A^T came to 57.9 -> 51.5 us at
+// the shorter launch.  Ranks 17 to 32, seven warps per 16 of them, were timed and taken out: beside the tiles X A^T came to 57.9 -> 51.5 us at
 // rank 32, but as a launch of its own (H recomputed for the gradients, 33 -> 43 us) the form is slower than the split kernel.
 constexpr int LDS_MASKED_TOKENS = 1025;
 static bool lds_masked(int M, int r) { return M >= LDS_MASKED_TOKENS && r <= 16; }
@@ -280,10 +281,7 @@ __global__ void __launch_bounds__(kThreads, 1) lora_down_stream_kernel(const Lds
     __syncthreads();
     pdl_wait();
     const int first = (int)blockIdx.x, stride = (int)gridDim.x;
-    if (L_IS_A && p.mask != nullptr) {
-        if (p.r <= 8) lora_down_stream<true, 1, false, LDS_MAXB, true>(p.M, p.T, p.r, p.In, p.L, p.P, first, stride, smem, p.stages, abort_flag_s, nullptr, nullptr, p.mask, p.out_scale);
-        else          lora_down_stream<true, 2, false, LDS_MAXB, true>(p.M, p.T, p.r, p.In, p.L, p.P, first, stride, smem, p.stages, abort_flag_s, nullptr, nullptr, p.mask, p.out_scale);
-    } else if (p.r <= 8) {
+    if (p.r <= 8) {
         lora_down_stream<L_IS_A, 1>(p.M, p.T, p.r, p.In, p.L, p.P, first, stride, smem, p.stages, abort_flag_s);
     } else {
         lora_down_stream<L_IS_A, 2>(p.M, p.T, p.r, p.In, p.L, p.P, first, stride, smem, p.stages, abort_flag_s);
@@ -294,7 +292,119 @@ __global__ void __launch_bounds__(kThreads, 1) lora_down_stream_kernel(const Lds
     }
 }
 
-// Stand-alone launch (r <= 16): one CTA per SM at most, each with up to LDS_MAXB row blocks.
+// The same product under a mask, as a launch of its own, bit for bit: the 14 partial sums of a row block are those of the ring form's warps, step by
+// step, and are added in their order.  But that form has one CTA of 15 warps per row block or more, which waits for its first rows, for the adapter words
+// of every chunk and for the slowest warp, and leaves SMs idle below 2368 tokens.  Here a warp loads DEPTH steps at a time straight into registers,
+// and a row block's sums are spread as wide as keeps two CTAs of seven warps per SM: over two CTAs, eight rows to each pair of them (ROWS = 8) or
+// sixteen; with more row blocks than SMs over one CTA, two sums to a warp (SUMS = 2).
+// Gradients that recompute H, INT4, rank 8, microseconds -- lora_down_split_kernel (other bits) / the ring form / this: 4096 x 4096, 1100 tokens 15.1 / 19.7 /
+// 15.9, 1800 tokens 23.1 / 25.3 / 23.6, 4096 tokens 39.0 / 46.4 / 39.3; 11008 -> 4096, 2048 tokens 41.3 / 52.9 / 42.2, 8192 tokens 134 / 203 / 142.
+constexpr int LDO_WARPS = LDS_CWARPS / 2;
+
+__device__ __forceinline__ float ld_cluster_f32(uint32_t cluster_addr) {
+    float v;
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(cluster_addr) : "memory");
+    return v;
+}
+
+template <int NT, int SUMS, int ROWS>
+__global__ void __launch_bounds__(LDO_WARPS * 32, 2)
+lora_down_masked_kernel(const LdsParams p) {
+    constexpr int DEPTH = NT == 1 ? 6 : 4, ELEMS = NT * 128, CTAS = 2 / SUMS;
+    __shared__ float red[SUMS * LDO_WARPS * ELEMS];
+    pdl_launch_dependents();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
+    const int rank = (int)blockIdx.x % CTAS, m_base = (int)blockIdx.x / CTAS * ROWS;
+    const int steps = p.T >> 5;                                     // (K is a multiple of 32)
+    const int r0 = m_base + g, r1 = r0 + 8;
+    const bool v0 = r0 < p.M, v1 = ROWS > 8 && r1 < p.M;
+    const size_t at0 = (size_t)r0 * p.T + q * 8, at1 = (size_t)r1 * p.T + q * 8;
+    const __nv_bfloat16* l0 = p.L + (size_t)g * p.T + q * 8;
+    const uint4 zero4 = make_uint4(0, 0, 0, 0);
+    const uint2 zero2 = make_uint2(0, 0);
+    float acc[SUMS][NT][4];
+    int next[SUMS], left[SUMS], skip[SUMS];                         // per sum: its next step; steps left in the chunk; from its last step in a chunk to the next one's first
+#pragma unroll
+    for (int v = 0; v < SUMS; ++v) {
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt) acc[v][nt][0] = acc[v][nt][1] = acc[v][nt][2] = acc[v][nt][3] = 0.f;
+        next[v] = (SUMS == 2 ? v : rank) * LDO_WARPS + warp;        // the ring form's consumer warp: steps w, w + 14, w + 28 of every chunk of 32
+        left[v] = (LDS_TC / 32 - next[v] + LDS_CWARPS - 1) / LDS_CWARPS;
+        skip[v] = LDS_TC / 32 - (left[v] - 1) * LDS_CWARPS;
+    }
+    int per_chunk[SUMS];
+#pragma unroll
+    for (int v = 0; v < SUMS; ++v) per_chunk[v] = left[v];
+    pdl_wait();
+#pragma unroll 1
+    while (next[0] < steps || next[SUMS - 1] < steps) {
+        uint4 xlo[DEPTH], xhi[DEPTH], l[DEPTH][NT];
+        uint2 mlo[DEPTH], mhi[DEPTH];
+        uint32_t in = 0;                                            // bit u: step u exists (warp-uniform)
+#pragma unroll
+        for (int u = 0; u < DEPTH; ++u) {
+            const int v = u % SUMS, k = next[v] * 32;
+            const bool ok = next[v] < steps;
+            if (ok) in |= 1u << u;
+            xlo[u] = v0 && ok ? __ldg(reinterpret_cast<const uint4*>(p.In + at0 + k)) : zero4;
+            xhi[u] = v1 && ok ? __ldg(reinterpret_cast<const uint4*>(p.In + at1 + k)) : zero4;
+            mlo[u] = v0 && ok ? __ldg(reinterpret_cast<const uint2*>(p.mask + at0 + k)) : zero2;
+            mhi[u] = v1 && ok ? __ldg(reinterpret_cast<const uint2*>(p.mask + at1 + k)) : zero2;
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt) l[u][nt] = ok && nt * 8 < p.r ? __ldg(reinterpret_cast<const uint4*>(l0 + (size_t)nt * 8 * p.T + k)) : zero4;
+            const bool last = --left[v] == 0;
+            next[v] += last ? skip[v] : LDS_CWARPS;
+            if (last) left[v] = per_chunk[v];
+        }
+#pragma unroll
+        for (int u = 0; u < DEPTH; ++u) {
+            if (!(in >> u & 1u)) continue;
+            xlo[u] = mask_eight(xlo[u], mlo[u]);
+            xhi[u] = mask_eight(xhi[u], mhi[u]);
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt) {
+                mma_bf16_16816(acc[u % SUMS][nt], xlo[u].x, xhi[u].x, xlo[u].y, xhi[u].y, l[u][nt].x, l[u][nt].y);
+                mma_bf16_16816(acc[u % SUMS][nt], xlo[u].z, xhi[u].z, xlo[u].w, xhi[u].w, l[u][nt].z, l[u][nt].w);
+            }
+        }
+    }
+#pragma unroll
+    for (int v = 0; v < SUMS; ++v)
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) red[(v * LDO_WARPS + warp) * ELEMS + (nt * 4 + c) * 32 + lane] = acc[v][nt][c];
+    __syncwarp();
+    if (CTAS == 2) cluster_sync_all();
+    else __syncthreads();
+    const uint32_t part0 = CTAS == 2 ? map_to_cta(smem_u32(red), 0) : 0u, part1 = CTAS == 2 ? map_to_cta(smem_u32(red), 1) : 0u;
+    for (int e = rank * (ELEMS / CTAS) + (int)threadIdx.x; e < (rank + 1) * (ELEMS / CTAS); e += LDO_WARPS * 32) {
+        float x[LDS_CWARPS], y = 0.f;
+#pragma unroll
+        for (int w = 0; w < LDS_CWARPS; ++w)
+            x[w] = CTAS == 2 ? ld_cluster_f32((w < LDO_WARPS ? part0 : part1) + (uint32_t)((w % LDO_WARPS) * ELEMS + e) * 4u) : red[(w % (SUMS * LDO_WARPS)) * ELEMS + e];
+#pragma unroll
+        for (int w = 0; w < LDS_CWARPS; ++w) y += x[w];
+        const int nt = e >> 7, c = (e >> 5) & 3, ln = e & 31;
+        const int row = m_base + (ln >> 2) + ((c & 2) ? 8 : 0), col = nt * 8 + (ln & 3) * 2 + (c & 1);
+        if (row < p.M && col < p.r && (ROWS > 8 || c < 2)) p.P[(size_t)row * p.r + col] = y * p.out_scale;
+    }
+    if (CTAS == 2) {
+        __syncwarp();
+        cluster_sync_all();                                         // nobody leaves while its peer may still read its parts
+    }
+}
+
+template <int NT>
+cudaError_t launch_lora_down_masked(const LdsParams& p, cudaStream_t st) {
+    const unsigned sms = (unsigned)sm_count(), eights = (unsigned)((p.M + 7) / 8), blocks = (unsigned)((p.M + 15) / 16);
+    const dim3 block(LDO_WARPS * 32);
+    if (eights <= sms) return launch_pdl(lora_down_masked_kernel<NT, 1, 8>, dim3(2 * eights), block, 0, st, 2, p);
+    if (blocks <= sms) return launch_pdl(lora_down_masked_kernel<NT, 1, 16>, dim3(2 * blocks), block, 0, st, 2, p);
+    return launch_pdl(lora_down_masked_kernel<NT, 2, 16>, dim3(blocks), block, 0, st, 1, p);
+}
+
+// Stand-alone launch (r <= 16): one CTA per SM at most, each with up to LDS_MAXB row blocks; under a mask the kernel above.
 int launch_lora_down_stream_impl(int M, int T, int r, bool l_is_A, const void* In, const void* L, float* P, cudaStream_t st, const uint8_t* mask,
                                  float out_scale) {
     if (M == 0 || r == 0) return QLORA_OK;
@@ -302,10 +412,14 @@ int launch_lora_down_stream_impl(int M, int T, int r, bool l_is_A, const void* I
     int grid = n_blocks < sm_count() ? n_blocks : sm_count();
     if ((n_blocks + grid - 1) / grid > LDS_MAXB) grid = (n_blocks + LDS_MAXB - 1) / LDS_MAXB;   // several waves of CTAs
     LdsParams p{};
-    p.M = M; p.T = T; p.r = r; p.stages = mask != nullptr ? 4 : 6; p.wait_limit_us = kWaitLimitUs;
+    p.M = M; p.T = T; p.r = r; p.stages = 6; p.wait_limit_us = kWaitLimitUs;
     p.In = (const __nv_bfloat16*)In; p.L = (const __nv_bfloat16*)L; p.P = P;
     p.mask = mask; p.out_scale = out_scale;
-    constexpr size_t smem_bytes = (6 * LDS_STAGE_BYTES > 4 * LDS_MASKED_STAGE_BYTES ? 6 * LDS_STAGE_BYTES : 4 * LDS_MASKED_STAGE_BYTES) + LDS_BAR_BYTES + 128;
+    if (mask != nullptr) {
+        const cudaError_t err = r <= 8 ? launch_lora_down_masked<1>(p, st) : launch_lora_down_masked<2>(p, st);
+        return err == cudaSuccess ? QLORA_OK : QLORA_ERR_CUDA;
+    }
+    constexpr size_t smem_bytes = 6 * LDS_STAGE_BYTES + LDS_BAR_BYTES + 128;
     static SmemLimit limit_a, limit_b;
     if (!limit_a.raise(lora_down_stream_kernel<true>, smem_bytes) || !limit_b.raise(lora_down_stream_kernel<false>, smem_bytes)) return QLORA_ERR_CUDA;
     const cudaError_t err = l_is_A ? launch_pdl(lora_down_stream_kernel<true>, dim3((unsigned)grid), dim3(kThreads), smem_bytes, st, 1, p)

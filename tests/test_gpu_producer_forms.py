@@ -57,3 +57,24 @@ def test_ranks_17_to_32_many_tokens(M, K, N, r):
         assert rel_err(to_f64(saved[name]), ref[name]) <= REL_TOL, name
     again = gl.run(save_hg=False)
     assert torch.equal(saved["dA"], again["dA"]) and torch.equal(saved["dB"], again["dB"])
+
+
+@pytest.mark.parametrize("M,K,N,r", [(1025, 64, 256, 8), (1184, 96, 64, 16), (1184, 1056, 64, 8), (1185, 2080, 128, 16), (2368, 480, 64, 8), (2369, 512, 64, 16),
+                                     (2400, 1472, 256, 8), (4800, 448, 64, 16)])
+def test_masked_product_as_a_launch_of_its_own(M, K, N, r):
+    """H recomputed for the gradients: eight rows to a pair of CTAs, sixteen, and one CTA to sixteen rows (borders at 1184 and 2368 tokens on 148 SMs);
+    one step of the contraction to a warp and none, a chunk that is not full; the bits of the H that the forward saved."""
+    import paper_2306_08162_b200 as ql
+    layer = qi.random_codes_layer(K=K, N=N, bits=4, group_size=32, r=r, alpha=2.0 * r, M=M, seed=M + K)
+    gl = GpuLayer(layer)
+    mask = torch.from_numpy((np.random.default_rng(M).random((M, K)) >= 0.25).astype(np.uint8)).cuda()
+    Y, H, G = torch.empty_like(gl.dY), torch.empty((M, r), device="cuda"), torch.randn((M, r), device="cuda")
+    ql.qlora_fwd_dropout(gl.desc, M, gl.X, mask, 1 / 0.75, gl.Q, gl.scales, gl.zeros, gl.A, gl.B, Y, H, gl.ws)
+    grads = [(torch.empty((r, K), device="cuda"), torch.empty((N, r), device="cuda")) for _ in range(2)]
+    for h, (dA, dB) in zip((H, None), grads):
+        ql.qlora_bwd_lora_dropout(gl.desc, M, gl.X, mask, 1 / 0.75, gl.dY, gl.A, gl.B, h, G, dA, dB, 0, gl.ws)
+    want = (gl.X.double() * mask / 0.75) @ gl.A.double().t()
+    assert rel_err(to_f64(H), to_f64(want)) < 1e-4                                  # fp32 sums of exact products
+    assert rel_err(to_f64(grads[1][1]), to_f64(gl.desc.alpha / r * gl.dY.double().t() @ want)) < 1e-2     # H once rounded to bf16 (2^-9)
+    assert torch.equal(grads[0][0], grads[1][0]) and torch.equal(grads[0][1], grads[1][1])
+    assert ql.qlora_device_status() == 0
