@@ -78,3 +78,19 @@ def test_masked_product_as_a_launch_of_its_own(M, K, N, r):
     assert rel_err(to_f64(grads[1][1]), to_f64(gl.desc.alpha / r * gl.dY.double().t() @ want)) < 1e-2     # H once rounded to bf16 (2^-9)
     assert torch.equal(grads[0][0], grads[1][0]) and torch.equal(grads[0][1], grads[1][1])
     assert ql.qlora_device_status() == 0
+
+
+@pytest.mark.parametrize("M,r", [(1536, 8), (1400, 16)])
+def test_dropout_with_a_split_last_wave(M, r):
+    """1024 -> 6656: 78 tiles on 74 SM pairs, so the forward's masked producers, their counters and four tiles that two pairs share are one launch."""
+    import paper_2306_08162_b200 as ql
+    test_dropout_beside_the_tiles(M, 1024, 6656, r)
+    layer = qi.random_codes_layer(K=1024, N=6656, bits=4, group_size=64, r=r, alpha=2.0 * r, M=M, seed=M + r)
+    gl = GpuLayer(layer)
+    mask = torch.from_numpy((np.random.default_rng(M).random((M, 1024)) >= 0.25).astype(np.uint8)).cuda()
+    runs = [(torch.empty_like(gl.dY), torch.empty((M, r), device="cuda")) for _ in range(3)]
+    for Y, H in runs:
+        ql.qlora_fwd_dropout(gl.desc, M, gl.X, mask, 1 / 0.75, gl.Q, gl.scales, gl.zeros, gl.A, gl.B, Y, H, gl.ws)
+    for Y, H in runs[1:]:
+        assert torch.equal(Y, runs[0][0]) and torch.equal(H, runs[0][1])
+    assert ql.qlora_device_status() == 0

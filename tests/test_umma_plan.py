@@ -111,3 +111,19 @@ def test_ranks_form_their_part_of_the_down_projection_where_that_pays(plan, bits
     out = (ctypes.c_int * 8)()
     assert plan.tiles(bits, 128, r, M, C, T, tr, 1, out)
     assert (out[2], out[3], out[4]) == (split, steps, down)
+
+
+def test_the_split_tile_tests_run_the_build_they_are_for(plan):
+    from test_gpu_split_tiles import CASES
+    out = (ctypes.c_int * 8)()
+    ranks = set()
+    for bits, g in ((2, 64), (3, 128), (4, 32), (8, 128)):
+        for M, K, N, r in CASES:
+            took = 0
+            for C, T, tr in ((N, K, 0), (K, N, 1)):
+                assert plan.tiles(bits, g if K % g == 0 else 64, r, M, C, T, tr, 1, out)
+                if out[4]:
+                    took += 1
+                    ranks.add((out[2], out[3]))
+            assert took, (bits, M, K, N, r)
+    assert {(4, 2), (2, 4), (4, 16), (4, 14), (4, 32)} <= ranks, ranks
