@@ -54,7 +54,7 @@ int launch_lora_masked_update(int M, int K, int r, float c, const float* G, cons
 // workspace, so calls that may overlap in time have different ones), otherwise by a down-projection launch ahead of it.
 bool umma_supported(const qlora_desc& d, int M);
 // dB = s dY^T H as a by-product of the backward call: the producer clusters of the CTA-pair kernel stream every row of dY
-// to form G, and the same pass gives dB (ranks up to 8).  `part`: workspace for one [N, r] fp32 part per producer CTA.
+// to form G, and the same pass gives dB (ranks up to 16).  `part`: workspace for one [N, r] fp32 part per producer CTA.
 // `done` is set when the launch took it on; otherwise dB is still to be computed by the caller.
 struct DbFuse {
     const float* H;

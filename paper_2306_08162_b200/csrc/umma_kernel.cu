@@ -41,7 +41,7 @@ __device__ unsigned int g_device_status = 0;   // sticky; bit 0: an mbarrier wai
 namespace {
 
 constexpr int kThreads = 480;
-constexpr int kDequantWarp0 = 7, kGroupWarps = 4;   // two dequant groups of four warps
+constexpr int kDequantWarp0 = 7, kGroupWarps = 4;   // two dequant groups of four warps (DOWN: a third in the epilogue's place)
 constexpr int kEpiWarp0 = 3, kEpiWarps = 4;
 constexpr int kSyncWords = 64;                       // counters in the workspace: [0], [1] producer clusters, [2 ..] one per split tile
 constexpr size_t kSplitTileBytes = 2 * 2 * 8 * 8 * 128 * 16;   // exchange area of one split tile: 2 halves x 2 CTAs x 8 chunks x 4 KiB
@@ -55,7 +55,7 @@ struct Params : TilePlan {
     const __nv_bfloat16* L;          // B [N, r] (forward) or A [r, K] (backward)
     __nv_bfloat16* Out;
     // producer clusters (n_prod > 0, as in the CTA-pair kernel): the first n_prod clusters of the grid compute
-    // P = In * Ldown into Pout (== Pmat) beside the tiles and publish it through counter pair `slot`
+    // P = In * Ldown into Pout (== Pmat) beside the tiles and publish it through the counter pair `sync`
     int n_prod, T, lds_stages;
     unsigned int* sync;   // the counter pair (n_prod > 0)
     int wait_limit_us;    // every wait inside the kernel gives up after this long
@@ -289,7 +289,7 @@ __device__ __forceinline__ uint4 lora_up_chunk(const Params& p, int wrow, int jc
     }
 }
 
-// DOWN (split tiles of short contractions, ranks 8 and 16): no producer clusters.  Every rank forms its part of P = In * Ldown beside its
+// DOWN (split tiles of ranks 8 and 16 up to 128 tokens, where down_pays says so): no producer clusters.  Every rank forms its part of P = In * Ldown beside its
 // part of the tile, from the activation stages it has anyway -- four more MMAs per stage, the adapter as their 64-row operand -- and the
 // parts of P meet where the tile's parts do; s P L is added in fp32 there.  So nothing has to be counted in device memory, nor the counters
 // set to zero by a launch ahead, and a tile waits for no other.
@@ -356,7 +356,6 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
     const int step0 = rank * p.steps;
 
     if (!DOWN && first_tile < 0) {
-        if constexpr (!DOWN) {
         // ------------------------------------------------------------------ producer cluster: LoRA down-projection on SMs
         // the tiles leave idle (one CTA per row block or more; lowest block indices, so they wait for nobody)
         const int n_ctas = p.n_prod * p.split;
@@ -391,7 +390,6 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
         __threadfence();       // every thread's rows of P are visible device-wide before the CTA is counted
         __syncthreads();
         if (threadIdx.x == 0) atomicAdd(&p.sync[0], 1u);
-        }
     } else if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer: activation tiles
         pdl_wait();
@@ -505,7 +503,7 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
             const int wt = tile / p.n_tok_tiles, tt = tile % p.n_tok_tiles;
             const int w0 = wt * kWRows, m0 = tt * p.BT;
             const uint32_t buf = tile_it & 1u;
-            if (!DOWN && p.n_prod > 0 && tile_it == 0 && rank == 0) {
+            if (p.n_prod > 0 && tile_it == 0 && rank == 0) {
                 // P is being computed by this launch's producer clusters: one thread waits for all of their CTAs, is counted
                 // as done with the counter, and the last such CTA of the launch zeroes the pair for the next one.
                 if (et == 0 && wait_counter(&p.sync[0], (unsigned)(p.n_prod * p.split), abort_flag)) {
@@ -577,9 +575,9 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
     } else if (warp >= (DOWN ? kEpiWarp0 : kDequantWarp0)) {
         // ------------------------------------------------------------------ unpack + dequant
         // (DOWN: one tile per CTA, so the epilogue's warps would be idle until the end; they are a third group.)
-        constexpr int kGroups = DOWN ? 3 : 2, kWarp0 = DOWN ? kEpiWarp0 : kDequantWarp0;
-        // Two groups of four warps take alternate pipeline stages, so each group has two stage times for its serial chain
-        // (wait, shared-memory loads, arithmetic, wait, stores, fence, arrive).  Inside a group a thread owns one column of
+        constexpr int kGroups = DOWN ? kDownGroups : kDequantGroups, kWarp0 = DOWN ? kEpiWarp0 : kDequantWarp0;
+        // The groups of four warps take the pipeline stages in turn, so each has as many stage times as there are groups for its serial chain
+        // (wait, shared-memory loads, arithmetic, wait, stores, fence, arrive); rings_sound says which ring lengths that allows.  Inside a group a thread owns one column of
         // the packed tile and two blocks of 32 consecutive-k codes.
         const int group = (warp - kWarp0) / kGroupWarps;
         const int gt = threadIdx.x - (kWarp0 + group * kGroupWarps) * 32;   // 0..127 inside the group

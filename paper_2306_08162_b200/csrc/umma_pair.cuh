@@ -54,7 +54,7 @@ struct PairParams {
     int r_down;                  // ranks of that product: r, or (r == 0) those of a product that the tiles do not use and do not wait for
     const uint8_t* mask;         // LoRA dropout, forward: mask on In (uint8 [M, T]), and the scale of the product
     float out_scale;
-    unsigned int* sync;          // the launch's counter pair (n_prod > 0)
+    unsigned int* sync;          // the launch's counters: [0], [1] the tiles wait for P (n_prod > 0, r > 0), [2 ..] split tiles (nsplit > 1); else NULL
     int wait_limit_us;           // every wait inside the kernel gives up after this long
     const __nv_bfloat16* In;     // [M, T]
     const __nv_bfloat16* Ldown;  // A [r, K] (forward) or B [N, r] (backward)

@@ -45,8 +45,8 @@ inline void plan_packed_stage(Plan& p, int bits, int g, bool transposed) {
     p.packed_slot_bytes = (p.words_bytes + 2 * p.scale_bytes + 127u) / 128u * 128u;
 }
 
-// Single-CTA kernel.  Offsets count from the 1024-byte aligned base of shared memory.  (The head of the kernel's parameters: their order
-// is that in which a CTA first reads them.)
+// Single-CTA kernel.  Offsets count from the 1024-byte aligned base of shared memory.  (The head of the kernel's parameters.  With the
+// fields in another order the smallest calls took 1 to 3 % longer: 512 x 512, 17 tokens, rank 8 4.98 -> 5.12 us.)
 struct TilePlan {
     int M, N, K, bits, g, r, r_pad;
     // r_pad: columns of the LoRA operands, a multiple of 16.  lora_lo: ranks [r, 2r) hold, beside the finite ones of the same adapter
