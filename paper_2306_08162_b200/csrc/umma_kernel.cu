@@ -1084,6 +1084,7 @@ static int launch_umma_pair(const qlora_desc& d, int M, bool transposed, const v
     const int grid = 2 * (p.n_tiles < pairs ? p.n_tiles + p.n_prod : pairs);
 #define QLORA_LAUNCH_PAIR(B)                                                                              \
     return transposed ? launch_pair_impl<B, true>(ta, tq, ts, tz, p, smem_bytes, grid, st)                \
+           : p.mask != nullptr && p.n_prod > 0 ? launch_pair_impl<B, false, true>(ta, tq, ts, tz, p, smem_bytes, grid, st) \
                       : launch_pair_impl<B, false>(ta, tq, ts, tz, p, smem_bytes, grid, st)
     switch (d.bits) {
         case 2: QLORA_LAUNCH_PAIR(2);

@@ -151,7 +151,9 @@ __device__ __forceinline__ PairItem pair_item(const PairParams& p, int w, int W,
     return r;
 }
 
-template <int BITS, bool TRANSPOSED>
+// MASKED: LoRA dropout, forward only (a build of its own: with these forms beside the plain ones the producers of a plain forward took some 0.8 us
+// longer, 768 -> 1280, 745 tokens 14.1 -> 14.9 us).
+template <int BITS, bool TRANSPOSED, bool MASKED>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 umma_pair_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_constant__ CUtensorMap tm_q,
                  const __grid_constant__ CUtensorMap tm_scales, const __grid_constant__ CUtensorMap tm_zeros,
@@ -219,25 +221,24 @@ umma_pair_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_consta
         // ------------------------------------------------------------------ producer cluster: LoRA down-projection first
         // (this CTA's row blocks: blockIdx.x, blockIdx.x + 2 n_prod, ...; the ring takes the operand area, below the barriers)
         pdl_wait();
-        bool done_here = false;
-        if constexpr (TRANSPOSED) {
-            if (p.with_db) {       // the same pass over dY also gives this CTA's part of dB
-                done_here = true;            // (the parts are added up by the tile CTAs, see the epilogue)
-                float* part = p.db_part + (size_t)blockIdx.x * p.T * p.r;
-                if (p.r <= 8) lora_down_stream<false, 1, true>(p.M, p.T, p.r, p.In, p.Ldown, p.Pout, (int)blockIdx.x, 2 * p.n_prod, smem_gen, p.lds_stages, abort_flag, p.Hmat, part);
-                else          lora_down_stream<false, 2, true, 3>(p.M, p.T, p.r, p.In, p.Ldown, p.Pout, (int)blockIdx.x, 2 * p.n_prod, smem_gen, p.lds_stages, abort_flag, p.Hmat, part);   // (two rank tiles: registers for three row blocks per CTA only; the host sees to it)
+        const int first = (int)blockIdx.x, stride = 2 * p.n_prod;
+        if constexpr (MASKED) {
+            if (p.r_down <= 8) lora_down_stream<true, 1, false, LDS_MAXB, true>(p.M, p.T, p.r_down, p.In, p.Ldown, p.Pout, first, stride, smem_gen, p.lds_stages, abort_flag, nullptr, nullptr, p.mask, p.out_scale);
+            else               lora_down_stream<true, 2, false, LDS_MAXB, true>(p.M, p.T, p.r_down, p.In, p.Ldown, p.Pout, first, stride, smem_gen, p.lds_stages, abort_flag, nullptr, nullptr, p.mask, p.out_scale);
+        } else {
+            bool db_here = false;                // (the parts are added up by the tile CTAs, see the epilogue)
+            if constexpr (TRANSPOSED) {
+                if (p.with_db) {       // the same pass over dY also gives this CTA's part of dB
+                    db_here = true;
+                    float* part = p.db_part + (size_t)blockIdx.x * p.T * p.r;
+                    if (p.r <= 8) lora_down_stream<false, 1, true>(p.M, p.T, p.r, p.In, p.Ldown, p.Pout, first, stride, smem_gen, p.lds_stages, abort_flag, p.Hmat, part);
+                    else          lora_down_stream<false, 2, true, 3>(p.M, p.T, p.r, p.In, p.Ldown, p.Pout, first, stride, smem_gen, p.lds_stages, abort_flag, p.Hmat, part);   // (two rank tiles: registers for three row blocks per CTA only; the host sees to it)
+                }
             }
-        }
-        if constexpr (!TRANSPOSED) {
-            if (p.mask != nullptr) {
-                done_here = true;
-                if (p.r_down <= 8) lora_down_stream<true, 1, false, LDS_MAXB, true>(p.M, p.T, p.r_down, p.In, p.Ldown, p.Pout, (int)blockIdx.x, 2 * p.n_prod, smem_gen, p.lds_stages, abort_flag, nullptr, nullptr, p.mask, p.out_scale);
-                else               lora_down_stream<true, 2, false, LDS_MAXB, true>(p.M, p.T, p.r_down, p.In, p.Ldown, p.Pout, (int)blockIdx.x, 2 * p.n_prod, smem_gen, p.lds_stages, abort_flag, nullptr, nullptr, p.mask, p.out_scale);
+            if (!db_here) {
+                if (p.r_down <= 8) lora_down_stream<!TRANSPOSED, 1>(p.M, p.T, p.r_down, p.In, p.Ldown, p.Pout, first, stride, smem_gen, p.lds_stages, abort_flag);
+                else               lora_down_stream<!TRANSPOSED, 2>(p.M, p.T, p.r_down, p.In, p.Ldown, p.Pout, first, stride, smem_gen, p.lds_stages, abort_flag);
             }
-        }
-        if (!done_here) {
-            if (p.r_down <= 8) lora_down_stream<!TRANSPOSED, 1>(p.M, p.T, p.r_down, p.In, p.Ldown, p.Pout, (int)blockIdx.x, 2 * p.n_prod, smem_gen, p.lds_stages, abort_flag);
-            else               lora_down_stream<!TRANSPOSED, 2>(p.M, p.T, p.r_down, p.In, p.Ldown, p.Pout, (int)blockIdx.x, 2 * p.n_prod, smem_gen, p.lds_stages, abort_flag);
         }
         __threadfence();       // every thread's rows of P (and of its part of dB) are visible device-wide before the CTA is counted
         __syncthreads();
@@ -647,11 +648,11 @@ done:
     }
 }
 
-template <int BITS, bool TRANSPOSED>
+template <int BITS, bool TRANSPOSED, bool MASKED = false>
 int launch_pair_impl(const CUtensorMap& ta, const CUtensorMap& tq, const CUtensorMap& ts, const CUtensorMap& tz, const PairParams& p,
                      size_t smem_bytes, int grid, cudaStream_t st) {
     static SmemLimit limit;
-    auto kern = umma_pair_kernel<BITS, TRANSPOSED>;
+    auto kern = umma_pair_kernel<BITS, TRANSPOSED, MASKED>;
     if (!limit.raise(kern, 232448 - 1024)) return QLORA_ERR_CUDA;
     return launch_pdl(kern, dim3((unsigned)grid), dim3(kThreads), smem_bytes, st, 1, ta, tq, ts, tz, p) == cudaSuccess
                ? QLORA_OK : QLORA_ERR_CUDA;   // (the cluster width of 2 is a compile-time attribute of the kernel)
