@@ -1034,22 +1034,31 @@ static int launch_umma_pair(const qlora_desc& d, int M, bool transposed, const v
     const bool want_p = (Ldown != nullptr || plan_only) && p.r_down > 0;
     if (plan_only) { sync = reinterpret_cast<unsigned int*>(sizeof(unsigned int)); split_buf = sync; split_bytes = ~(size_t)0; }   // (never dereferenced)
     const int n_blocks = (M + 15) / 16;
+    // Under a mask a producer CTA of several row blocks (48 bytes per row and element instead of 32) has to be through before the first tiles are, or the
+    // launch ahead is the shorter way.  Row blocks per CTA and contraction steps at which both were timed, forward, INT4, rank 8 / 16, beside
+    // the tiles against ahead: 2 at 8 steps -6 / +4 %, 3 at 18 -15 / -11, 5 at 18 -1 / +5, 5 at 24 -12 / -10, 6 at 24 -7 / -3, 7 at 18 +7 / +12, 7 at 32 -10 / -7.
+    auto masked_producers_pay = [&](int n_prod) {
+        return p.mask == nullptr || p.steps >= 4 * ((n_blocks + 2 * n_prod - 1) / (2 * n_prod)) + (p.r_down > 8 ? 2 : 0);
+    };
     auto producers = [&](int last) {
         // pairs with less to do: no tile at all, or one item fewer than the rest when the last wave is partly filled
         const int idle = p.n_tiles < pairs ? pairs - p.n_tiles : (last ? pairs - last : 0);
         int n_prod = (n_blocks + 3) / 4;                     // four row blocks per producer CTA pair when there is room
         if (n_prod > idle) n_prod = idle;
-        const bool fits = want_p && (sync != nullptr || d.r == 0) && r_fits && n_prod > 0 && n_prod * 2 * LDS_MAXB >= n_blocks && ring_fits;
-        return fits ? n_prod : 0;
+        const bool fits = want_p && n_prod > 0 && (sync != nullptr || d.r == 0) && r_fits && n_prod * 2 * LDS_MAXB >= n_blocks && ring_fits;
+        return fits && masked_producers_pay(n_prod) ? n_prod : 0;
     };
     // A partly filled last wave (more tiles than pairs, at most half a wave left over): each left-over tile goes to two
     // pairs, half of the contraction each, which exchange halves of the result through the workspace -- unless that
     // takes away the idle pairs that would otherwise have computed P beside the tiles (8192 tokens on 4096 x 4096: the
-    // down-projection launch it then needs costs what the split wins).
+    // down-projection launch it then needs costs what the split wins).  Under a mask the pairs are worth more to the longer product: a short contraction
+    // is not split (INT4, rank 8, per cent against neither split nor producers, split / whole: 18 steps, 3000 tokens -> 4096 -1 / -16; 24 steps, 3949 ->
+    // 3072 -8 / -15; 32 steps, 2374 -> 4096 -21 / -17).
+    constexpr int kMaskedSplitSteps = 28;
     p.n_full = p.n_tiles; p.nsplit = 1; p.split_buf = nullptr;
     const int rem = pair_split_tiles(p.n_tiles, p.steps, pairs);
     if (rem > 0 && sync != nullptr && split_buf != nullptr && (size_t)rem * kSplitTileBytes <= split_bytes &&
-        !(want_p && producers(2 * rem) == 0 && producers(p.n_tiles % pairs) > 0)) {
+        !(p.mask != nullptr && p.steps < kMaskedSplitSteps) && !(want_p && producers(2 * rem) == 0 && producers(p.n_tiles % pairs) > 0)) {
         p.n_full = p.n_tiles - rem; p.nsplit = 2; p.split_buf = static_cast<float4*>(split_buf);
     }
     if (want_p) p.n_prod = producers(p.nsplit > 1 ? 2 * rem : p.n_tiles % pairs);

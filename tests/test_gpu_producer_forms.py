@@ -94,3 +94,10 @@ def test_dropout_with_a_split_last_wave(M, r):
     for Y, H in runs[1:]:
         assert torch.equal(Y, runs[0][0]) and torch.equal(H, runs[0][1])
     assert ql.qlora_device_status() == 0
+
+
+@pytest.mark.parametrize("M,K,N,r", [(1600, 512, 4096, 8), (2400, 512, 256, 16), (1100, 1152, 8192, 16), (1100, 2048, 8192, 8)])
+def test_dropout_with_short_contractions(M, K, N, r):
+    """Where the masked product is a launch ahead because the tiles are through too soon, and where a left-over tile is kept whole (18 steps) and
+    split (32)."""
+    test_dropout_beside_the_tiles(M, K, N, r)
